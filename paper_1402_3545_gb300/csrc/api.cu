@@ -1989,7 +1989,7 @@ tpmg_status tpmg_nn_create(int cin, const float* params_host, tpmg_nn** out) {
     void** wb[] = {(void**)&b.w1, (void**)&b.w2f, (void**)&b.w2b, (void**)&b.w3f, (void**)&b.w3b, (void**)&b.w4};
     for (void** q : wb)
         if (st == TPMG_OK) st = dalloc(q, 16 * 16 * 27 * 2);
-    if (st == TPMG_OK) st = dalloc((void**)&b.part, sizeof(float) * 1024 * 16 * 16 * 27);
+    if (st == TPMG_OK) st = dalloc((void**)&b.part, sizeof(float) * NN_GRAD_PART);
     if (st == TPMG_OK) st = dalloc((void**)&b.dpart, sizeof(double) * 4096);
     if (st == TPMG_OK) st = dalloc((void**)&b.err, sizeof(int));
     if (st == TPMG_OK && cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess) st = set_err(TPMG_ERR_CUDA, "memset failed");

@@ -10,7 +10,7 @@
 // k_last_roll (16 -> 1). Other shapes use mma.sync kernels: k_conv16z (16 -> 16: tiles of 64 x 2
 // cells, each warp 16 consecutive cells as the M = 16 rows of mma.m16n8k16, K over the 27 taps x 16
 // input channels, operands by ldmatrix), k_first_z / k_first_tc2 and k_last_proj. The weight
-// gradients of the 16 -> 16 layers are tensor-core GEMMs too (cells are the K dimension).
+// gradients are in k_nn_grad.cu.
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -45,27 +45,7 @@ __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uin
 
 static constexpr int TXC = 64, TYC = 2;              // cells per block tile (x, y)
 static constexpr int HX = TXC + 2, HY = TYC + 2;     // halo tile
-static constexpr int HCELLS = HX * HY * 3;           // 3 planes
-static constexpr int HALO_BYTES = HCELLS * 32;       // 16 bf16 per cell
 static constexpr int W_BYTES = 27 * 16 * 16 * 2;
-
-// Loads the 66 x 4 x 3 halo tile of a 16-channel activation around plane k (zero beyond z ends).
-__device__ void load_halo16(const __nv_bfloat16* __restrict__ act, int nx, int ny, int nz, int x0, int y0, int k,
-                            unsigned char* H) {
-    const int tid = threadIdx.x;
-    for (int q = tid; q < HCELLS * 2; q += blockDim.x) {
-        const int v = q >> 1, half = q & 1;
-        const int xx = v % HX, yy = (v / HX) % HY, dz = v / (HX * HY);
-        const int kk = k - 1 + dz;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (kk >= 0 && kk < nz) {
-            const int i = nwrap(x0 - 1 + xx, nx), j = nwrap(y0 - 1 + yy, ny);
-            const size_t p = ((size_t)kk * ny + j) * nx + i;
-            val = __ldg(reinterpret_cast<const uint4*>(act + p * 16) + half);
-        }
-        reinterpret_cast<uint4*>(H)[q] = val;
-    }
-}
 
 // ---------------------------------------------------------------- 16 -> 16, marching in z
 // The same implicit GEMM as k_conv16, but a persistent block stages the weights once and walks
@@ -1486,282 +1466,6 @@ static int last_roll_grid(int nx, int ny) {
     return nb < ntiles ? nb : ntiles;
 }
 
-// partial weight gradient of the first layer: dW1[co][ci][tap] = sum_p d1[p][co] x[p + d(tap)][ci].
-// Thread t < 27 CIN G owns one (ci, tap) for all 16 co over the cells of group t / (27 CIN)
-// (G = 108 / (27 CIN) groups of the 128 tile cells); one partial per block and weight.
-template <int CIN>
-__global__ void __launch_bounds__(128) k_dwfirst_z(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
-                                                   float* __restrict__ partials, int nx, int ny, int nz) {
-    constexpr int NPAIR = 27 * CIN, G = 108 / NPAIR, CPG = TCELLS / G;
-    __shared__ __align__(16) __nv_bfloat16 ring[4 * PLANE_CELLS * CIN];
-    __shared__ __align__(16) __nv_bfloat16 dys[TCELLS * 16];
-    const int tid = threadIdx.x;
-    const bool act = tid < NPAIR * G;
-    const int pair = tid % NPAIR, grp = tid / NPAIR;
-    const int ci = pair % CIN, tap = pair / CIN;
-    const int dz = tap / 9, dyy = (tap / 3) % 3, dxx = tap % 3;
-    float acc[16];
-#pragma unroll
-    for (int co = 0; co < 16; ++co) acc[co] = 0.f;
-    const int tiles_x = nx / TXC, ntiles = tiles_x * (ny / TYC);
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int x0 = (tile % tiles_x) * TXC, y0 = (tile / tiles_x) * TYC;
-        __syncthreads();
-        load_thin<CIN>(x, ring, nx, ny, nz, x0, y0, -1);
-        load_thin<CIN>(x, ring, nx, ny, nz, x0, y0, 0);
-        for (int k = 0; k < nz; ++k) {
-            load_thin<CIN>(x, ring, nx, ny, nz, x0, y0, k + 1);
-            for (int q = tid; q < TCELLS * 2; q += blockDim.x) {
-                const int v = q >> 1, half = q & 1;
-                const size_t p = ((size_t)k * ny + y0 + v / TXC) * nx + x0 + v % TXC;
-                reinterpret_cast<uint4*>(dys)[q] = __ldg(reinterpret_cast<const uint4*>(dy + p * 16) + half);
-            }
-            __syncthreads();
-            if (act) {
-                const __nv_bfloat16* P = ring + ((k + dz) & 3) * (PLANE_CELLS * CIN);
-                for (int cc = grp * CPG; cc < (grp + 1) * CPG; ++cc) {
-                    const int cx = cc % TXC, cy = cc / TXC;
-                    const float xv = __bfloat162float(P[((cy + dyy) * HX + cx + dxx) * CIN + ci]);
-                    const uint4* g = reinterpret_cast<const uint4*>(dys + cc * 16);
-#pragma unroll
-                    for (int hq = 0; hq < 2; ++hq) {
-                        const uint4 gv = g[hq];
-                        const __nv_bfloat162* gb = reinterpret_cast<const __nv_bfloat162*>(&gv);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 f = __bfloat1622float2(gb[e]);
-                            acc[8 * hq + 2 * e] = fmaf(f.x, xv, acc[8 * hq + 2 * e]);
-                            acc[8 * hq + 2 * e + 1] = fmaf(f.y, xv, acc[8 * hq + 2 * e + 1]);
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-    // the groups of one (ci, tap) add up in shared memory, in group order
-    __shared__ float red[108 * 16];
-    if (act)
-#pragma unroll
-        for (int co = 0; co < 16; ++co) red[tid * 16 + co] = acc[co];
-    __syncthreads();
-    if (tid < NPAIR) {
-        float* dst = partials + (size_t)blockIdx.x * (16 * CIN * 27);
-        for (int co = 0; co < 16; ++co) {
-            float sm = 0.f;
-            for (int gq = 0; gq < G; ++gq) sm += red[(gq * NPAIR + tid) * 16 + co];
-            dst[(co * CIN + ci) * 27 + tap] = sm;
-        }
-    }
-}
-
-// partial weight gradient of the last layer: dW4[ci][tap] = sum_p d4[p] a3[p + d(tap)][ci];
-// thread t < 108 owns tap t % 27 for all 16 ci over the cells of group t / 27 (4 groups)
-__global__ void __launch_bounds__(128) k_dwlast_z(const __nv_bfloat16* __restrict__ a3, const float* __restrict__ d4,
-                                                  float* __restrict__ partials, int nx, int ny, int nz) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char* ring = smem;
-    float* ds = reinterpret_cast<float*>(smem + 4 * PLANE_BYTES);
-    const int tid = threadIdx.x;
-    const bool act = tid < 108;
-    const int tap = tid % 27, grp = tid / 27;
-    const int dz = tap / 9, dyy = (tap / 3) % 3, dxx = tap % 3;
-    float acc[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-    const int tiles_x = nx / TXC, ntiles = tiles_x * (ny / TYC);
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int x0 = (tile % tiles_x) * TXC, y0 = (tile / tiles_x) * TYC;
-        __syncthreads();
-        load_wide(a3, ring, nx, ny, nz, x0, y0, -1);
-        load_wide(a3, ring, nx, ny, nz, x0, y0, 0);
-        load_wide(a3, ring, nx, ny, nz, x0, y0, 1);
-        for (int k = 0; k < nz; ++k) {
-            load_wide(a3, ring, nx, ny, nz, x0, y0, k + 2);
-            {
-                const int v = tid;
-                const size_t p = ((size_t)k * ny + y0 + v / TXC) * nx + x0 + v % TXC;
-                ds[v] = __ldg(d4 + p);
-            }
-            cp_wait_nn<1>();
-            __syncthreads();
-            if (act) {
-                const unsigned char* P = ring + ((k + dz) & 3) * PLANE_BYTES;
-                for (int cc = grp * 32; cc < grp * 32 + 32; ++cc) {
-                    const int cx = cc % TXC, cy = cc / TXC;
-                    const float g = ds[cc];
-                    const int cell = (cy + dyy) * HX + cx + dxx;
-#pragma unroll
-                    for (int hq = 0; hq < 2; ++hq) {
-                        const uint4 av = *reinterpret_cast<const uint4*>(P + swz(cell, hq));
-                        const __nv_bfloat162* ab = reinterpret_cast<const __nv_bfloat162*>(&av);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 f = __bfloat1622float2(ab[e]);
-                            acc[8 * hq + 2 * e] = fmaf(g, f.x, acc[8 * hq + 2 * e]);
-                            acc[8 * hq + 2 * e + 1] = fmaf(g, f.y, acc[8 * hq + 2 * e + 1]);
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        cp_wait_nn<0>();
-    }
-    float* red = reinterpret_cast<float*>(smem);  // the ring is no longer read
-    __syncthreads();
-    if (act)
-#pragma unroll
-        for (int c = 0; c < 16; ++c) red[tid * 16 + c] = acc[c];
-    __syncthreads();
-    if (tid < 27) {
-        float* dst = partials + (size_t)blockIdx.x * (16 * 27);
-        for (int c = 0; c < 16; ++c) {
-            const float sm = (red[tid * 16 + c] + red[(27 + tid) * 16 + c]) + (red[(54 + tid) * 16 + c] + red[(81 + tid) * 16 + c]);
-            dst[c * 27 + tid] = sm;
-        }
-    }
-}
-
-// ---------------------------------------------------------------- backward of the last layer
-// d3[ci](p) = mask(a3) * sum_d W4[ci][d] d4(p - d): the transposed 16 <- 1 convolution
-__global__ void __launch_bounds__(256) k_bwd_last(const float* __restrict__ d4, const __nv_bfloat16* __restrict__ W,
-                                                  const __nv_bfloat16* __restrict__ a3, __nv_bfloat16* __restrict__ d3,
-                                                  int nx, int ny, int nz) {
-    __shared__ float w[16 * 27];
-    for (int q = threadIdx.x; q < 16 * 27; q += blockDim.x) w[q] = __bfloat162float(W[q]);
-    __syncthreads();
-    const size_t n = (size_t)nx * ny * nz;
-    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int i = (int)(p % nx), j = (int)((p / nx) % ny), k = (int)(p / ((size_t)nx * ny));
-    float acc[16];
-#pragma unroll
-    for (int ci = 0; ci < 16; ++ci) acc[ci] = 0.f;
-    for (int dz = -1; dz <= 1; ++dz) {
-        const int kk = k - dz;
-        if (kk < 0 || kk >= nz) continue;
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int tap = ((dz + 1) * 3 + dy + 1) * 3 + dx + 1;
-                const float g = __ldg(d4 + ((size_t)kk * ny + nwrap(j - dy, ny)) * nx + nwrap(i - dx, nx));
-#pragma unroll
-                for (int ci = 0; ci < 16; ++ci) acc[ci] = fmaf(w[ci * 27 + tap], g, acc[ci]);
-            }
-    }
-    __align__(16) __nv_bfloat16 m[16], o[16];
-    reinterpret_cast<uint4*>(m)[0] = __ldg(reinterpret_cast<const uint4*>(a3 + p * 16));
-    reinterpret_cast<uint4*>(m)[1] = __ldg(reinterpret_cast<const uint4*>(a3 + p * 16) + 1);
-#pragma unroll
-    for (int ci = 0; ci < 16; ++ci) o[ci] = __float2bfloat16_rn(__bfloat162float(m[ci]) > 0.f ? acc[ci] : 0.f);
-    reinterpret_cast<uint4*>(d3 + p * 16)[0] = reinterpret_cast<uint4*>(o)[0];
-    reinterpret_cast<uint4*>(d3 + p * 16)[1] = reinterpret_cast<uint4*>(o)[1];
-}
-
-// ---------------------------------------------------------------- weight gradient, 16 -> 16 layers
-// dW[co][ci][tap] = sum_p dy[co](p) x[ci](p + d): per tap a GEMM (16 co) x (cells) x (16 ci) on the
-// tensor cores; warp w accumulates the taps w, w+8, w+16, w+24 over the block's tiles, then writes
-// one partial sum per (block, tap, co, ci).
-__global__ void __launch_bounds__(256) k_dw16(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
-                                              float* __restrict__ partials, int nx, int ny, int nz) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char* H = smem;
-    unsigned char* D = smem + HALO_BYTES;  // 128 cells x 16 channels of dy
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float acc[4][2][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-    const int tiles_x = nx / TXC, tiles_y = ny / TYC;
-    const long ntiles = (long)tiles_x * tiles_y * nz;
-    const int q8 = lane >> 3, rr = lane & 7;
-    for (long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int tx = (int)(t % tiles_x), ty = (int)((t / tiles_x) % tiles_y), k = (int)(t / ((long)tiles_x * tiles_y));
-        const int x0 = tx * TXC, y0 = ty * TYC;
-        __syncthreads();
-        load_halo16(x, nx, ny, nz, x0, y0, k, H);
-        for (int q = threadIdx.x; q < TXC * TYC * 2; q += blockDim.x) {
-            const int v = q >> 1, half = q & 1;
-            const int xx = v % TXC, yy = v / TXC;
-            const size_t p = ((size_t)k * ny + y0 + yy) * nx + x0 + xx;
-            reinterpret_cast<uint4*>(D)[q] = __ldg(reinterpret_cast<const uint4*>(dy + p * 16) + half);
-        }
-        __syncthreads();
-        // 8 chunks of 16 cells: (row, 16-cell column block)
-#pragma unroll 1
-        for (int ch = 0; ch < 8; ++ch) {
-            const int yw = ch >> 2, xc = (ch & 3) * 16;
-            // A = dy^T (co x cells): stored [cell][co] -> transposed load
-            uint32_t a0, a1, a2, a3;
-            {
-                const int cellrow = (q8 >> 1) * 8 + rr, coff = (q8 & 1) * 8;
-                ldm_x4_t(saddr(D + ((yw * TXC + xc + cellrow) * 16 + coff) * 2), a0, a1, a2, a3);
-            }
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const int tap = warp + 8 * s;
-                if (tap >= 27) break;
-                const int dz = tap / 9, dyy = (tap / 3) % 3, dxx = tap % 3;
-                // B = shifted x (cells x ci): stored [cell][ci] -> transposed load
-                const int cellrow = (q8 & 1) * 8 + rr, cioff = (q8 >> 1) * 8;
-                const int cell = (dz * HY + yw + dyy) * HX + xc + cellrow + dxx;
-                uint32_t b0, b1, b2, b3;
-                ldm_x4_t(saddr(H + (cell * 16 + cioff) * 2), b0, b1, b2, b3);
-                mma16816(acc[s][0], a0, a1, a2, a3, b0, b1);
-                mma16816(acc[s][1], a0, a1, a2, a3, b2, b3);
-            }
-        }
-    }
-    const int g = lane >> 2, t2 = (lane & 3) * 2;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int tap = warp + 8 * s;
-        if (tap >= 27) break;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int co = g + 8 * h, ci = t2 + 8 * nt;
-                float* dst = partials + (size_t)blockIdx.x * (16 * 16 * 27);
-                dst[(co * 16 + ci) * 27 + tap] = acc[s][nt][2 * h];
-                dst[(co * 16 + ci + 1) * 27 + tap] = acc[s][nt][2 * h + 1];
-            }
-    }
-}
-
-// per-channel sums of dy (bias gradients): one partial per (block, channel)
-template <int C, bool F32>
-__global__ void k_chansum(const void* __restrict__ dyv, float* __restrict__ partials, size_t n, size_t cells_per_block) {
-    __shared__ float red[256];
-    const size_t p0 = blockIdx.x * cells_per_block, p1 = p0 + cells_per_block < n ? p0 + cells_per_block : n;
-    for (int c = 0; c < C; ++c) {
-        float s = 0.f;
-        for (size_t p = p0 + threadIdx.x; p < p1; p += blockDim.x)
-            s += F32 ? __ldg(reinterpret_cast<const float*>(dyv) + p)
-                     : __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(dyv)[p * C + c]);
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-            if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partials[(size_t)blockIdx.x * C + c] = red[0];
-        __syncthreads();
-    }
-}
-
-// out[e] = sum over blocks b of partials[b * nelem + e] (fixed order)
-__global__ void k_reduce_partials(const float* __restrict__ partials, int nblocks, int nelem, float* __restrict__ out) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nelem) return;
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * nelem + e];
-    out[e] = (float)s;
-}
-
 // ---------------------------------------------------------------- parameters
 // master fp32 params (flat, W[co][ci][tap] per layer) -> bf16 weights: W1, W4 as stored; W2, W3 as
 // [tap][co][ci] for the forward GEMM and [tap'][ci][co] with tap' the mirrored tap for the data
@@ -1928,55 +1632,24 @@ void nn_forward(const NNBufs& b, int nx, int ny, int nz, const __nv_bfloat16* x,
     note_launch();
 }
 
-int nn_grad_blocks(size_t n) {
-    size_t b = (n + 4095) / 4096;
-    return (int)(b < 1024 ? (b < 1 ? 1 : b) : 1024);
-}
-
 void nn_backward(const NNBufs& b, int nx, int ny, int nz, const __nv_bfloat16* x, const float* d4, float* grad,
                  cudaStream_t s) {
-    const size_t n = (size_t)nx * ny * nz;
-    const int cin = b.cin;
-    const int n1 = 16 * cin * 27, n2 = 16 * 16 * 27, n4 = 16 * 27;
-    float* gW1 = grad;
-    float* gb1 = gW1 + n1;
-    float* gW2 = gb1 + 16;
-    float* gb2 = gW2 + n2;
-    float* gW3 = gb2 + 16;
-    float* gb3 = gW3 + n2;
-    float* gW4 = gb3 + 16;
-    float* gb4 = gW4 + n4;
-    const int nb = nn_grad_blocks(n);
-    const size_t cpb = (n + nb - 1) / nb;
-    const int nbt = thin_grid(nx, ny, 1024);  // partial sums of the thin weight gradients
+    const int n1 = 16 * b.cin * 27, n2 = 16 * 16 * 27;
+    float* gW1 = grad;  // each layer's biases follow its weights
+    float* gW2 = gW1 + n1 + 16;
+    float* gW3 = gW2 + n2 + 16;
+    float* gW4 = gW3 + n2 + 16;
     // layer 4: dW4, db4 and d3 = mask(a3) * W4^T d4
-    k_dwlast_z<<<nbt, 128, 4 * PLANE_BYTES + TCELLS * 4, s>>>(b.a3, d4, b.part, nx, ny, nz);
-    k_reduce_partials<<<(n4 + 255) / 256, 256, 0, s>>>(b.part, nbt, n4, gW4);
-    k_chansum<1, true><<<nb, 256, 0, s>>>(d4, b.part, n, cpb);
-    k_reduce_partials<<<1, 256, 0, s>>>(b.part, nb, 1, gb4);
-    k_bwd_last<<<blocks_for(n), 256, 0, s>>>(d4, b.w4, b.a3, b.d1, nx, ny, nz);
-    for (int q = 0; q < 5; ++q) note_launch();
-    const size_t smem_dw = HALO_BYTES + TXC * TYC * 32;
-    cudaFuncSetAttribute(k_dw16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_dw);
-    // layer 3: dW3 from (a2, d3); d2 = mask(a2) * conv(d3, W3 flipped)
-    k_dw16<<<nb, 256, smem_dw, s>>>(b.a2, b.d1, b.part, nx, ny, nz);
-    k_reduce_partials<<<(n2 + 255) / 256, 256, 0, s>>>(b.part, nb, n2, gW3);
-    k_chansum<16, false><<<nb, 256, 0, s>>>(b.d1, b.part, n, cpb);
-    k_reduce_partials<<<1, 256, 0, s>>>(b.part, nb, 16, gb3);
+    nn_dw_last(b.a3, d4, b.part, gW4, nx, ny, nz, s);
+    nn_bwd_last(d4, b.w4, b.a3, b.d1, nx, ny, nz, s);
+    // layer 3: dW3, db3 from (a2, d3); d2 = mask(a2) * conv(d3, W3 flipped)
+    nn_dw16(b.a2, b.d1, b.part, gW3, nx, ny, nz, s);
     conv16<EPI_MASK>(b, b.d1, b.w3b, nullptr, b.a2, b.d2, nx, ny, nz, s);
-    // layer 2: dW2 from (a1, d2); d1 = mask(a1) * conv(d2, W2 flipped)
-    k_dw16<<<nb, 256, smem_dw, s>>>(b.a1, b.d2, b.part, nx, ny, nz);
-    k_reduce_partials<<<(n2 + 255) / 256, 256, 0, s>>>(b.part, nb, n2, gW2);
-    k_chansum<16, false><<<nb, 256, 0, s>>>(b.d2, b.part, n, cpb);
-    k_reduce_partials<<<1, 256, 0, s>>>(b.part, nb, 16, gb2);
+    // layer 2: dW2, db2 from (a1, d2); d1 = mask(a1) * conv(d2, W2 flipped)
+    nn_dw16(b.a1, b.d2, b.part, gW2, nx, ny, nz, s);
     conv16<EPI_MASK>(b, b.d2, b.w2b, nullptr, b.a1, b.d1, nx, ny, nz, s);
-    // layer 1: dW1 from (x, d1)
-    if (cin == 1) k_dwfirst_z<1><<<nbt, 128, 0, s>>>(x, b.d1, b.part, nx, ny, nz);
-    else k_dwfirst_z<2><<<nbt, 128, 0, s>>>(x, b.d1, b.part, nx, ny, nz);
-    k_reduce_partials<<<(n1 + 255) / 256, 256, 0, s>>>(b.part, nbt, n1, gW1);
-    k_chansum<16, false><<<nb, 256, 0, s>>>(b.d1, b.part, n, cpb);
-    k_reduce_partials<<<1, 256, 0, s>>>(b.part, nb, 16, gb1);
-    for (int q = 0; q < 12; ++q) note_launch();
+    // layer 1: dW1, db1 from (x, d1)
+    nn_dw_first(b.cin, x, b.d1, b.part, gW1, nx, ny, nz, s);
 }
 
 void nn_mse(const float* out, const float* target, float* d4, double* partials, size_t n, int nblocks, cudaStream_t s) {

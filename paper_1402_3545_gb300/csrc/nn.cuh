@@ -36,7 +36,19 @@ void nn_forward(const NNBufs& b, int nx, int ny, int nz, const __nv_bfloat16* x,
 // gradient of the loss w.r.t. all parameters into grad, given d4 = dLoss/dout (forward done before)
 void nn_backward(const NNBufs& b, int nx, int ny, int nz, const __nv_bfloat16* x, const float* d4, float* grad,
                  cudaStream_t s);
-int nn_grad_blocks(size_t n);
+// parameter gradients (k_nn_grad.cu): each writes its layer's weights and, behind them, biases to grad;
+// part holds NN_GRAD_MAX_BLOCKS partial gradients of a 16 -> 16 layer (weights and biases)
+static constexpr int NN_GRAD_MAX_BLOCKS = 1024;
+static constexpr size_t NN_GRAD_PART = (size_t)NN_GRAD_MAX_BLOCKS * (16 * 16 * 27 + 16);
+void nn_dw16(const __nv_bfloat16* x, const __nv_bfloat16* dy, float* part, float* grad, int nx, int ny, int nz,
+             cudaStream_t s);
+void nn_dw_first(int cin, const __nv_bfloat16* x, const __nv_bfloat16* d1, float* part, float* grad, int nx, int ny,
+                 int nz, cudaStream_t s);
+void nn_dw_last(const __nv_bfloat16* a3, const float* d4, float* part, float* grad, int nx, int ny, int nz,
+                cudaStream_t s);
+// d3 = mask(a3) * W4^T d4, the data gradient of the last layer
+void nn_bwd_last(const float* d4, const __nv_bfloat16* w4, const __nv_bfloat16* a3, __nv_bfloat16* d3, int nx, int ny,
+                 int nz, cudaStream_t s);
 void nn_mse(const float* out, const float* target, float* d4, double* partials, size_t n, int nblocks, cudaStream_t s);
 // residual loss: e = x[channel 0] - q (q = A NN(x)), tmp = -2 e / n, partial sums of e^2 / n
 void nn_res_loss(const __nv_bfloat16* x, int cin, const float* q, float* tmp, double* partials, size_t n, int nblocks,
