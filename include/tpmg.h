@@ -270,7 +270,7 @@ tpmg_status tpmg_measure_alu_rate(int which, int reps, double* ops_per_s, double
  * one-row tiles run as overlapping forward/backward stages; two-row tiles; one-row tiles with a
  * shallower ring). A level that was never tuned or set takes, in FP32, variant 8 where the level
  * fits one tile per resident warp (nx % 128 == 0), else 5; double-word takes 6 where nx % 64 == 0;
- * otherwise variant 3 (native FP64: variant 0). Variants 8-11 in other precisions run the default.
+ * otherwise (and in native FP64) variant 3. Variants 8-11 in other precisions run the default.
  * tpmg_autotune times each of them `reps` times on every level of precision `prec` (on the
  * operator's workspace, CUDA events on `stream`) and keeps the fastest per level; if variants_out
  * is not NULL it receives the choice of level l in variants_out[l] (host array of L+1 ints).

@@ -91,6 +91,7 @@ void launch_factor_k0(const Lv<P>& L, const typename P::S* finv, const typename 
 // ---------------------------------------------------------------- generic pipelined sweep
 
 // MODE_SMOOTH:    out = u + coef M^{-1}(f - A u), partial sums of ||f - A u||^2      (Eq. 11)
+// MODE_SMOOTHB:   the same as (1 - coef) u + coef M^{-1}(f + H u), without the sums (sweep_rhs)
 // MODE_RESIDUAL:  out = f - A u (stored in PO's precision), partial sums of ||f - A u||^2
 // MODE_LINESOLVE: out = coef M^{-1} u (u is the right-hand side; f unused)            (Eq. 9)
 //
@@ -206,6 +207,11 @@ __global__ void __launch_bounds__(32 * TY) k_sweep_pp(Lv<P> L, SweepK<P> K, cons
                 cp_wait<PD - 2>();  // planes k and k+1 (the upper neighbour) have landed
                 __syncthreads();    // ... including the halo values other threads fetched
                 const S* Us = ringU + slot * UPL;
+                if constexpr (MODE == MODE_SMOOTHB) {
+                    r = sweep_rhs<P>(P::ld_plain(ringF, slot * FPL + tid), P::ld_plain(Us, ctr - 1),
+                                     P::ld_plain(Us, ctr + 1), P::ld_plain(Us, ctr - 34), P::ld_plain(Us, ctr + 34), cx,
+                                     cy, iso);
+                } else {
                 if (k == 0) uc = P::ld_plain(Us, ctr);
                 const R up = (k + 1 < nz) ? P::ld_plain(ringU + nslot * UPL, ctr) : vzero;
                 const R diag = (nz == 1) ? dh : ((k == 0 || k == nz - 1) ? dh1 : dh2);
@@ -215,6 +221,7 @@ __global__ void __launch_bounds__(32 * TY) k_sweep_pp(Lv<P> L, SweepK<P> K, cons
                 if (want_norm) P::acc_dot(acc, cmp, r, r);
                 um = uc;
                 uc = up;
+                }
             } else {
                 cp_wait<PD - 1>();  // only this thread's own copies are read: no barrier needed
                 r = P::ld_plain(ringF, slot * FPL + tid);
@@ -251,7 +258,7 @@ __global__ void __launch_bounds__(32 * TY) k_sweep_pp(Lv<P> L, SweepK<P> K, cons
             __syncthreads();  // the backward ring reuses the forward ring's shared memory
             // back substitution, streaming v/m_k, (GS) the stacked values and (Smooth, unless
             // GFORM) u_k through the ring in reverse order; every thread reads only its own copies
-            constexpr bool NEED_U = MODE == MODE_SMOOTH && !GFORM;
+            constexpr bool NEED_U = (MODE == MODE_SMOOTH && !GFORM) || MODE == MODE_SMOOTHB;
             S* bW = reinterpret_cast<S*>(smem_raw);
             S* bD = bW + PD * NT;
             S* bU = bD + PD * NT;
@@ -275,6 +282,9 @@ __global__ void __launch_bounds__(32 * TY) k_sweep_pp(Lv<P> L, SweepK<P> K, cons
                 const size_t id = (size_t)k * pl + c;
                 if constexpr (GFORM)
                     P::st(reinterpret_cast<S*>(out), id, xn);
+                else if constexpr (MODE == MODE_SMOOTHB)
+                    P::st(reinterpret_cast<S*>(out), id,
+                          P::fma(cf, xn, P::mul_u(K.rest, P::ld_plain(bU, slot * NT + tid))));
                 else if constexpr (MODE == MODE_SMOOTH)
                     P::st(reinterpret_cast<S*>(out), id, P::fma(cf, xn, P::ld_plain(bU, slot * NT + tid)));
                 else
@@ -285,7 +295,7 @@ __global__ void __launch_bounds__(32 * TY) k_sweep_pp(Lv<P> L, SweepK<P> K, cons
             cp_wait<0>();
         }
     }
-    if (MODE != MODE_LINESOLVE && partials) {
+    if (MODE != MODE_LINESOLVE && MODE != MODE_SMOOTHB && partials) {
         double sm = block_sum(P::acc_get(acc, cmp));
         if (tid == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = sm;
     }
@@ -457,8 +467,8 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
 // (0-2), two persistent ones with the stack in global scratch (3, 4), and three persistent ones with
 // two columns per thread and L2 eviction hints (k_sweep_x2; 5-7); the autotuner (tpmg_autotune)
 // times them per level and stores its choice in Lv::variant. An untuned level takes variant 6
-// (double-word) or 5 (FP32) where the two-column form applies (nx % 64 == 0, aligned fields), else
-// variant 3; in native FP64, variant 0.
+// (double-word) or 8, 5 (FP32) where the two- or four-column form applies (nx % 64 or 128 == 0, aligned
+// fields), else variant 3; in native FP64, variant 3.
 template <class P>
 struct SmoothVariants;
 template <>
@@ -474,7 +484,7 @@ struct SmoothVariants<PolDW> {
     static constexpr int TY[3] = {1, 2, 2};
 };
 
-template <class P>
+template <class P, int MODE>
 static int smooth_dispatch(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                            typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
     int v = L.variant;
@@ -486,38 +496,41 @@ static int smooth_dispatch(const Lv<P>& L, double rho, const typename P::S* u, c
     }
     if (v < 0 || v >= TPMG_NUM_VARIANTS || v >= 8) {
         v = 0;
-        if (L.gstack && P::id != 0) {  // native FP64 is bound by its slow pipe: one column per thread
+        // native FP64 is bound by its slow pipe: one column per thread, many warps (512^2 x 128: 597 us, the
+        // two-column form 597-631, the shared-memory stack, six warps per SM, 748)
+        if (L.gstack && P::id == 0) v = 3;
+        if (L.gstack && P::id != 0) {
             const int nb = P::id == 1
-                               ? run_sweep_x2<P, P, 2, 4, MODE_SMOOTH, 1, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 8)
-                               : run_sweep_x2<P, P, 2, 4, MODE_SMOOTH, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
+                               ? run_sweep_x2<P, P, 2, 4, MODE, 1, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 8)
+                               : run_sweep_x2<P, P, 2, 4, MODE, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
             if (nb >= 0) return nb;
             v = 3;
         }
     }
     if (v >= 5 && L.gstack) {
         int nb = -1;
-        if (v == 5) nb = run_sweep_x2<P, P, 2, 4, MODE_SMOOTH, 1, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 8);
-        if (v == 6) nb = run_sweep_x2<P, P, 2, 4, MODE_SMOOTH, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
-        if (v == 7) nb = run_sweep_x2<P, P, 2, 6, MODE_SMOOTH, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
+        if (v == 5) nb = run_sweep_x2<P, P, 2, 4, MODE, 1, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 8);
+        if (v == 6) nb = run_sweep_x2<P, P, 2, 4, MODE, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
+        if (v == 7) nb = run_sweep_x2<P, P, 2, 6, MODE, 10, HINT_ALL>(L, rho, u, f, uo, partials, done, s, 12);
         if (nb >= 0) return nb;
     }
     if (P::id == 1) {  // FP32
-        if (v == 0 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 8, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
-        if (v == 1 && pp_fits<P, 4>(L)) return run_sweep_pp<P, P, 4, 6, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
-        if (v == 2 && pp_fits<P, 1>(L)) return run_sweep_pp<P, P, 1, 8, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
+        if (v == 0 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 8, MODE>(L, rho, u, f, uo, partials, done, s);
+        if (v == 1 && pp_fits<P, 4>(L)) return run_sweep_pp<P, P, 4, 6, MODE>(L, rho, u, f, uo, partials, done, s);
+        if (v == 2 && pp_fits<P, 1>(L)) return run_sweep_pp<P, P, 1, 8, MODE>(L, rho, u, f, uo, partials, done, s);
         if (L.gstack && v == 3 && pp_fits<P, 2>(L))
-            return run_sweep_pp<P, P, 2, 8, MODE_SMOOTH, true>(L, rho, u, f, uo, partials, done, s, 8);
+            return run_sweep_pp<P, P, 2, 8, MODE, true>(L, rho, u, f, uo, partials, done, s, 8);
         if (L.gstack && v == 4 && pp_fits<P, 2>(L))
-            return run_sweep_pp<P, P, 2, 8, MODE_SMOOTH, true>(L, rho, u, f, uo, partials, done, s, 16);
-        if (pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 8, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
+            return run_sweep_pp<P, P, 2, 8, MODE, true>(L, rho, u, f, uo, partials, done, s, 16);
+        if (pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 8, MODE>(L, rho, u, f, uo, partials, done, s);
     } else {  // 8-byte values
-        if (v == 1 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 4, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
-        if (v == 2 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 6, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
+        if (v == 1 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 4, MODE>(L, rho, u, f, uo, partials, done, s);
+        if (v == 2 && pp_fits<P, 2>(L)) return run_sweep_pp<P, P, 2, 6, MODE>(L, rho, u, f, uo, partials, done, s);
         if (L.gstack && v == 3 && pp_fits<P, 2>(L))
-            return run_sweep_pp<P, P, 2, 4, MODE_SMOOTH, true>(L, rho, u, f, uo, partials, done, s, 8);
+            return run_sweep_pp<P, P, 2, 4, MODE, true>(L, rho, u, f, uo, partials, done, s, 8);
         if (L.gstack && v == 4 && pp_fits<P, 2>(L))
-            return run_sweep_pp<P, P, 2, 4, MODE_SMOOTH, true>(L, rho, u, f, uo, partials, done, s, 16);
-        if (pp_fits<P, 1>(L)) return run_sweep_pp<P, P, 1, 6, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
+            return run_sweep_pp<P, P, 2, 4, MODE, true>(L, rho, u, f, uo, partials, done, s, 16);
+        if (pp_fits<P, 1>(L)) return run_sweep_pp<P, P, 1, 6, MODE>(L, rho, u, f, uo, partials, done, s);
     }
     return -1;
 }
@@ -526,7 +539,11 @@ template <class P>
 int launch_smooth_pp(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                      typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
     if (L.nz * 32 * 8 > 160 * 1024) return -1;  // stack too deep for shared memory
-    return smooth_dispatch<P>(L, rho, u, f, uo, partials, done, s);
+    // without a norm to give, the FP64-accurate policies take the form that needs no residual (12 -> 9
+    // arithmetic operations per cell); FP32 keeps one form, so that its results do not depend on the norm
+    if constexpr (P::id != 1)
+        if (!partials) return smooth_dispatch<P, MODE_SMOOTHB>(L, rho, u, f, uo, partials, done, s);
+    return smooth_dispatch<P, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
 }
 
 template <class P, class PO>

@@ -32,10 +32,14 @@ __device__ __forceinline__ void cp_wait() {
 }
 
 // MODE_APPLY: out = A u (f unused), formed as -(0 - A u) by the residual's stencil: negation is exact
-enum { MODE_SMOOTH = 0, MODE_RESIDUAL = 1, MODE_LINESOLVE = 2, MODE_RESTRICT = 3, MODE_APPLY = 4 };
+// MODE_SMOOTHB: the smoothing step in the form (1 - rho) u + rho M^{-1}(f + H u) (sweep_rhs), which
+// has no residual norm to give
+enum { MODE_SMOOTH = 0, MODE_RESIDUAL = 1, MODE_LINESOLVE = 2, MODE_RESTRICT = 3, MODE_APPLY = 4, MODE_SMOOTHB = 5 };
 // modes whose per-column Thomas stack lives in the block's scratch slot (MODE_RESTRICT keeps the
 // stack of the coarse column there)
-__host__ __device__ constexpr bool x2_stack(int mode) { return mode == MODE_SMOOTH || mode == MODE_LINESOLVE; }
+__host__ __device__ constexpr bool x2_stack(int mode) {
+    return mode == MODE_SMOOTH || mode == MODE_SMOOTHB || mode == MODE_LINESOLVE;
+}
 __host__ __device__ constexpr bool x2_slot(int mode) { return mode != MODE_RESIDUAL && mode != MODE_APPLY; }
 
 // MODE_RESTRICT: the fine level's residual r = f - A u is not stored; each 2 x 2 group of fine
@@ -218,6 +222,14 @@ __device__ __forceinline__ double sweep_x2_tiles(const Lv<P>& L, const SweepK<P>
                 cp_wait<PD - 2>();  // planes k and k+1 have landed
                 __syncthreads();    // ... including the halo values other threads fetched
                 const S* Us = ringU + slot * UPL;
+                if constexpr (MODE == MODE_SMOOTHB) {
+                    const R s0 = P::ld_plain(Us, ctr - UW), s1 = P::ld_plain(Us, ctr - UW + 1);
+                    const R n0 = P::ld_plain(Us, ctr + UW), n1 = P::ld_plain(Us, ctr + UW + 1);
+                    r0 = sweep_rhs<P>(P::ld_plain(ringF, slot * FPL + 2 * tid), P::ld_plain(Us, ctr - 1),
+                                      P::ld_plain(Us, ctr + 1), s0, n0, cx, cy, iso);
+                    r1 = sweep_rhs<P>(P::ld_plain(ringF, slot * FPL + 2 * tid + 1), P::ld_plain(Us, ctr),
+                                      P::ld_plain(Us, ctr + 2), s1, n1, cx, cy, iso);
+                } else {
                 if (k == 0) {
                     uc0 = P::ld_plain(Us, ctr);
                     uc1 = P::ld_plain(Us, ctr + 1);
@@ -249,6 +261,7 @@ __device__ __forceinline__ double sweep_x2_tiles(const Lv<P>& L, const SweepK<P>
                 if constexpr (RESTR) {
                     qv = P::add(r0, r1);  // the row pair's sum; the odd row hands it over
                     if (!even) P::st(xs, (k & 1) * 32 * CR + ci, qv);
+                }
                 }
             }
             if constexpr (MODE == MODE_APPLY) {
@@ -323,7 +336,7 @@ __device__ __forceinline__ double sweep_x2_tiles(const Lv<P>& L, const SweepK<P>
 
         if constexpr (STACK) {
             // back substitution from the stacked values and v/m_k (and u_k unless GFORM)
-            constexpr bool NEED_U = MODE == MODE_SMOOTH && !GFORM;
+            constexpr bool NEED_U = (MODE == MODE_SMOOTH && !GFORM) || MODE == MODE_SMOOTHB;
             __syncthreads();  // the backward ring reuses the forward ring's shared memory
             S* bW = reinterpret_cast<S*>(smem_raw);
             S* bD = bW + PD * 2 * NT;
@@ -368,9 +381,12 @@ __device__ __forceinline__ double sweep_x2_tiles(const Lv<P>& L, const SweepK<P>
                 x0 = P::fma_u(w0, x0, P::ld_plain(bD, o));  // the recurrence carries unnormalised pairs
                 x1 = P::fma_u(w1, x1, P::ld_plain(bD, o + 1));
                 const size_t id = (size_t)k * pl + c;
-                if constexpr (MODE == MODE_SMOOTH) {
+                if constexpr (MODE == MODE_SMOOTH || MODE == MODE_SMOOTHB) {
                     R o0 = x0, o1 = x1;  // GFORM: the recurrence already yields u'
-                    if constexpr (NEED_U) {
+                    if constexpr (MODE == MODE_SMOOTHB) {
+                        o0 = P::fma(cf, x0, P::mul_u(K.rest, P::ld_plain(bU, o)));  // u' = (1 - rho) u + rho x
+                        o1 = P::fma(cf, x1, P::mul_u(K.rest, P::ld_plain(bU, o + 1)));
+                    } else if constexpr (NEED_U) {
                         o0 = P::fma(cf, x0, P::ld_plain(bU, o));  // u' = u + rho x
                         o1 = P::fma(cf, x1, P::ld_plain(bU, o + 1));
                     }
