@@ -268,9 +268,13 @@ tpmg_status tpmg_measure_alu_rate(int which, int reps, double* ops_per_s, double
  * with eviction hints (5-7), and, in FP32 only, one warp per tile of 128 x 1 or 128 x 2 columns with
  * four columns per thread and the Thomas factors 1/m_k formed in registers (8-11: one-row tiles;
  * one-row tiles run as overlapping forward/backward stages; two-row tiles; one-row tiles with a
- * shallower ring). A level that was never tuned or set takes, in FP32, variant 8 where the level
- * fits one tile per resident warp (nx % 128 == 0), else 5; double-word takes 6 where nx % 64 == 0;
- * otherwise (and in native FP64) variant 3. Variants 8-11 in other precisions run the default.
+ * shallower ring). In FP32 and double-word variant 0 holds whole columns of a tile in shared memory
+ * and works on their planes in parallel where the level allows it (nz <= 128; nx a multiple of 512 bytes
+ * of values, or of 256 bytes with even ny, or of 128 bytes with ny a multiple of 4). A level that was
+ * never tuned or set takes variant 0 in those precisions where lambda^2 is constant or the level is
+ * small; otherwise, in FP32, variant 8 where the level fits one tile per resident warp (nx % 128 == 0),
+ * else 5; double-word takes 6 where nx % 64 == 0; otherwise (and in native FP64) variant 3. Variants
+ * 8-11 in other precisions run the default.
  * tpmg_autotune times each of them `reps` times on every level of precision `prec` (on the
  * operator's workspace, CUDA events on `stream`) and keeps the fastest per level; if variants_out
  * is not NULL it receives the choice of level l in variants_out[l] (host array of L+1 ints).

@@ -466,9 +466,10 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
 // Smooth: eight variants per precision -- three (TY, PD) tile shapes with the shared-memory stack
 // (0-2), two persistent ones with the stack in global scratch (3, 4), and three persistent ones with
 // two columns per thread and L2 eviction hints (k_sweep_x2; 5-7); the autotuner (tpmg_autotune)
-// times them per level and stores its choice in Lv::variant. An untuned level takes variant 6
-// (double-word) or 8, 5 (FP32) where the two- or four-column form applies (nx % 64 or 128 == 0, aligned
-// fields), else variant 3; in native FP64, variant 3.
+// times them per level and stores its choice in Lv::variant. In FP32 and double-word variant 0 is the
+// whole-column tile in shared memory (sweep_tile.cuh) where the level takes it. An untuned level takes
+// that where smooth_tile_pays, else variant 6 (double-word) or 8, 5 (FP32) where the four- or two-column
+// form applies (nx % 128 or 64 == 0, aligned fields), else variant 3; in native FP64, variant 3.
 template <class P>
 struct SmoothVariants;
 template <>
@@ -484,10 +485,37 @@ struct SmoothVariants<PolDW> {
     static constexpr int TY[3] = {1, 2, 2};
 };
 
+// policies with whole-column tiles in shared memory (sweep_tile.cuh)
+template <class P>
+constexpr bool tile_policy() {
+    return std::is_same<P, PolF32>::value || std::is_same<P, PolDW>::value;
+}
+// Where an untuned level smooths on whole columns in shared memory, from both sides' times over 15
+// horizontal sizes, nz = 8 .. 128 and both kinds of lambda^2 (tile / best sweep with its stack in L2, us):
+//  - below 16 planes the sweeps have no chain to speak of: FP32 512^2 x 8 13.5 / 12.2;
+//  - lambda^2 constant: FP32 everywhere else (128^2 x 128 13 / 57, 256^2 35 / 63, 512^2 121 / 124, 1024^2
+//    419 / 480); double-word (with conversions) above 64 planes everywhere (512^2 x 128 919 / 958), below
+//    only on levels of up to 65536 columns (320 x 200 x 32 72 / 74, 512^2 x 32 255 / 249);
+//  - lambda^2 varying: the factors of the planes share the shared memory, two blocks per SM remain, and
+//    only levels too small to fill the GPU gain: FP32 256^2 x 128 42 / 46, 448 x 256 62 / 67, but 512 x 256
+//    76 / 71; double-word 128^2 x 128 90 / 96, 160^2 136 / 143, but 256^2 319 / 265.
+template <class P>
+static bool smooth_tile_pays(const Lv<P>& L) {
+    const size_t cols = (size_t)L.nx * L.ny;
+    if (L.nz < 16) return false;
+    if (P::id == 1) return !L.fac_percol || cols < 131072;
+    return L.fac_percol ? cols <= 32768 : (L.nz >= 64 || cols <= 65536);
+}
+
 template <class P, int MODE>
 static int smooth_dispatch(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                            typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
     int v = L.variant;
+    if constexpr (tile_policy<P>())
+        if (v == 0 || ((v < 0 || v >= TPMG_NUM_VARIANTS) && smooth_tile_pays(L))) {
+            const int nb = launch_sweep_tile<P, MODE>(L, rho, u, f, uo, partials, done, s);
+            if (nb >= 0) return nb;
+        }
     if constexpr (std::is_same<P, PolF32>::value) {  // one tile of 128 x 2 columns per warp where the level takes it
         if ((v < 0 || v >= TPMG_NUM_VARIANTS || v >= 8) && L.gstack) {
             const int nb = launch_smooth_x4(L, rho, u, f, uo, partials, done, s, v >= 8 && v < TPMG_NUM_VARIANTS ? v - 8 : 0);
@@ -574,6 +602,13 @@ int launch_apply_A_x2(const Lv<P>& L, const typename P::S* x, typename P::S* y, 
 template <class P>
 int launch_line_solve_pp(const Lv<P>& L, const typename P::S* b, typename P::S* x, double scale, const int* done,
                          cudaStream_t s) {
+    if constexpr (tile_policy<P>())
+        // (the line solve has no stencil to form: it gains wherever the Smooth does, in FP32 on all levels of
+        // 16 planes and more: 1024^2 x 128 166 us / 349, 128^2 x 128 10 / 60, 512^2 x 128 varying 77 / 77)
+        if (smooth_tile_pays(L) || (P::id == 1 && L.nz >= 16)) {
+            const int nb = launch_sweep_tile<P, MODE_LINESOLVE>(L, scale, b, nullptr, x, nullptr, done, s);
+            if (nb >= 0) return nb;
+        }
     if constexpr (std::is_same<P, PolF32>::value) {
         if (L.gstack) {
             const int nb = launch_line_solve_x4(L, b, x, scale, done, s);

@@ -242,6 +242,12 @@ int launch_line_solve_pp(const Lv<P>& L, const typename P::S* b, typename P::S* 
 int launch_smooth_x4(const Lv<PolF32>& L, double rho, const float* u, const float* f, float* uo, double* partials,
                      const int* done, cudaStream_t s, int config);
 int launch_line_solve_x4(const Lv<PolF32>& L, const float* b, float* x, double scale, const int* done, cudaStream_t s);
+// Smooth and line solve on whole columns in shared memory (sweep_tile.cuh; F32, DW): nx a
+// multiple of 512 bytes (256 with even ny, 128 with ny a multiple of 4), nz <= 128, 16-byte aligned fields,
+// else -1. MODE as in sweep_x2.cuh
+template <class P, int MODE>
+int launch_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f, typename P::S* out,
+                      double* partials, const int* done, cudaStream_t s);
 // y = A x by the two-column sweep (nx % 64 == 0, 16-byte aligned fields), else -1
 template <class P>
 int launch_apply_A_x2(const Lv<P>& L, const typename P::S* x, typename P::S* y, cudaStream_t s);

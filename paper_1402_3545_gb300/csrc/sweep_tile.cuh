@@ -1,0 +1,479 @@
+// sweep_tile.cuh -- Smooth (Eq. 11) and line solve (Eq. 9) on tiles of whole columns held in shared
+// memory: the planes of a tile are worked on in parallel, only the recurrences run one plane after
+// the other.
+//
+// A block owns 4 rows of 128 bytes of x-adjacent columns (32 x 4 FP32 columns, 16 x 4 of 8 bytes) over
+// all nz planes: nz * 512 bytes of shared memory. Its eight warps take contiguous ranges of planes:
+//   1. form the right-hand side of the line solves (f - A u, or sweep_rhs' f + H u) of their planes:
+//      f arrives by cp.async for all planes at once and u is prefetched to L2 for all planes at once,
+//      so the whole tile's reads are in flight together; x neighbours and the tile's inner rows come
+//      from the other lanes by shuffles;
+//   2. one thread per column eliminates forward through shared memory (the only serial part, a chain
+//      of a multiply-add and a multiply per plane);
+//   3. FP32: all threads form g_k = u_k + rho d'_k - w_k u_{k+1} (see sweep_x2.cuh);
+//   4. one thread per column substitutes back;
+//   5. all threads write the result as 16-byte vectors.
+// The recurrences cost 1 us each per tile of 128 planes in FP32 and what remains is bound by the issue
+// and latency of step 1's loads (three rows of u per row; measured 3.8 TB/s of algorithmic traffic for the
+// FP32 Smooth on 1024^2 x 128, 6.4 TB/s for the line solve, which has no step 1).
+// Two or three blocks per SM overlap one another's phases. The plane-marching sweeps keep one plane's
+// loads, elimination and stack store of every column in one chain, and their Thomas stack in a
+// global scratch (8 or 16 bytes of L2 traffic per cell); here nothing but the fields moves.
+// The per-cell arithmetic and its order are those of the other sweeps, so the results are the same
+// bits in every precision.
+//
+// Factors: with lambda^2 varying, 1/m_k of the planes before the converged ones (Lv::fac_k0) comes with
+// the tile's other reads into shared memory, where the forward sweep replaces it by w_k = v/m_k (the
+// stored factor's bits) for the back substitution; with lambda^2 constant, two tables of nz values.
+#pragma once
+#include <type_traits>
+
+#include "kernels.cuh"
+#include "sweep_x2.cuh"
+
+namespace tpmg {
+
+namespace {
+
+constexpr int TNT = 256;  // threads of a block
+constexpr int TNW = TNT / 32;
+constexpr int TPB = 512;  // bytes of a tile plane: TR rows of TPB / TR bytes
+
+template <class P>
+struct TileVec {  // 16 bytes of adjacent columns
+    typedef typename P::S S;
+    typedef typename P::R R;
+    static constexpr int N = 16 / (int)sizeof(S);
+    R v[N];
+    __device__ __forceinline__ void from(const float4& t) {
+        const S* p = reinterpret_cast<const S*>(&t);
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[e] = P::ld_plain(p, e);
+    }
+    __device__ __forceinline__ void ldg(const S* p) { from(__ldg(reinterpret_cast<const float4*>(p))); }
+    __device__ __forceinline__ void lds(const S* p) { from(*reinterpret_cast<const float4*>(p)); }
+    __device__ __forceinline__ void sts(S* p) const {
+        float4 t;
+        S* q = reinterpret_cast<S*>(&t);
+#pragma unroll
+        for (int e = 0; e < N; ++e) P::sts(q, e, v[e]);
+        *reinterpret_cast<float4*>(p) = t;
+    }
+    __device__ __forceinline__ void stg(S* p) const {  // storage rounding (P::st) applied
+        float4 t;
+        S* q = reinterpret_cast<S*>(&t);
+#pragma unroll
+        for (int e = 0; e < N; ++e) P::sts(q, e, P::rnd(v[e]));
+        *reinterpret_cast<float4*>(p) = t;
+    }
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[e] = P::zero();
+    }
+};
+
+// CV adjacent columns of a plane in the recurrences
+template <class P, int CV>
+struct TileCol : TileVec<P> {
+    typedef typename P::R R;
+    static_assert(CV == TileVec<P>::N, "16 bytes, or one column");
+    __device__ __forceinline__ void fill(R x) {
+#pragma unroll
+        for (int q = 0; q < CV; ++q) this->v[q] = x;
+    }
+};
+template <class P>
+struct TileCol<P, 1> {
+    typedef typename P::S S;
+    typedef typename P::R R;
+    R v[1];
+    __device__ __forceinline__ void ldg(const S* p) { v[0] = P::ld(p, 0); }
+    __device__ __forceinline__ void lds(const S* p) { v[0] = P::ld_plain(p, 0); }
+    __device__ __forceinline__ void sts(S* p) const { P::sts(p, 0, v[0]); }
+    __device__ __forceinline__ void stg(S* p) const { P::st(p, 0, v[0]); }
+    __device__ __forceinline__ void zero() { v[0] = P::zero(); }
+    __device__ __forceinline__ void fill(R x) { v[0] = x; }
+};
+
+__device__ __forceinline__ float shfl_up_v(float x, int d) { return __shfl_up_sync(0xffffffffu, x, d); }
+__device__ __forceinline__ float shfl_dn_v(float x, int d) { return __shfl_down_sync(0xffffffffu, x, d); }
+__device__ __forceinline__ dw shfl_up_v(dw x, int d) { return dw{shfl_up_v(x.hi, d), shfl_up_v(x.lo, d)}; }
+__device__ __forceinline__ dw shfl_dn_v(dw x, int d) { return dw{shfl_dn_v(x.hi, d), shfl_dn_v(x.lo, d)}; }
+
+__device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+
+}  // namespace
+
+// kw: planes whose factors are kept per column in shared memory behind the nz planes of the tile (0
+// when lambda^2 is constant). ISO: square cells; NORM: partial sums of ||f - A u||^2 (both compile-time:
+// as runtime choices their instructions were issued either way)
+template <class P, int MODE, int TR, bool ISO, bool NORM>
+__global__ void __launch_bounds__(TNT, 3)
+    k_sweep_tile(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u, const typename P::S* __restrict__ f,
+                 typename P::S* __restrict__ out, double* partials, const int* done, int kw) {
+    typedef typename P::S S;
+    typedef typename P::R R;
+    typedef TileVec<P> V;
+    constexpr bool SM = MODE != MODE_LINESOLVE;  // a stencil, and u in the result
+    constexpr bool GFORM = MODE == MODE_SMOOTH && P::id == 1;
+    constexpr bool DIRECT = GFORM || MODE == MODE_LINESOLVE;  // the back substitution yields the result
+    constexpr int G = 32 / TR;                                // lanes of a tile row
+    constexpr int N = V::N, W = G * N, NC = TR * W;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (done && *(volatile const int*)done) return;
+    S* const Z = reinterpret_cast<S*>(smem_raw);
+    const int nx = L.nx, ny = L.ny, nz = L.nz;
+    S* const ZW = Z + (size_t)nz * NC;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, lx = lane % G, ry = lane / G;
+    const int i0 = blockIdx.x * W, j0 = blockIdx.y * TR;
+    const size_t pl = (size_t)nx * ny;
+    const size_t c = (size_t)(j0 + ry) * nx + i0 + lx * N;  // this thread's first column
+    const int zo = lane * N;                                // ... in a tile plane
+    const int ch = (nz + TNW - 1) / TNW, klo = warp * ch, khi = klo + ch < nz ? klo + ch : nz;
+    const bool percol = L.fac_percol != 0;
+    const R vzero = P::zero();
+    typename P::Acc acc = 0, cmp = 0;
+
+    // ---- 1. the right-hand side of the line solves
+    {
+        const S* src = (SM ? f : u) + (size_t)klo * pl + c;
+        const S* inv = L.finv + (size_t)klo * pl + c;
+        S* z = Z + klo * NC + zo;
+        for (int k = klo; k < khi; ++k, src += pl, z += NC) tile_cp16(z, src);
+        if (percol) {  // 1/m_k of the planes before the converged ones; the forward sweep turns them into w_k
+            z = ZW + klo * NC + zo;
+            for (int k = klo; k < khi && k < kw; ++k, inv += pl, z += NC) tile_cp16(z, inv);
+        } else {
+            for (int k = tid; k < nz; k += TNT) {
+                ZW[k] = L.finv[k];
+                ZW[nz + k] = L.fw[k];
+            }
+        }
+        cp_commit();
+    }
+    if constexpr (SM) {
+        if (klo < khi) {
+            // the rows next to the tile's first and last one (one row: both, two or more: a lane meets at
+            // most one of them), and the columns left and right of it (first and last lane of a row)
+            const int js = j0 == 0 ? ny - 1 : j0 - 1, jn = j0 + TR == ny ? 0 : j0 + TR;
+            const bool hrow = TR == 1 || ry == 0 || ry == TR - 1, hcol = lx == 0 || lx == G - 1;
+            const int hi = lx == 0 ? (i0 == 0 ? nx - 1 : i0 - 1) : (i0 + W == nx ? 0 : i0 + W);
+            const size_t p0 = (size_t)klo * pl;
+            const S* pu = u + p0 + c;
+            const S* ph = u + p0 + (size_t)(ry == 0 ? js : jn) * nx + i0 + lx * N;
+            const S* ph1 = u + p0 + (size_t)jn * nx + i0 + lx * N;  // TR == 1
+            const S* pe = u + p0 + (size_t)(j0 + ry) * nx + hi;
+            S* z = Z + klo * NC + zo;
+            constexpr int D = TR == 1 ? 2 : 3;  // planes fetched together
+            const R cx = K.cx, cy = K.cy, dh = K.dh;
+            V um, uc, vv, dg;
+            um.zero();
+            vv.zero();
+            dg.zero();
+            uc.ldg(pu);
+            if (MODE == MODE_SMOOTH) {
+                if (klo > 0) um.ldg(pu - pl);
+#pragma unroll
+                for (int q = 0; q < N; ++q) {
+                    vv.v[q] = P::ld(L.v, c + q);
+                    dg.v[q] = P::add(P::add(dh, vv.v[q]), vv.v[q]);
+                }
+            }
+            cp_wait<0>();  // this thread's pieces of f
+            // one batch of B planes from plane k: all their loads, then their arithmetic
+            auto batch = [&](auto bc, int k) {
+                constexpr int B = decltype(bc)::value;
+                V ru[B], rh[B], rh1[B];
+                R re[B];
+                const bool top = k + B == nz;  // the last plane has no upper neighbour
+#pragma unroll
+                for (int t = 0; t < B; ++t) {  // u of plane k+t+1, the halo of plane k+t
+                    if (MODE == MODE_SMOOTH || t + 1 < B || !top) ru[t].ldg(t + 1 == B && top ? pu : pu + pl);
+                    else ru[t].zero();
+                    rh[t].zero();
+                    re[t] = vzero;
+                    if (hrow) rh[t].ldg(ph);
+                    if (TR == 1) rh1[t].ldg(ph1);
+                    if (hcol) re[t] = P::ld(pe, 0);
+                    pu += pl;
+                    ph += pl;
+                    ph1 += pl;
+                    pe += pl;
+                }
+                if (top) ru[B - 1].zero();
+#pragma unroll
+                for (int t = 0; t < B; ++t, z += NC) {
+                    V r;
+                    r.lds(z);
+                    R wl = shfl_up_v(uc.v[N - 1], 1), el = shfl_dn_v(uc.v[0], 1);
+                    if (lx == 0) wl = re[t];
+                    if (lx == G - 1) el = re[t];
+                    V d = dg;
+                    if (MODE == MODE_SMOOTH && (k + t == 0 || k + t == nz - 1)) {
+#pragma unroll
+                        for (int q = 0; q < N; ++q) d.v[q] = nz == 1 ? dh : P::add(dh, vv.v[q]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < N; ++q) {
+                        R s = rh[t].v[q], n = rh[t].v[q];
+                        if (TR == 1) {
+                            n = rh1[t].v[q];
+                        } else {
+                            const R su = shfl_up_v(uc.v[q], G), nd = shfl_dn_v(uc.v[q], G);
+                            if (ry != 0) s = su;
+                            if (ry != TR - 1) n = nd;
+                        }
+                        const R w = q == 0 ? wl : uc.v[q > 0 ? q - 1 : 0];
+                        const R e = q == N - 1 ? el : uc.v[q < N - 1 ? q + 1 : q];
+                        if constexpr (MODE == MODE_SMOOTHB)
+                            r.v[q] = sweep_rhs<P>(r.v[q], w, e, s, n, cx, cy, ISO);
+                        else
+                            r.v[q] = sweep_residual<P>(r.v[q], d.v[q], uc.v[q], w, e, s, n, um.v[q], ru[t].v[q], cx, cy,
+                                                       vv.v[q], ISO);
+                        if (NORM) P::acc_dot(acc, cmp, r.v[q], r.v[q]);
+                    }
+                    r.sts(z);
+                    um = uc;
+                    uc = ru[t];
+                }
+            };
+            int k = klo;
+            for (; k + D <= khi; k += D) batch(std::integral_constant<int, D>(), k);
+            for (; k < khi; ++k) batch(std::integral_constant<int, 1>(), k);
+        }
+    }
+    cp_wait<0>();
+    __syncthreads();
+
+    // ---- 2. forward elimination, CV columns per thread, eight planes' values read at a time. FP32: one
+    // warp, four columns per thread (as many issue slots as one column each on four warps take for
+    // one); the longer chains of the 8-byte policies take one column per thread
+    constexpr int KB = 8, CV = P::id == 1 ? N : 1, CT = NC / CV;
+    constexpr int TAB = 0, COL = 1, CONV = 2;  // factors: per-plane table, per column and plane, converged
+    typedef TileCol<P, CV> C;
+    const bool col = tid < CT;
+    const int c0 = tid * CV;  // first column in the tile plane
+    const size_t gc = col ? (size_t)(j0 + c0 / W) * nx + i0 + c0 % W : 0;
+    const int clast = nz >= 2 ? nz - 2 : 0;  // plane of the converged factors
+    if (col) {
+        C v, d;
+        v.ldg(L.v + gc);
+        d.zero();
+        auto sweep = [&](auto kind, int k, int ke, const C& inv) {
+            constexpr int F = decltype(kind)::value;
+            S* z = Z + k * NC + c0;
+            S* zw = F == TAB ? ZW + k : ZW + k * NC + c0;
+            auto step = [&](S* zk, S* zwk, const C& r, const C& iv) {
+                if (F == COL) {
+                    C w;
+#pragma unroll
+                    for (int q = 0; q < CV; ++q) w.v[q] = P::mul(v.v[q], iv.v[q]);
+                    w.sts(zwk);
+                }
+#pragma unroll
+                for (int q = 0; q < CV; ++q) d.v[q] = P::mul_u(P::fma_u(v.v[q], d.v[q], r.v[q]), iv.v[q]);
+                d.sts(zk);
+            };
+            auto factor = [&](C& iv, const S* zwk) {
+                if (F == TAB) iv.fill(P::ld_plain(zwk, 0));
+                if (F == COL) iv.lds(zwk);
+                if (F == CONV) iv = inv;
+            };
+            constexpr int WS = F == TAB ? 1 : NC;
+            for (; k + KB <= ke; k += KB, z += KB * NC, zw += KB * WS) {
+                C r[KB], iv[KB];
+#pragma unroll
+                for (int q = 0; q < KB; ++q) {
+                    r[q].lds(z + q * NC);
+                    factor(iv[q], zw + q * WS);
+                }
+#pragma unroll
+                for (int q = 0; q < KB; ++q) step(z + q * NC, zw + q * WS, r[q], iv[q]);
+            }
+            for (; k < ke; ++k, z += NC, zw += WS) {
+                C r, iv;
+                r.lds(z);
+                factor(iv, zw);
+                step(z, zw, r, iv);
+            }
+        };
+        C cinv;
+        cinv.zero();
+        if (percol) {
+            C einv;
+            cinv.ldg(L.finv + (size_t)clast * pl + gc);
+            einv.ldg(L.finv + (size_t)(nz - 1) * pl + gc);
+            sweep(std::integral_constant<int, COL>(), 0, kw, cinv);
+            sweep(std::integral_constant<int, CONV>(), kw, nz - 1, cinv);
+            sweep(std::integral_constant<int, CONV>(), nz - 1, nz, einv);
+        } else {
+            sweep(std::integral_constant<int, TAB>(), 0, nz, cinv);
+        }
+    }
+    __syncthreads();
+
+    // ---- 3. FP32: g_k = u_k + rho d'_k - w_k u_{k+1}
+    if constexpr (GFORM) {
+        if (klo < khi) {
+            const R cf = K.coef;
+            V uc, up, cw;
+            cw.zero();
+            if (percol) {  // the converged v/m_k
+#pragma unroll
+                for (int q = 0; q < N; ++q) cw.v[q] = P::ld(L.fw, (size_t)clast * pl + c + q);
+            }
+            const S* pu = u + (size_t)klo * pl + c;
+            S* z = Z + klo * NC + zo;
+            uc.ldg(pu);
+#pragma unroll 4
+            for (int k = klo; k < khi; ++k, z += NC) {
+                pu += pl;
+                up.zero();
+                if (k + 1 < nz) up.ldg(pu);
+                V g, w = cw;
+                g.lds(z);
+                if (k < kw) w.lds(ZW + k * NC + zo);
+                if (!percol) {
+                    const R wk = P::ld_plain(ZW, nz + k);
+#pragma unroll
+                    for (int q = 0; q < N; ++q) w.v[q] = wk;
+                }
+#pragma unroll
+                for (int q = 0; q < N; ++q) g.v[q] = P::fma(P::neg(w.v[q]), up.v[q], P::fma(cf, g.v[q], uc.v[q]));
+                g.sts(z);
+                uc = up;
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- 4. back substitution
+    if (col) {
+        C x;
+        x.zero();
+        S* po = out + (size_t)(nz - 1) * pl + gc;
+        auto sweep = [&](auto kind, int k, int ke, const C& cw) {  // planes k-1 .. ke
+            constexpr int F = decltype(kind)::value;
+            S* z = Z + (k - 1) * NC + c0;
+            const S* zw = F == TAB ? ZW + nz + k - 1 : ZW + (k - 1) * NC + c0;
+            auto factor = [&](C& w, const S* zwk) {
+                if (F == TAB) w.fill(P::ld_plain(zwk, 0));
+                if (F == COL) w.lds(zwk);
+                if (F == CONV) w = cw;
+            };
+            auto step = [&](S* zk, const C& d, const C& w) {
+#pragma unroll
+                for (int q = 0; q < CV; ++q) x.v[q] = P::fma_u(w.v[q], x.v[q], d.v[q]);
+                if (DIRECT) {
+                    C o = x;
+                    if (MODE == MODE_LINESOLVE) {
+#pragma unroll
+                        for (int q = 0; q < CV; ++q) o.v[q] = P::mul(K.coef, x.v[q]);
+                    }
+                    o.stg(po);
+                    po -= pl;
+                } else {
+                    x.sts(zk);
+                }
+            };
+            constexpr int WS = F == TAB ? 1 : NC;
+            for (; k - KB >= ke; k -= KB, z -= KB * NC, zw -= KB * WS) {
+                C d[KB], w[KB];
+#pragma unroll
+                for (int q = 0; q < KB; ++q) {
+                    d[q].lds(z - q * NC);
+                    factor(w[q], zw - q * WS);
+                }
+#pragma unroll
+                for (int q = 0; q < KB; ++q) step(z - q * NC, d[q], w[q]);
+            }
+            for (; k > ke; --k, z -= NC, zw -= WS) {
+                C d, w;
+                d.lds(z);
+                factor(w, zw);
+                step(z, d, w);
+            }
+        };
+        C cw;
+        cw.zero();
+        if (percol) {
+            cw.ldg(L.fw + (size_t)clast * pl + gc);  // (that of plane nz-1 meets x = 0)
+            sweep(std::integral_constant<int, CONV>(), nz, kw, cw);
+            sweep(std::integral_constant<int, COL>(), kw, 0, cw);
+        } else {
+            sweep(std::integral_constant<int, TAB>(), nz, 0, cw);
+        }
+    }
+
+    // ---- 5. the result of the forms that add u
+    if constexpr (!DIRECT) {
+        __syncthreads();
+        const R cf = K.coef;
+        const S* pu = u + (size_t)klo * pl + c;
+        S* po = out + (size_t)klo * pl + c;
+        const S* z = Z + klo * NC + zo;
+#pragma unroll 4
+        for (int k = klo; k < khi; ++k, pu += pl, po += pl, z += NC) {
+            V x, uo;
+            uo.ldg(pu);
+            x.lds(z);
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                x.v[q] = P::fma(cf, x.v[q], MODE == MODE_SMOOTHB ? P::mul_u(K.rest, uo.v[q]) : uo.v[q]);
+            x.stg(po);
+        }
+    }
+    if (NORM) {
+        const double sm = block_sum(P::acc_get(acc, cmp));
+        if (tid == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = sm;
+    }
+}
+
+template <class P, int MODE, int TR, bool ISO, bool NORM>
+static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
+                          typename P::S* out, double* partials, const int* done, cudaStream_t s) {
+    typedef typename P::S S;
+    // planes whose factors differ from the converged ones (all but the last when none has converged)
+    int kw = 0;
+    if (L.fac_percol) kw = L.fac_k0 < L.nz - 1 ? (L.fac_k0 > 0 ? L.fac_k0 : 0) : L.nz - 1;
+    const size_t smem = (size_t)(L.nz + kw) * TPB + (L.fac_percol ? 0 : 2 * (size_t)L.nz * sizeof(S));
+    auto kern = k_sweep_tile<P, MODE, TR, ISO, NORM>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * TPB);
+    const dim3 grd(L.nx / (TPB / TR / (int)sizeof(S)), L.ny / TR);
+    kern<<<grd, TNT, smem, s>>>(L, sweep_k<P>(L.cx, L.cy, coef), u, f, out, partials, done, kw);
+    note_launch();
+    return (int)(grd.x * grd.y);
+}
+
+template <class P, int MODE, bool ISO, bool NORM>
+static int run_sweep_tile_rows(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
+                               typename P::S* out, double* partials, const int* done, cudaStream_t s) {
+    constexpr int W = TPB / (int)sizeof(typename P::S);
+    if (L.nx % W == 0) return run_sweep_tile<P, MODE, 1, ISO, NORM>(L, coef, u, f, out, partials, done, s);
+    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0)
+        return run_sweep_tile<P, MODE, 2, ISO, NORM>(L, coef, u, f, out, partials, done, s);
+    if (L.nx % (W / 4) == 0 && L.ny % 4 == 0)
+        return run_sweep_tile<P, MODE, 4, ISO, NORM>(L, coef, u, f, out, partials, done, s);
+    return -1;
+}
+
+template <class P, int MODE>
+int launch_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f, typename P::S* out,
+                      double* partials, const int* done, cudaStream_t s) {
+    if (L.nz > 128 || !L.finv || !L.fw) return -1;
+    auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+    if (!al(u) || (MODE != MODE_LINESOLVE && !al(f)) || !al(out) || !al(L.v) || (L.fac_percol && (!al(L.finv) || !al(L.fw))))
+        return -1;
+    // the line solve has no stencil and no norm
+    constexpr bool ONE = MODE == MODE_LINESOLVE, NN = MODE != MODE_SMOOTH;
+    if (ONE || L.cx == L.cy) {
+        if (NN || !partials) return run_sweep_tile_rows<P, MODE, true, false>(L, coef, u, f, out, partials, done, s);
+        return run_sweep_tile_rows<P, MODE, true, !NN>(L, coef, u, f, out, partials, done, s);
+    }
+    if (NN || !partials) return run_sweep_tile_rows<P, MODE, ONE, false>(L, coef, u, f, out, partials, done, s);
+    return run_sweep_tile_rows<P, MODE, ONE, !NN>(L, coef, u, f, out, partials, done, s);
+}
+
+}  // namespace tpmg
