@@ -110,6 +110,7 @@ struct tpmg_op {
     double* pgeo[MAXL + 1][3] = {};  // per level: |T|, x-face and y-face coefficients
     double* prad[3] = {};            // radial E = a - b - c, B = -b, C = -c
     double* pfac[MAXL + 1][3] = {};  // per level: Thomas factors 1/m, forward and backward multipliers
+    double* pchunk[MAXL + 1][2] = {};  // per small level: products of the multipliers per chunk of planes
     float* pgeo32[MAXL + 1][3] = {};  // FP32 copies for the mixed solve's inner V-cycles
     float* prad32[3] = {};
     float* pfac32[MAXL + 1][3] = {};
@@ -844,6 +845,7 @@ tpmg_status tpmg_destroy_operator(tpmg_op* op) {
         for (int l = 0; l <= MAXL; ++l) {
             dfree((void*&)op->pgeo[l][t]);
             dfree((void*&)op->pfac[l][t]);
+            if (t < 2) dfree((void*&)op->pchunk[l][t]);
             dfree((void*&)op->pgeo32[l][t]);
             dfree((void*&)op->pfac32[l][t]);
         }
@@ -2391,6 +2393,8 @@ static PanelLv panel_view(const tpmg_op* op, int l) {
     L.inv = op->pfac[l][0];
     L.fl = op->pfac[l][1];
     L.fw = op->pfac[l][2];
+    L.wf = op->pchunk[l][0];
+    L.wb = op->pchunk[l][1];
     return L;
 }
 
@@ -2463,7 +2467,13 @@ extern "C" tpmg_status tpmg_create_panel_operator(const tpmg_grid* g, double ome
         }
         for (int t = 0; t < 3; ++t)
             if ((st = dalloc((void**)&op->pfac[l][t], lvl_cells(op, l) * sizeof(double))) != TPMG_OK) return fail(st);
-        launch_panel_factors(panel_view(op, l), op->pfac[l][0], op->pfac[l][1], op->pfac[l][2], 0);
+        if (panel_chunked(nx, ny))
+            for (int t = 0; t < 2; ++t)
+                if ((st = dalloc((void**)&op->pchunk[l][t], (size_t)nx * ny * ((nz + panel_chunk_planes(nz) - 1) / panel_chunk_planes(nz)) *
+                                                                sizeof(double))) != TPMG_OK)
+                    return fail(st);
+        launch_panel_factors(panel_view(op, l), op->pfac[l][0], op->pfac[l][1], op->pfac[l][2], op->pchunk[l][0],
+                             op->pchunk[l][1], 0);
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(set_err(TPMG_ERR_CUDA, "panel setup kernels failed"));
     if (cudaStreamCreateWithFlags(&op->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||

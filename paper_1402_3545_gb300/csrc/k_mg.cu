@@ -345,7 +345,9 @@ Shape sweep_shape(int nx, int ny, int nz, int bytes_per_value, bool stack) {
 
 int max_partials(int nx, int ny) {
     const int col_kernels = ((nx + TX - 1) / TX) * ny;
-    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : 0;  // at most one block per column
+    // small levels: at most one block per column; chunked columns (native FP64): one per 8 columns. A level
+    // below the finest has a quarter of its columns or fewer, so that the finest level's count covers it.
+    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (nx * ny <= CHUNK_MAX_COLS ? (nx * ny + 7) / 8 : 0);
     return col_kernels > cell_kernels ? col_kernels : cell_kernels;
 }
 

@@ -16,14 +16,21 @@
 // factors of the column blocks are computed once per level (k_panel_factors): 1/m_k, the forward
 // multiplier |T| B_k / m_k and the backward one |T| C_k / m_k, per cell. The forward-eliminated
 // values go into the output field itself, which the back substitution then overwrites, so the
-// sweeps need no scratch. These kernels are bound by the FP64 pipe (about 14 FP64 instructions per
-// cell for a Smooth; at 54 resident warps per SM the pipe, not the load latency, sets the pace).
+// sweeps need no scratch. On large levels the FP64 kernels are bound by the FP64 pipe, so their
+// arithmetic is arranged for few instructions per cell: 9 for a residual, 9 for a Smooth without a
+// norm (in the form (1 - rho) u + rho M^{-1}(f + H u), H the horizontal couplings: the vertical part of
+// A u is not formed; 14 with the norm), 4 for the prolongation. Small levels leave most of the chip
+// idle with a thread per column and 2 nz dependent FP64 operations (about 80 cycles each) per sweep:
+// there a column is cut into chunks of planes (k_panel_chunk), and the pointwise kernels take a few
+// planes per thread. FP32 (the mixed solve's inner cycles) keeps one thread per column throughout.
 #include "kernels.cuh"
 #include "panel.cuh"
 
 namespace tpmg {
 
 namespace {
+
+constexpr int CB = 8, CH = 16;  // columns and chunks of a block of the chunked sweeps
 
 template <class T>
 struct PCol {
@@ -34,10 +41,10 @@ struct PCol {
 };
 
 template <class T>
-__device__ __forceinline__ PCol<T> panel_col(const PanelLvT<T>& L) {
+__device__ __forceinline__ PCol<T> panel_col(const PanelLvT<T>& L, int i, int j) {
     PCol<T> q;
-    q.i = blockIdx.x * blockDim.x + threadIdx.x;
-    q.j = blockIdx.y * blockDim.y + threadIdx.y;
+    q.i = i;
+    q.j = j;
     q.act = q.i < L.nx && q.j < L.ny;
     if (!q.act) return q;
     q.c = (size_t)q.j * L.nx + q.i;
@@ -52,6 +59,11 @@ __device__ __forceinline__ PCol<T> panel_col(const PanelLvT<T>& L) {
     q.an = __ldg(L.ay + (size_t)(q.j + 1) * L.nx + q.i);
     q.at = (q.aw + q.ae) + (q.as + q.an);
     return q;
+}
+
+template <class T>
+__device__ __forceinline__ PCol<T> panel_col(const PanelLvT<T>& L) {
+    return panel_col(L, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y);
 }
 
 // (A u)_{T,k} given the centre value, its vertical neighbours (0 beyond the column) and
@@ -72,17 +84,46 @@ __device__ __forceinline__ T panel_Au(const PanelLvT<T>& L, const PCol<T>& q, co
     return fma(-tc, up, s);
 }
 
+// f - A u at one cell in FP64, nine operations: the vertical and the |T| part of the diagonal share one
+// product with |T|
+__device__ __forceinline__ double panel_res(const PanelLv& L, const PCol<double>& q, const double* __restrict__ x, size_t b,
+                                            int k, double fk, double uc, double um, double up) {
+    const double xw = q.hw ? __ldg(x + b + q.c - 1) : 0.0;
+    const double xe = q.he ? __ldg(x + b + q.c + 1) : 0.0;
+    const double xs = q.hs ? __ldg(x + b + q.c - L.nx) : 0.0;
+    const double xn = q.hn ? __ldg(x + b + q.c + L.nx) : 0.0;
+    const double v = fma(-__ldg(L.C + k), up, fma(-__ldg(L.B + k), um, __ldg(L.E + k) * uc));
+    double r = fma(q.at, uc, fk);
+    r = fma(-q.aw, xw, r);
+    r = fma(-q.ae, xe, r);
+    r = fma(-q.as, xs, r);
+    r = fma(-q.an, xn, r);
+    return fma(-q.area, v, r);
+}
+// f + H u: the right-hand side of a smoothing step's line solves (four operations)
+__device__ __forceinline__ double panel_rhs(const PanelLv& L, const PCol<double>& q, const double* __restrict__ x, size_t b,
+                                            double fk) {
+    const double xw = q.hw ? __ldg(x + b + q.c - 1) : 0.0;
+    const double xe = q.he ? __ldg(x + b + q.c + 1) : 0.0;
+    const double xs = q.hs ? __ldg(x + b + q.c - L.nx) : 0.0;
+    const double xn = q.hn ? __ldg(x + b + q.c + L.nx) : 0.0;
+    return fma(-q.an, xn, fma(-q.as, xs, fma(-q.ae, xe, fma(-q.aw, xw, fk))));
+}
+
 }  // namespace
 
 // Thomas factors of every column block of level L: m_0 = D_0, m_k = D_k - (|T| B_k)^2 / m_{k-1}
 // with D_k = |T| E_k - alpha_T (the off-diagonals of row k are -|T| B_k below, -|T| C_k above, and
 // C_{k-1} = B_k); stored 1/m_k, |T| B_k / m_k and |T| C_k / m_k.
+// wf, wb (if not null): the products of the forward and of the backward multipliers over each chunk of
+// pp planes, [chunk][column] (k_panel_chunk).
 __global__ void __launch_bounds__(128) k_panel_factors(PanelLv L, double* __restrict__ inv, double* __restrict__ fl,
-                                                       double* __restrict__ fw) {
+                                                       double* __restrict__ fw, double* __restrict__ wf,
+                                                       double* __restrict__ wb, int pp) {
     const PCol<double> q = panel_col(L);
     if (!q.act) return;
     const size_t pl = (size_t)L.nx * L.ny;
-    double m_prev = 1.0;
+    double m_prev = 1.0, pf = 1.0, pb = 1.0;
     for (int k = 0; k < L.nz; ++k) {
         const double d = fma(q.area, L.E[k], -q.at);
         const double tb = q.area * L.B[k];
@@ -90,8 +131,18 @@ __global__ void __launch_bounds__(128) k_panel_factors(PanelLv L, double* __rest
         const double iv = 1.0 / m;
         inv[(size_t)k * pl + q.c] = iv;
         fl[(size_t)k * pl + q.c] = tb * iv;
-        fw[(size_t)k * pl + q.c] = q.area * L.C[k] * iv;
+        const double w = q.area * L.C[k] * iv;
+        fw[(size_t)k * pl + q.c] = w;
         m_prev = m;
+        if (wf) {
+            pf *= tb * iv;
+            pb *= w;
+            if ((k + 1) % pp == 0 || k + 1 == L.nz) {
+                wf[(size_t)(k / pp) * pl + q.c] = pf;
+                wb[(size_t)(k / pp) * pl + q.c] = pb;
+                pf = pb = 1.0;
+            }
+        }
     }
 }
 
@@ -101,7 +152,8 @@ __global__ void __launch_bounds__(128) k_panel_factors(PanelLv L, double* __rest
 // MODE 2 line solve: out = coef M^{-1} u (u is the right-hand side)
 // MODE 3 apply: out = A u
 // T is the arithmetic (double or float); the norm's partial sums are accumulated in T.
-template <int MODE, class T, class TO>
+// NORM (FP64 Smooth): with the sums; without them the Smooth takes the form that needs no residual.
+template <int MODE, class T, class TO, bool NORM>
 __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, const T* __restrict__ u,
                                                      const T* __restrict__ f, TO* out, double* partials,
                                                      const int* done) {
@@ -110,18 +162,30 @@ __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, cons
     const size_t pl = (size_t)L.nx * L.ny;
     const int nz = L.nz;
     T acc = 0;
+    constexpr bool RHS = MODE == 0 && sizeof(T) == 8 && !NORM;
     if (q.act) {
         T um = 0, uc = (MODE != 2) ? __ldg(u + q.c) : T(0), dp = 0;
         T tb = 0;  // |T| B_k (B_0 = 0); |T| C_k = |T| B_{k+1} is carried to the next plane
 #pragma unroll 2
         for (int k = 0; k < nz; ++k) {
             const size_t b = (size_t)k * pl;
+            if constexpr (RHS) {
+                const double r = panel_rhs(L, q, u, b, __ldg(f + b + q.c));
+                dp = fma(__ldg(L.fl + b + q.c), dp, r * __ldg(L.inv + b + q.c));
+                out[b + q.c] = dp;
+                continue;
+            }
             const T tc = (k + 1 < nz) ? q.area * __ldg(L.B + k + 1) : T(0);
             T r;
             if (MODE != 2) {
                 const T up = (k + 1 < nz) ? __ldg(u + b + pl + q.c) : T(0);
-                const T au = panel_Au(L, q, u, b, k, uc, um, up, tb, tc);
-                r = (MODE == 3) ? au : __ldg(f + b + q.c) - au;
+                if constexpr (sizeof(T) == 8) {
+                    r = panel_res(L, q, u, b, k, MODE == 3 ? 0.0 : __ldg(f + b + q.c), uc, um, up);
+                    if (MODE == 3) r = -r;
+                } else {
+                    const T au = panel_Au(L, q, u, b, k, uc, um, up, tb, tc);
+                    r = (MODE == 3) ? au : __ldg(f + b + q.c) - au;
+                }
                 um = uc;
                 uc = up;
             } else {
@@ -143,13 +207,162 @@ __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, cons
             for (int k = nz - 1; k >= 0; --k) {
                 const size_t id = (size_t)k * pl + q.c;
                 x = fma(__ldg(L.fw + id), x, (T)out[id]);
-                out[id] = (MODE == 0) ? fma(coef, x, __ldg(u + id)) : coef * x;
+                if constexpr (RHS) out[id] = fma(coef, x, (1.0 - coef) * __ldg(u + id));
+                else out[id] = (MODE == 0) ? fma(coef, x, __ldg(u + id)) : coef * x;
             }
         }
     }
     if ((MODE == 0 || MODE == 1) && partials) {
         const double s = block_sum((double)acc);
         if (threadIdx.x == 0 && threadIdx.y == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// ---------------------------------------------------------------- columns cut into chunks of planes
+// FP64 sweeps of the small levels: a block owns 8 columns, each cut into 16 chunks of PP planes with a thread
+// per chunk. Both recurrences (y_k = a_k + fl_k y_{k-1}, a_k = b_k / m_k; x_k = y_k + fw_k x_{k+1}) run
+// twice per chunk: from zero, for the value the chunk hands on, and, once the carried value is known
+// (the earlier chunks' values chained by the chunks' products of multipliers, wf and wb), for the
+// chunk's own values. That is one more operation per cell and direction and 2 (2 PP + 16) instead of
+// 2 nz dependent ones: on 64^2 x 128 a Smooth took 186 us with a thread per column.
+// MODE 0 Smooth, 2 line solve (u the right-hand side), 4 RestrictSmooth (u the fine residual r_f:
+// f_c = sum of the children to fc, out = coef M^{-1} f_c).
+template <int MODE, int PP, bool NORM>
+__global__ void __launch_bounds__(CB * CH) k_panel_chunk(PanelLv L, double coef, const double* __restrict__ u,
+                                                         const double* __restrict__ f, double* out,
+                                                         double* __restrict__ fc, double* partials, const int* done) {
+    __shared__ double sy[CH][CB], sx[CH][CB];
+    if (done && *(volatile const int*)done) return;
+    const int tx = threadIdx.x, w = threadIdx.y, nz = L.nz, k0 = w * PP;
+    // (a thread beyond the last column works on it and stores nothing)
+    const int col = blockIdx.x * CB + tx, ncol = L.nx * L.ny;
+    const bool act = col < ncol;
+    const int cc = act ? col : ncol - 1;
+    const PCol<double> q = panel_col(L, cc % L.nx, cc / L.nx);
+    const size_t pl = (size_t)L.nx * L.ny;
+    const int np = !act || k0 >= nz ? 0 : (nz - k0 < PP ? nz - k0 : PP);  // planes of this thread
+    // Every load is unconditional (planes beyond the column repeat its last one), so that a pass's loads
+    // are in flight together; planes beyond np get zeros and leave both chains at zero.
+    double a[PP], y = 0.0, acc = 0.0;
+    auto plane = [&](int p) { return (size_t)(k0 + p < nz ? k0 + p : nz - 1) * pl; };
+    {
+        const int kf = k0 < nz ? k0 : nz - 1;
+        double um = 0.0, uc = 0.0, fl[PP];
+        if (MODE == 0 && NORM) {
+            uc = __ldg(u + (size_t)kf * pl + q.c);
+            um = __ldg(u + (size_t)(kf > 0 ? kf - 1 : 0) * pl + q.c);
+            if (kf == 0) um = 0.0;
+        }
+#pragma unroll
+        for (int p = 0; p < PP; ++p) {
+            const bool in = p < np;
+            const int k = k0 + p < nz ? k0 + p : nz - 1;
+            const size_t b = plane(p), id = b + q.c;
+            double r;
+            if (MODE == 0 && NORM) {
+                double up = __ldg(u + (k + 1 < nz ? id + pl : id));
+                if (k + 1 == nz) up = 0.0;
+                r = panel_res(L, q, u, b, k, __ldg(f + id), uc, um, up);
+                if (in) acc = fma(r, r, acc);
+                um = uc;
+                uc = up;
+            } else if (MODE == 0) {
+                r = panel_rhs(L, q, u, b, __ldg(f + id));
+            } else if (MODE == 4) {
+                const size_t nxf = 2 * (size_t)L.nx;
+                const double* rf = u + 4 * b + (size_t)(2 * q.j) * nxf + 2 * q.i;
+                r = (__ldg(rf) + __ldg(rf + 1)) + (__ldg(rf + nxf) + __ldg(rf + nxf + 1));
+                if (in) fc[id] = r;
+            } else {
+                r = __ldg(u + id);
+            }
+            const double iv = __ldg(L.inv + id);
+            fl[p] = __ldg(L.fl + id);
+            a[p] = in ? r * iv : 0.0;
+        }
+#pragma unroll
+        for (int p = 0; p < PP; ++p) y = fma(p < np ? fl[p] : 0.0, y, a[p]);
+    }
+    sy[w][tx] = y;
+    const int last = (nz - 1) / PP;
+    __syncthreads();
+    if (w == 0) {  // one thread per column: each chunk's carried value in the place of what it hands on
+        y = 0.0;
+#pragma unroll 4
+        for (int c = 0; c <= last; ++c) {
+            const double e = sy[c][tx];
+            sy[c][tx] = y;
+            y = fma(__ldg(L.wf + (size_t)c * pl + q.c), y, e);
+        }
+    }
+    __syncthreads();
+    y = sy[w][tx];
+#pragma unroll
+    for (int p = 0; p < PP; ++p) {
+        const double m = __ldg(L.fl + plane(p) + q.c);
+        y = fma(p < np ? m : 0.0, y, a[p]);
+        a[p] = p < np ? y : 0.0;
+    }
+    double x = 0.0;
+#pragma unroll
+    for (int p = PP - 1; p >= 0; --p) {
+        const double m = __ldg(L.fw + plane(p) + q.c);
+        x = fma(p < np ? m : 0.0, x, a[p]);
+    }
+    sx[w][tx] = x;
+    __syncthreads();
+    if (w == 0) {
+        x = 0.0;
+#pragma unroll 4
+        for (int c = last; c >= 0; --c) {
+            const double e = sx[c][tx];
+            sx[c][tx] = x;
+            x = fma(__ldg(L.wb + (size_t)c * pl + q.c), x, e);
+        }
+    }
+    __syncthreads();
+    x = sx[w][tx];
+#pragma unroll
+    for (int p = PP - 1; p >= 0; --p) {
+        const size_t id = plane(p) + q.c;
+        const double m = __ldg(L.fw + id), uo = MODE == 0 ? __ldg(u + id) : 0.0;
+        x = fma(p < np ? m : 0.0, x, a[p]);
+        if (p < np) out[id] = MODE == 0 ? fma(coef, x, NORM ? uo : (1.0 - coef) * uo) : coef * x;
+    }
+    if (MODE == 0 && NORM) {
+        const double s = block_sum(acc);
+        if (tx == 0 && w == 0) partials[blockIdx.x] = s;
+    }
+}
+
+// FP64 Residual (MODE 1, stored in TO) and apply (MODE 3), pointwise: planes blockIdx.z * pz .. of each
+// column, partial sums of ||f - A u||^2
+template <int MODE, class TO>
+__global__ void __launch_bounds__(128) k_panel_point(PanelLv L, const double* __restrict__ u,
+                                                     const double* __restrict__ f, TO* __restrict__ out,
+                                                     double* partials, const int* done, int pz) {
+    if (done && *(volatile const int*)done) return;
+    const PCol<double> q = panel_col(L);
+    const size_t pl = (size_t)L.nx * L.ny;
+    const int nz = L.nz, k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
+    double acc = 0.0;
+    if (q.act && k0 < k1) {
+        size_t b = (size_t)k0 * pl;
+        double um = k0 > 0 ? __ldg(u + b - pl + q.c) : 0.0, uc = __ldg(u + b + q.c);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k, b += pl) {
+            const double up = k + 1 < nz ? __ldg(u + b + pl + q.c) : 0.0;
+            const double r = panel_res(L, q, u, b, k, MODE == 3 ? 0.0 : __ldg(f + b + q.c), uc, um, up);
+            out[b + q.c] = (TO)(MODE == 3 ? -r : r);
+            if (MODE == 1 && partials) acc = fma(r, r, acc);
+            um = uc;
+            uc = up;
+        }
+    }
+    if (MODE == 1 && partials) {
+        const double s = block_sum(acc);
+        if (threadIdx.x == 0 && threadIdx.y == 0)
+            partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
     }
 }
 
@@ -181,10 +394,11 @@ __global__ void __launch_bounds__(128) k_panel_restrict_smooth(PanelLvT<T> Lc, T
 }
 
 // u_f += P u_c: bilinear in the logical grid (weights 3/4 and 1/4 per direction), a coarse
-// neighbour beyond the panel boundary contributing 0. One thread per fine column.
+// neighbour beyond the panel boundary contributing 0. One thread per fine column and pz planes. In FP64 the
+// four products accumulate onto u_f (four operations); FP32 forms P u_c first.
 template <class T>
 __global__ void __launch_bounds__(128) k_panel_prolongate(int nxc, int nyc, int nz, const T* __restrict__ uc,
-                                                          T* __restrict__ uf, const int* done) {
+                                                          T* __restrict__ uf, const int* done, int pz) {
     if (done && *(volatile const int*)done) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     const int nxf = 2 * nxc, nyf = 2 * nyc;
@@ -195,13 +409,24 @@ __global__ void __launch_bounds__(128) k_panel_prolongate(int nxc, int nyc, int 
     const size_t plc = (size_t)nxc * nyc, plf = (size_t)nxf * nyf;
     const size_t c0 = (size_t)J * nxc + I, cx = (size_t)J * nxc + I2, cy = (size_t)J2 * nxc + I,
                  cxy = (size_t)J2 * nxc + I2, fo = (size_t)j * nxf + i;
-    for (int k = 0; k < nz; ++k) {
+    const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
+#pragma unroll 4
+    for (int k = k0; k < k1; ++k) {
         const T* p = uc + (size_t)k * plc;
-        T v = T(0.5625) * __ldg(p + c0);
-        if (in2) v = fma(T(0.1875), __ldg(p + cx), v);
-        if (jn2) v = fma(T(0.1875), __ldg(p + cy), v);
-        if (in2 && jn2) v = fma(T(0.0625), __ldg(p + cxy), v);
-        uf[(size_t)k * plf + fo] += v;
+        T& o = uf[(size_t)k * plf + fo];
+        if constexpr (sizeof(T) == 8) {
+            T v = fma(T(0.5625), __ldg(p + c0), o);
+            if (in2) v = fma(T(0.1875), __ldg(p + cx), v);
+            if (jn2) v = fma(T(0.1875), __ldg(p + cy), v);
+            if (in2 && jn2) v = fma(T(0.0625), __ldg(p + cxy), v);
+            o = v;
+        } else {
+            T v = T(0.5625) * __ldg(p + c0);
+            if (in2) v = fma(T(0.1875), __ldg(p + cx), v);
+            if (jn2) v = fma(T(0.1875), __ldg(p + cy), v);
+            if (in2 && jn2) v = fma(T(0.0625), __ldg(p + cxy), v);
+            o += v;
+        }
     }
 }
 
@@ -295,9 +520,48 @@ void launch_panel_cg_tridiag(const PanelLv& L, const Scalars* sc, double* r, con
     note_launch();
 }
 
-void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw, cudaStream_t s) {
-    k_panel_factors<<<panel_grid(L.nx, L.ny), dim3(32, 4), 0, s>>>(L, inv, fl, fw);
+void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw, double* wf, double* wb, cudaStream_t s) {
+    k_panel_factors<<<panel_grid(L.nx, L.ny), dim3(32, 4), 0, s>>>(L, inv, fl, fw, wf, wb, panel_chunk_planes(L.nz));
     note_launch();
+}
+
+// planes per block of the pointwise kernels: 16 where the level fills the GPU with them, else 4
+static int point_planes(int nx, int ny) { return (size_t)nx * ny > 65536 ? 16 : 4; }
+
+// The chunked sweep where the level has its chunk products (PanelLvT::wf). Returns the number of blocks, or
+// -1 where it does not apply.
+template <int MODE, int PP>
+static int run_panel_chunk(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
+                           double* partials, const int* done, cudaStream_t s) {
+    const int nb = (L.nx * L.ny + CB - 1) / CB;
+    const dim3 b(CB, CH);
+    if (MODE == 0 && partials) k_panel_chunk<MODE, PP, MODE == 0><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
+    else k_panel_chunk<MODE, PP, false><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
+    note_launch();
+    return nb;
+}
+template <int MODE>
+static int panel_chunk(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
+                       double* partials, const int* done, cudaStream_t s) {
+    if (!L.wf || !L.wb) return -1;
+    switch (panel_chunk_planes(L.nz)) {
+        case 4: return run_panel_chunk<MODE, 4>(L, coef, u, f, out, fc, partials, done, s);
+        case 8: return run_panel_chunk<MODE, 8>(L, coef, u, f, out, fc, partials, done, s);
+        default: return run_panel_chunk<MODE, 16>(L, coef, u, f, out, fc, partials, done, s);
+    }
+}
+
+template <int MODE, class TO>
+static int panel_point(const PanelLv& L, const double* u, const double* f, TO* out, double* partials, const int* done,
+                       cudaStream_t s) {
+    dim3 g = panel_grid(L.nx, L.ny);
+    int pz = point_planes(L.nx, L.ny);
+    // partial sums: at most one block per 32 columns (max_partials), that is four per 32 x 4 tile
+    if (partials) pz = L.ny >= 4 ? (L.nz + 3) / 4 : L.nz;
+    g.z = (L.nz + pz - 1) / pz;
+    k_panel_point<MODE, TO><<<g, dim3(32, 4), 0, s>>>(L, u, f, out, partials, done, pz);
+    note_launch();
+    return (int)(g.x * g.y * g.z);
 }
 
 template <class T>
@@ -305,11 +569,21 @@ int launch_panel_sweep(int mode, const PanelLvT<T>& L, double coef, const T* u, 
                        const int* done, cudaStream_t s) {
     const dim3 g = panel_grid(L.nx, L.ny), b(32, 4);
     const T c = (T)coef;
+    if constexpr (sizeof(T) == 8) {
+        if (mode == PANEL_RESIDUAL) return panel_point<1, double>(L, u, f, out, partials, done, s);
+        if (mode == PANEL_APPLY) return panel_point<3, double>(L, u, f, out, nullptr, done, s);
+        const int nb = mode == PANEL_SMOOTH ? panel_chunk<0>(L, coef, u, f, out, nullptr, partials, done, s)
+                                            : panel_chunk<2>(L, coef, u, f, out, nullptr, nullptr, done, s);
+        if (nb >= 0) return nb;
+    }
     switch (mode) {
-        case PANEL_SMOOTH: k_panel_sweep<0, T, T><<<g, b, 0, s>>>(L, c, u, f, out, partials, done); break;
-        case PANEL_RESIDUAL: k_panel_sweep<1, T, T><<<g, b, 0, s>>>(L, c, u, f, out, partials, done); break;
-        case PANEL_LINESOLVE: k_panel_sweep<2, T, T><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
-        default: k_panel_sweep<3, T, T><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
+        case PANEL_SMOOTH:
+            if (partials) k_panel_sweep<0, T, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done);
+            else k_panel_sweep<0, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done);
+            break;
+        case PANEL_RESIDUAL: k_panel_sweep<1, T, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done); break;
+        case PANEL_LINESOLVE: k_panel_sweep<2, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
+        default: k_panel_sweep<3, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
     }
     note_launch();
     return (int)(g.x * g.y);
@@ -317,22 +591,24 @@ int launch_panel_sweep(int mode, const PanelLvT<T>& L, double coef, const T* u, 
 
 int launch_panel_residual_to_f32(const PanelLv& L, const double* u, const double* f, float* r, double* partials,
                                  const int* done, cudaStream_t s) {
-    const dim3 g = panel_grid(L.nx, L.ny);
-    k_panel_sweep<1, double, float><<<g, dim3(32, 4), 0, s>>>(L, 1.0, u, f, r, partials, done);
-    note_launch();
-    return (int)(g.x * g.y);
+    return panel_point<1, float>(L, u, f, r, partials, done, s);
 }
 
 template <class T>
 void launch_panel_restrict_smooth(const PanelLvT<T>& Lc, double rho, const T* rf, T* fc, T* uc, const int* done,
                                   cudaStream_t s) {
+    if constexpr (sizeof(T) == 8)
+        if (panel_chunk<4>(Lc, rho, rf, nullptr, uc, fc, nullptr, done, s) >= 0) return;
     k_panel_restrict_smooth<T><<<panel_grid(Lc.nx, Lc.ny), dim3(32, 4), 0, s>>>(Lc, (T)rho, rf, fc, uc, done);
     note_launch();
 }
 
 template <class T>
 void launch_panel_prolongate(int nxc, int nyc, int nz, const T* uc, T* uf, const int* done, cudaStream_t s) {
-    k_panel_prolongate<T><<<panel_grid(2 * nxc, 2 * nyc), dim3(32, 4), 0, s>>>(nxc, nyc, nz, uc, uf, done);
+    dim3 g = panel_grid(2 * nxc, 2 * nyc);
+    const int pz = point_planes(2 * nxc, 2 * nyc);
+    g.z = (nz + pz - 1) / pz;
+    k_panel_prolongate<T><<<g, dim3(32, 4), 0, s>>>(nxc, nyc, nz, uc, uf, done, pz);
     note_launch();
 }
 

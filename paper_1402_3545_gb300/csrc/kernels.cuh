@@ -140,6 +140,9 @@ size_t gstack_bytes(int nz);
 // Levels with at most this many columns run the cell-parallel kernels (one thread per cell,
 // the column solve by parallel cyclic reduction): a thread per column leaves the GPU idle there.
 static constexpr int PCR_MAX_COLS = 4096;
+// Native FP64 levels of at most this many columns cut their columns into chunks of planes: above it a
+// thread per column fills the GPU
+static constexpr int CHUNK_MAX_COLS = 32768;
 inline int pcr_steps_for(int nz) {
     int s = 0;
     while ((1 << s) < nz) ++s;

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
+#include "kernels.cuh"
+
 namespace tpmg {
 
 // One multigrid level of the panel operator (Eq. (14)) as the kernels see it, in value type T
@@ -24,12 +26,22 @@ struct PanelLvT {
     const T* inv;
     const T* fl;
     const T* fw;
+    // FP64, small levels (panel_chunked): products of fl and of fw over each chunk of
+    // panel_chunk_planes(nz) planes, [chunk][column]; null elsewhere
+    const T* wf = nullptr;
+    const T* wb = nullptr;
 };
 typedef PanelLvT<double> PanelLv;
 
 enum { PANEL_SMOOTH = 0, PANEL_RESIDUAL = 1, PANEL_LINESOLVE = 2, PANEL_APPLY = 3 };
 
-void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw, cudaStream_t s);
+// planes per chunk of a column in the chunked sweeps: up to 16 chunks of 4, 8 or 16 planes
+inline int panel_chunk_planes(int nz) { return nz <= 64 ? 4 : (nz <= 128 ? 8 : 16); }
+// Levels that sweep their columns in chunks: where a thread per column leaves the GPU waiting on its
+// recurrences (128^2 x 128 Smooth 193 us with one thread per column at a floor of 36)
+inline bool panel_chunked(int nx, int ny) { return (size_t)nx * ny <= (size_t)CHUNK_MAX_COLS; }
+// wf, wb: the chunk products, or null
+void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw, double* wf, double* wb, cudaStream_t s);
 // mode PANEL_*: Smooth (coef = rho) and Residual write partial sums of ||f - A u||^2 when partials is
 // non-null; the line solve takes its right-hand side in u and scales by coef. Returns the number of
 // thread blocks (= partial sums written).
