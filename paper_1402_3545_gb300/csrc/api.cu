@@ -79,7 +79,8 @@ struct tpmg_op {
     float2* vdw[MAXL + 1] = {};
     Hier hier[3];  // by policy id (F64, F32, DW)
     void* finv[3][MAXL + 1] = {};  // Thomas factors 1/m_k per policy and level
-    void* pcr[3][MAXL + 1] = {};   // PCR factors of the small levels per policy and level
+    void* pcr[3][MAXL + 1] = {};   // PCR factors of the small levels per policy and level (not FP64)
+    double* chunkw[MAXL + 1] = {}; // native FP64, small levels: factor products per chunk of planes
     void* gstack = nullptr;        // Thomas-stack scratch of the persistent sweep variants
     void* fw[3][MAXL + 1] = {};    // Thomas factors v/m_k
     int percol[MAXL + 1] = {};     // 1 if lambda^2 varies over the level (factors per cell)
@@ -146,6 +147,7 @@ static Lv<P> level_view(const tpmg_op* op, int l) {
     L.fac_k0 = op->fac_k0[P::id][l];
     L.variant = op->variant[P::id][l];
     L.pcr = (const typename P::S*)op->pcr[P::id][l];
+    if constexpr (P::id == 0) L.chunkw = op->chunkw[l];
     L.gstack = op->gstack;
     L.pcr_steps = pcr_steps_for(op->g.nz);
     return L;
@@ -280,15 +282,16 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid) {
             CK(cudaMemcpy(&k0, dk, sizeof(int), cudaMemcpyDeviceToHost));
             op->fac_k0[pid][l] = k0;
         }
-        // small levels: parallel-cyclic-reduction factors for the cell-parallel kernels
-        if ((size_t)op->g.lnx[l] * op->g.lny[l] <= (size_t)PCR_MAX_COLS && op->g.nz <= 256) {
+        // small levels: factor products of the chunked columns (native FP64), parallel-cyclic-reduction
+        // factors of the cell-parallel kernels (the other policies)
+        const size_t cols = (size_t)op->g.lnx[l] * op->g.lny[l];
+        if (pid == 0 && cols <= (size_t)CHUNK_MAX_COLS) {
+            const Lv<PolF64> L = level_view<PolF64>(op, l);
+            TRY(dalloc((void**)&op->chunkw[l], chunk_count(L) * eb));
+            launch_chunk_products(L, op->chunkw[l], 0);
+        }
+        if (pid != 0 && cols <= (size_t)PCR_MAX_COLS && op->g.nz <= 256) {
             switch (pid) {
-                case 0: {
-                    Lv<PolF64> L = level_view<PolF64>(op, l);
-                    TRY(dalloc(&op->pcr[0][l], pcr_factor_count(L, op->percol[l]) * eb));
-                    launch_pcr_factors<PolF64>(L, (double*)op->pcr[0][l], op->percol[l], 0);
-                    break;
-                }
                 case 1: {
                     Lv<PolF32> L = level_view<PolF32>(op, l);
                     TRY(dalloc(&op->pcr[1][l], pcr_factor_count(L, op->percol[l]) * eb));
@@ -812,6 +815,7 @@ tpmg_status tpmg_destroy_operator(tpmg_op* op) {
         dfree((void*&)op->v64[l]);
         dfree((void*&)op->v32[l]);
         dfree((void*&)op->vdw[l]);
+        dfree((void*&)op->chunkw[l]);
         for (int p = 0; p < 3; ++p) {
             dfree(op->finv[p][l]);
             dfree(op->pcr[p][l]);

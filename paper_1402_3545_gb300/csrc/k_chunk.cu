@@ -1,0 +1,284 @@
+// k_chunk.cu -- native FP64 kernels of the small levels (128 x 256 columns and below): columns cut into
+// chunks of planes.
+//
+// With a thread per column these levels leave most of the chip waiting on 2 nz dependent FP64 operations
+// (about 80 cycles each); cyclic reduction (k_coarse.cu, the other policies) shortens the chain to log2 nz
+// steps but takes 2 log2(nz) + 1 operations per cell for the solve alone on a pipe that issues 1/74 of the
+// FP32 rate. Here a block owns 8 columns, each cut into 16 chunks of PP planes with a thread per chunk, and
+// both recurrences of the Thomas algorithm, y_k = b_k / m_k + w_k y_{k-1} and x_k = y_k + w_k x_{k+1}
+// (w_k = v / m_k), run twice per chunk: from zero, for the value the chunk hands on, and, once the carried
+// value is known (the earlier chunks' values chained by the chunks' products of w_k), for the chunk's own
+// values. One more operation per cell and direction (11 for a Smooth), 2 (2 PP + chunks) dependent ones.
+// The forward-error bound is that of the Thomas algorithm: the second pass is its recurrence, and the
+// carried value's own rounding enters damped by the products, all below 1.
+// Measured per Smooth inside a graph: 64^2 x 128 17 us (cyclic reduction 35), 128^2 x 128 65 us (thread per
+// column 95), 64^2 x 64 10 us (17), 8^2 x 128 9 us (6).
+#include "kernels.cuh"
+
+namespace tpmg {
+
+namespace {
+
+constexpr int CB = 8, CH = 16;  // columns and chunks of a block
+
+__device__ __forceinline__ int kwrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
+
+struct CCol {
+    int i, j;
+    bool act;
+    size_t c, w, e, s, n;  // in-plane offsets of the column and its neighbours
+};
+__device__ __forceinline__ CCol chunk_col(int nx, int ny, int col) {
+    CCol q;
+    q.act = col < nx * ny;
+    const int cc = q.act ? col : 0;
+    q.i = cc % nx;
+    q.j = cc / nx;
+    q.c = cc;
+    q.w = (size_t)q.j * nx + kwrap(q.i - 1, nx);
+    q.e = (size_t)q.j * nx + kwrap(q.i + 1, nx);
+    q.s = (size_t)kwrap(q.j - 1, ny) * nx + q.i;
+    q.n = (size_t)kwrap(q.j + 1, ny) * nx + q.i;
+    return q;
+}
+// f + cx (u_w + u_e) + cy (u_s + u_n) (sweep_rhs's form)
+__device__ __forceinline__ double chunk_rhs(const double* __restrict__ u, const CCol& q, double fk, double cx, double cy) {
+    return fma(cy, __ldg(u + q.s) + __ldg(u + q.n), fma(cx, __ldg(u + q.w) + __ldg(u + q.e), fk));
+}
+
+}  // namespace
+
+// product of w_k over each chunk of pp planes, [chunk][column] (lambda^2 varying) or [chunk]
+__global__ void __launch_bounds__(128) k_chunk_products(Lv<PolF64> L, double* __restrict__ out, int pp) {
+    const int ncol = L.fac_percol ? L.nx * L.ny : 1, col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= ncol) return;
+    double p = 1.0;
+    for (int k = 0; k < L.nz; ++k) {
+        p *= L.fw[(size_t)k * ncol + col];
+        if ((k + 1) % pp == 0 || k + 1 == L.nz) {
+            out[(size_t)(k / pp) * ncol + col] = p;
+            p = 1.0;
+        }
+    }
+}
+
+// MODE 0 Smooth: out = u + coef M^{-1}(f - A u); NORM with the partial sums of ||f - A u||^2, without them in
+// the form (1 - coef) u + coef M^{-1}(f + H u). MODE 1 line solve: out = coef M^{-1} u. MODE 2 RestrictSmooth:
+// fc = R u (u the fine residual in PF's storage), out = coef M^{-1} fc.
+template <class PF, int MODE, int PP, bool NORM>
+__global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, const typename PF::S* __restrict__ uin,
+                                                   const double* __restrict__ f, double* __restrict__ out,
+                                                   double* __restrict__ fc, double* partials, const int* done) {
+    __shared__ double sy[CH][CB], sx[CH][CB];
+    if (done && *(volatile const int*)done) return;
+    const double* u = reinterpret_cast<const double*>(uin);  // (MODE 2 reads uin)
+    const int tx = threadIdx.x, w = threadIdx.y, nz = L.nz, k0 = w * PP;
+    const CCol q = chunk_col(L.nx, L.ny, blockIdx.x * CB + tx);
+    const size_t pl = (size_t)L.nx * L.ny;
+    const int np = !q.act || k0 >= nz ? 0 : (nz - k0 < PP ? nz - k0 : PP);  // planes of this thread
+    // Every load is unconditional (planes beyond the column repeat its last one), so that a pass's loads
+    // are in flight together; planes beyond np get a = w = 0 and leave both chains at zero.
+    const size_t fs = L.fac_percol ? pl : 1, fo = L.fac_percol ? q.c : 0;  // factors of plane k at k * fs + fo
+    double a[PP], wk[PP], y = 0.0, acc = 0.0;
+    {
+        const int kf = k0 < nz ? k0 : nz - 1;
+        double um = 0.0, uc = 0.0, vv = 0.0, dh1 = 0.0, dh2 = 0.0;
+        if (MODE == 0 && NORM) {
+            uc = __ldg(u + (size_t)kf * pl + q.c);
+            um = __ldg(u + (size_t)(kf > 0 ? kf - 1 : 0) * pl + q.c);
+            if (kf == 0) um = 0.0;
+            vv = __ldg(L.v + q.c);
+            dh1 = (1.0 + 2.0 * L.cx + 2.0 * L.cy) + vv;
+            dh2 = dh1 + vv;
+        }
+#pragma unroll
+        for (int p = 0; p < PP; ++p) {
+            const bool in = p < np;
+            const int k = k0 + p < nz ? k0 + p : nz - 1;
+            const size_t b = (size_t)k * pl, id = b + q.c;
+            double r;
+            if (MODE == 0) {
+                r = chunk_rhs(u + b, q, __ldg(f + id), L.cx, L.cy);
+                if (NORM) {
+                    double up = __ldg(u + (k + 1 < nz ? id + pl : id));
+                    if (k + 1 == nz) up = 0.0;
+                    const double dg = nz == 1 ? dh1 - vv : (k == 0 || k == nz - 1 ? dh1 : dh2);
+                    r = fma(vv, um + up, fma(-dg, uc, r));
+                    if (in) acc = fma(r, r, acc);
+                    um = uc;
+                    uc = up;
+                }
+            } else if (MODE == 2) {
+                typedef Conv<PF, PolF64> CV;
+                const size_t nxf = 2 * (size_t)L.nx, c0 = (size_t)k * 4 * pl + (size_t)(2 * q.j) * nxf + 2 * q.i;
+                r = 0.25 * ((CV::f(PF::ld(uin, c0)) + CV::f(PF::ld(uin, c0 + 1))) +
+                            (CV::f(PF::ld(uin, c0 + nxf)) + CV::f(PF::ld(uin, c0 + nxf + 1))));
+                if (in) fc[id] = r;
+            } else {
+                r = __ldg(u + id);
+            }
+            const double iv = __ldg(L.finv + (size_t)k * fs + fo), wv = __ldg(L.fw + (size_t)k * fs + fo);
+            a[p] = in ? r * iv : 0.0;
+            wk[p] = in ? wv : 0.0;
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < PP; ++p) y = fma(wk[p], y, a[p]);
+    sy[w][tx] = y;
+    const double* cw = L.chunkw + fo;  // the chunks' products
+    const int last = (nz - 1) / PP;
+    __syncthreads();
+    if (w == 0) {  // one thread per column: each chunk's carried value in the place of what it hands on
+        y = 0.0;
+#pragma unroll 4
+        for (int c = 0; c <= last; ++c) {
+            const double e = sy[c][tx];
+            sy[c][tx] = y;
+            y = fma(__ldg(cw + (size_t)c * fs), y, e);
+        }
+    }
+    __syncthreads();
+    y = sy[w][tx];
+#pragma unroll
+    for (int p = 0; p < PP; ++p) {
+        y = fma(wk[p], y, a[p]);
+        a[p] = p < np ? y : 0.0;
+    }
+    double x = 0.0;
+#pragma unroll
+    for (int p = PP - 1; p >= 0; --p) x = fma(wk[p], x, a[p]);
+    sx[w][tx] = x;
+    double uo[MODE == 0 ? PP : 1];
+    if (MODE == 0) {
+#pragma unroll
+        for (int p = 0; p < PP; ++p) uo[p] = __ldg(u + (size_t)(k0 + p < nz ? k0 + p : nz - 1) * pl + q.c);
+    }
+    __syncthreads();
+    if (w == 0) {
+        x = 0.0;
+#pragma unroll 4
+        for (int c = last; c >= 0; --c) {
+            const double e = sx[c][tx];
+            sx[c][tx] = x;
+            x = fma(__ldg(cw + (size_t)c * fs), x, e);
+        }
+    }
+    __syncthreads();
+    x = sx[w][tx];
+    const double keep = 1.0 - coef;
+#pragma unroll
+    for (int p = PP - 1; p >= 0; --p) {
+        x = fma(wk[p], x, a[p]);
+        if (p < np) out[(size_t)(k0 + p) * pl + q.c] = MODE == 0 ? fma(coef, x, NORM ? uo[p] : keep * uo[p]) : coef * x;
+    }
+    if (MODE == 0 && NORM) {
+        const double s = block_sum(acc);
+        if (tx == 0 && w == 0) partials[blockIdx.x] = s;
+    }
+}
+
+// Residual, planes blockIdx.y * pz .. of a column per thread: seven operations per cell
+__global__ void __launch_bounds__(128) k_chunk_residual(Lv<PolF64> L, const double* __restrict__ u,
+                                                        const double* __restrict__ f, double* __restrict__ r,
+                                                        double* partials, const int* done, int pz) {
+    if (done && *(volatile const int*)done) return;
+    const CCol q = chunk_col(L.nx, L.ny, blockIdx.x * 128 + threadIdx.x);
+    const size_t pl = (size_t)L.nx * L.ny;
+    const int nz = L.nz, k0 = blockIdx.y * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
+    double acc = 0.0;
+    if (q.act && k0 < k1) {
+        const double vv = __ldg(L.v + q.c), dh = 1.0 + 2.0 * L.cx + 2.0 * L.cy, dh1 = dh + vv, dh2 = dh1 + vv;
+        double um = k0 > 0 ? __ldg(u + (size_t)(k0 - 1) * pl + q.c) : 0.0, uc = __ldg(u + (size_t)k0 * pl + q.c);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const size_t b = (size_t)k * pl, id = b + q.c;
+            const double up = k + 1 < nz ? __ldg(u + id + pl) : 0.0;
+            const double dg = nz == 1 ? dh : (k == 0 || k == nz - 1 ? dh1 : dh2);
+            const double rk = fma(vv, um + up, fma(-dg, uc, chunk_rhs(u + b, q, __ldg(f + id), L.cx, L.cy)));
+            r[id] = rk;
+            if (partials) acc = fma(rk, rk, acc);
+            um = uc;
+            uc = up;
+        }
+    }
+    if (partials) {
+        const double s = block_sum(acc);
+        if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// ---------------------------------------------------------------- launchers
+// 16 chunks of 4, 8 or 16 planes
+int chunk_planes(int nz) { return nz <= 4 * CH ? 4 : (nz <= 8 * CH ? 8 : 16); }
+
+size_t chunk_count(const Lv<PolF64>& L) {
+    return (size_t)((L.nz + chunk_planes(L.nz) - 1) / chunk_planes(L.nz)) * (L.fac_percol ? (size_t)L.nx * L.ny : 1);
+}
+
+void launch_chunk_products(const Lv<PolF64>& L, double* out, cudaStream_t s) {
+    const int ncol = L.fac_percol ? L.nx * L.ny : 1;
+    k_chunk_products<<<(ncol + 127) / 128, 128, 0, s>>>(L, out, chunk_planes(L.nz));
+    note_launch();
+}
+
+template <class PF, int MODE, int PP>
+static int run_chunk(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
+                     double* partials, const int* done, cudaStream_t s) {
+    const int nb = (L.nx * L.ny + CB - 1) / CB;
+    const dim3 b(CB, CH);
+    if (MODE == 0 && partials)
+        k_chunk<PF, MODE, PP, MODE == 0><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
+    else
+        k_chunk<PF, MODE, PP, false><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
+    note_launch();
+    return nb;
+}
+template <class PF, int MODE>
+static int chunk_sweep(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
+                       double* partials, const int* done, cudaStream_t s) {
+    if (!L.chunkw) return -1;
+    switch (chunk_planes(L.nz)) {
+        case 4: return run_chunk<PF, MODE, 4>(L, coef, u, f, out, fc, partials, done, s);
+        case 8: return run_chunk<PF, MODE, 8>(L, coef, u, f, out, fc, partials, done, s);
+        default: return run_chunk<PF, MODE, 16>(L, coef, u, f, out, fc, partials, done, s);
+    }
+}
+
+int launch_smooth_chunk(const Lv<PolF64>& L, double rho, const double* u, const double* f, double* uo, double* partials,
+                        const int* done, cudaStream_t s) {
+    // above PCR_MAX_COLS columns a tile variant that was chosen for the level takes precedence
+    if ((size_t)L.nx * L.ny > (size_t)PCR_MAX_COLS && L.variant >= 0) return -1;
+    return chunk_sweep<PolF64, 0>(L, rho, u, f, uo, nullptr, partials, done, s);
+}
+int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, double scale, const int* done, cudaStream_t s) {
+    return chunk_sweep<PolF64, 1>(L, scale, b, nullptr, x, nullptr, nullptr, done, s);
+}
+template <class PF>
+int launch_restrict_smooth_chunk(const Lv<PolF64>& Lc, double rho, const typename PF::S* rf, double* fc, double* uc,
+                                 const int* done, cudaStream_t s) {
+    // larger coarse levels: the column sweep, whose values the fused Residual + RestrictSmooth reproduces
+    if ((size_t)Lc.nx * Lc.ny > (size_t)PCR_MAX_COLS) return -1;
+    return chunk_sweep<PF, 2>(Lc, rho, rf, nullptr, uc, fc, nullptr, done, s);
+}
+template int launch_restrict_smooth_chunk<PolF64>(const Lv<PolF64>&, double, const double*, double*, double*, const int*,
+                                                  cudaStream_t);
+template int launch_restrict_smooth_chunk<PolDW>(const Lv<PolF64>&, double, const float2*, double*, double*, const int*,
+                                                 cudaStream_t);
+
+// planes per thread of the residual: at most 1024 blocks on PCR_MAX_COLS columns
+static int residual_planes(int nz) { return nz > 128 ? (nz + 31) / 32 : 4; }
+
+int residual_chunk_blocks(const Lv<PolF64>& L) {
+    const int pz = residual_planes(L.nz);
+    return (L.nx * L.ny + 127) / 128 * ((L.nz + pz - 1) / pz);
+}
+int launch_residual_chunk(const Lv<PolF64>& L, const double* u, const double* f, double* r, double* partials,
+                          const int* done, cudaStream_t s) {
+    const int pz = residual_planes(L.nz);
+    const dim3 g((L.nx * L.ny + 127) / 128, (L.nz + pz - 1) / pz);
+    k_chunk_residual<<<g, 128, 0, s>>>(L, u, f, r, partials, done, pz);
+    note_launch();
+    return (int)(g.x * g.y);
+}
+
+}  // namespace tpmg

@@ -2,8 +2,8 @@
 // PCR_MAX_COLS columns: 64 x 64 and below).
 //
 // The column kernels give each vertical column one thread, which leaves the GPU nearly idle on the
-// coarse levels (a 16 x 16 level has 256 columns) and, on the levels the double-word solver runs in
-// native FP64, serialises about 60 FP64 instructions per cell at 1/72 of the FP32 rate. Here every
+// coarse levels (a 16 x 16 level has 256 columns). Here (FP32 and double-word; native FP64, whose pipe the
+// extra operations would fill, cuts its columns into chunks, k_chunk.cu) every
 // cell has its own thread: the stencil and the transfers are pointwise, and the column block
 // M_c = tridiag(-v, D_k, -v) is solved by parallel cyclic reduction (PCR): with stride s = 1, 2, 4,
 // ... each row eliminates its neighbours at distance s,
@@ -274,6 +274,13 @@ __global__ void __launch_bounds__(256) k_prolongate_cell(int nxc, int nyc, int n
         const int I = i >> 1, J = j >> 1;
         const int I2 = cwrap((i & 1) ? I + 1 : I - 1, nxc), J2 = cwrap((j & 1) ? J + 1 : J - 1, nyc);
         const size_t bc = (size_t)k * plc;
+        if constexpr (P::id == 0 && PF::id == 0) {  // native FP64: four operations, accumulated onto u_f
+            R o = P::fma(w9, P::ld(uc, bc + (size_t)J * nxc + I), PF::ld_plain(uf, id));
+            o = P::fma(w3, P::ld(uc, bc + (size_t)J * nxc + I2), o);
+            o = P::fma(w3, P::ld(uc, bc + (size_t)J2 * nxc + I), o);
+            PF::st(uf, id, P::fma(w1, P::ld(uc, bc + (size_t)J2 * nxc + I2), o));
+            continue;
+        }
         R val = P::mul(w9, P::ld(uc, bc + (size_t)J * nxc + I));
         val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J * nxc + I2)));
         val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J2 * nxc + I)));
@@ -304,6 +311,24 @@ __global__ void __launch_bounds__(128) k_prolongate_x4(int nxc, int nyc, int nz,
     const R ym = P::ld(cp, rm + I), yp = P::ld(cp, rp + I);
     const R dmm = P::ld(cp, rm + Im), dpm = P::ld(cp, rm + Ip), dmp = P::ld(cp, rp + Im), dpp = P::ld(cp, rp + Ip);
     const R w9 = P::cst(0.5625), w3 = P::cst(0.1875), w1 = P::cst(0.0625);
+    if constexpr (P::id == 0 && PF::id == 0) {
+        // native FP64, bound by its pipe: the four products accumulate onto u_f, four operations per fine
+        // cell instead of 7.25 (64^2 to 128^2 x 128 18 us, 22 before)
+        const int nxf = 2 * nxc;
+        typename PF::S* p0 = uf + (size_t)k * 4 * plc + (size_t)(2 * J) * nxf + 2 * I;
+        auto row = [&](typename PF::S* p, R y, R dm, R dp) {
+            const double2 o = *reinterpret_cast<const double2*>(p);
+            double2 v;
+            v.x = P::fma(w1, dm, P::fma(w3, y, P::fma(w3, xm, P::fma(w9, c, o.x))));
+            v.y = P::fma(w1, dp, P::fma(w3, y, P::fma(w3, xp, P::fma(w9, c, o.y))));
+            *reinterpret_cast<double2*>(p) = v;
+        };
+        if (((uintptr_t)uf & 15) == 0) {
+            row(p0, ym, dmm, dpm);
+            row(p0 + nxf, yp, dmp, dpp);
+            return;
+        }
+    }
     const R c9 = P::mul(w9, c);
     // fine (a, b): a = 0 takes the x neighbour I-1, a = 1 takes I+1; likewise b in y
     const R v00 = P::add(P::add(c9, P::mul(w3, xm)), P::add(P::mul(w3, ym), P::mul(w1, dmm)));
@@ -414,7 +439,7 @@ int launch_prolongate_x4(int nxc, int nyc, int nz, const typename P::S* uc, type
     return (int)(grd.x * grd.y * grd.z);
 }
 
-#define TPMG_COARSE_INST(P)                                                                                 \
+#define TPMG_PCR_INST(P)                                                                                    \
     template size_t pcr_factor_count<P>(const Lv<P>&, int);                                                  \
     template void launch_pcr_factors<P>(const Lv<P>&, P::S*, int, cudaStream_t);                             \
     template int pcr_blocks<P>(const Lv<P>&);                                                                \
@@ -424,20 +449,22 @@ int launch_prolongate_x4(int nxc, int nyc, int nz, const typename P::S* uc, type
     template int launch_restrict_smooth_pcr<P, P>(const Lv<P>&, double, const P::S*, P::S*, P::S*, const int*, \
                                                   cudaStream_t);                                             \
     template int launch_residual_cell<P, P>(const Lv<P>&, const P::S*, const P::S*, P::S*, double*, const int*, \
-                                            cudaStream_t);                                                   \
+                                            cudaStream_t);
+#define TPMG_PROL_INST(P)                                                                                   \
     template int launch_prolongate_cell<P, P>(int, int, int, const P::S*, P::S*, const int*, cudaStream_t);     \
     template int launch_prolongate_x4<P, P>(int, int, int, const P::S*, P::S*, const int*, cudaStream_t);
 
-TPMG_COARSE_INST(PolF64)
-TPMG_COARSE_INST(PolF32)
-TPMG_COARSE_INST(PolDW)
-TPMG_COARSE_INST(PolF32B)
+TPMG_PROL_INST(PolF64)
+TPMG_PROL_INST(PolF32)
+TPMG_PROL_INST(PolDW)
+TPMG_PROL_INST(PolF32B)
+TPMG_PCR_INST(PolF32)
+TPMG_PCR_INST(PolDW)
+TPMG_PCR_INST(PolF32B)
 template int launch_restrict_smooth_pcr<PolF32, PolF32B>(const Lv<PolF32B>&, double, const float*, float*, float*,
                                                          const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
 template int launch_prolongate_x4<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
-template int launch_restrict_smooth_pcr<PolDW, PolF64>(const Lv<PolF64>&, double, const float2*, double*, double*,
-                                                       const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
 template int launch_prolongate_x4<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
 template int launch_residual_cell<PolDW, PolF32>(const Lv<PolDW>&, const float2*, const float2*, float*, double*,

@@ -14,6 +14,8 @@
 // Operator (Sec. 2.1.1, flat-box form of Eq. (6), periodic horizontally, Neumann at k = 0 and
 // k = nz-1): (A u)_k = D_k u_k - cx (u_W + u_E) - cy (u_S + u_N) - v (u_{k-1} + u_{k+1}) with
 // D_k = 1 + 2cx + 2cy + v * (number of vertical neighbours).
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace tpmg {
@@ -366,7 +368,11 @@ void launch_apply_A(const Lv<P>& L, const typename P::S* x, typename P::S* y, cu
 template <class P>
 void launch_line_solve(const Lv<P>& L, const typename P::S* b, typename P::S* x, double scale, const int* done,
                        cudaStream_t s) {
-    if (launch_line_solve_pcr<P>(L, b, x, scale, done, s) >= 0) return;
+    if constexpr (P::id == 0) {
+        if (launch_line_solve_chunk(L, b, x, scale, done, s) >= 0) return;
+    } else {
+        if (launch_line_solve_pcr<P>(L, b, x, scale, done, s) >= 0) return;
+    }
     if (launch_line_solve_pp<P>(L, b, x, scale, done, s) >= 0) return;
     Shape sh = sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), true);
     allow_smem(k_line_solve<P>, sh.smem);
@@ -376,7 +382,9 @@ void launch_line_solve(const Lv<P>& L, const typename P::S* b, typename P::S* x,
 template <class P>
 int launch_smooth(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                    typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
-    int nparts = launch_smooth_pcr<P>(L, rho, u, f, uo, partials, done, s);
+    int nparts;
+    if constexpr (P::id == 0) nparts = launch_smooth_chunk(L, rho, u, f, uo, partials, done, s);
+    else nparts = launch_smooth_pcr<P>(L, rho, u, f, uo, partials, done, s);
     if (nparts >= 0) return nparts;
     nparts = launch_smooth_pp<P>(L, rho, u, f, uo, partials, done, s);
     if (nparts >= 0) return nparts;
@@ -389,7 +397,10 @@ int launch_smooth(const Lv<P>& L, double rho, const typename P::S* u, const type
 template <class P, class PO>
 int residual_launch_blocks(const Lv<P>& L, const typename P::S* u, const typename P::S* f, typename PO::S* r) {
     // launch_residual's three choices in its order: pointwise, plane-pipelined, one thread per column
-    if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) return cell_blocks((size_t)L.nx * L.ny * L.nz);
+    if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) {
+        if constexpr (P::id == 0 && PO::id == 0) return residual_chunk_blocks(L);
+        return cell_blocks((size_t)L.nx * L.ny * L.nz);
+    }
     const int nb = residual_pp_blocks<P, PO>(L, u, f, r);
     if (nb >= 0) return nb;
     return sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false).nblocks();
@@ -397,8 +408,13 @@ int residual_launch_blocks(const Lv<P>& L, const typename P::S* u, const typenam
 template <class P, class PO>
 int launch_residual(const Lv<P>& L, const typename P::S* u, const typename P::S* f,
                     typename PO::S* r, double* partials, const int* done, cudaStream_t s) {
-    int nb = launch_residual_cell<P, PO>(L, u, f, r, partials, done, s);
-    if (nb >= 0) return nb;
+    int nb = -1;
+    if constexpr (P::id == 0 && PO::id == 0) {
+        if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) return launch_residual_chunk(L, u, f, r, partials, done, s);
+    } else {
+        nb = launch_residual_cell<P, PO>(L, u, f, r, partials, done, s);
+        if (nb >= 0) return nb;
+    }
     nb = launch_residual_pp<P, PO>(L, u, f, r, partials, done, s);
     if (nb >= 0) return nb;
     Shape sh = sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false);
@@ -409,7 +425,11 @@ int launch_residual(const Lv<P>& L, const typename P::S* u, const typename P::S*
 template <class PF, class P>
 void launch_restrict_smooth(const Lv<P>& Lc, double rho, const typename PF::S* rf,
                             typename P::S* fc, typename P::S* uc, const int* done, cudaStream_t s) {
-    if (launch_restrict_smooth_pcr<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
+    if constexpr (P::id == 0) {
+        if (launch_restrict_smooth_chunk<PF>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
+    } else {
+        if (launch_restrict_smooth_pcr<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
+    }
     // the pipelined kernel copies pairs of fine values: their address must be pair-aligned
     if (((uintptr_t)rf % (2 * sizeof(typename PF::S))) == 0 &&
         launch_restrict_smooth_pp<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0)

@@ -440,8 +440,8 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
     constexpr int PD = 4;
     if (L.nx % 64 || L.ny % 2 || !L.gstack || !Lc.finv || !Lc.fw || !Lc.v) return -1;
     if (Lc.nx * 2 != L.nx || Lc.ny * 2 != L.ny || Lc.nz != L.nz) return -1;
-    // small coarse levels solve their columns by cyclic reduction (k_coarse.cu)
-    if (Lc.pcr && (size_t)Lc.nx * Lc.ny <= (size_t)PCR_MAX_COLS && Lc.nz <= 256) return -1;
+    // small coarse levels solve their columns by cyclic reduction or in chunks (k_coarse.cu, k_chunk.cu)
+    if ((Lc.pcr || Lc.chunkw) && (size_t)Lc.nx * Lc.ny <= (size_t)PCR_MAX_COLS && Lc.nz <= 256) return -1;
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(u) || !al(f)) return -1;
     const size_t smem = sweep_x2_smem<P, 2, PD, MODE_RESTRICT>();

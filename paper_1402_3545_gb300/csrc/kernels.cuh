@@ -103,6 +103,9 @@ struct Lv {
     // 1/b of the decoupled rows; per cell when fac_percol, else one shared table of nz rows
     const typename P::S* pcr = nullptr;
     int pcr_steps = 0;
+    // native FP64 levels of at most CHUNK_MAX_COLS columns: products of w_k = v/m_k over chunks of planes
+    // (k_chunk.cu), else null
+    const typename P::S* chunkw = nullptr;
     // global scratch for the Thomas stacks of the persistent sweep variants (gstack_bytes(nz)
     // bytes, shared by the levels; null: those variants are not used)
     void* gstack = nullptr;
@@ -137,11 +140,12 @@ static constexpr int GS_BLOCKS_PER_SM = 16;
 static constexpr int GS_MAX_NT = 128;
 size_t gstack_bytes(int nz);
 
-// Levels with at most this many columns run the cell-parallel kernels (one thread per cell,
-// the column solve by parallel cyclic reduction): a thread per column leaves the GPU idle there.
+// Levels with at most this many columns run the cell-parallel kernels (one thread per cell, the column
+// solve by parallel cyclic reduction; native FP64: chunks of planes, k_chunk.cu): a thread per column
+// leaves the GPU idle there.
 static constexpr int PCR_MAX_COLS = 4096;
-// Native FP64 levels of at most this many columns cut their columns into chunks of planes: above it a
-// thread per column fills the GPU
+// Native FP64 levels of at most this many columns cut their columns into chunks of planes (k_chunk.cu):
+// above it a thread per column fills the GPU (256^2 x 128: 154 us; 128^2 x 128: 95 us in a cycle against 65 in chunks)
 static constexpr int CHUNK_MAX_COLS = 32768;
 inline int pcr_steps_for(int nz) {
     int s = 0;
@@ -299,6 +303,23 @@ int cell_blocks(size_t n);
 template <class P, class PF>
 int launch_prolongate_x4(int nxc, int nyc, int nz, const typename P::S* uc, typename PF::S* uf, const int* done,
                          cudaStream_t s);
+
+// ---------------------------------------------------------------- launchers (k_chunk.cu)
+// Native FP64 on small levels; -1 where the level has no chunk products (or takes another kernel).
+int chunk_planes(int nz);
+size_t chunk_count(const Lv<PolF64>& L);  // values of Lv::chunkw
+void launch_chunk_products(const Lv<PolF64>& L, double* out, cudaStream_t s);
+int launch_smooth_chunk(const Lv<PolF64>& L, double rho, const double* u, const double* f, double* uo, double* partials,
+                        const int* done, cudaStream_t s);
+int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, double scale, const int* done,
+                            cudaStream_t s);
+template <class PF>
+int launch_restrict_smooth_chunk(const Lv<PolF64>& Lc, double rho, const typename PF::S* rf, double* fc, double* uc,
+                                 const int* done, cudaStream_t s);
+// any level (the caller takes it up to PCR_MAX_COLS columns)
+int residual_chunk_blocks(const Lv<PolF64>& L);
+int launch_residual_chunk(const Lv<PolF64>& L, const double* u, const double* f, double* r, double* partials,
+                          const int* done, cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (k_mg.cu)
 template <class P>
