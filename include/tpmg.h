@@ -24,8 +24,8 @@
  *    arithmetic on the FP32 units (about 2^-47 relative accuracy per operation) and converts at the
  *    boundary through library-owned workspace; TPMG_F64 computes in native FP64.
  *  - `stream` is a cudaStream_t (NULL = the legacy default stream). Every entry point is stream
- *    ordered; only the solvers and tpmg_op_reserve synchronise (solvers: once per iteration, to
- *    read the convergence flag).
+ *    ordered; only the solvers and tpmg_op_reserve synchronise (solvers: at the end, to
+ *    read the convergence flag; with plain launches once per iteration).
  *  - Errors are returned as a tpmg_status, never thrown; nothing aborts the process. A failed
  *    CUDA call yields TPMG_ERR_CUDA and tpmg_last_error() describes it.
  *  - Workspace (coarse levels, ping-pong buffers, precision-conversion buffers, partial sums) is
@@ -171,7 +171,7 @@ typedef struct {
     double rho;      /* relaxation of the block-Jacobi smoother, Eq. (11) */
     double tol;      /* stop when ||f - A u|| / ||f - A u_0|| < tol, Eq. (10) */
     tpmg_precision prec;
-    int use_graph;   /* 1: replay each iteration from a CUDA graph (default), 0: plain launches */
+    int use_graph;   /* 1: the whole iteration loop as one CUDA graph (default), 0: plain launches */
     double timeout_s; /* time limit of every device-side wait (the batched solver's grid barrier);
                          default 1.0 s; when it runs out the solve ends with TPMG_ERR_TIMEOUT */
     int zero_guess;  /* 1: start from u = 0 without reading u (u is then output only), 0: start from

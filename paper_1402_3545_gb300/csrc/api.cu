@@ -4,8 +4,8 @@
 //
 // Solver control lives on the device: the finalize kernels compute the norms, CG's alpha/beta and
 // the convergence decision of Eq. (10) and raise a `done` flag that makes every later kernel of the
-// iteration return at once. One iteration is captured into a CUDA graph and replayed; the host
-// reads the flag once per iteration (one 64-byte device-to-host copy).
+// iteration return at once. The loop runs on the device too: one iteration is captured into the body of a
+// CUDA graph's WHILE node, and the host reads the scalars once, after the solve.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -466,43 +466,73 @@ struct Cycle {
     }
 };
 
-// ---------------------------------------------------------------- graph replay of one iteration
+static tpmg_status read_scalars(tpmg_op* op, cudaStream_t s) {
+    CK(cudaMemcpyAsync(op->sc_host, op->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return TPMG_OK;
+}
+
+// ---------------------------------------------------------------- the iteration loop
+// Runs body (one iteration, ending in a finalize kernel that updates the device scalars) until the
+// scalars say done, and leaves them in op->sc_host. With graphs the loop itself is on the device: the
+// iteration is captured into the body of a WHILE node whose condition the last kernel of the body sets
+// (launch_loop_cond), so a solve is one graph launch and one read of the scalars, not one of each per
+// iteration. The condition is bounded by max_iter as well as by done.
 template <class F>
-static tpmg_status run_iteration(tpmg_op* op, int slot, const std::vector<const void*>& key, bool use_graph,
-                                 cudaStream_t s, F&& body) {
-    if (!use_graph) {
-        body(s);
-        CK(cudaGetLastError());
+static tpmg_status run_loop(tpmg_op* op, const tpmg_params* prm, int slot, const std::vector<const void*>& key,
+                            cudaStream_t s, F&& body) {
+    if (!prm->use_graph) {
+        TRY(read_scalars(op, s));
+        int guard = 0;
+        while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
+            body(s);
+            CK(cudaGetLastError());
+            TRY(read_scalars(op, s));
+        }
         return TPMG_OK;
     }
     GraphCache& gc = op->graphs[slot];
     if (!gc.exec || gc.key != key) {
         if (gc.exec) cudaGraphExecDestroy(gc.exec);
         gc.exec = nullptr;
-        CK(cudaStreamBeginCapture(op->cap_stream, cudaStreamCaptureModeRelaxed));
+        cudaGraph_t graph = nullptr;
+        CK(cudaGraphCreate(&graph, 0));
+        cudaGraphConditionalHandle cond;
+        cudaGraphNode_t first = nullptr, loop = nullptr;
+        cudaGraphNodeParams np = {};
+        cudaError_t e = cudaGraphConditionalHandleCreate(&cond, graph, 0, 0);
+        if (e == cudaSuccess) e = add_loop_cond(graph, &first, cond, op->sc);
+        if (e == cudaSuccess) {
+            np.type = cudaGraphNodeTypeConditional;
+            np.conditional.handle = cond;
+            np.conditional.type = cudaGraphCondTypeWhile;
+            np.conditional.size = 1;
+            e = cudaGraphAddNode(&loop, graph, &first, nullptr, 1, &np);
+        }
         const unsigned long long c0 = launch_counter();
-        body(op->cap_stream);
+        if (e == cudaSuccess) {
+            cudaGraph_t inner = np.conditional.phGraph_out[0], captured = nullptr;
+            e = cudaStreamBeginCaptureToGraph(op->cap_stream, inner, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
+            if (e == cudaSuccess) {
+                body(op->cap_stream);
+                launch_loop_cond(cond, op->sc, op->cap_stream);
+                e = cudaStreamEndCapture(op->cap_stream, &captured);
+            }
+        }
         gc.nkernels = launch_counter() - c0;
         launch_counter() = c0;  // captured launches run only when the graph is replayed
-        cudaGraph_t graph = nullptr;
-        cudaError_t e = cudaStreamEndCapture(op->cap_stream, &graph);
-        if (e != cudaSuccess) return set_err(TPMG_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&gc.exec, graph, 0);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&gc.exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
             gc.exec = nullptr;
-            return set_err(TPMG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+            cudaGetLastError();
+            return set_err(TPMG_ERR_CUDA, std::string("iteration graph: ") + cudaGetErrorString(e));
         }
         gc.key = key;
     }
     CK(cudaGraphLaunch(gc.exec, s));
-    launch_counter() += gc.nkernels;
-    return TPMG_OK;
-}
-
-static tpmg_status read_scalars(tpmg_op* op, cudaStream_t s) {
-    CK(cudaMemcpyAsync(op->sc_host, op->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    TRY(read_scalars(op, s));
+    launch_counter() += 1 + gc.nkernels * (unsigned long long)op->sc_host->iters;
     return TPMG_OK;
 }
 
@@ -551,7 +581,6 @@ static tpmg_status mg_loop(tpmg_op* op, const tpmg_params* prm, typename PF::S* 
     const int nparts = launch_smooth<PF>(LL, prm->rho, A, fL, B, op->partials, done, s);
     launch_finalize_norm(op->partials, nparts, FIN_MG_INIT, op->sc, op->history, nullptr, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         Cycle<PF, PC> c2(op, prm, st, done, lsw);
         c2.u[L] = A;
@@ -566,11 +595,7 @@ static tpmg_status mg_loop(tpmg_op* op, const tpmg_params* prm, typename PF::S* 
     std::vector<const void*> key = {A, fL, B, op->history, (const void*)(size_t)prm->nu_pre,
                                     (const void*)(size_t)prm->nu_post, (const void*)(size_t)prm->n_coarse,
                                     (const void*)(size_t)(prm->rho * 1e12), (const void*)(size_t)lsw};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, PF::id, key, prm->use_graph != 0, s, body));
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, PF::id, key, s, body));
     return TPMG_OK;
 }
 
@@ -590,7 +615,6 @@ static tpmg_status mixed_loop(tpmg_op* op, const tpmg_params* prm, float2* uD, c
     const int nparts = launch_residual<PolDW, PolF32>(LD, uD, fD, r32, op->partials, done, s);
     launch_finalize_norm(op->partials, nparts, FIN_MG_INIT, op->sc, op->history, nullptr, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         void* cur = e;
         void* oth = eb;
@@ -610,11 +634,7 @@ static tpmg_status mixed_loop(tpmg_op* op, const tpmg_params* prm, float2* uD, c
     std::vector<const void*> key = {uD, fD, e, op->history, (const void*)(size_t)prm->nu_pre,
                                     (const void*)(size_t)prm->nu_post, (const void*)(size_t)prm->n_coarse,
                                     (const void*)(size_t)(prm->rho * 1e12), (const void*)(size_t)prm->coarse_bf16};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, 3, key, prm->use_graph != 0, s, body));
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, 3, key, s, body));
     return TPMG_OK;
 }
 
@@ -639,7 +659,6 @@ static tpmg_status cg_loop(tpmg_op* op, const tpmg_params* prm, typename P::S* u
     launch_cg_tridiag<P>(LL, op->sc, r, q, z, op->partials, s);
     launch_cg_beta(op->partials, nb_tri, 1, op->sc, op->history, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         launch_cg_spmv<P>(LL, op->sc, u, p, z, q, op->partials, st);
         launch_cg_alpha(op->partials, nb_spmv, op->sc, st);
@@ -647,11 +666,7 @@ static tpmg_status cg_loop(tpmg_op* op, const tpmg_params* prm, typename P::S* u
         launch_cg_beta(op->partials, nb_tri, 0, op->sc, op->history, st);
     };
     std::vector<const void*> key = {u, f, r, op->history};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, 4 + pid, key, prm->use_graph != 0, s, body));
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, 4 + pid, key, s, body));
     launch_cg_finish<P>(n, op->sc, u, p, s);
     CK(cudaGetLastError());
     return TPMG_OK;
@@ -2685,7 +2700,6 @@ static tpmg_status panel_mg_loop(tpmg_op* op, const tpmg_params* prm, double* A,
     const int nparts = launch_panel_sweep<double>(PANEL_SMOOTH, LL, prm->rho, A, fL, B, op->partials, done, s);
     launch_finalize_norm(op->partials, nparts, FIN_MG_INIT, op->sc, op->history, nullptr, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         PanelCycle<double> c{op, prm, st, done, fL};
         double* cur = c.rest(B, A);
@@ -2696,11 +2710,7 @@ static tpmg_status panel_mg_loop(tpmg_op* op, const tpmg_params* prm, double* A,
     std::vector<const void*> key = {A, fL, B, op->history, (const void*)(size_t)prm->nu_pre,
                                     (const void*)(size_t)prm->nu_post, (const void*)(size_t)prm->n_coarse,
                                     (const void*)(size_t)(prm->rho * 1e12)};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, 7, key, prm->use_graph != 0, s, body));
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, 7, key, s, body));
     return TPMG_OK;
 }
 
@@ -2720,7 +2730,6 @@ static tpmg_status panel_mixed_loop(tpmg_op* op, const tpmg_params* prm, double*
     const int nparts = launch_panel_residual_to_f32(LD, u, f, r32, op->partials, done, s);
     launch_finalize_norm(op->partials, nparts, FIN_MG_INIT, op->sc, op->history, nullptr, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         // first smoothing step from e = 0: e = rho M^{-1} r
         launch_panel_sweep<float>(PANEL_LINESOLVE, L32, prm->rho, r32, nullptr, e, nullptr, done, st);
@@ -2733,11 +2742,7 @@ static tpmg_status panel_mixed_loop(tpmg_op* op, const tpmg_params* prm, double*
     std::vector<const void*> key = {u, f, e, op->history, (const void*)(size_t)prm->nu_pre,
                                     (const void*)(size_t)prm->nu_post, (const void*)(size_t)prm->n_coarse,
                                     (const void*)(size_t)(prm->rho * 1e12)};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, 3, key, prm->use_graph != 0, s, body));  // a panel operator runs no flat mixed solve
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, 3, key, s, body));  // a panel operator runs no flat mixed solve
     return TPMG_OK;
 }
 
@@ -2790,7 +2795,6 @@ static tpmg_status panel_cg_solve(tpmg_op* op, const tpmg_params* prm, const voi
     launch_panel_cg_tridiag(LL, op->sc, r, q, z, op->partials, s);  // alpha = 0: z = M^{-1} r
     launch_cg_beta(op->partials, nb, 1, op->sc, op->history, s);
     CK(cudaGetLastError());
-    TRY(read_scalars(op, s));
     auto body = [&](cudaStream_t st) {
         launch_panel_cg_spmv(LL, op->sc, u, p, z, q, op->partials, st);
         launch_cg_alpha(op->partials, nb, op->sc, st);
@@ -2798,11 +2802,7 @@ static tpmg_status panel_cg_solve(tpmg_op* op, const tpmg_params* prm, const voi
         launch_cg_beta(op->partials, nb, 0, op->sc, op->history, st);
     };
     std::vector<const void*> key = {u, f, r, op->history};
-    int guard = 0;
-    while (!op->sc_host->done && guard++ <= prm->max_iter + 1) {
-        TRY(run_iteration(op, 4, key, prm->use_graph != 0, s, body));  // a panel operator runs no flat CG
-        TRY(read_scalars(op, s));
-    }
+    TRY(run_loop(op, prm, 4, key, s, body));  // a panel operator runs no flat CG
     launch_cg_finish<PolF64>(n, op->sc, u, p, s);
     CK(cudaEventRecord(op->ev1, s));
     CK(cudaGetLastError());

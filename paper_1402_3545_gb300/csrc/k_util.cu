@@ -225,6 +225,25 @@ void launch_scalars_init(Scalars* sc, double tol, int max_iter, cudaStream_t s) 
     k_scalars_init<<<1, 1, 0, s>>>(sc, tol, max_iter);
     note_launch();
 }
+// condition of a solve's WHILE node: another iteration unless done; pad counts the evaluations, so that the
+// loop ends whatever the body does
+__global__ void k_loop_cond(cudaGraphConditionalHandle cond, Scalars* sc) {
+    const bool go = !*(volatile int*)&sc->done && sc->pad <= sc->max_iter;
+    ++sc->pad;
+    cudaGraphSetConditional(cond, go ? 1u : 0u);
+}
+void launch_loop_cond(cudaGraphConditionalHandle cond, Scalars* sc, cudaStream_t s) {
+    k_loop_cond<<<1, 1, 0, s>>>(cond, sc);
+    note_launch();
+}
+cudaError_t add_loop_cond(cudaGraph_t graph, cudaGraphNode_t* node, cudaGraphConditionalHandle cond, Scalars* sc) {
+    void* args[] = {&cond, &sc};
+    cudaKernelNodeParams kp = {};
+    kp.func = (void*)k_loop_cond;
+    kp.gridDim = kp.blockDim = dim3(1);
+    kp.kernelParams = args;
+    return cudaGraphAddKernelNode(node, graph, nullptr, 0, &kp);
+}
 void launch_set_ab(Scalars* sc, double alpha, double beta, cudaStream_t s) {
     k_set_ab<<<1, 1, 0, s>>>(sc, alpha, beta);
     note_launch();

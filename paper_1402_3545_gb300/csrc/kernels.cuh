@@ -206,7 +206,7 @@ struct Scalars {
     double tol;
     double alpha, beta, kappa;  // CG: step, direction update, <r,z>
     double last_norm;
-    int iters, max_iter, done, converged, nonfinite, pad;
+    int iters, max_iter, done, converged, nonfinite, pad;  // pad: evaluations of the loop's condition
 };
 
 // process-wide count of kernel launches issued by the library (k_util.cu)
@@ -449,6 +449,9 @@ void launch_cg_alpha(const double* partials, int nparts, Scalars* sc, cudaStream
 void launch_cg_beta(const double* partials, int nparts, int init, Scalars* sc, double* history,
                     cudaStream_t s);
 void launch_scalars_init(Scalars* sc, double tol, int max_iter, cudaStream_t s);
+// the kernel that sets the condition of a solve's WHILE node, as a launch and as a graph node
+void launch_loop_cond(cudaGraphConditionalHandle cond, Scalars* sc, cudaStream_t s);
+cudaError_t add_loop_cond(cudaGraph_t graph, cudaGraphNode_t* node, cudaGraphConditionalHandle cond, Scalars* sc);
 void launch_set_ab(Scalars* sc, double alpha, double beta, cudaStream_t s);
 // dst = src (n elements of P's storage) unless *done is set
 template <class P>
