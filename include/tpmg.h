@@ -357,8 +357,9 @@ tpmg_status tpmg_fcg_solve(tpmg_op* op, tpmg_nn* nn, const float* aux, const tpm
  *
  * Scratch: one partial sum per thread block in a fixed file-scope device array of
  * TPMG_NOALLOC_MAX_BLOCKS doubles (512 KB), held by every GPU that loads the library until the
- * process exits. The number of blocks is that of the residual kernel the grid takes: at most 1024
- * on grids of at most 4096 columns; on grids with nx a multiple of 64, even ny and 16-byte aligned
+ * process exits. The number of blocks is that of the residual kernel the grid takes: at most 16
+ * per 128 columns (or 1024) on grids of at most 32768 columns; 4 per 128 columns on grids of at most 131072 columns with
+ * nx not a multiple of 32; on grids with nx a multiple of 64, even ny and 16-byte aligned
  * u, f, r (the two-column persistent sweep) at most 16 per SM whatever the size; otherwise
  * (nx/32)*(ny/4) blocks for nx a multiple of 32 and ny of 4, else one per 32 x 4 columns rounded
  * up. A call needing more than TPMG_NOALLOC_MAX_BLOCKS (above about 8.4 million columns on the

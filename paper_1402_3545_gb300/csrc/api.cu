@@ -285,7 +285,7 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid) {
         // small levels: factor products of the chunked columns (native FP64), parallel-cyclic-reduction
         // factors of the cell-parallel kernels (the other policies)
         const size_t cols = (size_t)op->g.lnx[l] * op->g.lny[l];
-        if (pid == 0 && cols <= (size_t)CHUNK_MAX_COLS) {
+        if (pid == 0 && chunk_level(op->g.lnx[l], op->g.lny[l])) {
             const Lv<PolF64> L = level_view<PolF64>(op, l);
             TRY(dalloc((void**)&op->chunkw[l], chunk_count(L) * eb));
             launch_chunk_products(L, op->chunkw[l], 0);

@@ -1,10 +1,10 @@
-// k_chunk.cu -- native FP64 kernels of the small levels (128 x 256 columns and below): columns cut into
-// chunks of planes.
+// k_chunk.cu -- native FP64 kernels of the small levels (128 x 256 columns and below) and of grids that fit no
+// tile: columns cut into chunks of planes; and the pointwise Residual of every policy.
 //
 // With a thread per column these levels leave most of the chip waiting on 2 nz dependent FP64 operations
 // (about 80 cycles each); cyclic reduction (k_coarse.cu, the other policies) shortens the chain to log2 nz
 // steps but takes 2 log2(nz) + 1 operations per cell for the solve alone on a pipe that issues 1/74 of the
-// FP32 rate. Here a block owns 8 columns, each cut into 16 chunks of PP planes with a thread per chunk, and
+// FP32 rate. Here a block owns 8 columns (2 or 4 on the smallest levels), each cut into 16 chunks of PP planes with a thread per chunk, and
 // both recurrences of the Thomas algorithm, y_k = b_k / m_k + w_k y_{k-1} and x_k = y_k + w_k x_{k+1}
 // (w_k = v / m_k), run twice per chunk: from zero, for the value the chunk hands on, and, once the carried
 // value is known (the earlier chunks' values chained by the chunks' products of w_k), for the chunk's own
@@ -19,7 +19,7 @@ namespace tpmg {
 
 namespace {
 
-constexpr int CB = 8, CH = 16;  // columns and chunks of a block
+constexpr int CH = 16;  // chunks of a column
 
 __device__ __forceinline__ int kwrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
@@ -40,6 +40,22 @@ __device__ __forceinline__ CCol chunk_col(int nx, int ny, int col) {
     q.s = (size_t)kwrap(q.j - 1, ny) * nx + q.i;
     q.n = (size_t)kwrap(q.j + 1, ny) * nx + q.i;
     return q;
+}
+// The value carried into chunk w of a column (lane = 2 w + column) from what the chunks before (UP) or behind
+// it hand on, e, and their products of multipliers, cw (0 beyond the column)
+template <bool UP>
+__device__ __forceinline__ double chunk_scan(double e, double cw, int w) {
+#pragma unroll
+    for (int d = 1; d < CH; d *= 2) {
+        const double ee = UP ? __shfl_up_sync(0xffffffffu, e, 2 * d) : __shfl_down_sync(0xffffffffu, e, 2 * d);
+        const double cc = UP ? __shfl_up_sync(0xffffffffu, cw, 2 * d) : __shfl_down_sync(0xffffffffu, cw, 2 * d);
+        if (UP ? w >= d : w + d < CH) {
+            e = fma(cw, ee, e);
+            cw *= cc;
+        }
+    }
+    const double c = UP ? __shfl_up_sync(0xffffffffu, e, 2) : __shfl_down_sync(0xffffffffu, e, 2);
+    return (UP ? w == 0 : w == CH - 1) ? 0.0 : c;
 }
 // f + cx (u_w + u_e) + cy (u_s + u_n) (sweep_rhs's form)
 __device__ __forceinline__ double chunk_rhs(const double* __restrict__ u, const CCol& q, double fk, double cx, double cy) {
@@ -65,7 +81,7 @@ __global__ void __launch_bounds__(128) k_chunk_products(Lv<PolF64> L, double* __
 // MODE 0 Smooth: out = u + coef M^{-1}(f - A u); NORM with the partial sums of ||f - A u||^2, without them in
 // the form (1 - coef) u + coef M^{-1}(f + H u). MODE 1 line solve: out = coef M^{-1} u. MODE 2 RestrictSmooth:
 // fc = R u (u the fine residual in PF's storage), out = coef M^{-1} fc.
-template <class PF, int MODE, int PP, bool NORM>
+template <class PF, int MODE, int PP, bool NORM, int CB>
 __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, const typename PF::S* __restrict__ uin,
                                                    const double* __restrict__ f, double* __restrict__ out,
                                                    double* __restrict__ fc, double* partials, const int* done) {
@@ -124,21 +140,31 @@ __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, co
     }
 #pragma unroll
     for (int p = 0; p < PP; ++p) y = fma(wk[p], y, a[p]);
-    sy[w][tx] = y;
     const double* cw = L.chunkw + fo;  // the chunks' products
     const int last = (nz - 1) / PP;
-    __syncthreads();
-    if (w == 0) {  // one thread per column: each chunk's carried value in the place of what it hands on
-        y = 0.0;
-#pragma unroll 4
-        for (int c = 0; c <= last; ++c) {
-            const double e = sy[c][tx];
-            sy[c][tx] = y;
-            y = fma(__ldg(cw + (size_t)c * fs), y, e);
+    double cwc = 0.0, pw[CB == 2 ? 1 : CH];
+    if constexpr (CB == 2) {  // a warp holds all chunks of its two columns: a scan of four steps
+        if (w <= last) cwc = __ldg(cw + (size_t)w * fs);
+        y = chunk_scan<true>(y, cwc, w);
+    } else {
+        if (w == 0) {
+#pragma unroll
+            for (int c = 0; c < CH; ++c) pw[c] = __ldg(cw + (size_t)(c <= last ? c : 0) * fs);
         }
+        sy[w][tx] = y;
+        __syncthreads();
+        if (w == 0) {  // one thread per column: each chunk's carried value in the place of what it hands on
+            y = 0.0;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const double e = sy[c][tx];
+                sy[c][tx] = y;
+                y = fma(pw[c], y, e);
+            }
+        }
+        __syncthreads();
+        y = sy[w][tx];
     }
-    __syncthreads();
-    y = sy[w][tx];
 #pragma unroll
     for (int p = 0; p < PP; ++p) {
         y = fma(wk[p], y, a[p]);
@@ -147,24 +173,28 @@ __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, co
     double x = 0.0;
 #pragma unroll
     for (int p = PP - 1; p >= 0; --p) x = fma(wk[p], x, a[p]);
-    sx[w][tx] = x;
     double uo[MODE == 0 ? PP : 1];
     if (MODE == 0) {
 #pragma unroll
         for (int p = 0; p < PP; ++p) uo[p] = __ldg(u + (size_t)(k0 + p < nz ? k0 + p : nz - 1) * pl + q.c);
     }
-    __syncthreads();
-    if (w == 0) {
-        x = 0.0;
-#pragma unroll 4
-        for (int c = last; c >= 0; --c) {
-            const double e = sx[c][tx];
-            sx[c][tx] = x;
-            x = fma(__ldg(cw + (size_t)c * fs), x, e);
+    if constexpr (CB == 2) {
+        x = chunk_scan<false>(x, cwc, w);
+    } else {
+        sx[w][tx] = x;
+        __syncthreads();
+        if (w == 0) {
+            x = 0.0;
+#pragma unroll
+            for (int c = CH - 1; c >= 0; --c) {  // (chunks beyond the column hand on zero)
+                const double e = sx[c][tx];
+                sx[c][tx] = x;
+                x = fma(pw[c], x, e);
+            }
         }
+        __syncthreads();
+        x = sx[w][tx];
     }
-    __syncthreads();
-    x = sx[w][tx];
     const double keep = 1.0 - coef;
 #pragma unroll
     for (int p = PP - 1; p >= 0; --p) {
@@ -177,32 +207,43 @@ __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, co
     }
 }
 
-// Residual, planes blockIdx.y * pz .. of a column per thread: seven operations per cell
-__global__ void __launch_bounds__(128) k_chunk_residual(Lv<PolF64> L, const double* __restrict__ u,
-                                                        const double* __restrict__ f, double* __restrict__ r,
-                                                        double* partials, const int* done, int pz) {
+// Residual, pointwise: planes blockIdx.y * pz .. of a column per thread, the sweeps' arithmetic in its order
+// (sweep_residual), so the same bits as their Residual. On levels of few tiles the marching Residual has one
+// chain per column: 128^2 x 128 FP64 110 us, 34 here; FP32 17 / 8.7; double-word 78 / 62
+// (both with its conversions).
+template <class P, class PO>
+__global__ void __launch_bounds__(128) k_residual_point(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u,
+                                                        const typename P::S* __restrict__ f,
+                                                        typename PO::S* __restrict__ r, double* partials,
+                                                        const int* done, int pz) {
+    typedef typename P::R R;
     if (done && *(volatile const int*)done) return;
     const CCol q = chunk_col(L.nx, L.ny, blockIdx.x * 128 + threadIdx.x);
     const size_t pl = (size_t)L.nx * L.ny;
     const int nz = L.nz, k0 = blockIdx.y * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
-    double acc = 0.0;
+    typename P::Acc acc = 0, cmp = 0;
     if (q.act && k0 < k1) {
-        const double vv = __ldg(L.v + q.c), dh = 1.0 + 2.0 * L.cx + 2.0 * L.cy, dh1 = dh + vv, dh2 = dh1 + vv;
-        double um = k0 > 0 ? __ldg(u + (size_t)(k0 - 1) * pl + q.c) : 0.0, uc = __ldg(u + (size_t)k0 * pl + q.c);
+        const R vv = P::ld(L.v, q.c), dh1 = P::add(K.dh, vv), dh2 = P::add(dh1, vv);
+        const bool iso = K.iso != 0;
+        R um = k0 > 0 ? P::ld(u, (size_t)(k0 - 1) * pl + q.c) : P::zero(), uc = P::ld(u, (size_t)k0 * pl + q.c);
 #pragma unroll 4
         for (int k = k0; k < k1; ++k) {
-            const size_t b = (size_t)k * pl, id = b + q.c;
-            const double up = k + 1 < nz ? __ldg(u + id + pl) : 0.0;
-            const double dg = nz == 1 ? dh : (k == 0 || k == nz - 1 ? dh1 : dh2);
-            const double rk = fma(vv, um + up, fma(-dg, uc, chunk_rhs(u + b, q, __ldg(f + id), L.cx, L.cy)));
-            r[id] = rk;
-            if (partials) acc = fma(rk, rk, acc);
+            const size_t b = (size_t)k * pl;
+            const R up = k + 1 < nz ? P::ld(u, b + pl + q.c) : P::zero();
+            const R dg = nz == 1 ? K.dh : (k == 0 || k == nz - 1 ? dh1 : dh2);
+            const R rk = sweep_residual<P>(P::ld(f, b + q.c), dg, uc, P::ld(u, b + q.w), P::ld(u, b + q.e),
+                                           P::ld(u, b + q.s), P::ld(u, b + q.n), um, up, K.cx, K.cy, vv, iso);
+            if constexpr (PO::id == P::id)
+                PO::st(reinterpret_cast<typename PO::S*>(r), b + q.c, rk);
+            else
+                PO::st(r, b + q.c, PO::from_f(P::to_f(rk)));
+            if (partials) P::acc_dot(acc, cmp, rk, rk);
             um = uc;
             uc = up;
         }
     }
     if (partials) {
-        const double s = block_sum(acc);
+        const double s = block_sum(P::acc_get(acc, cmp));
         if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
 }
@@ -221,17 +262,25 @@ void launch_chunk_products(const Lv<PolF64>& L, double* out, cudaStream_t s) {
     note_launch();
 }
 
-template <class PF, int MODE, int PP>
-static int run_chunk(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
-                     double* partials, const int* done, cudaStream_t s) {
+template <class PF, int MODE, int PP, int CB>
+static int run_chunk_cb(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
+                        double* partials, const int* done, cudaStream_t s) {
     const int nb = (L.nx * L.ny + CB - 1) / CB;
     const dim3 b(CB, CH);
     if (MODE == 0 && partials)
-        k_chunk<PF, MODE, PP, MODE == 0><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
+        k_chunk<PF, MODE, PP, MODE == 0, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
     else
-        k_chunk<PF, MODE, PP, false><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
+        k_chunk<PF, MODE, PP, false, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
     note_launch();
     return nb;
+}
+// columns per block: 8, fewer where the blocks would not reach every SM
+template <class PF, int MODE, int PP>
+static int run_chunk(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
+                     double* partials, const int* done, cudaStream_t s) {
+    if (L.nx * L.ny <= 512) return run_chunk_cb<PF, MODE, PP, 2>(L, coef, u, f, out, fc, partials, done, s);
+    if (L.nx * L.ny <= 2048) return run_chunk_cb<PF, MODE, PP, 4>(L, coef, u, f, out, fc, partials, done, s);
+    return run_chunk_cb<PF, MODE, PP, 8>(L, coef, u, f, out, fc, partials, done, s);
 }
 template <class PF, int MODE>
 static int chunk_sweep(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
@@ -246,8 +295,9 @@ static int chunk_sweep(const Lv<PolF64>& L, double coef, const typename PF::S* u
 
 int launch_smooth_chunk(const Lv<PolF64>& L, double rho, const double* u, const double* f, double* uo, double* partials,
                         const int* done, cudaStream_t s) {
-    // above PCR_MAX_COLS columns a tile variant that was chosen for the level takes precedence
-    if ((size_t)L.nx * L.ny > (size_t)PCR_MAX_COLS && L.variant >= 0) return -1;
+    // above PCR_MAX_COLS columns a tile variant that was chosen for the level takes precedence (where the
+    // level has tiles at all)
+    if ((size_t)L.nx * L.ny > (size_t)PCR_MAX_COLS && L.variant >= 0 && L.nx % 32 == 0) return -1;
     return chunk_sweep<PolF64, 0>(L, rho, u, f, uo, nullptr, partials, done, s);
 }
 int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, double scale, const int* done, cudaStream_t s) {
@@ -256,8 +306,9 @@ int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, dou
 template <class PF>
 int launch_restrict_smooth_chunk(const Lv<PolF64>& Lc, double rho, const typename PF::S* rf, double* fc, double* uc,
                                  const int* done, cudaStream_t s) {
-    // larger coarse levels: the column sweep, whose values the fused Residual + RestrictSmooth reproduces
-    if ((size_t)Lc.nx * Lc.ny > (size_t)PCR_MAX_COLS) return -1;
+    // larger coarse levels with tiles: the column sweep, whose values the fused Residual + RestrictSmooth
+    // reproduces
+    if ((size_t)Lc.nx * Lc.ny > (size_t)PCR_MAX_COLS && Lc.nx % 32 == 0) return -1;
     return chunk_sweep<PF, 2>(Lc, rho, rf, nullptr, uc, fc, nullptr, done, s);
 }
 template int launch_restrict_smooth_chunk<PolF64>(const Lv<PolF64>&, double, const double*, double*, double*, const int*,
@@ -265,20 +316,40 @@ template int launch_restrict_smooth_chunk<PolF64>(const Lv<PolF64>&, double, con
 template int launch_restrict_smooth_chunk<PolDW>(const Lv<PolF64>&, double, const float2*, double*, double*, const int*,
                                                  cudaStream_t);
 
-// planes per thread of the residual: at most 1024 blocks on PCR_MAX_COLS columns
-static int residual_planes(int nz) { return nz > 128 ? (nz + 31) / 32 : 4; }
+// planes per thread of the residual: at most 16 blocks per 128 columns, or 1024, on small levels (room for one
+// partial sum per 8 columns, and for 1216, max_partials), 4 on larger ones, where the columns alone fill the GPU
+static int residual_planes(int nx, int ny, int nz) {
+    if ((size_t)nx * ny > (size_t)CHUNK_MAX_COLS) return (nz + 3) / 4;
+    const int four = (nx * ny + 127) / 128 * ((nz + 3) / 4);  // blocks of four planes per thread
+    return four > 1024 ? (nz + 15) / 16 : 4;
+}
 
-int residual_chunk_blocks(const Lv<PolF64>& L) {
-    const int pz = residual_planes(L.nz);
+template <class P>
+int residual_point_blocks(const Lv<P>& L) {
+    const int pz = residual_planes(L.nx, L.ny, L.nz);
     return (L.nx * L.ny + 127) / 128 * ((L.nz + pz - 1) / pz);
 }
-int launch_residual_chunk(const Lv<PolF64>& L, const double* u, const double* f, double* r, double* partials,
-                          const int* done, cudaStream_t s) {
-    const int pz = residual_planes(L.nz);
+template <class P, class PO>
+int launch_residual_point(const Lv<P>& L, const typename P::S* u, const typename P::S* f, typename PO::S* r,
+                          double* partials, const int* done, cudaStream_t s) {
+    const int pz = residual_planes(L.nx, L.ny, L.nz);
     const dim3 g((L.nx * L.ny + 127) / 128, (L.nz + pz - 1) / pz);
-    k_chunk_residual<<<g, 128, 0, s>>>(L, u, f, r, partials, done, pz);
+    k_residual_point<P, PO><<<g, 128, 0, s>>>(L, sweep_k<P>(L.cx, L.cy, 1.0), u, f, r, partials, done, pz);
     note_launch();
     return (int)(g.x * g.y);
 }
+#define TPMG_POINT_INST(P, PO)                                                                              \
+    template int launch_residual_point<P, PO>(const Lv<P>&, const P::S*, const P::S*, PO::S*, double*, const int*, \
+                                              cudaStream_t);
+TPMG_POINT_INST(PolF64, PolF64)
+TPMG_POINT_INST(PolF32, PolF32)
+TPMG_POINT_INST(PolF32B, PolF32B)
+TPMG_POINT_INST(PolDW, PolDW)
+TPMG_POINT_INST(PolDW, PolF32)
+TPMG_POINT_INST(PolF64, PolF32)
+template int residual_point_blocks<PolF64>(const Lv<PolF64>&);
+template int residual_point_blocks<PolF32>(const Lv<PolF32>&);
+template int residual_point_blocks<PolF32B>(const Lv<PolF32B>&);
+template int residual_point_blocks<PolDW>(const Lv<PolDW>&);
 
 }  // namespace tpmg

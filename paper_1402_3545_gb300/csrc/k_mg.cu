@@ -349,7 +349,7 @@ int max_partials(int nx, int ny) {
     const int col_kernels = ((nx + TX - 1) / TX) * ny;
     // small levels: at most one block per column; chunked columns (native FP64): one per 8 columns. A level
     // below the finest has a quarter of its columns or fewer, so that the finest level's count covers it.
-    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (nx * ny <= CHUNK_MAX_COLS ? (nx * ny + 7) / 8 : 0);
+    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (chunk_level(nx, ny) ? (nx * ny + 127) / 128 * 16 : 0);
     return col_kernels > cell_kernels ? col_kernels : cell_kernels;
 }
 
@@ -394,13 +394,20 @@ int launch_smooth(const Lv<P>& L, double rho, const typename P::S* u, const type
     note_launch();
     return sh.nblocks();
 }
+// Where the Residual runs pointwise: native FP64 on every level up to CHUNK_MAX_COLS columns, up to four times
+// that without tiles; the other policies on the levels between the cell kernels' and that size whose tiles
+// (residual_pp_blocks) it replaces bit for bit.
+template <class P, class PO>
+static bool residual_pointwise(const Lv<P>& L, const typename P::S* u, const typename P::S* f, const typename PO::S* r) {
+    const size_t cols = (size_t)L.nx * L.ny;
+    if (P::id == 0 && PO::id == 0) return cols <= (size_t)CHUNK_MAX_COLS || (L.nx % 32 != 0 && cols <= 4 * (size_t)CHUNK_MAX_COLS);
+    return cols > (size_t)PCR_MAX_COLS && cols <= (size_t)CHUNK_MAX_COLS && L.nx % 32 == 0 && (L.ny % 4 == 0 || (L.nx % 64 == 0 && L.ny % 2 == 0));
+}
 template <class P, class PO>
 int residual_launch_blocks(const Lv<P>& L, const typename P::S* u, const typename P::S* f, typename PO::S* r) {
-    // launch_residual's three choices in its order: pointwise, plane-pipelined, one thread per column
-    if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) {
-        if constexpr (P::id == 0 && PO::id == 0) return residual_chunk_blocks(L);
-        return cell_blocks((size_t)L.nx * L.ny * L.nz);
-    }
+    // launch_residual's choices in its order: pointwise, plane-pipelined, one thread per column
+    if (residual_pointwise<P, PO>(L, u, f, r)) return residual_point_blocks(L);
+    if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) return cell_blocks((size_t)L.nx * L.ny * L.nz);
     const int nb = residual_pp_blocks<P, PO>(L, u, f, r);
     if (nb >= 0) return nb;
     return sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false).nblocks();
@@ -408,10 +415,9 @@ int residual_launch_blocks(const Lv<P>& L, const typename P::S* u, const typenam
 template <class P, class PO>
 int launch_residual(const Lv<P>& L, const typename P::S* u, const typename P::S* f,
                     typename PO::S* r, double* partials, const int* done, cudaStream_t s) {
-    int nb = -1;
-    if constexpr (P::id == 0 && PO::id == 0) {
-        if ((size_t)L.nx * L.ny <= (size_t)PCR_MAX_COLS) return launch_residual_chunk(L, u, f, r, partials, done, s);
-    } else {
+    if (residual_pointwise<P, PO>(L, u, f, r)) return launch_residual_point<P, PO>(L, u, f, r, partials, done, s);
+    int nb;
+    if constexpr (P::id != 0 || PO::id != 0) {  // (native FP64's small levels are pointwise above)
         nb = launch_residual_cell<P, PO>(L, u, f, r, partials, done, s);
         if (nb >= 0) return nb;
     }

@@ -30,7 +30,7 @@ namespace tpmg {
 
 namespace {
 
-constexpr int CB = 8, CH = 16;  // columns and chunks of a block of the chunked sweeps
+constexpr int CH = 16;  // chunks of a column in the chunked sweeps
 
 template <class T>
 struct PCol {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, cons
 // 2 nz dependent ones: on 64^2 x 128 a Smooth took 186 us with a thread per column.
 // MODE 0 Smooth, 2 line solve (u the right-hand side), 4 RestrictSmooth (u the fine residual r_f:
 // f_c = sum of the children to fc, out = coef M^{-1} f_c).
-template <int MODE, int PP, bool NORM>
+template <int MODE, int PP, bool NORM, int CB>
 __global__ void __launch_bounds__(CB * CH) k_panel_chunk(PanelLv L, double coef, const double* __restrict__ u,
                                                          const double* __restrict__ f, double* out,
                                                          double* __restrict__ fc, double* partials, const int* done) {
@@ -530,15 +530,23 @@ static int point_planes(int nx, int ny) { return (size_t)nx * ny > 65536 ? 16 : 
 
 // The chunked sweep where the level has its chunk products (PanelLvT::wf). Returns the number of blocks, or
 // -1 where it does not apply.
+template <int MODE, int PP, int CB>
+static int run_panel_chunk_cb(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
+                              double* partials, const int* done, cudaStream_t s) {
+    const int nb = (L.nx * L.ny + CB - 1) / CB;
+    const dim3 b(CB, CH);
+    if (MODE == 0 && partials) k_panel_chunk<MODE, PP, MODE == 0, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
+    else k_panel_chunk<MODE, PP, false, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
+    note_launch();
+    return nb;
+}
+// columns per block: 8, fewer where the blocks would not reach every SM
 template <int MODE, int PP>
 static int run_panel_chunk(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
                            double* partials, const int* done, cudaStream_t s) {
-    const int nb = (L.nx * L.ny + CB - 1) / CB;
-    const dim3 b(CB, CH);
-    if (MODE == 0 && partials) k_panel_chunk<MODE, PP, MODE == 0><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
-    else k_panel_chunk<MODE, PP, false><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
-    note_launch();
-    return nb;
+    if (L.nx * L.ny <= 512) return run_panel_chunk_cb<MODE, PP, 2>(L, coef, u, f, out, fc, partials, done, s);
+    if (L.nx * L.ny <= 2048) return run_panel_chunk_cb<MODE, PP, 4>(L, coef, u, f, out, fc, partials, done, s);
+    return run_panel_chunk_cb<MODE, PP, 8>(L, coef, u, f, out, fc, partials, done, s);
 }
 template <int MODE>
 static int panel_chunk(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,

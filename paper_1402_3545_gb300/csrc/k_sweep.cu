@@ -415,6 +415,11 @@ static int run_sweep_x2(const Lv<P>& L, double coef, const typename P::S* u, con
     return nb;
 }
 
+// policies with whole-column tiles in shared memory (sweep_tile.cuh)
+template <class P>
+constexpr bool tile_policy() {
+    return std::is_same<P, PolF32>::value || std::is_same<P, PolDW>::value;
+}
 // ---------------------------------------------------------------- Residual + RestrictSmooth, fused
 // One pass over the fine level L: r = f - A u per fine cell (not stored), f_c = R r and
 // u_c = rho M_c^{-1} f_c on the coarse level Lc (sweep_x2_tiles in MODE_RESTRICT). Per fine cell it
@@ -444,6 +449,15 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
     if ((Lc.pcr || Lc.chunkw) && (size_t)Lc.nx * Lc.ny <= (size_t)PCR_MAX_COLS && Lc.nz <= 256) return -1;
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(u) || !al(f)) return -1;
+    // whole-column tiles (us, tile / marching): FP32 everywhere (1024 x 512 x 64 83 / 134, 512^2 x 128 83-87 /
+    // 126-132, 256^2 x 128 17-19 / 62); double-word, whose arithmetic rather than the chain bounds large levels,
+    // where the marching form leaves the GPU idle (with conversions: 256 x 72 x 128 83 / 131, 256^2 x 128
+    // 233-239 / 256-264, 384 x 256 347 / 351, but 512^2 x 128 854 / 834 and 384 x 256 x 8 38 / 36)
+    if constexpr (tile_policy<P>())
+        if (P::id == 1 || (L.nx * L.ny <= 98304 && L.nz >= 16)) {
+            const int nb = launch_restrict_tile<P>(L, Lc, rho, u, f, fc, uc, done, s);
+            if (nb >= 0) return nb;
+        }
     const size_t smem = sweep_x2_smem<P, 2, PD, MODE_RESTRICT>();
     auto kern = k_residual_restrict_x2<P, PD>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -468,7 +482,7 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
 // two columns per thread and L2 eviction hints (k_sweep_x2; 5-7); the autotuner (tpmg_autotune)
 // times them per level and stores its choice in Lv::variant. In FP32 and double-word variant 0 is the
 // whole-column tile in shared memory (sweep_tile.cuh) where the level takes it. An untuned level takes
-// that where smooth_tile_pays, else variant 6 (double-word) or 8, 5 (FP32) where the four- or two-column
+// that where tile_pays, else variant 6 (double-word) or 8, 5 (FP32) where the four- or two-column
 // form applies (nx % 128 or 64 == 0, aligned fields), else variant 3; in native FP64, variant 3.
 template <class P>
 struct SmoothVariants;
@@ -485,11 +499,6 @@ struct SmoothVariants<PolDW> {
     static constexpr int TY[3] = {1, 2, 2};
 };
 
-// policies with whole-column tiles in shared memory (sweep_tile.cuh)
-template <class P>
-constexpr bool tile_policy() {
-    return std::is_same<P, PolF32>::value || std::is_same<P, PolDW>::value;
-}
 // Where an untuned level smooths on whole columns in shared memory, from both sides' times over 15
 // horizontal sizes, nz = 8 .. 128 and both kinds of lambda^2 (tile / best sweep with its stack in L2, us):
 //  - below 16 planes the sweeps have no chain to speak of: FP32 512^2 x 8 13.5 / 12.2;
@@ -500,7 +509,7 @@ constexpr bool tile_policy() {
 //    only levels too small to fill the GPU gain: FP32 256^2 x 128 42 / 46, 448 x 256 62 / 67, but 512 x 256
 //    76 / 71; double-word 128^2 x 128 90 / 96, 160^2 136 / 143, but 256^2 319 / 265.
 template <class P>
-static bool smooth_tile_pays(const Lv<P>& L) {
+bool tile_pays(const Lv<P>& L) {
     const size_t cols = (size_t)L.nx * L.ny;
     if (L.nz < 16) return false;
     if (P::id == 1) return !L.fac_percol || cols < 131072;
@@ -512,7 +521,7 @@ static int smooth_dispatch(const Lv<P>& L, double rho, const typename P::S* u, c
                            typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
     int v = L.variant;
     if constexpr (tile_policy<P>())
-        if (v == 0 || ((v < 0 || v >= TPMG_NUM_VARIANTS) && smooth_tile_pays(L))) {
+        if (v == 0 || ((v < 0 || v >= TPMG_NUM_VARIANTS) && tile_pays(L))) {
             const int nb = launch_sweep_tile<P, MODE>(L, rho, u, f, uo, partials, done, s);
             if (nb >= 0) return nb;
         }
@@ -605,7 +614,7 @@ int launch_line_solve_pp(const Lv<P>& L, const typename P::S* b, typename P::S* 
     if constexpr (tile_policy<P>())
         // (the line solve has no stencil to form: it gains wherever the Smooth does, in FP32 on all levels of
         // 16 planes and more: 1024^2 x 128 166 us / 349, 128^2 x 128 10 / 60, 512^2 x 128 varying 77 / 77)
-        if (smooth_tile_pays(L) || (P::id == 1 && L.nz >= 16)) {
+        if (tile_pays(L) || (P::id == 1 && L.nz >= 16)) {
             const int nb = launch_sweep_tile<P, MODE_LINESOLVE>(L, scale, b, nullptr, x, nullptr, done, s);
             if (nb >= 0) return nb;
         }
@@ -760,6 +769,9 @@ int launch_restrict_smooth_pp(const Lv<P>& Lc, double rho, const typename PF::S*
     note_launch();
     return 1;
 }
+
+template bool tile_pays<PolF32>(const Lv<PolF32>&);
+template bool tile_pays<PolDW>(const Lv<PolDW>&);
 
 #define TPMG_SWEEP_INST(P)                                                                                  \
     template void launch_factors<P>(const Lv<P>&, P::S*, P::S*, int, cudaStream_t);                         \

@@ -144,9 +144,10 @@ size_t gstack_bytes(int nz);
 // solve by parallel cyclic reduction; native FP64: chunks of planes, k_chunk.cu): a thread per column
 // leaves the GPU idle there.
 static constexpr int PCR_MAX_COLS = 4096;
-// Native FP64 levels of at most this many columns cut their columns into chunks of planes (k_chunk.cu):
-// above it a thread per column fills the GPU (256^2 x 128: 154 us; 128^2 x 128: 95 us in a cycle against 65 in chunks)
+// Native FP64 levels of at most this many columns cut their columns into chunks of planes (k_chunk.cu), and so
+// do larger ones whose nx has no 32-column tiles; above it a thread per column fills the GPU (256^2 x 128: 154 us; 128^2 x 128: 95 us in a cycle against 65 in chunks)
 static constexpr int CHUNK_MAX_COLS = 32768;
+inline bool chunk_level(int nx, int ny) { return (size_t)nx * ny <= (size_t)CHUNK_MAX_COLS || nx % 32 != 0; }
 inline int pcr_steps_for(int nz) {
     int s = 0;
     while ((1 << s) < nz) ++s;
@@ -252,6 +253,8 @@ int launch_line_solve_x4(const Lv<PolF32>& L, const float* b, float* x, double s
 // Smooth and line solve on whole columns in shared memory (sweep_tile.cuh; F32, DW): nx a
 // multiple of 512 bytes (256 with even ny, 128 with ny a multiple of 4), nz <= 128, 16-byte aligned fields,
 // else -1. MODE as in sweep_x2.cuh
+template <class P>
+bool tile_pays(const Lv<P>& L);  // where an untuned level smooths on such tiles (k_sweep.cu)
 template <class P, int MODE>
 int launch_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f, typename P::S* out,
                       double* partials, const int* done, cudaStream_t s);
@@ -269,6 +272,11 @@ template <class P>
 int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const typename P::S* u,
                              const typename P::S* f, typename P::S* fc, typename P::S* uc, const int* done,
                              cudaStream_t s);
+// the same on whole-column tiles (k_restrict_tile.cu; F32 and DW): fine nx a multiple of 512 bytes, even ny,
+// 16-byte aligned fields, else -1
+template <class P>
+int launch_restrict_tile(const Lv<P>& L, const Lv<P>& Lc, double rho, const typename P::S* u, const typename P::S* f,
+                         typename P::S* fc, typename P::S* uc, const int* done, cudaStream_t s);
 // number of blocks launch_residual_pp would launch for these fields (= partial sums it writes),
 // -1 where it would return -1; nothing is launched
 template <class P, class PO>
@@ -316,10 +324,12 @@ int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, dou
 template <class PF>
 int launch_restrict_smooth_chunk(const Lv<PolF64>& Lc, double rho, const typename PF::S* rf, double* fc, double* uc,
                                  const int* done, cudaStream_t s);
-// any level (the caller takes it up to PCR_MAX_COLS columns)
-int residual_chunk_blocks(const Lv<PolF64>& L);
-int launch_residual_chunk(const Lv<PolF64>& L, const double* u, const double* f, double* r, double* partials,
-                          const int* done, cudaStream_t s);
+// Residual, pointwise, any level and policy; the number of its blocks (= partial sums)
+template <class P>
+int residual_point_blocks(const Lv<P>& L);
+template <class P, class PO>
+int launch_residual_point(const Lv<P>& L, const typename P::S* u, const typename P::S* f, typename PO::S* r,
+                          double* partials, const int* done, cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (k_mg.cu)
 template <class P>
@@ -363,6 +373,13 @@ int launch_cg_spmv(const Lv<P>& L, const Scalars* sc, typename P::S* u, typename
 template <class P>
 int launch_cg_tridiag(const Lv<P>& L, const Scalars* sc, typename P::S* r, const typename P::S* q,
                       typename P::S* z, double* partials, cudaStream_t s);
+// the fused Tridiag on whole columns in shared memory (sweep_tile.cuh; F32 and DW; 16-byte aligned fields) and
+// its number of blocks, -1 where the level does not take it
+template <class P>
+int cg_tile_blocks(const Lv<P>& L);
+template <class P>
+int launch_cg_tile(const Lv<P>& L, const Scalars* sc, typename P::S* r, const typename P::S* q, typename P::S* z,
+                   double* partials, cudaStream_t s);
 template <class P>
 void launch_cg_finish(size_t n, const Scalars* sc, typename P::S* u, const typename P::S* p,
                       cudaStream_t s);
