@@ -62,67 +62,136 @@ __global__ void __launch_bounds__(256) k_cg_spmv(Lv<P> L, const Scalars* __restr
     if (threadIdx.x == 0 && threadIdx.y == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 
-// The fused SpMV pointwise: the stencil has no recurrence along the column, so every pair of
-// x-adjacent cells of a plane is a thread (grid-stride over the pairs, a fixed number of blocks for
-// the partial sums); neighbours come through the read-only cache. Requires nx even.
-template <class P>
-__global__ void __launch_bounds__(256) k_cg_spmv_cell(Lv<P> L, const Scalars* __restrict__ sc,
-                                                      typename P::S* __restrict__ u, typename P::S* __restrict__ p,
-                                                      const typename P::S* __restrict__ z,
-                                                      typename P::S* __restrict__ q, double* partials) {
+// The fused SpMV with two x-adjacent columns per thread and SPMV_PZ planes per block: the vertical neighbours
+// stay in registers, the x neighbours come from the adjacent lanes, and a plane's six 16-byte loads (DW; 8 bytes
+// in FP32) are in flight together. Bound by DRAM (seven fields); 512^2 x 128 double-word 378 us, 390 with
+// a thread per pair of cells, whose 64-bit divisions for the cell's indices and five stencil loads it does
+// without. Requires nx even; ALIGNED: pair-aligned fields.
+constexpr int SPMV_PZ = 16, SPMV_TY = 8;
+template <class P, bool ALIGNED>
+struct CgPair {
+    typedef typename P::S S;
+    typename P::R a, b;
+    __device__ __forceinline__ void ldg(const S* p) {
+        if constexpr (!ALIGNED) {
+            a = P::ld(p, 0);
+            b = P::ld(p, 1);
+        } else if constexpr (sizeof(S) == 8) {
+            const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+            get(reinterpret_cast<const S*>(&t));
+        } else {
+            const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+            get(reinterpret_cast<const S*>(&t));
+        }
+    }
+    __device__ __forceinline__ void ld(const S* p) {  // a field that is written too
+        if constexpr (!ALIGNED) {
+            get(p);
+        } else if constexpr (sizeof(S) == 8) {
+            const float4 t = *reinterpret_cast<const float4*>(p);
+            get(reinterpret_cast<const S*>(&t));
+        } else {
+            const float2 t = *reinterpret_cast<const float2*>(p);
+            get(reinterpret_cast<const S*>(&t));
+        }
+    }
+    __device__ __forceinline__ void get(const S* q) {
+        a = P::ld_plain(q, 0);
+        b = P::ld_plain(q, 1);
+    }
+    __device__ __forceinline__ void st(S* p) const {
+        if constexpr (!ALIGNED) {
+            P::st(p, 0, a);
+            P::st(p, 1, b);
+        } else if constexpr (sizeof(S) == 8) {
+            float4 t;
+            P::st(reinterpret_cast<S*>(&t), 0, a);
+            P::st(reinterpret_cast<S*>(&t), 1, b);
+            *reinterpret_cast<float4*>(p) = t;
+        } else {
+            float2 t;
+            P::st(reinterpret_cast<S*>(&t), 0, a);
+            P::st(reinterpret_cast<S*>(&t), 1, b);
+            *reinterpret_cast<float2*>(p) = t;
+        }
+    }
+    __device__ __forceinline__ void zero() { a = b = P::zero(); }
+};
+__device__ __forceinline__ float lane_up(float x) { return __shfl_up_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ float lane_dn(float x) { return __shfl_down_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ dw lane_up(dw x) { return dw{lane_up(x.hi), lane_up(x.lo)}; }
+__device__ __forceinline__ dw lane_dn(dw x) { return dw{lane_dn(x.hi), lane_dn(x.lo)}; }
+
+template <class P, bool ALIGNED>
+__global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<P> K, const Scalars* __restrict__ sc,
+                                                                typename P::S* __restrict__ u,
+                                                                typename P::S* __restrict__ p,
+                                                                const typename P::S* __restrict__ z,
+                                                                typename P::S* __restrict__ q, double* partials, int pz) {
     typedef typename P::R R;
+    typedef CgPair<P, ALIGNED> V;
     if (*(volatile const int*)&sc->done) return;
-    const int nx = L.nx, ny = L.ny, nz = L.nz, hx2 = nx / 2;
-    const size_t pl = (size_t)nx * ny, npairs = (size_t)hx2 * ny * nz;
+    const int nx = L.nx, ny = L.ny, nz = L.nz, lane = threadIdx.x;
+    const int i = 2 * (blockIdx.x * 32 + lane), j = blockIdx.y * SPMV_TY + threadIdx.y;
+    const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
+    const size_t pl = (size_t)nx * ny;
     const R alpha = P::cst(sc->alpha), beta = P::cst(sc->beta);
-    const R cx = P::cst(L.cx), cy = P::cst(L.cy);
-    const R dh = P::cst(1.0 + 2.0 * L.cx + 2.0 * L.cy);
-    const bool iso = L.cx == L.cy;
     typename P::Acc acc = 0, cmp = 0;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < npairs; t += (size_t)gridDim.x * blockDim.x) {
-        const int ip = (int)(t % hx2), j = (int)((t / hx2) % ny), k = (int)(t / ((size_t)hx2 * ny));
-        const int i = 2 * ip;
-        const size_t c = (size_t)j * nx + i, b = (size_t)k * pl, id = b + c;
-        const size_t rs = (size_t)wrapc(j - 1, ny) * nx + i, rn = (size_t)wrapc(j + 1, ny) * nx + i;
-        const R z0 = P::ld(z, id), z1 = P::ld(z, id + 1);
-        const R zw = P::ld(z, b + (size_t)j * nx + wrapc(i - 1, nx)), ze = P::ld(z, b + (size_t)j * nx + wrapc(i + 2, nx));
-        const R zs0 = P::ld(z, b + rs), zs1 = P::ld(z, b + rs + 1), zn0 = P::ld(z, b + rn), zn1 = P::ld(z, b + rn + 1);
-        R zm0 = P::zero(), zm1 = P::zero(), zp0 = P::zero(), zp1 = P::zero();
-        if (k > 0) {
-            zm0 = P::ld(z, id - pl);
-            zm1 = P::ld(z, id - pl + 1);
-        }
-        if (k + 1 < nz) {
-            zp0 = P::ld(z, id + pl);
-            zp1 = P::ld(z, id + pl + 1);
-        }
+    if (j < ny) {  // (a whole warp: one row)
+        const bool act = i < nx;
+        const int ii = act ? i : nx - 2;  // lanes beyond the row repeat its last pair and store nothing
+        const size_t row = (size_t)j * nx, c = row + ii, b0 = (size_t)k0 * pl;
+        const size_t rs = (size_t)wrapc(j - 1, ny) * nx + ii, rn = (size_t)wrapc(j + 1, ny) * nx + ii;
+        // the pair's x neighbours beyond the warp or the row are loaded
+        const bool lw = lane == 0, le = lane == 31 || i + 2 >= nx;
+        const size_t cw = row + wrapc(ii - 1, nx), ce = row + wrapc(ii + 2, nx);
         const R v0 = P::ld(L.v, c), v1 = P::ld(L.v, c + 1);
-        R d0 = dh, d1 = dh;
-        if (k > 0) {
-            d0 = P::add(d0, v0);
-            d1 = P::add(d1, v1);
+        const R d1a = P::add(K.dh, v0), d1b = P::add(K.dh, v1), d2a = P::add(d1a, v0), d2b = P::add(d1b, v1);
+        const bool iso = K.iso != 0;
+        V zm, zc;
+        zm.zero();
+        zc.ldg(z + b0 + c);
+        if (k0 > 0) zm.ldg(z + b0 - pl + c);
+#pragma unroll 2
+        for (int k = k0; k < k1; ++k) {
+            const size_t b = (size_t)k * pl, id = b + c;
+            V zp, zs, zn, po, qo, uo;
+            zp.ldg(z + (k + 1 < nz ? id + pl : id));
+            zs.ldg(z + b + rs);
+            zn.ldg(z + b + rn);
+            po.ld(p + id);
+            qo.ld(q + id);
+            uo.ld(u + id);
+            R zw = lane_up(zc.b), ze = lane_dn(zc.a);
+            if (lw) zw = P::ld(z, b + cw);
+            if (le) ze = P::ld(z, b + ce);
+            if (k + 1 == nz) zp.zero();
+            const bool end = k == 0 || k == nz - 1;
+            const R da = nz == 1 ? K.dh : (end ? d1a : d2a), db = nz == 1 ? K.dh : (end ? d1b : d2b);
+            // A z = -(f - A z) with f = 0: the sweep residual of a zero right-hand side, negated
+            const R az0 = P::neg(sweep_residual<P>(P::zero(), da, zc.a, zw, zc.b, zs.a, zn.a, zm.a, zp.a, K.cx, K.cy, v0, iso));
+            const R az1 = P::neg(sweep_residual<P>(P::zero(), db, zc.b, zc.a, ze, zs.b, zn.b, zm.b, zp.b, K.cx, K.cy, v1, iso));
+            V un, pn, qn;
+            un.a = P::fma(alpha, po.a, uo.a);
+            un.b = P::fma(alpha, po.b, uo.b);
+            pn.a = P::fma(beta, po.a, zc.a);
+            pn.b = P::fma(beta, po.b, zc.b);
+            qn.a = P::fma(beta, qo.a, az0);
+            qn.b = P::fma(beta, qo.b, az1);
+            if (act) {
+                un.st(u + id);
+                pn.st(p + id);
+                qn.st(q + id);
+                P::acc_dot(acc, cmp, pn.a, qn.a);
+                P::acc_dot(acc, cmp, pn.b, qn.b);
+            }
+            zm = zc;
+            zc = zp;
         }
-        if (k + 1 < nz) {
-            d0 = P::add(d0, v0);
-            d1 = P::add(d1, v1);
-        }
-        // A z = -(f - A z) with f = 0: the sweep residual of a zero right-hand side, negated
-        const R az0 = P::neg(sweep_residual<P>(P::zero(), d0, z0, zw, z1, zs0, zn0, zm0, zp0, cx, cy, v0, iso));
-        const R az1 = P::neg(sweep_residual<P>(P::zero(), d1, z1, z0, ze, zs1, zn1, zm1, zp1, cx, cy, v1, iso));
-        const R po0 = P::ld_plain(p, id), po1 = P::ld_plain(p, id + 1);
-        P::st(u, id, P::fma(alpha, po0, P::ld_plain(u, id)));
-        P::st(u, id + 1, P::fma(alpha, po1, P::ld_plain(u, id + 1)));
-        const R pn0 = P::fma(beta, po0, z0), pn1 = P::fma(beta, po1, z1);
-        const R qn0 = P::fma(beta, P::ld_plain(q, id), az0), qn1 = P::fma(beta, P::ld_plain(q, id + 1), az1);
-        P::st(p, id, pn0);
-        P::st(p, id + 1, pn1);
-        P::st(q, id, qn0);
-        P::st(q, id + 1, qn1);
-        P::acc_dot(acc, cmp, pn0, qn0);
-        P::acc_dot(acc, cmp, pn1, qn1);
     }
     const double s = block_sum(P::acc_get(acc, cmp));
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    if (threadIdx.x == 0 && threadIdx.y == 0)
+        partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
 }
 
 template <class P>
@@ -413,25 +482,41 @@ __global__ void k_cg_finish(size_t n, const Scalars* __restrict__ sc, typename P
         P::st(u, t, P::add(P::ld_plain(u, t), P::mul(alpha, P::ld(p, t))));
 }
 
-// the pointwise SpMV for the FP32-pipe policies (native FP64 keeps the column kernel, which reuses
-// the vertical neighbours from registers and runs faster on the slow FP64 pipe)
+// the marching SpMV for the FP32-pipe policies (native FP64 keeps the column kernel, bound by its pipe)
+template <class P>
+static dim3 spmv_march_grid(const Lv<P>& L, int& pz) {
+    dim3 g((L.nx / 2 + 31) / 32, (L.ny + SPMV_TY - 1) / SPMV_TY);
+    // one partial sum per block: as many slabs of planes as max_partials leaves room for
+    const int room = max_partials(L.nx, L.ny) / (int)(g.x * g.y);
+    int nzs = (L.nz + SPMV_PZ - 1) / SPMV_PZ;
+    if (nzs > room) nzs = room < 1 ? 1 : room;
+    pz = (L.nz + nzs - 1) / nzs;
+    g.z = (L.nz + pz - 1) / pz;
+    return g;
+}
 template <class P>
 int cg_spmv_blocks(const Lv<P>& L) {
     if (L.nx % 2 == 0 && P::id != 0) {
-        const size_t b = ((size_t)L.nx / 2 * L.ny * L.nz + 255) / 256;
-        return (int)(b < 152 * 8 ? (b ? b : 1) : 152 * 8);
+        int pz;
+        const dim3 g = spmv_march_grid(L, pz);
+        return (int)(g.x * g.y * g.z);
     }
     return sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false).nblocks();
 }
 template <class P>
 int launch_cg_spmv(const Lv<P>& L, const Scalars* sc, typename P::S* u, typename P::S* p,
                    const typename P::S* z, typename P::S* q, double* partials, cudaStream_t s) {
-    if (L.nx % 2 == 0 && P::id != 0) {
-        const int nb = cg_spmv_blocks(L);
-        k_cg_spmv_cell<P><<<nb, 256, 0, s>>>(L, sc, u, p, z, q, partials);
-        note_launch();
-        return nb;
-    }
+    if constexpr (P::id != 0)
+        if (L.nx % 2 == 0) {
+            int pz;
+            const dim3 g = spmv_march_grid(L, pz), b(32, SPMV_TY);
+            const SweepK<P> K = sweep_k<P>(L.cx, L.cy, 1.0);
+            const bool al = (((uintptr_t)u | (uintptr_t)p | (uintptr_t)z | (uintptr_t)q) & (2 * sizeof(typename P::S) - 1)) == 0;
+            if (al) k_cg_spmv_march<P, true><<<g, b, 0, s>>>(L, K, sc, u, p, z, q, partials, pz);
+            else k_cg_spmv_march<P, false><<<g, b, 0, s>>>(L, K, sc, u, p, z, q, partials, pz);
+            note_launch();
+            return (int)(g.x * g.y * g.z);
+        }
     Shape sh = sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false);
     k_cg_spmv<P><<<sh.grid, sh.block, 0, s>>>(L, sc, u, p, z, q, partials);
     note_launch();
@@ -441,6 +526,10 @@ int launch_cg_spmv(const Lv<P>& L, const Scalars* sc, typename P::S* u, typename
 // its factors and the scratch
 template <class P>
 int cg_tridiag_blocks(const Lv<P>& L) {
+    if constexpr (P::id != 0) {
+        const int nb = cg_tile_blocks(L);
+        if (nb >= 0) return nb;
+    }
     if (cg_x2_fits(L)) return cg_x2_blocks(L);
     if (L.gstack && L.finv && L.fw) {
         static int per_sm = 0;
@@ -461,6 +550,11 @@ int cg_tridiag_blocks(const Lv<P>& L) {
 template <class P>
 int launch_cg_tridiag(const Lv<P>& L, const Scalars* sc, typename P::S* r, const typename P::S* q,
                       typename P::S* z, double* partials, cudaStream_t s) {
+    if constexpr (P::id != 0)
+        if ((((uintptr_t)r | (uintptr_t)q | (uintptr_t)z) & 15) == 0) {
+            const int nb = launch_cg_tile(L, sc, r, q, z, partials, s);
+            if (nb >= 0) return nb;
+        }
     if (cg_x2_fits(L)) {
         const int nb = cg_x2_blocks(L);
         k_cg_tridiag_x2<P, CGX_TY, CGX_PD><<<nb, dim3(32, CGX_TY), cg_x2_smem<P>(), s>>>(L, sc, r, q, z, partials);

@@ -9,5 +9,7 @@ template int launch_sweep_tile<PolDW, MODE_SMOOTHB>(const Lv<PolDW>&, double, co
     const int*, cudaStream_t);
 template int launch_sweep_tile<PolDW, MODE_LINESOLVE>(const Lv<PolDW>&, double, const PolDW::S*, const PolDW::S*, PolDW::S*, double*,
     const int*, cudaStream_t);
+template int cg_tile_blocks<PolDW>(const Lv<PolDW>&);
+template int launch_cg_tile<PolDW>(const Lv<PolDW>&, const Scalars*, PolDW::S*, const PolDW::S*, PolDW::S*, double*, cudaStream_t);
 
 }  // namespace tpmg

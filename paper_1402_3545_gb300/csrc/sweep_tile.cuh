@@ -106,19 +106,25 @@ __device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
 
 }  // namespace
 
+// MODE_CGTRI: the fused Tridiag of CG, u the residual r (rewritten: r -= alpha q), f = q, out = z = M^{-1} r,
+// partial sums of <r, r> and, behind them, of <r, z>: with M = U^T D U the elimination gives yh = U^{-T} r
+// and d' = D^{-1} yh, so <r, M^{-1} r> = sum_k yh_k d'_k, and the back substitution does not read r again.
+constexpr int MODE_CGTRI = 16;
+
 // kw: planes whose factors are kept per column in shared memory behind the nz planes of the tile (0
 // when lambda^2 is constant). ISO: square cells; NORM: partial sums of ||f - A u||^2 (both compile-time:
 // as runtime choices their instructions were issued either way)
 template <class P, int MODE, int TR, bool ISO, bool NORM>
 __global__ void __launch_bounds__(TNT, 3)
     k_sweep_tile(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u, const typename P::S* __restrict__ f,
-                 typename P::S* __restrict__ out, double* partials, const int* done, int kw) {
+                 typename P::S* __restrict__ out, double* partials, const int* done, int kw, const Scalars* sc) {
     typedef typename P::S S;
     typedef typename P::R R;
     typedef TileVec<P> V;
-    constexpr bool SM = MODE != MODE_LINESOLVE;  // a stencil, and u in the result
+    constexpr bool CG = MODE == MODE_CGTRI;
+    constexpr bool SM = MODE != MODE_LINESOLVE && !CG;  // a stencil, and u in the result
     constexpr bool GFORM = MODE == MODE_SMOOTH && P::id == 1;
-    constexpr bool DIRECT = GFORM || MODE == MODE_LINESOLVE;  // the back substitution yields the result
+    constexpr bool DIRECT = GFORM || MODE == MODE_LINESOLVE || CG;  // the back substitution yields the result
     constexpr int G = 32 / TR;                                // lanes of a tile row
     constexpr int N = V::N, W = G * N, NC = TR * W;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -134,7 +140,7 @@ __global__ void __launch_bounds__(TNT, 3)
     const int ch = (nz + TNW - 1) / TNW, klo = warp * ch, khi = klo + ch < nz ? klo + ch : nz;
     const bool percol = L.fac_percol != 0;
     const R vzero = P::zero();
-    typename P::Acc acc = 0, cmp = 0;
+    typename P::Acc acc = 0, cmp = 0, az = 0, cz = 0;
 
     // ---- 1. the right-hand side of the line solves
     {
@@ -244,6 +250,30 @@ __global__ void __launch_bounds__(TNT, 3)
             for (; k < khi; ++k) batch(std::integral_constant<int, 1>(), k);
         }
     }
+    if constexpr (CG) {
+        const R nalpha = P::neg(P::cst(sc->alpha));
+        const S* pq = f + (size_t)klo * pl + c;
+        S* pr = const_cast<S*>(u) + (size_t)klo * pl + c;
+        S* z = Z + klo * NC + zo;
+        bool landed = false;
+#pragma unroll 4
+        for (int k = klo; k < khi; ++k, pq += pl, pr += pl, z += NC) {
+            V q, r;
+            q.ldg(pq);
+            if (!landed) {
+                cp_wait<0>();  // this thread's pieces of r
+                landed = true;
+            }
+            r.lds(z);
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                r.v[t] = P::fma(nalpha, q.v[t], r.v[t]);
+                P::acc_dot(acc, cmp, r.v[t], r.v[t]);
+            }
+            r.stg(pr);
+            r.sts(z);
+        }
+    }
     cp_wait<0>();
     __syncthreads();
 
@@ -273,7 +303,15 @@ __global__ void __launch_bounds__(TNT, 3)
                     w.sts(zwk);
                 }
 #pragma unroll
-                for (int q = 0; q < CV; ++q) d.v[q] = P::mul_u(P::fma_u(v.v[q], d.v[q], r.v[q]), iv.v[q]);
+                for (int q = 0; q < CV; ++q) {
+                    if constexpr (CG) {
+                        const R yh = P::fma(v.v[q], d.v[q], r.v[q]);
+                        d.v[q] = P::mul(yh, iv.v[q]);
+                        P::acc_dot(az, cz, yh, d.v[q]);
+                    } else {
+                        d.v[q] = P::mul_u(P::fma_u(v.v[q], d.v[q], r.v[q]), iv.v[q]);
+                    }
+                }
                 d.sts(zk);
             };
             auto factor = [&](C& iv, const S* zwk) {
@@ -365,7 +403,8 @@ __global__ void __launch_bounds__(TNT, 3)
             };
             auto step = [&](S* zk, const C& d, const C& w) {
 #pragma unroll
-                for (int q = 0; q < CV; ++q) x.v[q] = P::fma_u(w.v[q], x.v[q], d.v[q]);
+                for (int q = 0; q < CV; ++q)
+                    x.v[q] = CG ? P::fma(w.v[q], x.v[q], d.v[q]) : P::fma_u(w.v[q], x.v[q], d.v[q]);
                 if (DIRECT) {
                     C o = x;
                     if (MODE == MODE_LINESOLVE) {
@@ -428,12 +467,18 @@ __global__ void __launch_bounds__(TNT, 3)
     if (NORM) {
         const double sm = block_sum(P::acc_get(acc, cmp));
         if (tid == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = sm;
+        if constexpr (CG) {
+            __syncthreads();
+            const double sz = block_sum(P::acc_get(az, cz));
+            if (tid == 0) partials[gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = sz;
+        }
     }
 }
 
 template <class P, int MODE, int TR, bool ISO, bool NORM>
 static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
-                          typename P::S* out, double* partials, const int* done, cudaStream_t s) {
+                          typename P::S* out, double* partials, const int* done, cudaStream_t s,
+                          const Scalars* sc = nullptr) {
     typedef typename P::S S;
     // planes whose factors differ from the converged ones (all but the last when none has converged)
     int kw = 0;
@@ -442,7 +487,7 @@ static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, c
     auto kern = k_sweep_tile<P, MODE, TR, ISO, NORM>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * TPB);
     const dim3 grd(L.nx / (TPB / TR / (int)sizeof(S)), L.ny / TR);
-    kern<<<grd, TNT, smem, s>>>(L, sweep_k<P>(L.cx, L.cy, coef), u, f, out, partials, done, kw);
+    kern<<<grd, TNT, smem, s>>>(L, sweep_k<P>(L.cx, L.cy, coef), u, f, out, partials, done, kw, sc);
     note_launch();
     return (int)(grd.x * grd.y);
 }
@@ -457,6 +502,29 @@ static int run_sweep_tile_rows(const Lv<P>& L, double coef, const typename P::S*
     if (L.nx % (W / 4) == 0 && L.ny % 4 == 0)
         return run_sweep_tile<P, MODE, 4, ISO, NORM>(L, coef, u, f, out, partials, done, s);
     return -1;
+}
+
+template <class P>
+int cg_tile_blocks(const Lv<P>& L) {
+    constexpr int W = TPB / (int)sizeof(typename P::S);
+    if (L.nz > 128 || !L.finv || !L.fw || !(tile_pays(L) || (P::id == 1 && L.nz >= 16))) return -1;
+    auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+    if (!al(L.v) || (L.fac_percol && (!al(L.finv) || !al(L.fw)))) return -1;
+    if (L.nx % W == 0) return L.nx / W * L.ny;
+    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0) return L.nx / (W / 2) * (L.ny / 2);
+    if (L.nx % (W / 4) == 0 && L.ny % 4 == 0) return L.nx / (W / 4) * (L.ny / 4);
+    return -1;
+}
+template <class P>
+int launch_cg_tile(const Lv<P>& L, const Scalars* sc, typename P::S* r, const typename P::S* q, typename P::S* z,
+                   double* partials, cudaStream_t s) {
+    constexpr int W = TPB / (int)sizeof(typename P::S);
+    if (cg_tile_blocks(L) < 0) return -1;
+    const int* done = &sc->done;
+    if (L.nx % W == 0) return run_sweep_tile<P, MODE_CGTRI, 1, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
+    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0)
+        return run_sweep_tile<P, MODE_CGTRI, 2, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
+    return run_sweep_tile<P, MODE_CGTRI, 4, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
 }
 
 template <class P, int MODE>
