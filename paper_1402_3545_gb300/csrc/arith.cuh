@@ -23,6 +23,47 @@ struct dw {
     float hi, lo;
 };
 
+// ---------------------------------------------------------------- conversions on the integer pipe
+// FP64 values taken apart and put together from the IEEE 754 formats, without FP64 instructions, where all parts
+// are normal floats (or zero); else by the conversion instructions. The same bits either way.
+// Exponents for which the rounded value and its remainder's scale 2^(E-52) are both normal floats
+constexpr int CVT_EMIN = -74, CVT_EMAX = 126;
+
+// true if the fast form holds; hi = fl32(v), rem = signed units of 2^(E-52) of v - hi
+__device__ __forceinline__ bool split_f64(double v, float& hi, int& rem, int& e) {
+    const unsigned w1 = (unsigned)__double2hiint(v), w0 = (unsigned)__double2loint(v);
+    e = (int)((w1 >> 20) & 0x7ffu) - 1023;
+    const unsigned low = w0 & 0x1fffffffu;                        // the 29 fraction bits below a float's
+    const unsigned m = ((w1 & 0xfffffu) << 3) | (w0 >> 29);       // the upper 23
+    const unsigned up = (low + (m & 1u)) > 0x10000000u ? 1u : 0u;  // above the tie, or on it with an odd m
+    hi = __uint_as_float((w1 & 0x80000000u) | ((((unsigned)(e + 127)) << 23) + m + up));
+    rem = (int)low - (int)(up << 29);
+    if ((int)w1 < 0) rem = -rem;
+    return e >= CVT_EMIN && e <= CVT_EMAX;
+}
+__device__ __forceinline__ dw dw_of(double v) {
+    float hi;
+    int rem, e;
+    if (split_f64(v, hi, rem, e))  // |rem| <= 2^28: rounded to 24 bits, then scaled exactly
+        return dw{hi, __int2float_rn(rem) * __uint_as_float((unsigned)(e - 52 + 127) << 23)};
+    if (v == 0.0) return dw{__int_as_float(__double2hiint(v)), 0.f};  // the zero keeps its sign
+    hi = __double2float_rn(v);
+    return dw{hi, __double2float_rn(v - (double)hi)};
+}
+__device__ __forceinline__ float f32_of(double v) {
+    float hi;
+    int rem, e;
+    if (split_f64(v, hi, rem, e)) return hi;
+    return __double2float_rn(v);
+}
+__device__ __forceinline__ double f64_of(float v) {
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)  // normal: the exponent field moves by 1023 - 127
+        return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+    if (a == 0) return __hiloint2double((int)b, 0);
+    return (double)v;
+}
+
 // ---------------------------------------------------------------- error-free transformations
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = __fadd_rn(a, b);

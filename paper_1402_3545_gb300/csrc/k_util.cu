@@ -170,26 +170,66 @@ __global__ void k_copy(size_t n, const S* __restrict__ src, S* __restrict__ dst,
         dst[t] = src[t];
 }
 
+// Conversions between the caller's FP64 fields and the stored formats. They should run at memory speed, but
+// with conversion instructions and FP64 arithmetic (four a value for FP64 -> double-word, three back) they were
+// bound by the FP64 pipe: 249 and 189 us on 33.5M values, where the bytes need 79; now 79 and 84. Values whose parts are all
+// normal floats are therefore taken apart and put together on the integer pipe, from the IEEE 754 formats: round
+// to nearest even of the 52-bit fraction to 23 bits, the remainder as a signed integer times a power of two. All
+// others (float denormals, overflow, inf, NaN) take the conversion instructions. Both give the same bits
+// (split_f64 and its users in arith.cuh).
+// two values a thread where both arrays are 16-byte aligned (VEC), else one
+template <bool VEC>
 __global__ void k_f64_to_dw(size_t n, const double* __restrict__ x, float2* __restrict__ y) {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-        double v = x[t];
-        float h = __double2float_rn(v);
-        y[t] = make_float2(h, __double2float_rn(v - (double)h));
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        for (size_t t = t0; t < n / 2; t += nt) {
+            const double2 v = reinterpret_cast<const double2*>(x)[t];
+            const dw a = dw_of(v.x), b = dw_of(v.y);
+            reinterpret_cast<float4*>(y)[t] = make_float4(a.hi, a.lo, b.hi, b.lo);
+        }
+        if (t0 == 0 && (n & 1)) PolDW::st(y, n - 1, dw_of(x[n - 1]));
+    } else {
+        for (size_t t = t0; t < n; t += nt) PolDW::st(y, t, dw_of(x[t]));
     }
 }
+template <bool VEC>
 __global__ void k_dw_to_f64(size_t n, const float2* __restrict__ x, double* __restrict__ y) {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
-        float2 v = x[t];
-        y[t] = (double)v.x + (double)v.y;
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        for (size_t t = t0; t < n / 2; t += nt) {
+            const float4 v = reinterpret_cast<const float4*>(x)[t];
+            reinterpret_cast<double2*>(y)[t] = make_double2(f64_of(v.x) + f64_of(v.y), f64_of(v.z) + f64_of(v.w));
+        }
+        if (t0 == 0 && (n & 1)) y[n - 1] = f64_of(x[n - 1].x) + f64_of(x[n - 1].y);
+    } else {
+        for (size_t t = t0; t < n; t += nt) y[t] = f64_of(x[t].x) + f64_of(x[t].y);
     }
 }
+template <bool VEC>
 __global__ void k_f64_to_f32(size_t n, const double* __restrict__ x, float* __restrict__ y) {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
-        y[t] = __double2float_rn(x[t]);
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        for (size_t t = t0; t < n / 2; t += nt) {
+            const double2 v = reinterpret_cast<const double2*>(x)[t];
+            reinterpret_cast<float2*>(y)[t] = make_float2(f32_of(v.x), f32_of(v.y));
+        }
+        if (t0 == 0 && (n & 1)) y[n - 1] = f32_of(x[n - 1]);
+    } else {
+        for (size_t t = t0; t < n; t += nt) y[t] = f32_of(x[t]);
+    }
 }
+template <bool VEC>
 __global__ void k_f32_to_f64(size_t n, const float* __restrict__ x, double* __restrict__ y) {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
-        y[t] = (double)x[t];
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        for (size_t t = t0; t < n / 2; t += nt) {
+            const float2 v = reinterpret_cast<const float2*>(x)[t];
+            reinterpret_cast<double2*>(y)[t] = make_double2(f64_of(v.x), f64_of(v.y));
+        }
+        if (t0 == 0 && (n & 1)) y[n - 1] = f64_of(x[n - 1]);
+    } else {
+        for (size_t t = t0; t < n; t += nt) y[t] = f64_of(x[t]);
+    }
 }
 // coarse vertical coefficient: the average of the 2x2 children
 __global__ void k_coarsen_v(int nxf, int nyf, const double* __restrict__ vf, double* __restrict__ vc) {
@@ -200,6 +240,7 @@ __global__ void k_coarsen_v(int nxf, int nyf, const double* __restrict__ vf, dou
     vc[(size_t)J * nxc + I] = 0.25 * (vf[a] + vf[a + 1] + vf[b] + vf[b + 1]);
 }
 
+static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 static unsigned grid_for(size_t n) {
     size_t b = (n + 255) / 256;
     if (b > 152 * 16) b = 152 * 16;
@@ -258,19 +299,23 @@ template void launch_copy<PolF32>(size_t, const float*, float*, const int*, cuda
 template void launch_copy<PolDW>(size_t, const float2*, float2*, const int*, cudaStream_t);
 
 void launch_f64_to_dw(size_t n, const double* x, float2* y, cudaStream_t s) {
-    k_f64_to_dw<<<grid_for(n), 256, 0, s>>>(n, x, y);
+    if (aligned16(x) && aligned16(y)) k_f64_to_dw<true><<<grid_for((n + 1) / 2), 256, 0, s>>>(n, x, y);
+    else k_f64_to_dw<false><<<grid_for(n), 256, 0, s>>>(n, x, y);
     note_launch();
 }
 void launch_dw_to_f64(size_t n, const float2* x, double* y, cudaStream_t s) {
-    k_dw_to_f64<<<grid_for(n), 256, 0, s>>>(n, x, y);
+    if (aligned16(x) && aligned16(y)) k_dw_to_f64<true><<<grid_for((n + 1) / 2), 256, 0, s>>>(n, x, y);
+    else k_dw_to_f64<false><<<grid_for(n), 256, 0, s>>>(n, x, y);
     note_launch();
 }
 void launch_f64_to_f32(size_t n, const double* x, float* y, cudaStream_t s) {
-    k_f64_to_f32<<<grid_for(n), 256, 0, s>>>(n, x, y);
+    if (aligned16(x) && aligned16(y)) k_f64_to_f32<true><<<grid_for((n + 1) / 2), 256, 0, s>>>(n, x, y);
+    else k_f64_to_f32<false><<<grid_for(n), 256, 0, s>>>(n, x, y);
     note_launch();
 }
 void launch_f32_to_f64(size_t n, const float* x, double* y, cudaStream_t s) {
-    k_f32_to_f64<<<grid_for(n), 256, 0, s>>>(n, x, y);
+    if (aligned16(x) && aligned16(y)) k_f32_to_f64<true><<<grid_for((n + 1) / 2), 256, 0, s>>>(n, x, y);
+    else k_f32_to_f64<false><<<grid_for(n), 256, 0, s>>>(n, x, y);
     note_launch();
 }
 void launch_coarsen_v_f64(int nxf, int nyf, const double* vf, double* vc, cudaStream_t s) {

@@ -197,6 +197,14 @@ template <class P>
 struct Conv<P, P> {
     __device__ __forceinline__ static typename P::R f(typename P::R x) { return x; }
 };
+template <>
+struct Conv<PolF64, PolDW> {  // the same values without the FP64 pipe's conversions (one addition back)
+    __device__ __forceinline__ static dw f(double x) { return dw_of(x); }
+};
+template <>
+struct Conv<PolDW, PolF64> {
+    __device__ __forceinline__ static double f(dw x) { return f64_of(x.hi) + f64_of(x.lo); }
+};
 
 // Device-resident solver scalars (one struct per running solve). All solver control decisions
 // are taken on the device by the finalize kernels so a whole iteration can be replayed from a
