@@ -1572,7 +1572,7 @@ struct BatchCache {
     int nu_pre = 0, nu_post = 0, n_coarse = 0, max_iter = 0;
     double rho = 0, tol = 0, timeout_s = 0;
     std::vector<const void*> io_key;
-    int nprob = 0, nphase = 0, ntasks = 0, total_parts = 0, nz_max = 0, grid = 0;
+    int nprob = 0, nphase = 0, ntasks = 0, total_parts = 0, grid = 0;
     size_t smem = 0;
     BProbDesc* d_probs = nullptr;
     BState* d_state = nullptr;
@@ -1585,7 +1585,6 @@ struct BatchCache {
     int* d_flags = nullptr;     // error, n_active
     int* h_flags = nullptr;     // pinned: initial flags and results
     double* d_hist = nullptr;
-    float* d_scratch = nullptr;  // the persistent blocks' Thomas stacks
     cudaGraphExec_t graph = nullptr;
     unsigned long long graph_kernels = 0;
     std::vector<BTask> h_tasks;
@@ -1593,7 +1592,7 @@ struct BatchCache {
     ~BatchCache() {
         if (graph) cudaGraphExecDestroy(graph);
         void* ptrs[] = {d_probs,    d_state, d_tasks, d_phase_begin, d_phase_tiles, d_partials,
-                        d_bar,      d_flags, d_hist,  d_scratch};
+                        d_bar,      d_flags, d_hist};
         for (void* p : ptrs) dev_free(p);
         if (h_state) cudaFreeHost(h_state);
         if (h_flags) cudaFreeHost(h_flags);
@@ -1618,6 +1617,11 @@ static void drop_batches_of(const tpmg_op* op) {
 static void cycle_tasks(tpmg_op* op, int b, const tpmg_params* prm, std::vector<BTask>& out) {
     Hier& h = op->hier[1];
     const int L = op->g.L;
+    auto form_of = [&](int type, int level) {
+        const int lf = type == BT_RRS ? level - 1 : level;  // whose factors it uses
+        return batched_form(type, op->g.lnx[level], op->g.lny[level], op->g.nz, op->percol[lf],
+                            factor_planes(level_view<PolF32>(op, lf)), op->cx[level] == op->cy[level]);
+    };
     auto task = [&](int type, int level, const void* a, const void* rhs, void* o, void* o2) {
         BTask t;
         t.type = type;
@@ -1627,12 +1631,8 @@ static void cycle_tasks(tpmg_op* op, int b, const tpmg_params* prm, std::vector<
         t.b = rhs;
         t.out = o;
         t.out2 = o2;
-        const int nxl = op->g.lnx[level];
-        const int nyl = op->g.lny[level];
-        t.x2 = (type == BT_SMOOTH || type == BT_RESID || type == BT_LS0 || type == BT_RRS) &&
-               batched_x2_fits(nxl, nyl, a ? a : rhs, rhs, type == BT_RRS ? a : o);
-        t.tiles_x = t.x2 ? nxl / 64 : (nxl + 31) / 32;
-        t.tiles_y = (nyl + BTY - 1) / BTY;
+        t.form = form_of(type, level);
+        t.tiles = batched_tiles(type, t.form, op->g.lnx[level], op->g.lny[level], op->g.nz);
         t.tile_base = 0;
         out.push_back(t);
     };
@@ -1653,9 +1653,9 @@ static void cycle_tasks(tpmg_op* op, int b, const tpmg_params* prm, std::vector<
             loth[l] = h.ub[l];
         }
         // Residual of level l, then RestrictSmooth onto l-1: one fused task where level l takes
-        // two-column tiles (the same arithmetic), else the two tasks; returns whether it fused
+        // its tiles (the same arithmetic), else the two tasks; returns whether it fused
         auto residual_restrict = [&](int l, const void* u_l) {
-            if (op->fuse_restrict && batched_x2_fits(op->g.lnx[l], op->g.lny[l], u_l, h.f[l], u_l)) {
+            if (op->fuse_restrict && form_of(BT_RRS, l) >= 0) {
                 task(BT_RRS, l, u_l, h.f[l], h.f[l - 1], lcur[l - 1]);
                 return true;
             }
@@ -1689,7 +1689,7 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
     bc->nprob = np;
     std::vector<BProbDesc> probs(np);
     std::vector<std::vector<BTask>> lists(np);
-    int parts = 0, maxlen = 0, nz_max = 1;
+    int parts = 0, maxlen = 0;
     for (int b = 0; b < np; ++b) {
         tpmg_op* op = bc->ops[b];
         const int L = op->g.L;
@@ -1697,13 +1697,13 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
         memset(&pd, 0, sizeof(pd));
         pd.L = L;
         pd.nz = op->g.nz;
-        nz_max = op->g.nz > nz_max ? op->g.nz : nz_max;
         for (int l = 1; l <= L; ++l) {
             BLevelDesc& ld = pd.lev[l];
             ld.nx = op->g.lnx[l];
             ld.ny = op->g.lny[l];
             ld.nz = op->g.nz;
             ld.percol = op->percol[l];
+            ld.kw = op->percol[l] ? factor_planes(level_view<PolF32>(op, l)) : 0;
             ld.cx = op->cx[l];
             ld.cy = op->cy[l];
             ld.v = op->v32[l];
@@ -1717,14 +1717,12 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
         pd.fD = (const float2*)op->hier[2].f[L];
         pd.vD = op->vdw[L];
         pd.r32 = (float*)op->hier[1].f[L];
-        pd.fine_x2 = batched_x2_fits(op->g.lnx[L], op->g.lny[L], pd.uD, pd.fD, pd.r32) ? 1 : 0;
-        pd.fine_tiles = (pd.fine_x2 ? op->g.lnx[L] / 64 : (op->g.lnx[L] + 31) / 32) * ((op->g.lny[L] + BTY - 1) / BTY);
+        pd.fine_tiles = batched_tiles(BT_OUTRES, BF_COLS, op->g.lnx[L], op->g.lny[L], op->g.nz);
         pd.part_base = parts;
         parts += pd.fine_tiles;
         cycle_tasks(op, b, prm, lists[b]);
         maxlen = (int)lists[b].size() > maxlen ? (int)lists[b].size() : maxlen;
     }
-    bc->nz_max = nz_max;
     bc->total_parts = parts;
     // phases: outer residual, convergence decision, then the p-th step of every problem's cycle
     std::vector<BTask>& tasks = bc->h_tasks;
@@ -1735,7 +1733,7 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
         int tiles = 0;
         for (size_t t = first; t < tasks.size(); ++t) {
             tasks[t].tile_base = tiles;
-            tiles += tasks[t].tiles_x * tasks[t].tiles_y;
+            tiles += tasks[t].tiles;
         }
         bc->h_phase_tiles.push_back(tiles);
     };
@@ -1750,9 +1748,8 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
             t.level = op->g.L;
             if (ph < 2) {
                 t.type = ph == 0 ? BT_OUTRES : BT_FINAL;
-                t.x2 = ph == 0 ? probs[b].fine_x2 : 0;
-                t.tiles_x = ph == 0 ? (t.x2 ? op->g.lnx[op->g.L] / 64 : (op->g.lnx[op->g.L] + 31) / 32) : 1;
-                t.tiles_y = ph == 0 ? (op->g.lny[op->g.L] + BTY - 1) / BTY : 1;
+                t.form = BF_COLS;
+                t.tiles = ph == 0 ? probs[b].fine_tiles : 1;
                 tasks.push_back(t);
             } else if (ph - 2 < (int)lists[b].size()) {
                 tasks.push_back(lists[b][ph - 2]);
@@ -1784,13 +1781,16 @@ static tpmg_status build_batch(BatchCache* bc, const tpmg_params* prm) {
                   cudaMemcpyHostToDevice));
     CK(cudaMemcpy(bc->d_phase_tiles, bc->h_phase_tiles.data(), sizeof(int) * bc->h_phase_tiles.size(),
                   cudaMemcpyHostToDevice));
-    bc->smem = batched_smem_bytes();
-    int per_sm = batched_blocks_per_sm();
+    bc->smem = 0;
+    for (const BTask& t : tasks) {
+        const BLevelDesc& ld = probs[t.prob].lev[t.type == BT_RRS ? t.level - 1 : t.level];
+        bc->smem = std::max(bc->smem, batched_smem(t.type, t.form, ld.nz, ld.percol, ld.kw));
+    }
+    const int per_sm = batched_blocks_per_sm(bc->smem);
     int nsm = 0;
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, bc->ops[0]->device));
     if (per_sm < 1) return set_err(TPMG_ERR_ARG, "batched kernel does not fit on an SM");
     bc->grid = per_sm * nsm;
-    TRY(dalloc((void**)&bc->d_scratch, sizeof(float) * batched_scratch_floats(bc->grid, nz_max)));
     return TPMG_OK;
 }
 
@@ -1865,8 +1865,6 @@ extern "C" tpmg_status tpmg_mg_solve_batched(int nprob, tpmg_op* const* ops, con
     d.tol = prm->tol;
     d.max_iter = prm->max_iter;
     d.timeout_ns = (unsigned long long)(timeout_s * 1e9);
-    d.nz_max = bc->nz_max;
-    d.scratch = bc->d_scratch;
     std::vector<const void*> io_key;
     for (int b = 0; b < nprob; ++b) {
         io_key.push_back(f[b]);

@@ -5,19 +5,37 @@
 // (stored FP32), one FP32 V-cycle of Algorithm 1 on A e = r from e = 0, u += e. The host turns the
 // cycle of every problem into a list of phases; phase p holds one task per problem (the problem's
 // p-th step: a Smooth, Residual, RestrictSmooth, Prolongate, ... on one of its levels), each task cut
-// into tiles of 32 x BTY columns. The persistent blocks stride over the tiles of a phase and then
+// into tiles. The persistent blocks stride over the tiles of a phase and then
 // meet at a grid barrier; problems of fewer levels simply have no task in the late phases. The
 // barrier is a counter plus generation word; every wait is bounded by a time limit after which
 // the kernel raises an error flag and all blocks return (TPMG_ERR_TIMEOUT on the host).
 //
-// One thread per column sweeps k with the Thomas recurrence (precomputed factors: a table of nz
-// entries when lambda^2 is constant on the level, which is the batched workload's case), the
-// forward-eliminated values on a per-block stack in global scratch (L2-resident; a stack in shared
-// memory would leave room for only three blocks per SM).
+// Forms of a task (batched_form):
+//  - BF_TILE1, BF_TILE4: Smooth and first line solve on whole columns in shared memory, 128 x 1 or 32 x 4 FP32
+//    columns a tile, as the single-problem solver's (sweep_tile.cuh); the fused Residual + RestrictSmooth on
+//    tiles of 128 x 2 fine columns (restrict_tile.cuh);
+//  - BF_COLS: 32 columns of the level in order, planes in parallel over the eight warps, one warp running the
+//    recurrences in shared memory: all other shapes;
+//  - Residuals (FP32 and the outer double-word one), Prolongate and the correction: pointwise.
+// Three blocks of 256 threads per SM, set by the tiles' 65 KB at 128 planes. Before, 128-thread blocks marched
+// every column plane by plane, its Thomas values on a stack in L2 (a chain of loads, elimination and stack store
+// per plane, and on the narrow levels one column per thread): 12 problems of 64 .. 512 squared x 32 .. 128 to 1e-9
+// 43.2 ms, 29.1 here, the same bits. What is left: the FP32 tiles (0.55 of the copy rate), the outer residual
+// and correction (20 bytes per cell each) and, once most problems have converged, too few tiles per phase.
+#include <type_traits>
+
 #include "kernels.cuh"
-#include "sweep_x2.cuh"
+#include "restrict_tile.cuh"
+#include "sweep_tile.cuh"
 
 namespace tpmg {
+
+constexpr int BNT = 256, BNW = BNT / 32;
+static_assert(BNT == TNT && BNT == RNT, "the tiles' block");
+constexpr int BPZ = 16;             // planes of a column a pointwise residual tile takes
+constexpr int BCH = 4096;           // cells of a correction tile
+constexpr int BPU = 1024;           // coarse segments of a Prolongate tile
+constexpr size_t BTILE_SMEM = 72 * 1024;  // three blocks of it fit an SM
 
 __device__ __forceinline__ int bwrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
@@ -31,7 +49,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 __device__ bool grid_barrier(const BatchDesc& d) {
     __syncthreads();
     __shared__ int ok;
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
+    if (threadIdx.x == 0) {
         ok = 1;
         volatile unsigned* gen = d.bar_gen;
         const unsigned g = *gen;
@@ -62,210 +80,301 @@ __device__ bool grid_barrier(const BatchDesc& d) {
     return ok != 0;
 }
 
-// ---------------------------------------------------------------- FP32 tile operations
-struct TileIdx {
-    int i, j, tid, nt;
+// ---------------------------------------------------------------- tile operations
+// Fields are read by ordinary loads: they are written by this kernel, and the read-only path need not see that.
+
+struct BCol {  // a column of a level and its horizontal neighbours
+    size_t c, w, e, s, n;
     bool act;
 };
-__device__ __forceinline__ TileIdx tile_idx(int i0, int j0, int nx, int ny) {
-    TileIdx t;
-    t.i = i0 + threadIdx.x;
-    t.j = j0 + threadIdx.y;
-    t.tid = threadIdx.y * 32 + threadIdx.x;
-    t.nt = 32 * BTY;
-    t.act = t.i < nx && t.j < ny;
-    return t;
+__device__ __forceinline__ BCol bcol(int nx, int ny, int col) {
+    BCol q;
+    q.act = col < nx * ny;
+    if (!q.act) col = nx * ny - 1;
+    const int j = col / nx, i = col - j * nx;
+    q.c = (size_t)col;
+    q.w = (size_t)j * nx + bwrap(i - 1, nx);
+    q.e = (size_t)j * nx + bwrap(i + 1, nx);
+    q.s = (size_t)bwrap(j - 1, ny) * nx + i;
+    q.n = (size_t)bwrap(j + 1, ny) * nx + i;
+    return q;
 }
-
-__device__ __forceinline__ float fac(const float* a, int percol, int k, size_t pl, size_t c) {
-    return __ldg(a + (percol ? (size_t)k * pl + c : (size_t)k));
+// FP32 residual of a cell
+template <bool SW>
+__device__ __forceinline__ float bresidual(const SweepK<PolF32>& K, float diag, float vv, float fk, float uc, float w, float e,
+                                           float s, float n, float um, float up) {
+    if (SW) return sweep_residual<PolF32>(fk, diag, uc, w, e, s, n, um, up, K.cx, K.cy, vv, K.iso != 0);
+    const float cx = K.cx, cy = K.cy, hx = w + e, hy = s + n;
+    return fk - (diag * uc - cx * hx - cy * hy - vv * (um + up));
 }
+template <class P>
+__device__ __forceinline__ typename P::R bload(const typename P::S* p, size_t i) { return P::ld_plain(p, i); }
 
-// MODE 0: out = u + rho M^{-1}(f - A u); MODE 1: out = f - A u; MODE 2: out = rho M^{-1} f (u unused)
-template <int MODE>
-__device__ void t_sweep(const BLevelDesc& L, float rho, const float* __restrict__ u, const float* __restrict__ f,
-                        float* __restrict__ out, int i0, int j0, float* stack) {
-    TileIdx t = tile_idx(i0, j0, L.nx, L.ny);
-    if (!t.act) return;
-    const int nx = L.nx, ny = L.ny, nz = L.nz;
-    const size_t pl = (size_t)nx * ny, c = (size_t)t.j * nx + t.i;
-    const size_t cw = (size_t)t.j * nx + bwrap(t.i - 1, nx), ce = (size_t)t.j * nx + bwrap(t.i + 1, nx);
-    const size_t cs = (size_t)bwrap(t.j - 1, ny) * nx + t.i, cn = (size_t)bwrap(t.j + 1, ny) * nx + t.i;
-    const float cx = L.k1.cx, cy = L.k1.cy, vv = __ldg(L.v + c);  // converted on the host
-    const float dh = L.k1.dh, dh1 = dh + vv, dh2 = dh1 + vv;
-    float um = 0.f, uc = (MODE != 2) ? __ldg(u + c) : 0.f, d_prev = 0.f;
-    float fnext = __ldg(f + c);
-    #pragma unroll 2
-    for (int k = 0; k < nz; ++k) {
-        const size_t b = (size_t)k * pl;
-        const float fk = fnext;
-        if (k + 1 < nz) fnext = __ldg(f + b + pl + c);
-        float r;
-        if (MODE == 2) {
-            r = fk;
-        } else {
-            const float up = (k + 1 < nz) ? __ldg(u + b + pl + c) : 0.f;
-            const float diag = (nz == 1) ? dh : ((k == 0 || k == nz - 1) ? dh1 : dh2);
-            const float hx = __ldg(u + b + cw) + __ldg(u + b + ce), hy = __ldg(u + b + cs) + __ldg(u + b + cn);
-            r = fk - (diag * uc - cx * hx - cy * hy - vv * (um + up));
-            um = uc;
-            uc = up;
-        }
-        if (MODE == 1) {
-            out[b + c] = r;
-        } else {
-            const float d = (r + vv * d_prev) * fac(L.finv, L.percol, k, pl, c);
-            stack[(size_t)k * t.nt + t.tid] = d;
-            d_prev = d;
-        }
-    }
-    if (MODE == 1) return;
-    float xn = 0.f;
-    #pragma unroll 4
-    for (int k = nz - 1; k >= 0; --k) {
-        const size_t id = (size_t)k * pl + c;
-        xn = stack[(size_t)k * t.nt + t.tid] + fac(L.fw, L.percol, k, pl, c) * xn;
-        out[id] = (MODE == 0) ? __ldg(u + id) + rho * xn : rho * xn;
-    }
-}
-
-// coarse level Lc from the fine residual rf: f_c = R r_f, u_c = rho M_c^{-1} f_c
-__device__ void t_restrict_smooth(const BLevelDesc& Lc, float rho, const float* __restrict__ rf, float* __restrict__ fc,
-                                  float* __restrict__ uc, int i0, int j0, float* stack) {
-    TileIdx t = tile_idx(i0, j0, Lc.nx, Lc.ny);
-    if (!t.act) return;
-    const int nxc = Lc.nx, nz = Lc.nz, nxf = 2 * nxc;
-    const size_t plc = (size_t)nxc * Lc.ny, plf = 4 * plc, c = (size_t)t.j * nxc + t.i;
-    const size_t f00 = (size_t)(2 * t.j) * nxf + 2 * t.i, f01 = f00 + nxf;
-    const float vv = __ldg(Lc.v + c);
-    float d_prev = 0.f;
-    auto fine = [&](int k) {
-        const size_t bf = (size_t)k * plf;
-        return 0.25f * ((__ldg(rf + bf + f00) + __ldg(rf + bf + f00 + 1)) +
-                        (__ldg(rf + bf + f01) + __ldg(rf + bf + f01 + 1)));
-    };
-    auto fwd = [&](int k, float fk) {
-        fc[(size_t)k * plc + c] = fk;
-        const float d = (fk + vv * d_prev) * fac(Lc.finv, Lc.percol, k, plc, c);
-        stack[(size_t)k * t.nt + t.tid] = d;
-        d_prev = d;
-    };
-    // the children of four planes are loaded before their recurrence steps
-    int k = 0;
-    for (; k + 4 <= nz; k += 4) {
-        float fk[4];
+// r = f - A u on planes of BNT columns; the sum of squares of the thread's residuals (SUM)
+template <class P, class PO, bool SW, bool SUM>
+__device__ double t_residual(int nx, int ny, int nz, const SweepK<P>& K, const typename P::S* vp, const typename P::S* u,
+                             const typename P::S* f, typename PO::S* r, int tile) {
+    typedef typename P::R R;
+    const int tx = (nx * ny + BNT - 1) / BNT;
+    const BCol q = bcol(nx, ny, (tile % tx) * BNT + threadIdx.x);
+    const size_t pl = (size_t)nx * ny;
+    const int k0 = tile / tx * BPZ, k1 = k0 + BPZ < nz ? k0 + BPZ : nz;
+    typename P::Acc acc = 0, cmp = 0;
+    if (q.act) {
+        const R vv = P::ld(vp, q.c), dh1 = P::add(K.dh, vv), dh2 = P::add(dh1, vv);
+        const bool iso = K.iso != 0;
+        const size_t b0 = (size_t)k0 * pl;
+        const typename P::S *pw = u + b0 + q.w, *pe = u + b0 + q.e, *ps = u + b0 + q.s, *pn = u + b0 + q.n,
+                            *pu = u + b0 + q.c, *pf = f + b0 + q.c;
+        typename PO::S* pr = r + b0 + q.c;
+        R um = k0 > 0 ? bload<P>(pu - pl, 0) : P::zero(), uc = bload<P>(pu, 0);
+        // two planes' loads are issued together
+        constexpr int D = 2;
+        for (int k = k0; k < k1; k += D) {
+            R up[D], w[D], e[D], s[D], n[D], fk[D];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) fk[q] = fine(k + q);
+            for (int t = 0; t < D; ++t) {
+                const size_t o = (size_t)(k + t < nz ? t : 0) * pl;       // past the end: plane k again, not used
+                const size_t o1 = (size_t)(k + t + 1 < nz ? t + 1 : 0) * pl;
+                up[t] = bload<P>(pu, o1);
+                w[t] = bload<P>(pw, o);
+                e[t] = bload<P>(pe, o);
+                s[t] = bload<P>(ps, o);
+                n[t] = bload<P>(pn, o);
+                fk[t] = bload<P>(pf, o);
+            }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) fwd(k + q, fk[q]);
-    }
-    for (; k < nz; ++k) fwd(k, fine(k));
-    float xn = 0.f;
-    k = nz - 1;
-    for (; k >= 3; k -= 4) {
-        float st[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) st[q] = stack[(size_t)(k - q) * t.nt + t.tid];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            xn = st[q] + fac(Lc.fw, Lc.percol, k - q, plc, c) * xn;
-            uc[(size_t)(k - q) * plc + c] = rho * xn;
-        }
-    }
-    for (; k >= 0; --k) {
-        xn = stack[(size_t)k * t.nt + t.tid] + fac(Lc.fw, Lc.percol, k, plc, c) * xn;
-        uc[(size_t)k * plc + c] = rho * xn;
-    }
-}
-
-// fine level Lf: u_f += P u_c (bilinear, cell centred, periodic)
-__device__ void t_prolongate(const BLevelDesc& Lf, const float* __restrict__ ucrs, float* __restrict__ uf, int i0, int j0) {
-    TileIdx t = tile_idx(i0, j0, Lf.nx, Lf.ny);
-    if (!t.act) return;
-    const int nxc = Lf.nx / 2, nyc = Lf.ny / 2, nz = Lf.nz;
-    const int I = t.i >> 1, J = t.j >> 1;
-    const int I2 = bwrap((t.i & 1) ? I + 1 : I - 1, nxc), J2 = bwrap((t.j & 1) ? J + 1 : J - 1, nyc);
-    const size_t plc = (size_t)nxc * nyc, plf = (size_t)Lf.nx * Lf.ny;
-    const size_t a = (size_t)J * nxc + I, bq = (size_t)J * nxc + I2, cq = (size_t)J2 * nxc + I,
-                 dq = (size_t)J2 * nxc + I2, o = (size_t)t.j * Lf.nx + t.i;
-    auto pv = [&](int k) {
-        const size_t bc = (size_t)k * plc;
-        return 0.5625f * __ldg(ucrs + bc + a) + 0.1875f * __ldg(ucrs + bc + bq) + 0.1875f * __ldg(ucrs + bc + cq) +
-               0.0625f * __ldg(ucrs + bc + dq);
-    };
-    // four planes per step: all loads issued before the stores (the planes are disjoint)
-    int k = 0;
-    for (; k + 4 <= nz; k += 4) {
-        float val[4], old[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            val[q] = pv(k + q);
-            old[q] = uf[(size_t)(k + q) * plf + o];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) uf[(size_t)(k + q) * plf + o] = old[q] + val[q];
-    }
-    for (; k < nz; ++k) uf[(size_t)k * plf + o] += pv(k);
-}
-
-// ---------------------------------------------------------------- double-word outer steps
-// r32 = f - A u in double-word arithmetic (finest level), partial sum of ||r||^2 per tile
-__device__ double t_outres(const BProbDesc& pb, int i0, int j0) {
-    typedef PolDW P;
-    typedef P::R R;
-    const BLevelDesc& L = pb.lev[pb.L];
-    TileIdx t = tile_idx(i0, j0, L.nx, L.ny);
-    P::Acc acc = 0, cmp = 0;
-    if (t.act) {
-        const int nx = L.nx, ny = L.ny, nz = L.nz;
-        const size_t pl = (size_t)nx * ny, c = (size_t)t.j * nx + t.i;
-        const size_t cw = (size_t)t.j * nx + bwrap(t.i - 1, nx), ce = (size_t)t.j * nx + bwrap(t.i + 1, nx);
-        const size_t cs = (size_t)bwrap(t.j - 1, ny) * nx + t.i, cn = (size_t)bwrap(t.j + 1, ny) * nx + t.i;
-        const R cx = pb.kD.cx, cy = pb.kD.cy, vv = P::ld(pb.vD, c);  // converted on the host
-        const R dh = pb.kD.dh, dh1 = P::add(dh, vv), dh2 = P::add(dh1, vv);
-        R um = P::zero(), uc = P::ld_plain(pb.uD, c);
-        for (int k = 0; k < nz; ++k) {
-            const size_t b = (size_t)k * pl;
-            const R up = (k + 1 < nz) ? P::ld_plain(pb.uD, b + pl + c) : P::zero();
-            const R hx = P::add(P::ld_plain(pb.uD, b + cw), P::ld_plain(pb.uD, b + ce));
-            const R hy = P::add(P::ld_plain(pb.uD, b + cs), P::ld_plain(pb.uD, b + cn));
-            const R diag = (nz == 1) ? dh : ((k == 0 || k == nz - 1) ? dh1 : dh2);
-            R au = P::mul(diag, uc);
-            au = P::sub(au, P::mul(cx, hx));
-            au = P::sub(au, P::mul(cy, hy));
-            au = P::sub(au, P::mul(vv, P::add(um, up)));
-            const R r = P::sub(P::ld(pb.fD, b + c), au);
-            P::acc_dot(acc, cmp, r, r);
-            pb.r32[b + c] = P::to_f(r);
-            um = uc;
-            uc = up;
+            for (int t = 0; t < D; ++t) {
+                if (k + t >= k1) break;
+                if (k + t + 1 == nz) up[t] = P::zero();
+                const R dg = nz == 1 ? K.dh : (k + t == 0 || k + t == nz - 1 ? dh1 : dh2);
+                R rk;
+                if constexpr (P::id == 1) rk = bresidual<SW>(K, dg, vv, fk[t], uc, w[t], e[t], s[t], n[t], um, up[t]);
+                else rk = sweep_residual<P>(fk[t], dg, uc, w[t], e[t], s[t], n[t], um, up[t], K.cx, K.cy, vv, iso);
+                if constexpr (PO::id == P::id) P::st(reinterpret_cast<typename P::S*>(pr), (size_t)t * pl, rk);
+                else PO::st(pr, (size_t)t * pl, PO::from_f(P::to_f(rk)));
+                if (SUM) P::acc_dot(acc, cmp, rk, rk);
+                um = uc;
+                uc = up[t];
+            }
+            pw += D * pl;
+            pe += D * pl;
+            ps += D * pl;
+            pn += D * pl;
+            pu += D * pl;
+            pf += D * pl;
+            pr += D * pl;
         }
     }
     return P::acc_get(acc, cmp);
 }
 
-// u += e (double-word plus FP32), finest level
-__device__ void t_correct(const BProbDesc& pb, const float* __restrict__ e, int i0, int j0) {
-    const BLevelDesc& L = pb.lev[pb.L];
-    TileIdx t = tile_idx(i0, j0, L.nx, L.ny);
-    if (!t.act) return;
-    const size_t pl = (size_t)L.nx * L.ny, c = (size_t)t.j * L.nx + t.i;
-    // four planes per step: all loads issued before the stores (the planes are disjoint)
-    int k = 0;
-    for (; k + 4 <= L.nz; k += 4) {
-        PolDW::R uv[4];
-        float ev[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uv[q] = PolDW::ld_plain(pb.uD, (size_t)(k + q) * pl + c);
-            ev[q] = __ldg(e + (size_t)(k + q) * pl + c);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) PolDW::st(pb.uD, (size_t)(k + q) * pl + c, PolDW::add(uv[q], PolDW::from_f(ev[q])));
+enum { BM_SMOOTH = 0, BM_LINE = 1, BM_RESTRICT = 2 };
+
+// Levels of 64-column multiples (and ny of 4) have the arithmetic of the single-problem sweeps in every form (SW:
+// sweep_residual's order, the Smooth's back substitution over g_k = u_k + rho d_k - w_k u_{k+1}), the others the
+// plain one; a form that takes a level over gives the same bits.
+__host__ __device__ __forceinline__ bool bsweeps(int nx, int ny) { return nx % 64 == 0 && ny % 4 == 0; }
+
+// The right-hand side of a column's line solve at plane k: f - A u (Smooth), f, or the restricted residual
+template <int MODE, bool SW>
+struct BRhs {
+    const float *u, *f;
+    BCol q;
+    size_t pl;
+    float vv, dh1, dh2;
+    size_t f00;  // BM_RESTRICT: the first of the column's four fine ones
+    int nxf;
+    __device__ BRhs(const BLevelDesc& L, const float* u_, const float* f_, int col) : u(u_), f(f_) {
+        q = bcol(L.nx, L.ny, col);
+        pl = (size_t)L.nx * L.ny;
+        vv = __ldg(L.v + q.c);
+        dh1 = L.krho.dh + vv;
+        dh2 = dh1 + vv;
+        nxf = 2 * L.nx;
+        const int j = (int)(q.c / L.nx), i = (int)(q.c - (size_t)j * L.nx);
+        f00 = (size_t)(2 * j) * nxf + 2 * i;
     }
-    for (; k < L.nz; ++k) {
-        const size_t id = (size_t)k * pl + c;
-        PolDW::st(pb.uD, id, PolDW::add(PolDW::ld_plain(pb.uD, id), PolDW::from_f(__ldg(e + id))));
+    __device__ __forceinline__ float at(const BLevelDesc& L, int k) const {
+        const size_t b = (size_t)k * pl;
+        if (MODE == BM_LINE) return f[b + q.c];
+        if (MODE == BM_RESTRICT) {
+            const float* p = u + 4 * b + f00;
+            return 0.25f * ((p[0] + p[1]) + (p[nxf] + p[nxf + 1]));
+        }
+        const int nz = L.nz;
+        const float um0 = u[b - (k > 0 ? pl : 0) + q.c], up0 = u[b + (k + 1 < nz ? pl : 0) + q.c];
+        const float um = k > 0 ? um0 : 0.f, up = k + 1 < nz ? up0 : 0.f;
+        const float dg = nz == 1 ? L.krho.dh : (k == 0 || k == nz - 1 ? dh1 : dh2);
+        return bresidual<SW>(L.krho, dg, vv, f[b + q.c], u[b + q.c], u[b + q.w], u[b + q.e], u[b + q.s], u[b + q.n], um, up);
+    }
+};
+
+// BF_COLS: out = u + rho M^{-1}(f - A u), rho M^{-1} f, or (u the fine residual) fc = R u, out = rho M^{-1} fc
+template <int MODE, bool SW>
+__device__ void t_cols(const BLevelDesc& L, float rho, const float* u, const float* f, float* fc, float* out, int tile,
+                       unsigned char* smem) {
+    float* const Z = reinterpret_cast<float*>(smem);
+    const int nz = L.nz, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* const T = Z + (size_t)nz * 32;  // the factor tables where lambda^2 is constant
+    const BRhs<MODE, SW> R(L, u, f, tile * 32 + lane);
+    constexpr bool GF = MODE == BM_SMOOTH && SW;  // the back substitution yields the result
+    const size_t pl = R.pl, c = R.q.c;
+    if (!L.percol)
+        for (int k = threadIdx.x; k < nz; k += BNT) {
+            T[k] = __ldg(L.finv + k);
+            T[nz + k] = __ldg(L.fw + k);
+        }
+    constexpr int D = MODE == BM_SMOOTH ? 2 : 4;
+    for (int k = warp; k < nz; k += D * BNW) {
+        float r[D];
+#pragma unroll
+        for (int t = 0; t < D; ++t) r[t] = R.at(L, k + t * BNW < nz ? k + t * BNW : k);
+#pragma unroll
+        for (int t = 0; t < D; ++t) {
+            const int kk = k + t * BNW;
+            if (kk >= nz) break;
+            Z[kk * 32 + lane] = r[t];
+            if (MODE == BM_RESTRICT && R.q.act) fc[(size_t)kk * pl + c] = r[t];
+        }
+    }
+    __syncthreads();
+    constexpr int KB = 8;
+    auto fac = [&](int which, int k) {
+        if (!L.percol) return T[which * nz + k];
+        return __ldg((which ? L.fw : L.finv) + (size_t)k * pl + c);
+    };
+    if (warp == 0) {
+        const float vv = R.vv;
+        float d = 0.f;
+        int k = 0;
+        for (; k + KB <= nz; k += KB) {
+            float r[KB], iv[KB];
+#pragma unroll
+            for (int t = 0; t < KB; ++t) {
+                r[t] = Z[(k + t) * 32 + lane];
+                iv[t] = fac(0, k + t);
+            }
+#pragma unroll
+            for (int t = 0; t < KB; ++t) {
+                d = PolF32::mul(PolF32::fma(vv, d, r[t]), iv[t]);
+                Z[(k + t) * 32 + lane] = d;
+            }
+        }
+        for (; k < nz; ++k) {
+            d = PolF32::mul(PolF32::fma(vv, d, Z[k * 32 + lane]), fac(0, k));
+            Z[k * 32 + lane] = d;
+        }
+    }
+    if (GF) {
+        __syncthreads();
+        for (int k = warp; k < nz; k += BNW) {
+            const float u0 = u[(size_t)k * pl + c], u1 = u[(size_t)(k + 1 < nz ? k + 1 : k) * pl + c];
+            Z[k * 32 + lane] = PolF32::fma(-fac(1, k), k + 1 < nz ? u1 : 0.f, PolF32::fma(rho, Z[k * 32 + lane], u0));
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {
+        float x = 0.f;
+        auto put = [&](int kk, float xk) {
+            if (MODE == BM_SMOOTH && !GF) Z[kk * 32 + lane] = xk;
+            else if (R.q.act) out[(size_t)kk * pl + c] = GF ? xk : PolF32::mul(rho, xk);
+        };
+        int k = nz;
+        for (; k - KB >= 0; k -= KB) {
+            float dk[KB], w[KB];
+#pragma unroll
+            for (int t = 0; t < KB; ++t) {
+                dk[t] = Z[(k - 1 - t) * 32 + lane];
+                w[t] = fac(1, k - 1 - t);
+            }
+#pragma unroll
+            for (int t = 0; t < KB; ++t) {
+                x = PolF32::fma(w[t], x, dk[t]);
+                put(k - 1 - t, x);
+            }
+        }
+        for (; k > 0; --k) {
+            x = PolF32::fma(fac(1, k - 1), x, Z[(k - 1) * 32 + lane]);
+            put(k - 1, x);
+        }
+    }
+    if (MODE == BM_SMOOTH && !GF) {
+        __syncthreads();
+        if (R.q.act)
+            for (int kk = warp; kk < nz; kk += BNW)
+                out[(size_t)kk * pl + c] = PolF32::fma(rho, Z[kk * 32 + lane], u[(size_t)kk * pl + c]);
+    }
+}
+
+// u_f += P u_c (bilinear, cell centred, periodic). A segment is the 2 x 2 fine cells of one coarse column in one
+// plane; where nxc is even, two adjacent ones (16 bytes of both fine rows).
+__device__ void t_prolongate(const BLevelDesc& Lf, const float* uc, float* uf, int tile) {
+    const int nxc = Lf.nx / 2, nyc = Lf.ny / 2;
+    const size_t plc = (size_t)nxc * nyc;
+    const bool two = nxc % 2 == 0;
+    const int nu = two ? nxc / 2 : nxc;
+    const long long n = (long long)nu * nyc * Lf.nz;
+    long long id = (long long)tile * BPU + threadIdx.x;
+    for (int t = 0; t < BPU / BNT && id < n; ++t, id += BNT) {
+        const int kJ = (int)(id / nu), I = (int)(id - (long long)kJ * nu) * (two ? 2 : 1), J = kJ % nyc, k = kJ / nyc;
+        const float* cp = uc + (size_t)k * plc;
+        float* p0 = uf + (size_t)k * 4 * plc + (size_t)(2 * J) * (2 * nxc) + 2 * I;
+        float* p1 = p0 + 2 * nxc;
+        const int Im = bwrap(I - 1, nxc), Ip = bwrap(I + (two ? 2 : 1), nxc);
+        const float* rows[3] = {cp + (size_t)bwrap(J - 1, nyc) * nxc, cp + (size_t)J * nxc, cp + (size_t)bwrap(J + 1, nyc) * nxc};
+        auto val = [](float c, float x, float y, float d) {
+            return __fmaf_rn(0.0625f, d, __fmaf_rn(0.1875f, y, __fmaf_rn(0.5625f, c, __fmul_rn(0.1875f, x))));
+        };
+        if (two) {
+            float4 o0 = *reinterpret_cast<const float4*>(p0), o1 = *reinterpret_cast<const float4*>(p1);
+            float a[3][4];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float2 m = *reinterpret_cast<const float2*>(rows[r] + I);
+                a[r][0] = rows[r][Im];
+                a[r][1] = m.x;
+                a[r][2] = m.y;
+                a[r][3] = rows[r][Ip];
+            }
+            o0.x = __fadd_rn(o0.x, val(a[1][1], a[1][0], a[0][1], a[0][0]));
+            o0.y = __fadd_rn(o0.y, val(a[1][1], a[1][2], a[0][1], a[0][2]));
+            o0.z = __fadd_rn(o0.z, val(a[1][2], a[1][1], a[0][2], a[0][1]));
+            o0.w = __fadd_rn(o0.w, val(a[1][2], a[1][3], a[0][2], a[0][3]));
+            o1.x = __fadd_rn(o1.x, val(a[1][1], a[1][0], a[2][1], a[2][0]));
+            o1.y = __fadd_rn(o1.y, val(a[1][1], a[1][2], a[2][1], a[2][2]));
+            o1.z = __fadd_rn(o1.z, val(a[1][2], a[1][1], a[2][2], a[2][1]));
+            o1.w = __fadd_rn(o1.w, val(a[1][2], a[1][3], a[2][2], a[2][3]));
+            *reinterpret_cast<float4*>(p0) = o0;
+            *reinterpret_cast<float4*>(p1) = o1;
+        } else {
+            const float c = rows[1][I], xm = rows[1][Im], xp = rows[1][Ip];
+            p0[0] = __fadd_rn(p0[0], val(c, xm, rows[0][I], rows[0][Im]));
+            p0[1] = __fadd_rn(p0[1], val(c, xp, rows[0][I], rows[0][Ip]));
+            p1[0] = __fadd_rn(p1[0], val(c, xm, rows[2][I], rows[2][Im]));
+            p1[1] = __fadd_rn(p1[1], val(c, xp, rows[2][I], rows[2][Ip]));
+        }
+    }
+}
+
+// u += e (double-word plus FP32), finest level: four cells a thread, their loads before the stores
+__device__ void t_correct(const BProbDesc& pb, const float* e, int tile) {
+    const BLevelDesc& L = pb.lev[pb.L];
+    const size_t n = (size_t)L.nx * L.ny * L.nz, n4 = n / 4;
+    const size_t q0 = (size_t)tile * (BCH / 4);
+    for (int t = 0; t < BCH / 4 / BNT; ++t) {
+        const size_t q = q0 + t * BNT + threadIdx.x;
+        if (q >= n4) break;
+        float4* pu = reinterpret_cast<float4*>(pb.uD) + 2 * q;
+        const float4 a = pu[0], b = pu[1], ev = reinterpret_cast<const float4*>(e)[q];
+        auto add = [](float hi, float lo, float x) { return PolDW::add(dw{hi, lo}, PolDW::from_f(x)); };
+        const dw r0 = add(a.x, a.y, ev.x), r1 = add(a.z, a.w, ev.y), r2 = add(b.x, b.y, ev.z), r3 = add(b.z, b.w, ev.w);
+        pu[0] = make_float4(r0.hi, r0.lo, r1.hi, r1.lo);
+        pu[1] = make_float4(r2.hi, r2.lo, r3.hi, r3.lo);
+    }
+    if (tile == 0 && threadIdx.x < n - 4 * n4) {  // the last one to three cells
+        const size_t id = 4 * n4 + threadIdx.x;
+        PolDW::st(pb.uD, id, PolDW::add(PolDW::ld_plain(pb.uD, id), PolDW::from_f(e[id])));
     }
 }
 
@@ -275,8 +384,8 @@ __device__ void t_final(const BatchDesc& d, int prob, int it) {
     // a problem that has finished keeps its iteration count, residual and place in the count of
     // active problems (only this block writes this problem's state, before the next barrier)
     if (!*(volatile int*)&d.state[prob].active) return;
-    __shared__ double buf[32 * BTY];
-    const int tid = threadIdx.y * 32 + threadIdx.x, nt = 32 * BTY;
+    __shared__ double buf[BNT];
+    const int tid = threadIdx.x, nt = BNT;
     double s = 0.0;
     for (int q = tid; q < pb.fine_tiles; q += nt) s += d.partials[pb.part_base + q];
     buf[tid] = s;
@@ -316,13 +425,7 @@ __device__ void t_final(const BatchDesc& d, int prob, int it) {
     __syncthreads();
 }
 
-// ---------------------------------------------------------------- two-column tiles
-// Levels whose nx is a multiple of 64 (and ny of BTY) run their Smooth, Residual and first line
-// solve, and the outer double-word residual, on tiles of 64 x BTY columns with the plane-pipelined
-// two-column sweep of the single-problem solver (sweep_x2.cuh): the block's dynamic shared memory
-// holds the rings, its scratch slot the Thomas stack.
-constexpr int BPD = 4;  // ring depth of the two-column sweeps
-
+// ---------------------------------------------------------------- the persistent kernel
 __device__ __forceinline__ Lv<PolF32> lv32(const BLevelDesc& b) {
     Lv<PolF32> L;
     L.nx = b.nx;
@@ -338,127 +441,89 @@ __device__ __forceinline__ Lv<PolF32> lv32(const BLevelDesc& b) {
     return L;
 }
 
-bool batched_x2_fits(int nx, int ny, const void* a, const void* b, const void* out) {
-    auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
-    return nx % 64 == 0 && ny % BTY == 0 && al(a) && al(b) && al(out);
+// Smooth or first line solve of a task on whole-column tiles
+template <int MODE, int TR>
+__device__ __forceinline__ void tile_task(const BTask& tk, const BLevelDesc& bl, int loc, unsigned char* smem) {
+    constexpr int W = TPB / TR / (int)sizeof(float);
+    const int tx = bl.nx / W, by = loc / tx, bx = loc - by * tx;
+    const float* u = (const float*)(MODE == MODE_LINESOLVE ? tk.b : tk.a);
+    sweep_tile_body<PolF32, MODE, TR, true, false, false>(lv32(bl), bl.krho, u, (const float*)tk.b, (float*)tk.out, nullptr,
+                                                          bl.kw, nullptr, bx, by, 0, 0, smem);
 }
 
-size_t batched_smem_bytes() {
-    size_t m = sweep_x2_smem<PolDW, BTY, BPD, MODE_RESIDUAL>();
-    const size_t s1 = sweep_x2_smem<PolF32, BTY, BPD, MODE_SMOOTH>();
-    const size_t s2 = sweep_x2_smem<PolF32, BTY, BPD, MODE_LINESOLVE>();
-    const size_t s3 = sweep_x2_smem<PolF32, BTY, BPD, MODE_RESTRICT>();
-    m = s1 > m ? s1 : m;
-    m = s3 > m ? s3 : m;
-    return s2 > m ? s2 : m;
-}
-
-// ---------------------------------------------------------------- the persistent kernel
-__global__ void __launch_bounds__(32 * BTY, 4) k_batched(BatchDesc d) {
+__global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
     extern __shared__ __align__(16) unsigned char bsmem[];
-    float* stack = d.scratch + (size_t)blockIdx.x * d.nz_max * 64 * BTY;
-    __shared__ double red[32];
+    constexpr int TB = 128;  // tasks of a phase whose first tiles are kept in shared memory
+    __shared__ int base[TB];
     const float rho = (float)d.rho;
     for (int it = 0; it <= d.max_iter; ++it) {
         for (int ph = 0; ph < d.nphase; ++ph) {
             const int tb = d.phase_begin[ph], te = d.phase_begin[ph + 1];
             const int ntiles = d.phase_tiles[ph];
+            for (int t = threadIdx.x; t < te - tb && t < TB; t += BNT) base[t] = d.tasks[tb + t].tile_base;
+            __syncthreads();
             for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
                 // the task owning tile t (tasks of a phase are sorted by tile_base)
-                int lo = tb, hi = te - 1;
+                int lo = 0, hi = te - tb - 1;
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
-                    if (d.tasks[mid].tile_base <= t) lo = mid;
+                    if ((mid < TB ? base[mid] : d.tasks[tb + mid].tile_base) <= t) lo = mid;
                     else hi = mid - 1;
                 }
-                const BTask& tk = d.tasks[lo];
+                const BTask& tk = d.tasks[tb + lo];
                 if (tk.type == BT_FINAL) {
                     t_final(d, tk.prob, it);
                     continue;
                 }
                 if (!*(volatile int*)&d.state[tk.prob].active) continue;
-                const int loc = t - tk.tile_base;
-                const int i0 = (loc % tk.tiles_x) * 32, j0 = (loc / tk.tiles_x) * BTY;
+                const int loc = t - tk.tile_base, form = tk.form;
                 const BProbDesc& pb = d.probs[tk.prob];
-                if (tk.x2) {
-                    switch (tk.type) {
-                        case BT_OUTRES: {
-                            Lv<PolDW> LD;
-                            const BLevelDesc& bl = pb.lev[pb.L];
-                            LD.nx = bl.nx;
-                            LD.ny = bl.ny;
-                            LD.nz = bl.nz;
-                            LD.cx = bl.cx;
-                            LD.cy = bl.cy;
-                            LD.v = pb.vD;
-                            LD.finv = LD.fw = nullptr;
-                            LD.fac_percol = 0;
-                            LD.variant = -1;
-                            const double s = sweep_x2_tiles<PolDW, PolF32, BTY, BPD, MODE_RESIDUAL, 0>(
-                                LD, pb.kD, pb.uD, pb.fD, pb.r32, true, loc, loc + 1, 1, nullptr, bsmem);
-                            if (threadIdx.x == 0 && threadIdx.y == 0) d.partials[pb.part_base + loc] = s;
-                            break;
-                        }
-                        case BT_LS0:
-                            sweep_x2_tiles<PolF32, PolF32, BTY, BPD, MODE_LINESOLVE, HINT_ALL>(
-                                lv32(pb.lev[tk.level]), pb.lev[tk.level].krho, (const float*)tk.b, nullptr, (float*)tk.out, false, loc,
-                                loc + 1, 1, stack, bsmem);
-                            break;
-                        case BT_SMOOTH:
-                            sweep_x2_tiles<PolF32, PolF32, BTY, BPD, MODE_SMOOTH, HINT_ALL>(
-                                lv32(pb.lev[tk.level]), pb.lev[tk.level].krho, (const float*)tk.a, (const float*)tk.b, (float*)tk.out,
-                                false, loc, loc + 1, 1, stack, bsmem);
-                            break;
-                        case BT_RESID:
-                            sweep_x2_tiles<PolF32, PolF32, BTY, BPD, MODE_RESIDUAL, 0>(
-                                lv32(pb.lev[tk.level]), pb.lev[tk.level].k1, (const float*)tk.a, (const float*)tk.b, (float*)tk.out,
-                                false, loc, loc + 1, 1, nullptr, bsmem);
-                            break;
-                        case BT_RRS: {
-                            const XRestrict<PolF32> xr{lv32(pb.lev[tk.level - 1]), pb.lev[tk.level - 1].krho.coef,
-                                                       0.25f, (float*)tk.out, (float*)tk.out2};
-                            sweep_x2_tiles<PolF32, PolF32, BTY, BPD, MODE_RESTRICT, 0>(
-                                lv32(pb.lev[tk.level]), pb.lev[tk.level].k1, (const float*)tk.a, (const float*)tk.b, nullptr, false,
-                                loc, loc + 1, 1, stack, bsmem, &xr);
-                            break;
-                        }
-                        default:
-                            break;
-                    }
-                    continue;
-                }
+                const BLevelDesc& bl = pb.lev[tk.level];
+                const bool sw = bsweeps(bl.nx, bl.ny);
+                const float *a = (const float*)tk.a, *b = (const float*)tk.b;
+                float *o = (float*)tk.out, *o2 = (float*)tk.out2;
                 switch (tk.type) {
                     case BT_OUTRES: {
-                        double s = t_outres(pb, i0, j0);
-                        s = block_sum(s);
-                        if (threadIdx.x == 0 && threadIdx.y == 0) d.partials[pb.part_base + loc] = s;
-                        (void)red;
+                        const double s = block_sum(t_residual<PolDW, PolF32, true, true>(bl.nx, bl.ny, bl.nz, pb.kD, pb.vD, pb.uD,
+                                                                                   pb.fD, pb.r32, loc));
+                        if (threadIdx.x == 0) d.partials[pb.part_base + loc] = s;
                         break;
                     }
                     case BT_LS0:
-                        t_sweep<2>(pb.lev[tk.level], rho, nullptr, (const float*)tk.b, (float*)tk.out, i0, j0, stack);
+                        if (form == BF_TILE1) tile_task<MODE_LINESOLVE, 1>(tk, bl, loc, bsmem);
+                        else if (form == BF_TILE4) tile_task<MODE_LINESOLVE, 4>(tk, bl, loc, bsmem);
+                        else t_cols<BM_LINE, true>(bl, rho, nullptr, b, nullptr, o, loc, bsmem);
                         break;
                     case BT_SMOOTH:
-                        t_sweep<0>(pb.lev[tk.level], rho, (const float*)tk.a, (const float*)tk.b, (float*)tk.out, i0, j0,
-                                   stack);
+                        if (form == BF_TILE1) tile_task<MODE_SMOOTH, 1>(tk, bl, loc, bsmem);
+                        else if (form == BF_TILE4) tile_task<MODE_SMOOTH, 4>(tk, bl, loc, bsmem);
+                        else if (sw) t_cols<BM_SMOOTH, true>(bl, rho, a, b, nullptr, o, loc, bsmem);
+                        else t_cols<BM_SMOOTH, false>(bl, rho, a, b, nullptr, o, loc, bsmem);
                         break;
                     case BT_RESID:
-                        t_sweep<1>(pb.lev[tk.level], rho, (const float*)tk.a, (const float*)tk.b, (float*)tk.out, i0, j0,
-                                   stack);
+                        if (sw) t_residual<PolF32, PolF32, true, false>(bl.nx, bl.ny, bl.nz, bl.k1, bl.v, a, b, o, loc);
+                        else t_residual<PolF32, PolF32, false, false>(bl.nx, bl.ny, bl.nz, bl.k1, bl.v, a, b, o, loc);
                         break;
                     case BT_RS:
-                        t_restrict_smooth(pb.lev[tk.level], rho, (const float*)tk.a, (float*)tk.out, (float*)tk.out2, i0,
-                                          j0, stack);
+                        t_cols<BM_RESTRICT, true>(bl, rho, a, nullptr, o, o2, loc, bsmem);
                         break;
+                    case BT_RRS: {
+                        const BLevelDesc& bc = pb.lev[tk.level - 1];
+                        const XRestrict<PolF32> xr{lv32(bc), bc.krho.coef, 0.25f, o, o2};
+                        const int tx = bl.nx / 128, by = loc / tx, bx = loc - by * tx;
+                        restrict_tile_body<PolF32, true, false>(lv32(bl), bl.k1, xr, a, b, bc.kw, bx, by, bsmem);
+                        break;
+                    }
                     case BT_PROL:
-                        t_prolongate(pb.lev[tk.level], (const float*)tk.a, (float*)tk.out, i0, j0);
+                        t_prolongate(bl, a, o, loc);
                         break;
                     case BT_CORR:
-                        t_correct(pb, (const float*)tk.a, i0, j0);
+                        t_correct(pb, a, loc);
                         break;
                     default:
                         break;
                 }
+                __syncthreads();  // before the next tile takes the shared memory
             }
             if (!grid_barrier(d)) return;
             // after the convergence phase every block sees the same count of active problems
@@ -467,19 +532,54 @@ __global__ void __launch_bounds__(32 * BTY, 4) k_batched(BatchDesc d) {
     }
 }
 
-int batched_blocks_per_sm() {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batched, 32 * BTY, batched_smem_bytes()) != cudaSuccess)
-        return 0;
-    return nb < 8 ? nb : 8;  // 8 x 128 threads per SM; more only grows the scratch
+// ---------------------------------------------------------------- tasks and launch
+// The vector tiles (cx == cy: their square-cell form) take the levels with the sweeps' arithmetic, all others the
+// 32-column form.
+int batched_form(int type, int nx, int ny, int nz, int percol, int kw, bool square) {
+    const size_t tile = (size_t)nz * TPB + (percol ? (size_t)kw * TPB : 2 * (size_t)nz * sizeof(float));
+    if (type == BT_SMOOTH || type == BT_LS0) {
+        if (square && bsweeps(nx, ny) && tile <= BTILE_SMEM) {
+            return nx % 128 == 0 ? BF_TILE1 : BF_TILE4;
+        }
+        return BF_COLS;
+    }
+    if (type == BT_RRS)  // nx, ny of the fine level, percol and kw of the coarse one
+        return square && bsweeps(nx, ny) && nx % 128 == 0 && batched_smem(BT_RRS, BF_TILE1, nz, percol, kw) <= BTILE_SMEM ? BF_TILE1 : -1;
+    return BF_COLS;
 }
-
-size_t batched_scratch_floats(int grid, int nz_max) { return (size_t)grid * nz_max * 64 * BTY; }
-
+size_t batched_smem(int type, int form, int nz, int percol, int kw) {
+    const size_t tables = percol ? 0 : 2 * (size_t)nz * sizeof(float);
+    if (type == BT_RRS) return (size_t)(nz + (percol ? kw : 0)) * 256 + tables;
+    if (type != BT_SMOOTH && type != BT_LS0 && type != BT_RS) return 0;
+    if (form == BF_COLS) return (size_t)nz * 128 + 2 * (size_t)nz * sizeof(float);
+    return (size_t)(nz + (percol ? kw : 0)) * TPB + tables;
+}
+int batched_tiles(int type, int form, int nx, int ny, int nz) {
+    const long long cols = (long long)nx * ny;
+    auto up = [](long long a, long long b) { return (int)((a + b - 1) / b); };
+    switch (type) {
+        case BT_SMOOTH:
+        case BT_LS0:
+        case BT_RS: return up(cols, form == BF_COLS ? 32 : 128);
+        case BT_RRS: return nx / 128 * (ny / 2);
+        case BT_RESID:
+        case BT_OUTRES: return up(cols, BNT) * up(nz, BPZ);
+        case BT_PROL: return up((long long)(nx / 2 % 2 == 0 ? nx / 4 : nx / 2) * (ny / 2) * nz, BPU);
+        case BT_CORR: return up(cols * nz, BCH);
+        default: return 1;
+    }
+}
+int batched_blocks_per_sm(size_t smem) {
+    int nb = 0;
+    if (cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BTILE_SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batched, BNT, smem) != cudaSuccess)
+        return 0;
+    return nb;
+}
 cudaError_t launch_batched(const BatchDesc& d, int grid, size_t smem, cudaStream_t s) {
     BatchDesc arg = d;
     void* args[] = {&arg};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_batched, dim3(grid), dim3(32, BTY), args, smem, s);
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_batched, dim3(grid), dim3(BNT), args, smem, s);
     if (e == cudaSuccess) note_launch();
     return e;
 }

@@ -237,6 +237,9 @@ int max_partials(int nx, int ny);
 // Thomas factors of level L into finv/fw (per cell when percol, else a table of nz entries).
 template <class P>
 void launch_factors(const Lv<P>& L, typename P::S* finv, typename P::S* fw, int percol, cudaStream_t s);
+// planes before the converged per-cell factors (all but the last when none has converged)
+template <class P>
+inline int factor_planes(const Lv<P>& L) { return L.fac_k0 < L.nz - 1 ? (L.fac_k0 > 0 ? L.fac_k0 : 0) : L.nz - 1; }
 // first plane of the converged range of per-cell factors (see Lv::fac_k0), written to *k0 (device
 // int, initialised by the caller to 0): the maximum over the columns
 template <class P>
@@ -401,11 +404,13 @@ void launch_cg_finish(size_t n, const Scalars* sc, typename P::S* u, const typen
 // (a = u, b = f of the fine level, out = f_c, out2 = u_c), where the fine level takes 64 x BTY tiles
 enum { BT_OUTRES = 0, BT_FINAL = 1, BT_LS0 = 2, BT_SMOOTH = 3, BT_RESID = 4, BT_RS = 5, BT_PROL = 6, BT_CORR = 7,
        BT_RRS = 8 };
-static constexpr int BTY = 4;  // rows of columns per tile (block = 32 x BTY threads)
+// forms of a task's tiles (k_batched.cu)
+enum { BF_TILE1 = 0, BF_TILE4 = 1, BF_COLS = 2 };
 static constexpr int BMAXL = 16;
 
 struct BLevelDesc {  // FP32 view of one level of one problem
     int nx, ny, nz, percol;
+    int kw;  // percol: planes whose factors differ from the converged ones
     double cx, cy;
     const float* v;
     const float* finv;
@@ -422,7 +427,6 @@ struct BProbDesc {
     float* r32;         // FP32 right-hand side of the inner cycle (finest level)
     int part_base;      // first partial-sum slot of this problem's outer residual norm
     int fine_tiles;     // tiles of the outer residual (= its partial sums)
-    int fine_x2;        // 1: the outer residual runs on two-column tiles
     double* history;    // relative residual history (max_iter + 1 doubles)
 };
 struct BTask {
@@ -431,8 +435,7 @@ struct BTask {
     const void* b;  // right-hand side
     void* out;
     void* out2;
-    int tiles_x, tiles_y, tile_base;
-    int x2;  // 1: tiles of 64 x BTY columns run by the two-column sweep (Smooth, Residual, line solve, RRS)
+    int form, tiles, tile_base;
 };
 struct BState {
     double r0, rel;
@@ -453,17 +456,15 @@ struct BatchDesc {
     double rho, tol;
     int max_iter;
     unsigned long long timeout_ns;
-    int nz_max;
-    float* scratch;  // Thomas stacks: nz_max x 64 BTY floats per block
 };
 // cooperative launch of the persistent kernel; returns the CUDA status of the launch
 cudaError_t launch_batched(const BatchDesc& d, int grid, size_t smem, cudaStream_t s);
-// blocks per SM of the persistent kernel and its dynamic shared memory (the two-column sweep's rings)
-int batched_blocks_per_sm();
-size_t batched_smem_bytes();
-size_t batched_scratch_floats(int grid, int nz_max);
-// whether a level of nx x ny columns and its fields suit the two-column sweep tiles
-bool batched_x2_fits(int nx, int ny, const void* a, const void* b, const void* out);
+// The form a task's tiles take (BT_RRS: nx, ny of the fine level, percol and kw of the coarse one; -1: the two
+// separate tasks), the number of tiles, and the dynamic shared memory of a block
+int batched_form(int type, int nx, int ny, int nz, int percol, int kw, bool square);
+int batched_tiles(int type, int form, int nx, int ny, int nz);
+size_t batched_smem(int type, int form, int nz, int percol, int kw);
+int batched_blocks_per_sm(size_t smem);
 
 // ---------------------------------------------------------------- scalar kernels (k_util.cu)
 // modes of finalize_norm

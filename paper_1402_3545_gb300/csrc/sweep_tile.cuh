@@ -52,6 +52,12 @@ struct TileVec {  // 16 bytes of adjacent columns
     }
     __device__ __forceinline__ void ldg(const S* p) { from(__ldg(reinterpret_cast<const float4*>(p))); }
     __device__ __forceinline__ void lds(const S* p) { from(*reinterpret_cast<const float4*>(p)); }
+    // a field: through the read-only cache, or by ordinary loads where this kernel itself writes it
+    template <bool RO>
+    __device__ __forceinline__ void ldf(const S* p) {
+        if (RO) ldg(p);
+        else lds(p);
+    }
     __device__ __forceinline__ void sts(S* p) const {
         float4 t;
         S* q = reinterpret_cast<S*>(&t);
@@ -111,13 +117,16 @@ __device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
 // and d' = D^{-1} yh, so <r, M^{-1} r> = sum_k yh_k d'_k, and the back substitution does not read r again.
 constexpr int MODE_CGTRI = 16;
 
+// One tile: columns bx * W .., rows by * TR ...
 // kw: planes whose factors are kept per column in shared memory behind the nz planes of the tile (0
-// when lambda^2 is constant). ISO: square cells; NORM: partial sums of ||f - A u||^2 (both compile-time:
-// as runtime choices their instructions were issued either way)
-template <class P, int MODE, int TR, bool ISO, bool NORM>
-__global__ void __launch_bounds__(TNT, 3)
-    k_sweep_tile(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u, const typename P::S* __restrict__ f,
-                 typename P::S* __restrict__ out, double* partials, const int* done, int kw, const Scalars* sc) {
+// when lambda^2 is constant). ISO: square cells; NORM: partial sums of ||f - A u||^2, this tile's at part of
+// nparts (both compile-time: as runtime choices their instructions were issued either way). RO: the fields read
+// are not written by the kernel
+template <class P, int MODE, int TR, bool ISO, bool NORM, bool RO>
+__device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>& K, const typename P::S* u,
+                                                const typename P::S* f, typename P::S* out, double* partials, int kw,
+                                                const Scalars* sc, int bx, int by, int part, int nparts,
+                                                unsigned char* smem_raw) {
     typedef typename P::S S;
     typedef typename P::R R;
     typedef TileVec<P> V;
@@ -127,13 +136,11 @@ __global__ void __launch_bounds__(TNT, 3)
     constexpr bool DIRECT = GFORM || MODE == MODE_LINESOLVE || CG;  // the back substitution yields the result
     constexpr int G = 32 / TR;                                // lanes of a tile row
     constexpr int N = V::N, W = G * N, NC = TR * W;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (done && *(volatile const int*)done) return;
     S* const Z = reinterpret_cast<S*>(smem_raw);
     const int nx = L.nx, ny = L.ny, nz = L.nz;
     S* const ZW = Z + (size_t)nz * NC;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, lx = lane % G, ry = lane / G;
-    const int i0 = blockIdx.x * W, j0 = blockIdx.y * TR;
+    const int i0 = bx * W, j0 = by * TR;
     const size_t pl = (size_t)nx * ny;
     const size_t c = (size_t)(j0 + ry) * nx + i0 + lx * N;  // this thread's first column
     const int zo = lane * N;                                // ... in a tile plane
@@ -178,9 +185,9 @@ __global__ void __launch_bounds__(TNT, 3)
             um.zero();
             vv.zero();
             dg.zero();
-            uc.ldg(pu);
+            uc.template ldf<RO>(pu);
             if (MODE == MODE_SMOOTH) {
-                if (klo > 0) um.ldg(pu - pl);
+                if (klo > 0) um.template ldf<RO>(pu - pl);
 #pragma unroll
                 for (int q = 0; q < N; ++q) {
                     vv.v[q] = P::ld(L.v, c + q);
@@ -196,13 +203,13 @@ __global__ void __launch_bounds__(TNT, 3)
                 const bool top = k + B == nz;  // the last plane has no upper neighbour
 #pragma unroll
                 for (int t = 0; t < B; ++t) {  // u of plane k+t+1, the halo of plane k+t
-                    if (MODE == MODE_SMOOTH || t + 1 < B || !top) ru[t].ldg(t + 1 == B && top ? pu : pu + pl);
+                    if (MODE == MODE_SMOOTH || t + 1 < B || !top) ru[t].template ldf<RO>(t + 1 == B && top ? pu : pu + pl);
                     else ru[t].zero();
                     rh[t].zero();
                     re[t] = vzero;
-                    if (hrow) rh[t].ldg(ph);
-                    if (TR == 1) rh1[t].ldg(ph1);
-                    if (hcol) re[t] = P::ld(pe, 0);
+                    if (hrow) rh[t].template ldf<RO>(ph);
+                    if (TR == 1) rh1[t].template ldf<RO>(ph1);
+                    if (hcol) re[t] = RO ? P::ld(pe, 0) : P::ld_plain(pe, 0);
                     pu += pl;
                     ph += pl;
                     ph1 += pl;
@@ -259,7 +266,7 @@ __global__ void __launch_bounds__(TNT, 3)
 #pragma unroll 4
         for (int k = klo; k < khi; ++k, pq += pl, pr += pl, z += NC) {
             V q, r;
-            q.ldg(pq);
+            q.template ldf<RO>(pq);
             if (!landed) {
                 cp_wait<0>();  // this thread's pieces of r
                 landed = true;
@@ -364,12 +371,12 @@ __global__ void __launch_bounds__(TNT, 3)
             }
             const S* pu = u + (size_t)klo * pl + c;
             S* z = Z + klo * NC + zo;
-            uc.ldg(pu);
+            uc.template ldf<RO>(pu);
 #pragma unroll 4
             for (int k = klo; k < khi; ++k, z += NC) {
                 pu += pl;
                 up.zero();
-                if (k + 1 < nz) up.ldg(pu);
+                if (k + 1 < nz) up.template ldf<RO>(pu);
                 V g, w = cw;
                 g.lds(z);
                 if (k < kw) w.lds(ZW + k * NC + zo);
@@ -456,7 +463,7 @@ __global__ void __launch_bounds__(TNT, 3)
 #pragma unroll 4
         for (int k = klo; k < khi; ++k, pu += pl, po += pl, z += NC) {
             V x, uo;
-            uo.ldg(pu);
+            uo.template ldf<RO>(pu);
             x.lds(z);
 #pragma unroll
             for (int q = 0; q < N; ++q)
@@ -466,13 +473,23 @@ __global__ void __launch_bounds__(TNT, 3)
     }
     if (NORM) {
         const double sm = block_sum(P::acc_get(acc, cmp));
-        if (tid == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = sm;
+        if (tid == 0) partials[part] = sm;
         if constexpr (CG) {
             __syncthreads();
             const double sz = block_sum(P::acc_get(az, cz));
-            if (tid == 0) partials[gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = sz;
+            if (tid == 0) partials[nparts + part] = sz;
         }
     }
+}
+
+template <class P, int MODE, int TR, bool ISO, bool NORM>
+__global__ void __launch_bounds__(TNT, 3)
+    k_sweep_tile(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u, const typename P::S* __restrict__ f,
+                 typename P::S* __restrict__ out, double* partials, const int* done, int kw, const Scalars* sc) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (done && *(volatile const int*)done) return;
+    sweep_tile_body<P, MODE, TR, ISO, NORM, true>(L, K, u, f, out, partials, kw, sc, blockIdx.x, blockIdx.y,
+                                                  blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, smem_raw);
 }
 
 template <class P, int MODE, int TR, bool ISO, bool NORM>
@@ -480,9 +497,8 @@ static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, c
                           typename P::S* out, double* partials, const int* done, cudaStream_t s,
                           const Scalars* sc = nullptr) {
     typedef typename P::S S;
-    // planes whose factors differ from the converged ones (all but the last when none has converged)
     int kw = 0;
-    if (L.fac_percol) kw = L.fac_k0 < L.nz - 1 ? (L.fac_k0 > 0 ? L.fac_k0 : 0) : L.nz - 1;
+    if (L.fac_percol) kw = factor_planes(L);
     const size_t smem = (size_t)(L.nz + kw) * TPB + (L.fac_percol ? 0 : 2 * (size_t)L.nz * sizeof(S));
     auto kern = k_sweep_tile<P, MODE, TR, ISO, NORM>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * TPB);
