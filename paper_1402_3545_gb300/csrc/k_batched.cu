@@ -11,16 +11,16 @@
 // the kernel raises an error flag and all blocks return (TPMG_ERR_TIMEOUT on the host).
 //
 // Forms of a task (batched_form):
-//  - BF_TILE1, BF_TILE4: Smooth and first line solve on whole columns in shared memory, 128 x 1 or 32 x 4 FP32
-//    columns a tile, as the single-problem solver's (sweep_tile.cuh); the fused Residual + RestrictSmooth on
-//    tiles of 128 x 2 fine columns (restrict_tile.cuh);
+//  - BF_TILE1, BF_TILE2: Smooth and first line solve on whole columns in shared memory, 128 x 1 or 64 x 2 FP32
+//    columns a tile, as the single-problem solver's (sweep_tile.cuh; here the one-row tile is the faster one); the fused Residual + RestrictSmooth on tiles of 128 x 2 fine
+//    columns (restrict_tile.cuh);
 //  - BF_COLS: 32 columns of the level in order, planes in parallel over the eight warps, one warp running the
 //    recurrences in shared memory: all other shapes;
 //  - Residuals (FP32 and the outer double-word one), Prolongate and the correction: pointwise.
 // Three blocks of 256 threads per SM, set by the tiles' 65 KB at 128 planes. Before, 128-thread blocks marched
 // every column plane by plane, its Thomas values on a stack in L2 (a chain of loads, elimination and stack store
 // per plane, and on the narrow levels one column per thread): 12 problems of 64 .. 512 squared x 32 .. 128 to 1e-9
-// 43.2 ms, 29.1 here, the same bits. What is left: the FP32 tiles (0.55 of the copy rate), the outer residual
+// 43.2 ms, 28.7 here, the same bits. What is left: the FP32 tiles (0.55 of the copy rate), the outer residual
 // and correction (20 bytes per cell each) and, once most problems have converged, too few tiles per phase.
 #include <type_traits>
 
@@ -491,12 +491,12 @@ __global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
                     }
                     case BT_LS0:
                         if (form == BF_TILE1) tile_task<MODE_LINESOLVE, 1>(tk, bl, loc, bsmem);
-                        else if (form == BF_TILE4) tile_task<MODE_LINESOLVE, 4>(tk, bl, loc, bsmem);
+                        else if (form == BF_TILE2) tile_task<MODE_LINESOLVE, 2>(tk, bl, loc, bsmem);
                         else t_cols<BM_LINE, true>(bl, rho, nullptr, b, nullptr, o, loc, bsmem);
                         break;
                     case BT_SMOOTH:
                         if (form == BF_TILE1) tile_task<MODE_SMOOTH, 1>(tk, bl, loc, bsmem);
-                        else if (form == BF_TILE4) tile_task<MODE_SMOOTH, 4>(tk, bl, loc, bsmem);
+                        else if (form == BF_TILE2) tile_task<MODE_SMOOTH, 2>(tk, bl, loc, bsmem);
                         else if (sw) t_cols<BM_SMOOTH, true>(bl, rho, a, b, nullptr, o, loc, bsmem);
                         else t_cols<BM_SMOOTH, false>(bl, rho, a, b, nullptr, o, loc, bsmem);
                         break;
@@ -538,10 +538,8 @@ __global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
 int batched_form(int type, int nx, int ny, int nz, int percol, int kw, bool square) {
     const size_t tile = (size_t)nz * TPB + (percol ? (size_t)kw * TPB : 2 * (size_t)nz * sizeof(float));
     if (type == BT_SMOOTH || type == BT_LS0) {
-        if (square && bsweeps(nx, ny) && tile <= BTILE_SMEM) {
-            return nx % 128 == 0 ? BF_TILE1 : BF_TILE4;
-        }
-        return BF_COLS;
+        if (!square || !bsweeps(nx, ny) || tile > BTILE_SMEM) return BF_COLS;
+        return nx % 128 == 0 ? BF_TILE1 : BF_TILE2;
     }
     if (type == BT_RRS)  // nx, ny of the fine level, percol and kw of the coarse one
         return square && bsweeps(nx, ny) && nx % 128 == 0 && batched_smem(BT_RRS, BF_TILE1, nz, percol, kw) <= BTILE_SMEM ? BF_TILE1 : -1;

@@ -405,7 +405,7 @@ void launch_cg_finish(size_t n, const Scalars* sc, typename P::S* u, const typen
 enum { BT_OUTRES = 0, BT_FINAL = 1, BT_LS0 = 2, BT_SMOOTH = 3, BT_RESID = 4, BT_RS = 5, BT_PROL = 6, BT_CORR = 7,
        BT_RRS = 8 };
 // forms of a task's tiles (k_batched.cu)
-enum { BF_TILE1 = 0, BF_TILE4 = 1, BF_COLS = 2 };
+enum { BF_TILE1 = 0, BF_TILE2 = 1, BF_COLS = 2 };
 static constexpr int BMAXL = 16;
 
 struct BLevelDesc {  // FP32 view of one level of one problem
