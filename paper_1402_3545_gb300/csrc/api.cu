@@ -87,7 +87,7 @@ struct tpmg_op {
     int fac_k0[3][MAXL + 1];       // first plane of the converged factor range (Lv::fac_k0)
     double kappa_M[MAXL + 1] = {}; // condition number of the level's column blocks
     int lsw_dw = 1;                // the double-word solver uses native FP64 below this level
-    bool fac_ready[3] = {false, false, false};
+    int fac_top[3] = {0, 0, 0};  // levels up to which the factors are ready
     int variant[3][MAXL + 1];      // autotuned tile variant of the pipelined Smooth (-1: default)
     int fuse_restrict = 1;         // V-cycles fuse Residual and RestrictSmooth where the kernel applies
     void* cgbuf[3][4] = {};  // r, z, p, q per policy
@@ -254,13 +254,15 @@ static tpmg_status ensure_history(tpmg_op* op, int n) {
     return TPMG_OK;
 }
 
-// Thomas factors of every level in precision pid, computed once (they depend on the operator only)
-static tpmg_status ensure_factors(tpmg_op* op, int pid) {
-    if (op->fac_ready[pid]) return TPMG_OK;
+// Thomas factors of the levels up to `top` (0: all) in precision pid, computed once (they depend on the
+// operator only)
+static tpmg_status ensure_factors(tpmg_op* op, int pid, int top = 0) {
+    if (top < 1) top = op->g.L;
+    if (op->fac_top[pid] >= top) return TPMG_OK;
     TRY(ensure_common(op));
     TRY(dalloc(&op->gstack, gstack_bytes(op->g.nz)));
     const size_t eb = elem_bytes(pid);
-    for (int l = 1; l <= op->g.L; ++l) {
+    for (int l = op->fac_top[pid] + 1; l <= top; ++l) {
         size_t nvals = op->percol[l] ? lvl_cells(op, l) : (size_t)op->g.nz;
         TRY(dalloc(&op->finv[pid][l], nvals * eb));
         TRY(dalloc(&op->fw[pid][l], nvals * eb));
@@ -308,7 +310,7 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid) {
         }
     }
     CK(cudaDeviceSynchronize());
-    op->fac_ready[pid] = true;
+    op->fac_top[pid] = top;
     return TPMG_OK;
 }
 
@@ -889,7 +891,7 @@ tpmg_status tpmg_op_reserve(tpmg_op* op, tpmg_precision prec) {
             TRY(ensure_hier(op, 2, true));
             TRY(ensure_cg(op, 2));
             TRY(ensure_io(op));
-            if (op->lsw_dw > 1) TRY(ensure_factors(op, 0));  // the levels that run in native FP64
+            if (op->lsw_dw > 1) TRY(ensure_factors(op, 0, op->lsw_dw - 1));  // the levels that run in native FP64
             break;
         case TPMG_MIXED: TRY(ensure_hier(op, 2, true)); TRY(ensure_hier(op, 1, true)); break;
         default: return set_err(TPMG_ERR_ARG, "unknown precision");
@@ -946,9 +948,11 @@ static void out_back(tpmg_op* op, cudaStream_t s, int slot, void* y, size_t n) {
     if (P::id == 2) DWIO{op, s}.out(slot, y, n);
 }
 
-static tpmg_status prep_unit(tpmg_op* op, tpmg_precision prec) {
+// low: a double-word call on a level that runs in native FP64 (prec is TPMG_F64): only those levels' factors
+static tpmg_status prep_unit(tpmg_op* op, tpmg_precision prec, bool low = false) {
     if (prec == TPMG_DW) TRY(ensure_io(op));
-    if (prec == TPMG_F64 || prec == TPMG_F32 || prec == TPMG_DW) TRY(ensure_factors(op, pid_of(prec)));
+    if (low) TRY(ensure_factors(op, 0, op->lsw_dw - 1));
+    else if (prec == TPMG_F64 || prec == TPMG_F32 || prec == TPMG_DW) TRY(ensure_factors(op, pid_of(prec)));
     return ensure_common(op);
 }
 
@@ -957,9 +961,10 @@ extern "C" {
 tpmg_status tpmg_apply_A(tpmg_op* op, int level, tpmg_precision prec, const void* x, void* y, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    const bool low = prec == TPMG_DW && level < op->lsw_dw;
+    if (low) prec = TPMG_F64;  // see DW_KAPPA_MAX
     if (!x || !y) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = lvl_cells(op, level);
     DISPATCH_PREC(prec, {
@@ -975,9 +980,10 @@ tpmg_status tpmg_apply_A(tpmg_op* op, int level, tpmg_precision prec, const void
 tpmg_status tpmg_line_solve(tpmg_op* op, int level, tpmg_precision prec, const void* b, void* x, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    const bool low = prec == TPMG_DW && level < op->lsw_dw;
+    if (low) prec = TPMG_F64;  // see DW_KAPPA_MAX
     if (!x || !b) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = lvl_cells(op, level);
     DISPATCH_PREC(prec, {
@@ -994,9 +1000,10 @@ tpmg_status tpmg_smooth(tpmg_op* op, int level, tpmg_precision prec, double rho,
                         const void* f, void* u_out, double* norm_out, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    const bool low = prec == TPMG_DW && level < op->lsw_dw;
+    if (low) prec = TPMG_F64;  // see DW_KAPPA_MAX
     if (!u || !f || !u_out) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = lvl_cells(op, level);
     DISPATCH_PREC(prec, {
@@ -1016,9 +1023,10 @@ tpmg_status tpmg_residual(tpmg_op* op, int level, tpmg_precision prec, const voi
                           void* r, double* norm_out, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    const bool low = prec == TPMG_DW && level < op->lsw_dw;
+    if (low) prec = TPMG_F64;  // see DW_KAPPA_MAX
     if (!u || !f || !r) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = lvl_cells(op, level);
     DISPATCH_PREC(prec, {
@@ -1038,10 +1046,11 @@ tpmg_status tpmg_restrict_smooth(tpmg_op* op, int level, tpmg_precision prec, do
                                  void* f_c, void* u_c, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    const bool low = prec == TPMG_DW && level < op->lsw_dw;
+    if (low) prec = TPMG_F64;  // see DW_KAPPA_MAX
     if (level >= op->g.L) return set_err(TPMG_ERR_ARG, "restrict_smooth needs a coarse level < L");
     if (!r_fine || !f_c || !u_c) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nc = lvl_cells(op, level), nf = lvl_cells(op, level + 1);
     DISPATCH_PREC(prec, {
@@ -1063,10 +1072,11 @@ tpmg_status tpmg_residual_restrict_smooth(tpmg_op* op, int level, tpmg_precision
     TRY(check_level(op, level));
     if (level >= op->g.L) return set_err(TPMG_ERR_ARG, "residual_restrict_smooth needs a coarse level < L");
     if (!u_fine || !f_fine || !f_c || !u_c) return set_err(TPMG_ERR_ARG, "NULL field");
-    if (prec == TPMG_DW && level + 1 < op->lsw_dw) prec = TPMG_F64;  // see DW_KAPPA_MAX
+    // see DW_KAPPA_MAX; a small coarse level has no fused form
+    if (prec == TPMG_DW && level + 1 < op->lsw_dw && lvl_cells(op, level) / op->g.nz > (size_t)PCR_MAX_COLS) prec = TPMG_F64;
     if (prec == TPMG_DW && level < op->lsw_dw) {
-        // double-word fine level over a native-FP64 coarse level: the two kernels, the residual
-        // handed over in FP64 through a staging buffer
+        // a native-FP64 coarse level, the fine one in either: the two kernels, the residual handed over in FP64
+        // through a staging buffer
         TRY(prep_unit(op, prec));
         TRY(tpmg_residual(op, level + 1, prec, u_fine, f_fine, op->io[3], nullptr, stream));
         return tpmg_restrict_smooth(op, level, prec, rho, op->io[3], f_c, u_c, stream);
@@ -1119,10 +1129,11 @@ tpmg_status tpmg_set_fusion(tpmg_op* op, int enable) {
 tpmg_status tpmg_prolongate(tpmg_op* op, int level, tpmg_precision prec, const void* u_c, void* u_f, void* stream) {
     TRY(flat_only(op));
     TRY(check_level(op, level));
-    if (prec == TPMG_DW && level - 1 < op->lsw_dw) prec = TPMG_F64;
     if (level <= 1) return set_err(TPMG_ERR_ARG, "prolongate needs a fine level > 1");
+    const bool low = prec == TPMG_DW && level - 1 < op->lsw_dw;
+    if (low) prec = TPMG_F64;
     if (!u_c || !u_f) return set_err(TPMG_ERR_ARG, "NULL field");
-    TRY(prep_unit(op, prec));
+    TRY(prep_unit(op, prec, low));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nc = lvl_cells(op, level - 1), nf = lvl_cells(op, level);
     DISPATCH_PREC(prec, {
