@@ -79,7 +79,7 @@ struct tpmg_op {
     float2* vdw[MAXL + 1] = {};
     Hier hier[3];  // by policy id (F64, F32, DW)
     void* finv[3][MAXL + 1] = {};  // Thomas factors 1/m_k per policy and level
-    void* pcr[3][MAXL + 1] = {};   // PCR factors of the small levels per policy and level (not FP64)
+    void* pcr[3][MAXL + 1] = {};   // PCR factors of the small levels per policy and level
     double* chunkw[MAXL + 1] = {}; // native FP64, small levels: factor products per chunk of planes
     void* gstack = nullptr;        // Thomas-stack scratch of the persistent sweep variants
     void* fw[3][MAXL + 1] = {};    // Thomas factors v/m_k
@@ -284,16 +284,24 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid, int top = 0) {
             CK(cudaMemcpy(&k0, dk, sizeof(int), cudaMemcpyDeviceToHost));
             op->fac_k0[pid][l] = k0;
         }
-        // small levels: factor products of the chunked columns (native FP64), parallel-cyclic-reduction
-        // factors of the cell-parallel kernels (the other policies)
+        // small levels: factor products of the columns in chunks (native FP64), parallel-cyclic-reduction factors
+        // of the cell-parallel kernels
         const size_t cols = (size_t)op->g.lnx[l] * op->g.lny[l];
-        if (pid == 0 && chunk_level(op->g.lnx[l], op->g.lny[l])) {
+        const int f64 = f64_columns(op->g.lnx[l], op->g.lny[l], op->g.nz);
+        if (pid == 0 && f64 == F64_CHUNK) {
             const Lv<PolF64> L = level_view<PolF64>(op, l);
             TRY(dalloc((void**)&op->chunkw[l], chunk_count(L) * eb));
             launch_chunk_products(L, op->chunkw[l], 0);
         }
-        if (pid != 0 && cols <= (size_t)PCR_MAX_COLS && op->g.nz <= 256) {
+        const bool low = pid == 2 && l < op->lsw_dw;  // these run in native FP64
+        if (pid == 0 ? f64 == F64_PCR : !low && cols <= (size_t)PCR_MAX_COLS && op->g.nz <= 256) {
             switch (pid) {
+                case 0: {
+                    Lv<PolF64> L = level_view<PolF64>(op, l);
+                    TRY(dalloc(&op->pcr[0][l], pcr_factor_count(L, op->percol[l]) * eb));
+                    launch_pcr_factors<PolF64>(L, (double*)op->pcr[0][l], op->percol[l], 0);
+                    break;
+                }
                 case 1: {
                     Lv<PolF32> L = level_view<PolF32>(op, l);
                     TRY(dalloc(&op->pcr[1][l], pcr_factor_count(L, op->percol[l]) * eb));

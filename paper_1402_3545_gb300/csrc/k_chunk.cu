@@ -1,18 +1,20 @@
-// k_chunk.cu -- native FP64 kernels of the small levels (128 x 256 columns and below) and of grids that fit no
-// tile: columns cut into chunks of planes; and the pointwise Residual of every policy.
+// k_chunk.cu -- native FP64 kernels of small levels and of grids that fit no tile (f64_columns): columns cut into
+// chunks of planes; and the pointwise Residual of every policy.
 //
 // With a thread per column these levels leave most of the chip waiting on 2 nz dependent FP64 operations
 // (about 80 cycles each); cyclic reduction (k_coarse.cu, the other policies) shortens the chain to log2 nz
 // steps but takes 2 log2(nz) + 1 operations per cell for the solve alone on a pipe that issues 1/74 of the
-// FP32 rate. Here a block owns 8 columns (2 or 4 on the smallest levels), each cut into 16 chunks of PP planes with a thread per chunk, and
+// FP32 rate. Here a block owns 8 columns (2 or 4 on the smallest levels), each cut into up to 16 chunks of PP
+// planes with a thread per chunk (only those that nz planes have: idle ones would take the pipe all the same,
+// 450 x 330 x 4 200 us with all 16), and
 // both recurrences of the Thomas algorithm, y_k = b_k / m_k + w_k y_{k-1} and x_k = y_k + w_k x_{k+1}
 // (w_k = v / m_k), run twice per chunk: from zero, for the value the chunk hands on, and, once the carried
 // value is known (the earlier chunks' values chained by the chunks' products of w_k), for the chunk's own
 // values. One more operation per cell and direction (11 for a Smooth), 2 (2 PP + chunks) dependent ones.
 // The forward-error bound is that of the Thomas algorithm: the second pass is its recurrence, and the
 // carried value's own rounding enters damped by the products, all below 1.
-// Measured per Smooth inside a graph: 64^2 x 128 17 us (cyclic reduction 35), 128^2 x 128 65 us (thread per
-// column 95), 64^2 x 64 10 us (17), 8^2 x 128 9 us (6).
+// Measured per Smooth inside a graph: 64^2 x 128 16 us (cyclic reduction 30), 128^2 x 128 49 us (thread per
+// column 72), 64^2 x 64 10 us (17); 300 x 150 x 60 with the norm 119 us, 185 with a thread per column.
 #include "kernels.cuh"
 
 namespace tpmg {
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, co
             y = 0.0;
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
+                if (c > last) break;
                 const double e = sy[c][tx];
                 sy[c][tx] = y;
                 y = fma(pw[c], y, e);
@@ -186,7 +189,8 @@ __global__ void __launch_bounds__(CB * CH) k_chunk(Lv<PolF64> L, double coef, co
         if (w == 0) {
             x = 0.0;
 #pragma unroll
-            for (int c = CH - 1; c >= 0; --c) {  // (chunks beyond the column hand on zero)
+            for (int c = CH - 1; c >= 0; --c) {
+                if (c > last) continue;
                 const double e = sx[c][tx];
                 sx[c][tx] = x;
                 x = fma(pw[c], x, e);
@@ -266,7 +270,10 @@ template <class PF, int MODE, int PP, int CB>
 static int run_chunk_cb(const Lv<PolF64>& L, double coef, const typename PF::S* u, const double* f, double* out, double* fc,
                         double* partials, const int* done, cudaStream_t s) {
     const int nb = (L.nx * L.ny + CB - 1) / CB;
-    const dim3 b(CB, CH);
+    // the chunks that the column has, in whole warps (the scan of CB == 2 takes all of its warp)
+    constexpr int WR = 32 / CB;
+    const int rows = ((L.nz + PP - 1) / PP + WR - 1) / WR * WR;
+    const dim3 b(CB, CB == 2 ? CH : rows);
     if (MODE == 0 && partials)
         k_chunk<PF, MODE, PP, MODE == 0, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
     else

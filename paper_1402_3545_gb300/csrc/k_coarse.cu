@@ -2,8 +2,8 @@
 // PCR_MAX_COLS columns: 64 x 64 and below).
 //
 // The column kernels give each vertical column one thread, which leaves the GPU nearly idle on the
-// coarse levels (a 16 x 16 level has 256 columns). Here (FP32 and double-word; native FP64, whose pipe the
-// extra operations would fill, cuts its columns into chunks, k_chunk.cu) every
+// coarse levels (a 16 x 16 level has 256 columns). Here (FP32 and double-word; of native FP64, whose pipe the
+// extra operations fill, only the levels that f64_columns picks, the others in chunks, k_chunk.cu) every
 // cell has its own thread: the stencil and the transfers are pointwise, and the column block
 // M_c = tridiag(-v, D_k, -v) is solved by parallel cyclic reduction (PCR): with stride s = 1, 2, 4,
 // ... each row eliminates its neighbours at distance s,
@@ -515,6 +515,7 @@ TPMG_PROL_INST(PolF64)
 TPMG_PROL_INST(PolF32)
 TPMG_PROL_INST(PolDW)
 TPMG_PROL_INST(PolF32B)
+TPMG_PCR_INST(PolF64)
 TPMG_PCR_INST(PolF32)
 TPMG_PCR_INST(PolDW)
 TPMG_PCR_INST(PolF32B)
@@ -522,6 +523,8 @@ template int launch_restrict_smooth_pcr<PolF32, PolF32B>(const Lv<PolF32B>&, dou
                                                          const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
 template int launch_prolongate_x4<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
+template int launch_restrict_smooth_pcr<PolDW, PolF64>(const Lv<PolF64>&, double, const float2*, double*, double*,
+                                                       const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
 template int launch_prolongate_x4<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
 template int launch_residual_cell<PolDW, PolF32>(const Lv<PolDW>&, const float2*, const float2*, float*, double*,

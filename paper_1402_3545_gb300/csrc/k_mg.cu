@@ -349,7 +349,7 @@ int max_partials(int nx, int ny) {
     const int col_kernels = ((nx + TX - 1) / TX) * ny;
     // small levels: at most one block per column; chunked columns (native FP64): one per 8 columns. A level
     // below the finest has a quarter of its columns or fewer, so that the finest level's count covers it.
-    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (chunk_level(nx, ny) ? (nx * ny + 127) / 128 * 16 : 0);
+    const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (nx * ny <= CHUNK_MAX_COLS || nx % 32 != 0 ? (nx * ny + 127) / 128 * 16 : 0);
     return col_kernels > cell_kernels ? col_kernels : cell_kernels;
 }
 
@@ -368,11 +368,9 @@ void launch_apply_A(const Lv<P>& L, const typename P::S* x, typename P::S* y, cu
 template <class P>
 void launch_line_solve(const Lv<P>& L, const typename P::S* b, typename P::S* x, double scale, const int* done,
                        cudaStream_t s) {
-    if constexpr (P::id == 0) {
+    if constexpr (P::id == 0)
         if (launch_line_solve_chunk(L, b, x, scale, done, s) >= 0) return;
-    } else {
-        if (launch_line_solve_pcr<P>(L, b, x, scale, done, s) >= 0) return;
-    }
+    if (launch_line_solve_pcr<P>(L, b, x, scale, done, s) >= 0) return;
     if (launch_line_solve_pp<P>(L, b, x, scale, done, s) >= 0) return;
     Shape sh = sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), true);
     allow_smem(k_line_solve<P>, sh.smem);
@@ -382,9 +380,9 @@ void launch_line_solve(const Lv<P>& L, const typename P::S* b, typename P::S* x,
 template <class P>
 int launch_smooth(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                    typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
-    int nparts;
+    int nparts = -1;
     if constexpr (P::id == 0) nparts = launch_smooth_chunk(L, rho, u, f, uo, partials, done, s);
-    else nparts = launch_smooth_pcr<P>(L, rho, u, f, uo, partials, done, s);
+    if (nparts < 0) nparts = launch_smooth_pcr<P>(L, rho, u, f, uo, partials, done, s);
     if (nparts >= 0) return nparts;
     nparts = launch_smooth_pp<P>(L, rho, u, f, uo, partials, done, s);
     if (nparts >= 0) return nparts;
@@ -431,11 +429,9 @@ int launch_residual(const Lv<P>& L, const typename P::S* u, const typename P::S*
 template <class PF, class P>
 void launch_restrict_smooth(const Lv<P>& Lc, double rho, const typename PF::S* rf,
                             typename P::S* fc, typename P::S* uc, const int* done, cudaStream_t s) {
-    if constexpr (P::id == 0) {
+    if constexpr (P::id == 0)
         if (launch_restrict_smooth_chunk<PF>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
-    } else {
-        if (launch_restrict_smooth_pcr<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
-    }
+    if (launch_restrict_smooth_pcr<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0) return;
     // the pipelined kernel copies pairs of fine values: their address must be pair-aligned
     if (((uintptr_t)rf % (2 * sizeof(typename PF::S))) == 0 &&
         launch_restrict_smooth_pp<PF, P>(Lc, rho, rf, fc, uc, done, s) >= 0)

@@ -534,7 +534,8 @@ template <int MODE, int PP, int CB>
 static int run_panel_chunk_cb(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
                               double* partials, const int* done, cudaStream_t s) {
     const int nb = (L.nx * L.ny + CB - 1) / CB;
-    const dim3 b(CB, CH);
+    constexpr int WR = 32 / CB;  // the chunks that the column has, in whole warps
+    const dim3 b(CB, ((L.nz + PP - 1) / PP + WR - 1) / WR * WR);
     if (MODE == 0 && partials) k_panel_chunk<MODE, PP, MODE == 0, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, partials, done);
     else k_panel_chunk<MODE, PP, false, CB><<<nb, b, 0, s>>>(L, coef, u, f, out, fc, nullptr, done);
     note_launch();

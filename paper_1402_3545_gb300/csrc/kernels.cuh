@@ -103,7 +103,7 @@ struct Lv {
     // 1/b of the decoupled rows; per cell when fac_percol, else one shared table of nz rows
     const typename P::S* pcr = nullptr;
     int pcr_steps = 0;
-    // native FP64 levels of at most CHUNK_MAX_COLS columns: products of w_k = v/m_k over chunks of planes
+    // native FP64 levels in chunks (f64_columns): products of w_k = v/m_k over chunks of planes
     // (k_chunk.cu), else null
     const typename P::S* chunkw = nullptr;
     // global scratch for the Thomas stacks of the persistent sweep variants (gstack_bytes(nz)
@@ -144,10 +144,32 @@ size_t gstack_bytes(int nz);
 // solve by parallel cyclic reduction; native FP64: chunks of planes, k_chunk.cu): a thread per column
 // leaves the GPU idle there.
 static constexpr int PCR_MAX_COLS = 4096;
-// Native FP64 levels of at most this many columns cut their columns into chunks of planes (k_chunk.cu), and so
-// do larger ones whose nx has no 32-column tiles; above it a thread per column fills the GPU (256^2 x 128: 154 us; 128^2 x 128: 95 us in a cycle against 65 in chunks)
+// Levels of at most this many columns have too few of them to fill the GPU with a thread each: pointwise kernels
+// and, in native FP64, columns in chunks of planes below (f64_columns, and the panel's)
 static constexpr int CHUNK_MAX_COLS = 32768;
-inline bool chunk_level(int nx, int ny) { return (size_t)nx * ny <= (size_t)CHUNK_MAX_COLS || nx % 32 != 0; }
+// What a native FP64 level's columns run on, from all forms' times over 14 horizontal sizes and nz = 4 .. 256, with
+// and without the norm (Smooth without it, us; chunks / the other form):
+//  - cyclic reduction (k_coarse.cu) on small levels of few planes, where the chunks' three barriers outweigh its
+//    operations: 32^2 x 8 5.5 / 3.6, x 32 6.0 / 5.4, x 48 6.4 / 6.8; 64^2 x 8 5.7 / 4.0, x 12 5.9 / 5.9, x 20 6.5 / 7.3;
+//    up to 512 columns a warp scans the chunks: 16^2 x 8 4.5 / 3.6, x 12 4.3 / 4.8; and on the smallest of many
+//    planes, where a level is one wave of either: 8^2 x 160 9.6 / 6.7, 16^2 x 128 6.7 / 6.0;
+//  - the sweep (a thread per column) where the columns alone fill the GPU. With tiles: 96^2 x 8 7.4 / 6.3, x 16
+//    7.3 / 10.4; 128^2 x 24 15.8 / 15.3, x 32 16.0 / 19.7; 192 x 160 x 64 49 / 47. Without (nx % 32 != 0, a slower
+//    sweep): 150^2 x 4 12 / 8; 182 x 178 x 20 29 / 37 but 47 / 41 with the norm, x 32 30 / 48; 450 x 330 x 20
+//    121 / 125, x 32 125 / 207, x 64 229 / 552;
+//  - chunks of planes (k_chunk.cu) else.
+enum { F64_SWEEP = 0, F64_CHUNK = 1, F64_PCR = 2 };
+inline int f64_columns(int nx, int ny, int nz) {
+    const size_t cols = (size_t)nx * ny;
+    if (nz > 256) return F64_SWEEP;
+    if (cols <= (size_t)PCR_MAX_COLS) {
+        const int few = cols <= 512 ? 8 : (cols <= 2048 ? 32 : 12);
+        return nz <= few || (cols <= 256 && nz > 64) ? F64_PCR : F64_CHUNK;
+    }
+    const bool small = cols <= (size_t)CHUNK_MAX_COLS / 2;
+    if (nx % 32 == 0) return small && (nz > 24 || (nz > 8 && cols <= 10240)) ? F64_CHUNK : F64_SWEEP;
+    return nz > 24 || (small && nz > 4) ? F64_CHUNK : F64_SWEEP;
+}
 inline int pcr_steps_for(int nz) {
     int s = 0;
     while ((1 << s) < nz) ++s;
