@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) k_cg_spmv(Lv<P> L, const Scalars* __restr
 
 // The fused SpMV with two x-adjacent columns per thread and SPMV_PZ planes per block: the vertical neighbours
 // stay in registers, the x neighbours come from the adjacent lanes, and a plane's six 16-byte loads (DW; 8 bytes
-// in FP32) are in flight together. Bound by DRAM (seven fields); 512^2 x 128 double-word 378 us, 390 with
+// in FP32) are in flight together. Bound by DRAM (seven fields); 512^2 x 128 double-word 372 us, 390 with
 // a thread per pair of cells, whose 64-bit divisions for the cell's indices and five stencil loads it does
 // without. Requires nx even; ALIGNED: pair-aligned fields.
 constexpr int SPMV_PZ = 16, SPMV_TY = 8;
@@ -142,9 +142,10 @@ __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<
         const int ii = act ? i : nx - 2;  // lanes beyond the row repeat its last pair and store nothing
         const size_t row = (size_t)j * nx, c = row + ii, b0 = (size_t)k0 * pl;
         const size_t rs = (size_t)wrapc(j - 1, ny) * nx + ii, rn = (size_t)wrapc(j + 1, ny) * nx + ii;
-        // the pair's x neighbours beyond the warp or the row are loaded
+        // the columns beyond the warp's ends or the row's: every lane loads both (one sector each)
         const bool lw = lane == 0, le = lane == 31 || i + 2 >= nx;
-        const size_t cw = row + wrapc(ii - 1, nx), ce = row + wrapc(ii + 2, nx);
+        const int iw = i - 2 * lane;
+        const size_t cw = row + wrapc(iw - 1, nx), ce = row + (iw + 64 < nx ? iw + 64 : 0);
         const R v0 = P::ld(L.v, c), v1 = P::ld(L.v, c + 1);
         const R d1a = P::add(K.dh, v0), d1b = P::add(K.dh, v1), d2a = P::add(d1a, v0), d2b = P::add(d1b, v1);
         const bool iso = K.iso != 0;
@@ -162,9 +163,10 @@ __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<
             po.ld(p + id);
             qo.ld(q + id);
             uo.ld(u + id);
+            const R zl = P::ld(z, b + cw), zr = P::ld(z, b + ce);
             R zw = lane_up(zc.b), ze = lane_dn(zc.a);
-            if (lw) zw = P::ld(z, b + cw);
-            if (le) ze = P::ld(z, b + ce);
+            if (lw) zw = zl;
+            if (le) ze = zr;
             if (k + 1 == nz) zp.zero();
             const bool end = k == 0 || k == nz - 1;
             const R da = nz == 1 ? K.dh : (end ? d1a : d2a), db = nz == 1 ? K.dh : (end ? d1b : d2b);
