@@ -313,13 +313,37 @@ __global__ void __launch_bounds__(256) k_prolongate(int nxc, int nyc, int nz,
 }
 
 // ---------------------------------------------------------------- u += e (FP32 correction)
-template <class P>
+// Bound by memory. VEC: four values a thread, their loads before the stores (16-byte aligned fields): a thread that
+// adds one value at a time has only its own 12 bytes in flight. 1024^2 x 128 double-word 403 us, 444 before.
+template <class P, bool VEC>
 __global__ void k_correct(size_t n, typename P::S* __restrict__ u, const float* __restrict__ e,
                           const int* done) {
+    typedef typename P::S S;
     if (done && *(volatile const int*)done) return;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
-         t += (size_t)gridDim.x * blockDim.x)
-        P::st(u, t, P::add(P::ld_plain(u, t), P::from_f(__ldg(e + t))));
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    size_t n4 = 0;
+    if (VEC) {
+        constexpr int V = sizeof(S) / 4;  // 16-byte pieces of four values
+        union Four {
+            float4 q[V];
+            S v[4];
+            __device__ Four() {}
+        };
+        n4 = n / 4;
+        for (size_t t = t0; t < n4; t += nt) {
+            float4* pu = reinterpret_cast<float4*>(u) + V * t;
+            Four a;
+#pragma unroll
+            for (int q = 0; q < V; ++q) a.q[q] = pu[q];
+            const float4 ev = __ldg(reinterpret_cast<const float4*>(e) + t);
+            const float x[4] = {ev.x, ev.y, ev.z, ev.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) P::st(a.v, q, P::add(P::ld_plain(a.v, q), P::from_f(x[q])));
+#pragma unroll
+            for (int q = 0; q < V; ++q) pu[q] = a.q[q];
+        }
+    }
+    for (size_t t = 4 * n4 + t0; t < n; t += nt) P::st(u, t, P::add(P::ld_plain(u, t), P::from_f(__ldg(e + t))));
 }
 
 // ---------------------------------------------------------------- launch shapes
@@ -452,9 +476,11 @@ void launch_prolongate(int nxc, int nyc, int nz, const typename P::S* uc, typena
 }
 template <class P>
 void launch_correct(size_t n, typename P::S* u, const float* e, const int* done, cudaStream_t s) {
-    size_t blocks = (n + 255) / 256;
+    const bool vec = (((uintptr_t)u | (uintptr_t)e) & 15) == 0;
+    size_t blocks = ((vec ? (n + 3) / 4 : n) + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    k_correct<P><<<(unsigned)blocks, 256, 0, s>>>(n, u, e, done);
+    if (vec) k_correct<P, true><<<(unsigned)blocks, 256, 0, s>>>(n, u, e, done);
+    else k_correct<P, false><<<(unsigned)blocks, 256, 0, s>>>(n, u, e, done);
     note_launch();
 }
 
