@@ -100,10 +100,13 @@ def test_restrict_tile_equals_the_two_kernels(prec, shape, square, lam):
     op.close()
 
 
-# chunk sizes change above 64 and 128 planes and end at 256; 8, 4 or 2 columns a block by the level's size; 182^2 is
-# a level of more than 32768 columns whose nx has no 32-column tiles
+# chunk sizes change above 64 and 128 planes and end at 256; 8, 4 or 2 columns a block by the level's size; whole and
+# part-filled rows of chunks. The rule's edges: cyclic reduction up to 8, 32 or 12 planes and on 256 columns above 64;
+# 10240 and 16384 columns with tiles, 4 and 24 planes without
 @pytest.mark.parametrize("shape", [(2, 2, 64), (6, 4, 65), (34, 10, 128), (66, 62, 129), (34, 10, 256), (66, 62, 1),
-                                   (182, 182, 5)], ids=lambda s: "x".join(map(str, s)))
+                                   (182, 182, 5), (130, 130, 24), (130, 130, 25), (16, 16, 9), (16, 16, 65), (32, 32, 32),
+                                   (32, 32, 33), (64, 64, 12), (64, 64, 13), (128, 80, 9), (128, 128, 24), (128, 128, 25)],
+                         ids=lambda s: "x".join(map(str, s)))
 def test_chunked_columns_match_oracle(shape):
     nx, ny, nz = shape
     p = make_problem(nx, ny, nz)
