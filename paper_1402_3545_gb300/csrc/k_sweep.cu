@@ -576,9 +576,12 @@ template <class P>
 int launch_smooth_pp(const Lv<P>& L, double rho, const typename P::S* u, const typename P::S* f,
                      typename P::S* uo, double* partials, const int* done, cudaStream_t s) {
     if (L.nz * 32 * 8 > 160 * 1024) return -1;  // stack too deep for shared memory
-    // without a norm to give, the FP64-accurate policies take the form that needs no residual (12 -> 9
-    // arithmetic operations per cell); FP32 keeps one form, so that its results do not depend on the norm
-    if constexpr (P::id != 1)
+    // without a norm to give, native FP64 takes the form that needs no residual (9 instead of 12 FP64 instructions
+    // per cell). Double-word and FP32 keep the correction form: there the line solve's rounding is relative to the
+    // correction, in the other to u itself, and the pairs' line solve rounds more than their storage does (attainable
+    // residual of a double-word solve, 128^3, lambda^2 varying: 2.5e-12 of the first, 1.3e-11 in the other form).
+    // FP64's line solve does not: 8.6e-14 and 9.2e-14.
+    if constexpr (P::id == 0)
         if (!partials) return smooth_dispatch<P, MODE_SMOOTHB>(L, rho, u, f, uo, partials, done, s);
     return smooth_dispatch<P, MODE_SMOOTH>(L, rho, u, f, uo, partials, done, s);
 }

@@ -5,8 +5,6 @@ namespace tpmg {
 
 template int launch_sweep_tile<PolDW, MODE_SMOOTH>(const Lv<PolDW>&, double, const PolDW::S*, const PolDW::S*, PolDW::S*, double*,
     const int*, cudaStream_t);
-template int launch_sweep_tile<PolDW, MODE_SMOOTHB>(const Lv<PolDW>&, double, const PolDW::S*, const PolDW::S*, PolDW::S*, double*,
-    const int*, cudaStream_t);
 template int launch_sweep_tile<PolDW, MODE_LINESOLVE>(const Lv<PolDW>&, double, const PolDW::S*, const PolDW::S*, PolDW::S*, double*,
     const int*, cudaStream_t);
 template int cg_tile_blocks<PolDW>(const Lv<PolDW>&);

@@ -4,7 +4,7 @@
 //
 // A block owns 512 bytes of columns over all nz planes, in one, two or four rows: nz * 512 bytes of shared
 // memory. Its eight warps take contiguous ranges of planes:
-//   1. form the right-hand side of the line solves (f - A u, or sweep_rhs' f + H u) of their planes:
+//   1. form the right-hand side of the line solves (Smooth: f - A u) of their planes:
 //      f arrives by cp.async for all planes at once, u by batches of planes whose loads are issued together;
 //      x neighbours and the tile's inner rows come from the other lanes by shuffles;
 //   2. one thread per column (FP32: per four) eliminates forward through shared memory (the only serial part, a
@@ -134,7 +134,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
     // 12 problems against 28.7)
     constexpr bool AHEAD = RO;
     constexpr bool CG = MODE == MODE_CGTRI;
-    constexpr bool SM = MODE != MODE_LINESOLVE && !CG;  // a stencil, and u in the result
+    constexpr bool SM = MODE == MODE_SMOOTH;  // a stencil, and u in the result
     constexpr bool GFORM = MODE == MODE_SMOOTH && P::id == 1;
     constexpr bool DIRECT = GFORM || MODE == MODE_LINESOLVE || CG;  // the back substitution yields the result
     constexpr int G = 32 / TR;                                // lanes of a tile row
@@ -186,13 +186,10 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
             const R cx = K.cx, cy = K.cy, dh = K.dh;
             V um, uc, vv, dg;
             um.zero();
-            vv.zero();
             dg.zero();
             uc.template ldf<RO>(pu);
-            if (MODE == MODE_SMOOTH) {
-                if (klo > 0) um.template ldf<RO>(pu - pl);
-                vv.ldg(L.v + c);
-            }
+            if (klo > 0) um.template ldf<RO>(pu - pl);
+            vv.ldg(L.v + c);
             bool first = true;
             // one batch of B planes from plane k: all their loads, then their arithmetic
             auto batch = [&](auto bc, int k) {
@@ -202,8 +199,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
                 const bool top = k + B == nz;  // the last plane has no upper neighbour
 #pragma unroll
                 for (int t = 0; t < B; ++t) {  // u of plane k+t+1, the halo of plane k+t
-                    if (MODE == MODE_SMOOTH || t + 1 < B || !top) ru[t].template ldf<RO>(t + 1 == B && top ? pu : pu + pl);
-                    else ru[t].zero();
+                    ru[t].template ldf<RO>(t + 1 == B && top ? pu : pu + pl);
                     if (!hrow) rh[t].zero();
                     if (hrow) rh[t].template ldf<RO>(ph);
                     if (TR == 1) rh1[t].template ldf<RO>(ph1);
@@ -215,10 +211,8 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
                 }
                 if (first) {  // (the first batch's loads are on their way too)
                     cp_wait<0>();  // this thread's pieces of f
-                    if (MODE == MODE_SMOOTH) {
 #pragma unroll
-                        for (int q = 0; q < N; ++q) dg.v[q] = P::add(P::add(dh, vv.v[q]), vv.v[q]);
-                    }
+                    for (int q = 0; q < N; ++q) dg.v[q] = P::add(P::add(dh, vv.v[q]), vv.v[q]);
                     first = false;
                 }
                 if (top) ru[B - 1].zero();
@@ -230,7 +224,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
                     if (lx == 0) wl = re[t];
                     if (lx == G - 1) el = re[t];
                     V d = dg;
-                    if (MODE == MODE_SMOOTH && (k + t == 0 || k + t == nz - 1)) {
+                    if (k + t == 0 || k + t == nz - 1) {
 #pragma unroll
                         for (int q = 0; q < N; ++q) d.v[q] = nz == 1 ? dh : P::add(dh, vv.v[q]);
                     }
@@ -249,11 +243,8 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
                         }
                         const R w = q == 0 ? wl : uc.v[q > 0 ? q - 1 : 0];
                         const R e = q == N - 1 ? el : uc.v[q < N - 1 ? q + 1 : q];
-                        if constexpr (MODE == MODE_SMOOTHB)
-                            r.v[q] = sweep_rhs<P>(r.v[q], w, e, s, n, cx, cy, ISO);
-                        else
-                            r.v[q] = sweep_residual<P>(r.v[q], d.v[q], uc.v[q], w, e, s, n, um.v[q], ru[t].v[q], cx, cy,
-                                                       vv.v[q], ISO);
+                        r.v[q] = sweep_residual<P>(r.v[q], d.v[q], uc.v[q], w, e, s, n, um.v[q], ru[t].v[q], cx, cy,
+                                                   vv.v[q], ISO);
                         if (NORM) P::acc_dot(acc, cmp, r.v[q], r.v[q]);
                     }
                     r.sts(z);
@@ -551,8 +542,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
                 V x;
                 x.lds(z);
 #pragma unroll
-                for (int q = 0; q < N; ++q)
-                    x.v[q] = P::fma(cf, x.v[q], MODE == MODE_SMOOTHB ? P::mul_u(K.rest, ua[t].v[q]) : ua[t].v[q]);
+                for (int q = 0; q < N; ++q) x.v[q] = P::fma(cf, x.v[q], ua[t].v[q]);
                 x.stg(po);
             }
         }
