@@ -6,11 +6,13 @@
 // operands and FP32 accumulators (M = 16 is all a layer has, far below the 128 rows of a tcgen05 tile).
 // The steps (tile of 64 x 8 columns, plane) of the whole grid are numbered tile by tile and dealt to
 // the blocks in equal contiguous ranges: each block marches in z through rings of planes fetched two
-// planes ahead, keeps all its sums in registers, and writes one partial per weight and bias at its
-// end (at most 2 blocks per SM, so the final reduction reads a few MB). On the training crop
-// (256^2 x 64, cin = 2) the backward pass's weight and bias gradients took 4.1 ms with one-plane tiles
-// loaded synchronously, per-weight FP32 loops for the thin layers, separate bias sums and serial
-// reductions over 1024 partials; 0.66 ms now.
+// planes ahead, and writes one partial per weight and bias at its end (at most 2 blocks per SM, so the
+// final reduction reads a few MB).
+// Rounding: the tensor cores cut an accumulator's low bits off instead of rounding them, an error that does not
+// average out: same-signed sums lose about half a unit in the last place per MMA (2.6e-5 of the sum in 430 of
+// them). So no accumulator lives long: the thin layers add each MMA's 16 cells to FP32 sums by ordinary
+// additions, the 16 -> 16 layers pass theirs on every D16_FLUSH planes, and biases are ordinary additions, FP32 over 32
+// planes and FP64 from there.
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
@@ -22,7 +24,6 @@ namespace {
 
 constexpr int GX = 64, GY = 8;         // cells of a tile plane in x and y
 constexpr int ROWB = 32;               // bytes of a cell's 16 channels
-constexpr unsigned BF16_ONES = 0x3f803f80u;
 
 __device__ __forceinline__ int gwrap(int a, int n) {
     a %= n;
@@ -56,6 +57,12 @@ __device__ __forceinline__ void gmma(float (&c)[4], const uint32_t (&a)[4], uint
 // the 8 rows of an ldmatrix phase fall on distinct banks
 __device__ __forceinline__ int gswz(int r, int h) { return r * ROWB + ((h ^ ((r >> 2) & 1)) << 4); }
 
+// sum of the four cells that a lane's registers of one row of an A fragment hold
+__device__ __forceinline__ float gsum(uint32_t lo, uint32_t hi) {
+    return (__uint_as_float(lo << 16) + __uint_as_float(lo & 0xffff0000u)) +
+           (__uint_as_float(hi << 16) + __uint_as_float(hi & 0xffff0000u));
+}
+
 // the block's contiguous share [s0, s1) of the steps
 __device__ __forceinline__ void share(long nsteps, long& s0, long& s1) {
     s0 = nsteps * blockIdx.x / gridDim.x;
@@ -68,14 +75,16 @@ __device__ __forceinline__ void share(long nsteps, long& s0, long& s1) {
 // Twelve warps: warp w owns the x-shift dx = w / 4 (its nine (dz, dy) taps: 72 accumulators) on the
 // 16-cell column w % 4 of the tile. The x rows (B, shifted by dx) are each read once; the dy rows (A)
 // they meet, planes k-1 .. k+1 and rows y-1 .. y+1, stay in a rolling 3 x 3 window of fragments that
-// takes three new ones per row: 4 ldmatrix for 18 MMAs, against one per tap. The bias gradient is one
-// more MMA with a B of ones (dx = 1 warps). Rings: 5 planes of dy (10 rows), 3 of x (66 cells a row).
-// Measured on 256^2 x 64 (4.2 M cells, 58 GFLOP): 160 us, bound by mma.sync issue; 758 us before (one
-// plane per tile, three planes of halo loaded synchronously for it, an ldmatrix per tap) plus 291 us
-// for the bias sums.
+// takes three new ones per row: 4 ldmatrix for 18 MMAs, against one per tap. The bias gradient adds up
+// the dx = 1 warps' dy fragments. Rings: 5 planes of dy (10 rows), 3 of x (66 cells a row). Every D16_FLUSH
+// planes (256 MMAs to an accumulator) and at the end the four 16-cell columns add their sums, in order, to the
+// block's in shared memory, [x-shift, dz, dy, half of ci][lane][4], 16 bytes a lane.
+// Measured on 256^2 x 64 (4.2 M cells, 58 GFLOP): 165 us.
 constexpr int D16_NT = 384, D16_DYP = (GY + 2) * GX * ROWB, D16_XP = GY * (GX + 2) * ROWB;
-constexpr int D16_SMEM = 5 * D16_DYP + 3 * D16_XP;
+constexpr int D16_RING = 5 * D16_DYP + 3 * D16_XP;
 constexpr int D16_OUT = 27 * 256 + 16;  // weights, then biases
+constexpr int D16_SMEM = D16_RING + 27 * 256 * (int)sizeof(float);
+constexpr int D16_FLUSH = 32;
 
 __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __restrict__ x,
                                                        const __nv_bfloat16* __restrict__ dy,
@@ -83,11 +92,13 @@ __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __re
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* const DY = smem;
     unsigned char* const X = smem + 5 * D16_DYP;
+    float* const red = reinterpret_cast<float*>(smem + D16_RING);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int dx = warp >> 2, xc = (warp & 3) * 16;
     const int q8 = lane >> 3, rr = lane & 7;
     float acc[3][3][2][4];
-    float accb[4] = {0.f, 0.f, 0.f, 0.f};
+    __shared__ double redb[16];
+    float b0 = 0.f, b1 = 0.f;  // biases of output channels lane / 4 and 8 + lane / 4
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -96,6 +107,43 @@ __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __re
             for (int c = 0; c < 2; ++c)
 #pragma unroll
                 for (int d = 0; d < 4; ++d) acc[a][b][c][d] = 0.f;
+    for (int q = tid; q < 27 * 256; q += D16_NT) red[q] = 0.f;
+    if (tid < 16) redb[tid] = 0.0;
+    // this thread's sums to the block's
+    auto flush = [&]() {
+        for (int c = 0; c < 4; ++c) {
+            __syncthreads();
+            if ((warp & 3) != c) continue;
+#pragma unroll
+            for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+                for (int t = 0; t < 3; ++t)
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt) {
+                        float4* r = reinterpret_cast<float4*>(red) + (((dx * 3 + dz) * 3 + t) * 2 + nt) * 32 + lane;
+                        float* a = acc[dz][t][nt];
+                        float4 v = *r;
+                        v.x += a[0];
+                        v.y += a[1];
+                        v.z += a[2];
+                        v.w += a[3];
+                        *r = v;
+                        a[0] = a[1] = a[2] = a[3] = 0.f;
+                    }
+            if (dx == 1) {
+                for (int h = 1; h < 4; h <<= 1) {
+                    b0 += __shfl_xor_sync(0xffffffffu, b0, h);
+                    b1 += __shfl_xor_sync(0xffffffffu, b1, h);
+                }
+                if ((lane & 3) == 0) {  // (the block's in FP64)
+                    redb[lane >> 2] += b0;
+                    redb[8 + (lane >> 2)] += b1;
+                }
+                b0 = b1 = 0.f;
+            }
+        }
+    };
+    int since = 0;
     const int tiles_x = nx / GX, tiles_y = (ny + GY - 1) / GY;
     long s0, s1;
     share((long)tiles_x * tiles_y * nz, s0, s1);
@@ -152,6 +200,7 @@ __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __re
             const int acell = xc + (q8 >> 1) * 8 + rr, ah = q8 & 1;   // A = dy^T: stored [cell][co]
             const int bcell = xc + dx + (q8 & 1) * 8 + rr, bh = q8 >> 1;  // B = x: stored [cell][ci]
             uint32_t A[3][3][4];  // [dz][halo row mod 3]
+            float p0 = 0.f, p1 = 0.f;  // the plane's bias sums
 #pragma unroll
             for (int dz = 0; dz < 3; ++dz)
 #pragma unroll
@@ -170,50 +219,43 @@ __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __re
                             gmma(acc[dz][t][0], A[dz][(y + 2 - t) % 3], B[0], B[1]);
                             gmma(acc[dz][t][1], A[dz][(y + 2 - t) % 3], B[2], B[3]);
                         }
-                    if (dx == 1) gmma(accb, A[1][(y + 1) % 3], BF16_ONES, BF16_ONES);
+                    if (dx == 1) {
+                        const uint32_t(&a)[4] = A[1][(y + 1) % 3];
+                        p0 += gsum(a[0], a[2]);
+                        p1 += gsum(a[1], a[3]);
+                    }
                 }
+            }
+            b0 += p0;
+            b1 += p1;
+            if (++since == D16_FLUSH) {
+                flush();
+                since = 0;
             }
         }
         gwait<0>();
     }
-    // the four 16-cell columns of each x-shift add up in shared memory, in order
-    float* red = reinterpret_cast<float*>(smem);
-    const int g = lane >> 2, t2 = (lane & 3) * 2;
-    for (int c = 0; c < 4; ++c) {
-        __syncthreads();
-        if ((warp & 3) != c) continue;
-#pragma unroll
-        for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-            for (int t = 0; t < 3; ++t)
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int co = g + 8 * (e >> 1), ci = 8 * nt + t2 + (e & 1), tap = (dz * 3 + t) * 3 + dx;
-                        float* r = red + (co * 16 + ci) * 27 + tap;
-                        *r = c == 0 ? acc[dz][t][nt][e] : *r + acc[dz][t][nt][e];
-                    }
-        if (dx == 1 && t2 == 0) {
-            float* r = red + 27 * 256 + g;
-            r[0] = c == 0 ? accb[0] : r[0] + accb[0];
-            r[8] = c == 0 ? accb[2] : r[8] + accb[2];
-        }
-    }
+    flush();
     __syncthreads();
-    for (int q = tid; q < D16_OUT; q += D16_NT) partials[(size_t)blockIdx.x * D16_OUT + q] = red[q];
+    float* const out = partials + (size_t)blockIdx.x * D16_OUT;
+    for (int q = tid; q < 27 * 256; q += D16_NT) {  // weight (co, ci, tap): where the fragments keep it
+        const int co = q / 432, ci = q / 27 % 16, tap = q % 27;
+        const int part = ((tap % 3 * 3 + tap / 9) * 3 + tap / 3 % 3) * 2 + ci / 8;
+        out[q] = red[(part * 32 + co % 8 * 4 + ci % 8 / 2) * 4 + co / 8 * 2 + ci % 2];
+    }
+    if (tid < 16) out[27 * 256 + tid] = (float)redb[tid];
 }
 
 // ---------------------------------------------------------------- first and last layer
 // The thin layers as the same GEMM. First layer: M = co, A = d1 (16 channels), N = (tap, ci) of the
 // input, read at p + d. Last layer (LAST): M = ci, A = a3, N = the 27 taps of d4, read at p - d; d4
 // is FP32 and enters as the exact sum of three BF16 parts (8 + 8 + 8 significant bits), one MMA
-// each, so nothing of it is rounded. Eight warps, one row of the tile each; A by ldmatrix from a
+// each, the smallest first, so nothing of it is rounded. Eight warps, one row of the tile each; A by ldmatrix from a
 // 3-plane ring; the thin operand from a 4-plane ring of channel-separated rows, kept twice, once
 // shifted by a cell, so that a lane's pair of cells is one aligned word for every x-shift. Bias
-// gradients: a B of ones (first layer), or the sum of d4 as it is loaded (last layer).
-// Measured on 256^2 x 64: 62 us (first, cin = 2) and 86 us (last); 564 and 336 us with FP32 loops per
-// weight.
+// gradients: the sum of the A fragments (first layer), or of d4 as it is loaded (last layer).
+// Measured on 256^2 x 64: 65 us (first, cin = 2) and 87 us (last).
+constexpr int THIN_FLUSH = 32;
 template <int CIN, bool LAST>
 struct ThinShape {
     static constexpr int NCH = LAST ? 3 : CIN;            // thin rows stored per plane row
@@ -237,7 +279,13 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
     __nv_bfloat16* const T = reinterpret_cast<__nv_bfloat16*>(smem + 3 * SH::AP);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q8 = lane >> 3, rr = lane & 7, g = lane >> 2, t = lane & 3;
-    float acc[SH::NTL][4], accb[4] = {0.f, 0.f, 0.f, 0.f}, bsum = 0.f;
+    __shared__ double redb[8][16];
+    float acc[SH::NTL][4];
+    // biases: of channels lane / 4 and 8 + lane / 4, or (LAST) of this thread's cells; FP32 sums of up to THIN_FLUSH
+    // planes
+    float f0 = 0.f, f1 = 0.f;
+    double b0 = 0.0, b1 = 0.0;
+    int since = 0;
     int off[SH::NTL], ddz[SH::NTL];  // word offset within a thin plane, plane offset 0..2, of the lane's columns
 #pragma unroll
     for (int j = 0; j < SH::NTL; ++j) {
@@ -299,7 +347,7 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
                 if (LAST) {
                     const float v = __uint_as_float(tv[q]);
                     const bool own = row >= 1 && row <= GY && y0 + row - 1 < ny && col >= 1 && col <= GX;
-                    if (own && z >= zb && z < ze) bsum += v;
+                    if (own && z >= zb && z < ze) f0 += v;
                     part[0] = __float2bfloat16_rn(v);
                     const float r1 = v - __bfloat162float(part[0]);
                     part[1 % SH::NCH] = __float2bfloat16_rn(r1);
@@ -333,6 +381,7 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
             if (z + 1 < ze) fetch(z + 2);
             if (y0 + warp < ny) {
                 const unsigned pa = gsa(AR + (z % 3) * SH::AP);
+                float p0 = 0.f, p1 = 0.f;  // the plane's bias sums
                 const uint32_t* base[SH::NTL];
 #pragma unroll
                 for (int j = 0; j < SH::NTL; ++j)
@@ -341,19 +390,50 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
                 for (int c = 0; c < GX / 16; ++c) {
                     uint32_t A[4];
                     gldm_t(pa + gswz(warp * GX + c * 16 + (q8 >> 1) * 8 + rr, q8 & 1), A);
+                    float d[SH::NTL][4];
 #pragma unroll
-                    for (int pc = 0; pc < (LAST ? 3 : 1); ++pc)
+                    for (int pc = LAST ? 2 : 0; pc >= 0; --pc) {
+                        if (pc != 1)  // (the two small parts share an accumulator)
+#pragma unroll
+                            for (int j = 0; j < SH::NTL; ++j) d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.f;
 #pragma unroll
                         for (int j = 0; j < SH::NTL; ++j) {
                             const uint32_t* b = base[j] + pc * SH::CP + c * 8;
-                            gmma(acc[j], A, b[0], b[4]);
+                            gmma(d[j], A, b[0], b[4]);
                         }
-                    if (!LAST) gmma(accb, A, BF16_ONES, BF16_ONES);
+                        if (pc != 2)
+#pragma unroll
+                            for (int j = 0; j < SH::NTL; ++j)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) acc[j][e] += d[j][e];
+                    }
+                    if (!LAST) {
+                        p0 += gsum(A[0], A[2]);
+                        p1 += gsum(A[1], A[3]);
+                    }
                 }
+                f0 += p0;
+                f1 += p1;
             }
             if (z + 1 < ze) store(z + 2);
+            if (++since == THIN_FLUSH) {
+                b0 += f0;
+                b1 += f1;
+                f0 = f1 = 0.f;
+                since = 0;
+            }
         }
         gwait<0>();
+    }
+    b0 += f0;
+    b1 += f1;
+    for (int h = 1; h < (LAST ? 32 : 4); h <<= 1) {
+        b0 += __shfl_xor_sync(0xffffffffu, b0, h);
+        if (!LAST) b1 += __shfl_xor_sync(0xffffffffu, b1, h);
+    }
+    if (t == 0) {
+        redb[warp][g] = b0;
+        redb[warp][8 + g] = b1;
     }
     // the warps' sums add up in shared memory, in order
     float* red = reinterpret_cast<float*>(smem);
@@ -370,15 +450,12 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
                     *r = w == 0 ? acc[j][e] : *r + acc[j][e];
                 }
             }
-        if (!LAST && t == 0) {
-            float* r = red + 16 * SH::N + g;
-            r[0] = w == 0 ? accb[0] : r[0] + accb[0];
-            r[8] = w == 0 ? accb[2] : r[8] + accb[2];
-        }
-        if (LAST) {
-            for (int h = 16; h > 0; h >>= 1) bsum += __shfl_xor_sync(0xffffffffu, bsum, h);
-            if (lane == 0) red[16 * SH::N] = w == 0 ? bsum : red[16 * SH::N] + bsum;
-        }
+    }
+    __syncthreads();
+    if (tid < SH::OUT - 16 * SH::N) {
+        double b = redb[0][tid];
+        for (int w = 1; w < 8; ++w) b += redb[w][tid];
+        red[16 * SH::N + tid] = (float)b;
     }
     __syncthreads();
     for (int q = tid; q < SH::OUT; q += 256) partials[(size_t)blockIdx.x * SH::OUT + q] = red[q];

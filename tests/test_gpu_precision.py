@@ -25,3 +25,52 @@ def test_double_word_attains_the_refinement_s_residual(shape, lam):
         level[prec] = np.median(res["history"][-10:])
     assert level[tpmg.DW] < 2.0 * level[tpmg.MIXED], level
     op.close()
+
+
+@pytest.mark.parametrize("cin,shape", [(2, (64, 256, 256)), (1, (64, 1024, 1024))], ids=["2^22", "2^26"])
+def test_gradient_sums_of_one_sign_match_64_bit_sums(cin, shape):
+    """A network whose layers pass channel 0 of x on (centre taps 1, the last layer's 1/16) and a target x - d: with
+    the values chosen here no activation and no data gradient rounds (BF16 x in [1, 2), d of 8 bits down to 2^-12, a
+    power of two of cells), so what remains are the gradients' own sums of 2^22 and 2^26 terms of one sign:
+    S_ci(tap) = sum_p d4(p) x_ci(p + tap) and sum_p d4(p), times 1/16 below the last layer.
+
+    Tolerances, of each element: the tensor cores cut off at most a unit in the last place (2^-23) per MMA. 16 -> 16
+    layers: 256 MMAs to an accumulator. First and last: one, and the result's own rounding, below 2^-22. Biases: the
+    result's rounding and those of many partial sums, which average out, below 2^-23."""
+    nz, ny, nx = shape
+    n = nx * ny * nz
+    W = [np.zeros((16, cin, 27)), np.zeros((16, 16, 27)), np.zeros((16, 16, 27)), np.zeros((1, 16, 27))]
+    W[0][:, 0, 13] = 1.0
+    for w in W[1:3]:
+        w[:, :, 13] = np.eye(16)
+    W[3][0, :, 13] = 1.0 / 16.0
+    net = tpmg.Network(cin, np.concatenate([np.concatenate([w.ravel(), np.zeros(w.shape[0])]) for w in W]).astype(np.float32))
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+
+    def mantissa():
+        return 1.0 + torch.randint(0, 128, shape, generator=g, device="cuda").float() / 128.0
+
+    x = torch.stack([mantissa() for _ in range(cin)], dim=-1)
+    d = torch.ldexp(mantissa(), -torch.randint(1, 13, shape, generator=g, device="cuda"))
+    loss, grad = net.loss_grad(x.reshape(-1), (x[..., 0] - d).reshape(-1), shape)
+    grad = grad.double().cpu().numpy()
+    S = np.zeros((cin, 27))
+    for dz in (-1, 0, 1):
+        to, frm = slice(max(0, -dz), nz - max(0, dz)), slice(max(0, dz), nz - max(0, -dz))
+        for dy in (-1, 0, 1):
+            for dx in (-1, 0, 1):
+                for ci in range(cin):
+                    S[ci, ((dz + 1) * 3 + dy + 1) * 3 + dx + 1] = float(
+                        (d[to].double() * x[frm][..., ci].roll((-dy, -dx), (1, 2))).sum())
+    S, B = S * 2.0 / n, float(d.double().sum()) * 2.0 / n
+    n1, n2 = 16 * cin * 27, 16 * 16 * 27
+    at = np.cumsum([0, n1, 16, n2, 16, n2, 16, 16 * 27, 1])
+    part = [grad[a:b] for a, b in zip(at[:-1], at[1:])]
+    cut = 2.0 ** -23
+    want = [np.tile(S.ravel() / 16, 16), B / 16, np.tile(S[0] / 16, 256), B / 16, np.tile(S[0] / 16, 256), B / 16,
+            np.tile(S[0], 16), B]
+    tol = [2 * cut, cut, 256 * cut, cut, 256 * cut, cut, 2 * cut, cut]
+    off = [np.abs(p / w - 1.0).max() for p, w in zip(part, want)]
+    assert all(o < t for o, t in zip(off, tol)), off
+    net.close()
