@@ -274,13 +274,6 @@ __global__ void __launch_bounds__(256) k_prolongate_cell(int nxc, int nyc, int n
         const int I = i >> 1, J = j >> 1;
         const int I2 = cwrap((i & 1) ? I + 1 : I - 1, nxc), J2 = cwrap((j & 1) ? J + 1 : J - 1, nyc);
         const size_t bc = (size_t)k * plc;
-        if constexpr (P::id == 0 && PF::id == 0) {  // native FP64: four operations, accumulated onto u_f
-            R o = P::fma(w9, P::ld(uc, bc + (size_t)J * nxc + I), PF::ld_plain(uf, id));
-            o = P::fma(w3, P::ld(uc, bc + (size_t)J * nxc + I2), o);
-            o = P::fma(w3, P::ld(uc, bc + (size_t)J2 * nxc + I), o);
-            PF::st(uf, id, P::fma(w1, P::ld(uc, bc + (size_t)J2 * nxc + I2), o));
-            continue;
-        }
         R val = P::mul(w9, P::ld(uc, bc + (size_t)J * nxc + I));
         val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J * nxc + I2)));
         val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J2 * nxc + I)));
@@ -365,13 +358,15 @@ __global__ void __launch_bounds__(128) k_prolongate_vec(int nxc, int nyc, int nz
     for (int q = 0; q < CW; ++q) {
         const R xm = c[1][q], xc = c[1][q + 1], xp = c[1][q + 2];
         if constexpr (P::id == 0 && PF::id == 0) {
-            // native FP64, bound by its pipe: the four products accumulate onto u_f, four operations per fine
-            // cell instead of 7.25 (64^2 to 128^2 x 128 18 us, 22 before)
-            auto acc = [&](SF& o, R x, R y, R d) { o = P::fma(w1, d, P::fma(w3, y, P::fma(w3, x, P::fma(w9, xc, o)))); };
-            acc(o0.v[2 * q], xm, c[0][q + 1], c[0][q]);
-            acc(o0.v[2 * q + 1], xp, c[0][q + 1], c[0][q + 2]);
-            acc(o1.v[2 * q], xm, c[2][q + 1], c[2][q]);
-            acc(o1.v[2 * q + 1], xp, c[2][q + 1], c[2][q + 2]);
+            // native FP64, bound by its pipe: both rows share their x part, four operations per fine cell instead of
+            // 7.25. P u_c is formed before it is added, so that only the last rounding is relative to u_f, of which
+            // the correction is a small part
+            const R hm = P::fma(w9, xc, P::mul(w3, xm)), hp = P::fma(w9, xc, P::mul(w3, xp));
+            auto acc = [&](SF& o, R h, R y, R d) { o = P::add(o, P::fma(w1, d, P::fma(w3, y, h))); };
+            acc(o0.v[2 * q], hm, c[0][q + 1], c[0][q]);
+            acc(o0.v[2 * q + 1], hp, c[0][q + 1], c[0][q + 2]);
+            acc(o1.v[2 * q], hm, c[2][q + 1], c[2][q]);
+            acc(o1.v[2 * q + 1], hp, c[2][q + 1], c[2][q + 2]);
         } else {
             // (FP32: the contractions of the general form, written out, so that both give the same bits)
             auto val = [&](R x, R y, R d) {

@@ -394,39 +394,35 @@ __global__ void __launch_bounds__(128) k_panel_restrict_smooth(PanelLvT<T> Lc, T
 }
 
 // u_f += P u_c: bilinear in the logical grid (weights 3/4 and 1/4 per direction), a coarse
-// neighbour beyond the panel boundary contributing 0. One thread per fine column and pz planes. In FP64 the
-// four products accumulate onto u_f (four operations); FP32 forms P u_c first.
+// neighbour beyond the panel boundary contributing 0. A thread takes the two fine rows of a coarse one, which
+// share their x part: four operations per fine cell. P u_c is formed before it is added, so that only the last
+// rounding is relative to u_f, of which the correction is a small part.
 template <class T>
 __global__ void __launch_bounds__(128) k_panel_prolongate(int nxc, int nyc, int nz, const T* __restrict__ uc,
                                                           T* __restrict__ uf, const int* done, int pz) {
     if (done && *(volatile const int*)done) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int nxf = 2 * nxc, nyf = 2 * nyc;
-    if (i >= nxf || j >= nyf) return;
-    const int I = i >> 1, J = j >> 1;
-    const int I2 = (i & 1) ? I + 1 : I - 1, J2 = (j & 1) ? J + 1 : J - 1;
-    const bool in2 = I2 >= 0 && I2 < nxc, jn2 = J2 >= 0 && J2 < nyc;
-    const size_t plc = (size_t)nxc * nyc, plf = (size_t)nxf * nyf;
-    const size_t c0 = (size_t)J * nxc + I, cx = (size_t)J * nxc + I2, cy = (size_t)J2 * nxc + I,
-                 cxy = (size_t)J2 * nxc + I2, fo = (size_t)j * nxf + i;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
+    const int nxf = 2 * nxc;
+    if (i >= nxf || J >= nyc) return;
+    const int I = i >> 1, I2 = (i & 1) ? I + 1 : I - 1;
+    const bool in2 = I2 >= 0 && I2 < nxc, js = J > 0, jn = J + 1 < nyc;
+    const size_t plc = (size_t)nxc * nyc, c0 = (size_t)J * nxc + I, cx = (size_t)J * nxc + I2,
+                 fo = (size_t)(2 * J) * nxf + i;
     const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
-#pragma unroll 4
+#pragma unroll 2
     for (int k = k0; k < k1; ++k) {
         const T* p = uc + (size_t)k * plc;
-        T& o = uf[(size_t)k * plf + fo];
-        if constexpr (sizeof(T) == 8) {
-            T v = fma(T(0.5625), __ldg(p + c0), o);
-            if (in2) v = fma(T(0.1875), __ldg(p + cx), v);
-            if (jn2) v = fma(T(0.1875), __ldg(p + cy), v);
-            if (in2 && jn2) v = fma(T(0.0625), __ldg(p + cxy), v);
-            o = v;
-        } else {
-            T v = T(0.5625) * __ldg(p + c0);
-            if (in2) v = fma(T(0.1875), __ldg(p + cx), v);
-            if (jn2) v = fma(T(0.1875), __ldg(p + cy), v);
-            if (in2 && jn2) v = fma(T(0.0625), __ldg(p + cxy), v);
-            o += v;
-        }
+        T* o = uf + (size_t)k * 4 * plc + fo;
+        const T o0 = o[0], o1 = o[nxf];
+        T h = T(0.5625) * __ldg(p + c0);
+        if (in2) h = fma(T(0.1875), __ldg(p + cx), h);
+        T v0 = h, v1 = h;
+        if (js) v0 = fma(T(0.1875), __ldg(p + c0 - nxc), v0);
+        if (js && in2) v0 = fma(T(0.0625), __ldg(p + cx - nxc), v0);
+        if (jn) v1 = fma(T(0.1875), __ldg(p + c0 + nxc), v1);
+        if (jn && in2) v1 = fma(T(0.0625), __ldg(p + cx + nxc), v1);
+        o[0] = o0 + v0;
+        o[nxf] = o1 + v1;
     }
 }
 
@@ -614,7 +610,7 @@ void launch_panel_restrict_smooth(const PanelLvT<T>& Lc, double rho, const T* rf
 
 template <class T>
 void launch_panel_prolongate(int nxc, int nyc, int nz, const T* uc, T* uf, const int* done, cudaStream_t s) {
-    dim3 g = panel_grid(2 * nxc, 2 * nyc);
+    dim3 g = panel_grid(2 * nxc, nyc);
     const int pz = point_planes(2 * nxc, 2 * nyc);
     g.z = (nz + pz - 1) / pz;
     k_panel_prolongate<T><<<g, dim3(32, 4), 0, s>>>(nxc, nyc, nz, uc, uf, done, pz);

@@ -74,3 +74,34 @@ def test_gradient_sums_of_one_sign_match_64_bit_sums(cin, shape):
     off = [np.abs(p / w - 1.0).max() for p, w in zip(part, want)]
     assert all(o < t for o, t in zip(off, tol)), off
     net.close()
+
+
+@pytest.mark.parametrize("what,shape,by", [("box", (130, 66, 3), 0), ("box", (130, 66, 3), 1), ("box", (32, 32, 8), 0),
+                                           ("panel", (66, 64, 5), 0)], ids=["vector", "any-alignment", "cells", "panel"])
+def test_prolongation_rounds_once_relative_to_the_fine_field(what, shape, by):
+    """u_f + P u_c with a correction of a tenth of u_f, as in a V-cycle, in native FP64 against extended precision.
+    The correctly rounded sum has the r.m.s. error e of one rounding; P u_c adds at most five of a tenth of its size:
+    sqrt(1 + 5 / 100) e. 1.25 e leaves room for that, not for more than one rounding at u_f's size."""
+    nx, ny, nz = shape
+    n, nc = nx * ny * nz, nx * ny * nz // 4
+    rng = np.random.default_rng(17)
+    uf, uc = rng.standard_normal((nz, ny, nx)), 0.1 * rng.standard_normal((nz, ny // 2, nx // 2))
+    t = torch.empty(n + 2, dtype=torch.float64, device="cuda")[by:by + n]
+    t.copy_(torch.from_numpy(uf.ravel()))
+    if what == "box":
+        op = tpmg.Operator(nx, ny, nz, 1e-2, 1.0 / nx, 1.0 / ny, 1.0 / nz, 1e3, nlevels=2)
+        tpmg.prolongate(op.op, 2, tpmg.F64, dev(uc, tpmg.F64), t, nc, n)
+        e = np.pad(uc.astype(np.longdouble), ((0, 0), (1, 1), (1, 1)), mode="wrap")
+    else:
+        op = tpmg.PanelOperator(nx, ny, nz, 1e-4, 1.0, 1e-3, nlevels=2)
+        tpmg.panel_prolongate(op.op, 2, dev(uc, tpmg.F64), t, nc, n)
+        e = np.pad(uc.astype(np.longdouble), ((0, 0), (1, 1), (1, 1)))
+    exact = uf.astype(np.longdouble)
+    c, ldx = e[:, 1:-1, 1:-1], {0: e[:, 1:-1, :-2], 1: e[:, 1:-1, 2:]}
+    for b, y in ((0, slice(None, -2)), (1, slice(2, None))):
+        for a, x in ((0, slice(None, -2)), (1, slice(2, None))):
+            exact[:, b::2, a::2] += (9 * c + 3 * ldx[a] + 3 * e[:, y, 1:-1] + e[:, y, x]) / 16
+    rms = lambda v: float(np.sqrt(np.mean((v.astype(np.longdouble) - exact) ** 2)))
+    got = t.cpu().numpy().reshape(nz, ny, nx)
+    assert rms(got) < 1.25 * rms(exact.astype(np.float64)), (rms(got), rms(exact.astype(np.float64)))
+    op.close()
