@@ -322,14 +322,14 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid, int top = 0) {
     return TPMG_OK;
 }
 
-// hierarchy of precision pid; the finest level's u and f are allocated only when `own_fine`
-// (DW: internal copies of the caller's FP64 fields; mixed inner FP32 cycle: e and r).
-static tpmg_status ensure_hier(tpmg_op* op, int pid, bool own_fine) {
-    TRY(ensure_factors(op, pid));
+// hierarchy of precision pid up to level `top` (0: all); the finest level's u and f are allocated only when
+// `own_fine` (DW: internal copies of the caller's FP64 fields; mixed inner FP32 cycle: e and r).
+static tpmg_status ensure_hier(tpmg_op* op, int pid, bool own_fine, int top = 0) {
+    TRY(ensure_factors(op, pid, top));
     Hier& h = op->hier[pid];
     const size_t eb = elem_bytes(pid);
     const int L = op->g.L;
-    for (int l = 1; l <= L; ++l) {
+    for (int l = 1; l <= (top < 1 ? L : top); ++l) {
         size_t bytes = lvl_cells(op, l) * eb;
         TRY(dalloc(&h.ub[l], bytes));
         TRY(dalloc(&h.r[l], bytes));
@@ -338,8 +338,13 @@ static tpmg_status ensure_hier(tpmg_op* op, int pid, bool own_fine) {
             TRY(dalloc(&h.f[l], bytes));
         }
     }
-    h.ready = true;
     return ensure_common(op);
+}
+
+// the double-word solver's hierarchy: its own levels and the coarse ones that run in native FP64
+static tpmg_status ensure_hier_dw(tpmg_op* op) {
+    TRY(ensure_hier(op, 2, true));
+    return op->lsw_dw > 1 ? ensure_hier(op, 0, false, op->lsw_dw - 1) : TPMG_OK;
 }
 
 static tpmg_status ensure_io(tpmg_op* op) {
@@ -896,10 +901,9 @@ tpmg_status tpmg_op_reserve(tpmg_op* op, tpmg_precision prec) {
         case TPMG_F64: TRY(ensure_hier(op, 0, false)); TRY(ensure_cg(op, 0)); break;
         case TPMG_F32: TRY(ensure_hier(op, 1, false)); TRY(ensure_cg(op, 1)); break;
         case TPMG_DW:
-            TRY(ensure_hier(op, 2, true));
-            TRY(ensure_cg(op, 2));
+            TRY(ensure_hier_dw(op));
+            TRY(ensure_cg(op, op->lsw_dw > op->g.L ? 0 : 2));
             TRY(ensure_io(op));
-            if (op->lsw_dw > 1) TRY(ensure_factors(op, 0, op->lsw_dw - 1));  // the levels that run in native FP64
             break;
         case TPMG_MIXED: TRY(ensure_hier(op, 2, true)); TRY(ensure_hier(op, 1, true)); break;
         default: return set_err(TPMG_ERR_ARG, "unknown precision");
@@ -1081,7 +1085,8 @@ tpmg_status tpmg_residual_restrict_smooth(tpmg_op* op, int level, tpmg_precision
     if (level >= op->g.L) return set_err(TPMG_ERR_ARG, "residual_restrict_smooth needs a coarse level < L");
     if (!u_fine || !f_fine || !f_c || !u_c) return set_err(TPMG_ERR_ARG, "NULL field");
     // see DW_KAPPA_MAX; a small coarse level has no fused form
-    if (prec == TPMG_DW && level + 1 < op->lsw_dw && lvl_cells(op, level) / op->g.nz > (size_t)PCR_MAX_COLS) prec = TPMG_F64;
+    const bool low = prec == TPMG_DW && level + 1 < op->lsw_dw && lvl_cells(op, level) / op->g.nz > (size_t)PCR_MAX_COLS;
+    if (low) prec = TPMG_F64;
     if (prec == TPMG_DW && level < op->lsw_dw) {
         // a native-FP64 coarse level, the fine one in either: the two kernels, the residual handed over in FP64
         // through a staging buffer
@@ -1089,8 +1094,8 @@ tpmg_status tpmg_residual_restrict_smooth(tpmg_op* op, int level, tpmg_precision
         TRY(tpmg_residual(op, level + 1, prec, u_fine, f_fine, op->io[3], nullptr, stream));
         return tpmg_restrict_smooth(op, level, prec, rho, op->io[3], f_c, u_c, stream);
     }
-    TRY(prep_unit(op, prec));
-    TRY(ensure_hier(op, pid_of(prec), true));  // the fine residual buffer of the unfused fallback
+    TRY(prep_unit(op, prec, low));
+    TRY(ensure_hier(op, pid_of(prec), true, low ? op->lsw_dw - 1 : 0));  // the fine residual buffer of the unfused fallback
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nc = lvl_cells(op, level), nf = lvl_cells(op, level + 1);
     DISPATCH_PREC(prec, {
@@ -1265,8 +1270,7 @@ tpmg_status tpmg_mg_solve(tpmg_op* op, const tpmg_params* prm, const void* f, vo
             TRY((mg_loop<PolF32, PolF32>(op, prm, (float*)u, (float*)f, 1, s)));
             break;
         case TPMG_DW: {
-            TRY(ensure_hier(op, 2, true));
-            TRY(ensure_hier(op, 0, false));
+            TRY(ensure_hier_dw(op));
             float2* uD = (float2*)op->hier[2].u[L];
             float2* fD = (float2*)op->hier[2].f[L];
             CK(cudaEventRecord(op->ev0, s));
@@ -1396,8 +1400,7 @@ tpmg_status tpmg_vcycle(tpmg_op* op, const tpmg_params* prm, const void* f, void
             TRY(one(PolF32(), PolF32(), (float*)u, (float*)f, 1));
             break;
         case TPMG_DW: {
-            TRY(ensure_hier(op, 2, true));
-            TRY(ensure_hier(op, 0, false));
+            TRY(ensure_hier_dw(op));
             float2* uD = (float2*)op->hier[2].u[L];
             float2* fD = (float2*)op->hier[2].f[L];
             launch_f64_to_dw(n, (const double*)u, uD, s);
