@@ -17,7 +17,7 @@ int launch_restrict_tile(const Lv<P>& L, const Lv<P>& Lc, double rho, const type
                          typename P::S* fc, typename P::S* uc, const int* done, cudaStream_t s) {
     typedef typename P::S S;
     constexpr int W = 512 / (int)sizeof(S), PLANE = 256;
-    if (L.nx % W || L.ny % 2) return -1;
+    if (L.nx % W || L.ny % 2 || L.ny / 2 > 65535) return -1;  // (rows of tiles that a launch takes)
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(fc) || !al(uc) || (Lc.fac_percol && !al(Lc.finv))) return -1;
     int kw = 0;

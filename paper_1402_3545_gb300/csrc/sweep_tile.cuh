@@ -570,8 +570,7 @@ __global__ void __launch_bounds__(TNT, 3)
 
 template <class P, int MODE, int TR, bool ISO, bool NORM>
 static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
-                          typename P::S* out, double* partials, const int* done, cudaStream_t s,
-                          const Scalars* sc = nullptr) {
+                          typename P::S* out, double* partials, const int* done, cudaStream_t s, const Scalars* sc) {
     typedef typename P::S S;
     int kw = 0;
     if (L.fac_percol) kw = factor_planes(L);
@@ -584,43 +583,41 @@ static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, c
     return (int)(grd.x * grd.y);
 }
 
+// Rows of a level's tiles, 0 where it has none. two: two rows wherever they fit. The launch takes 65535 rows of tiles.
+template <class P>
+static int tile_rows(int nx, int ny, bool two) {
+    constexpr int W = TPB / (int)sizeof(typename P::S), MAXR = 65535;
+    if (nx % W == 0 && !(two && ny % 2 == 0) && ny <= MAXR) return 1;
+    if (nx % (W / 2) == 0 && ny % 2 == 0 && ny / 2 <= MAXR) return 2;
+    return nx % (W / 4) == 0 && ny % 4 == 0 && ny / 4 <= MAXR ? 4 : 0;
+}
 template <class P, int MODE, bool ISO, bool NORM>
 static int run_sweep_tile_rows(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
-                               typename P::S* out, double* partials, const int* done, cudaStream_t s) {
-    constexpr int W = TPB / (int)sizeof(typename P::S);
+                               typename P::S* out, double* partials, const int* done, cudaStream_t s,
+                               const Scalars* sc = nullptr) {
     // FP32 Smooth: two rows of 64 columns share their inner rows and so load two rows of u per row instead of
     // three (1024^2 x 128 396 us, 429 with one row of 128, 436 with four of 32)
-    constexpr bool TWO = P::id == 1 && MODE == MODE_SMOOTH;
-    if (L.nx % W == 0 && !(TWO && L.ny % 2 == 0))
-        return run_sweep_tile<P, MODE, 1, ISO, NORM>(L, coef, u, f, out, partials, done, s);
-    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0)
-        return run_sweep_tile<P, MODE, 2, ISO, NORM>(L, coef, u, f, out, partials, done, s);
-    if (L.nx % (W / 4) == 0 && L.ny % 4 == 0)
-        return run_sweep_tile<P, MODE, 4, ISO, NORM>(L, coef, u, f, out, partials, done, s);
-    return -1;
+    switch (tile_rows<P>(L.nx, L.ny, P::id == 1 && MODE == MODE_SMOOTH)) {
+        case 1: return run_sweep_tile<P, MODE, 1, ISO, NORM>(L, coef, u, f, out, partials, done, s, sc);
+        case 2: return run_sweep_tile<P, MODE, 2, ISO, NORM>(L, coef, u, f, out, partials, done, s, sc);
+        case 4: return run_sweep_tile<P, MODE, 4, ISO, NORM>(L, coef, u, f, out, partials, done, s, sc);
+        default: return -1;
+    }
 }
 
 template <class P>
 int cg_tile_blocks(const Lv<P>& L) {
-    constexpr int W = TPB / (int)sizeof(typename P::S);
     if (L.nz > 128 || !L.finv || !L.fw || !(tile_pays(L) || (P::id == 1 && L.nz >= 16))) return -1;
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(L.v) || (L.fac_percol && (!al(L.finv) || !al(L.fw)))) return -1;
-    if (L.nx % W == 0) return L.nx / W * L.ny;
-    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0) return L.nx / (W / 2) * (L.ny / 2);
-    if (L.nx % (W / 4) == 0 && L.ny % 4 == 0) return L.nx / (W / 4) * (L.ny / 4);
-    return -1;
+    const int tr = tile_rows<P>(L.nx, L.ny, false);
+    return tr ? L.nx / (TPB / tr / (int)sizeof(typename P::S)) * (L.ny / tr) : -1;
 }
 template <class P>
 int launch_cg_tile(const Lv<P>& L, const Scalars* sc, typename P::S* r, const typename P::S* q, typename P::S* z,
                    double* partials, cudaStream_t s) {
-    constexpr int W = TPB / (int)sizeof(typename P::S);
     if (cg_tile_blocks(L) < 0) return -1;
-    const int* done = &sc->done;
-    if (L.nx % W == 0) return run_sweep_tile<P, MODE_CGTRI, 1, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
-    if (L.nx % (W / 2) == 0 && L.ny % 2 == 0)
-        return run_sweep_tile<P, MODE_CGTRI, 2, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
-    return run_sweep_tile<P, MODE_CGTRI, 4, true, true>(L, 1.0, r, q, z, partials, done, s, sc);
+    return run_sweep_tile_rows<P, MODE_CGTRI, true, true>(L, 1.0, r, q, z, partials, &sc->done, s, sc);
 }
 
 template <class P, int MODE>
