@@ -371,8 +371,8 @@ Shape sweep_shape(int nx, int ny, int nz, int bytes_per_value, bool stack) {
 
 int max_partials(int nx, int ny) {
     const int col_kernels = ((nx + TX - 1) / TX) * ny;
-    // small levels: at most one block per column; chunked columns (native FP64): one per 8 columns. A level
-    // below the finest has a quarter of its columns or fewer, so that the finest level's count covers it.
+    // small levels: at most one block per column; chunked columns (native FP64) and the pointwise Residual: one per
+    // 8 columns. (A coarse level's count can be above the finest one's: 112 x 100 takes 1408, 224 x 200 1400.)
     const int cell_kernels = nx * ny <= PCR_MAX_COLS ? nx * ny : (nx * ny <= CHUNK_MAX_COLS || nx % 32 != 0 ? (nx * ny + 127) / 128 * 16 : 0);
     return col_kernels > cell_kernels ? col_kernels : cell_kernels;
 }

@@ -23,6 +23,8 @@
 // idle with a thread per column and 2 nz dependent FP64 operations (about 80 cycles each) per sweep:
 // there a column is cut into chunks of planes (k_panel_chunk), and the pointwise kernels take a few
 // planes per thread. FP32 (the mixed solve's inner cycles) keeps one thread per column throughout.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "panel.cuh"
 
@@ -561,8 +563,10 @@ static int panel_point(const PanelLv& L, const double* u, const double* f, TO* o
                        cudaStream_t s) {
     dim3 g = panel_grid(L.nx, L.ny);
     int pz = point_planes(L.nx, L.ny);
-    // partial sums: at most one block per 32 columns (max_partials), that is four per 32 x 4 tile
-    if (partials) pz = L.ny >= 4 ? (L.nz + 3) / 4 : L.nz;
+    if (partials) {  // as many slabs of planes as max_partials leaves room for
+        const int room = max_partials(L.nx, L.ny) / (int)(g.x * g.y);
+        pz = std::max(pz, room > 1 ? (L.nz + room - 1) / room : L.nz);
+    }
     g.z = (L.nz + pz - 1) / pz;
     k_panel_point<MODE, TO><<<g, dim3(32, 4), 0, s>>>(L, u, f, out, partials, done, pz);
     note_launch();
