@@ -302,9 +302,6 @@ static int chunk_sweep(const Lv<PolF64>& L, double coef, const typename PF::S* u
 
 int launch_smooth_chunk(const Lv<PolF64>& L, double rho, const double* u, const double* f, double* uo, double* partials,
                         const int* done, cudaStream_t s) {
-    // above PCR_MAX_COLS columns a tile variant that was chosen for the level takes precedence (where the
-    // level has tiles at all)
-    if ((size_t)L.nx * L.ny > (size_t)PCR_MAX_COLS && L.variant >= 0 && L.nx % 32 == 0) return -1;
     return chunk_sweep<PolF64, 0>(L, rho, u, f, uo, nullptr, partials, done, s);
 }
 int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, double scale, const int* done, cudaStream_t s) {
