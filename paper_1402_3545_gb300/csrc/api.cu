@@ -1448,8 +1448,9 @@ tpmg_status tpmg_autotune(tpmg_op* op, tpmg_precision prec, int reps, int* varia
                 typedef decltype(tag) P;
                 typedef typename P::S S;
                 Hier& h = op->hier[pid];
-                launch_smooth<P>(level_view<P>(op, l), 0.8, (const S*)h.u[l], (const S*)h.f[l], (S*)h.ub[l],
-                                 op->partials, nullptr, s);
+                // without the norm, as all but one Smooth of a cycle run (in native FP64 another kernel)
+                launch_smooth<P>(level_view<P>(op, l), 0.8, (const S*)h.u[l], (const S*)h.f[l], (S*)h.ub[l], nullptr,
+                                 nullptr, s);
             };
             auto once = [&]() {
                 if (pid == 0) run(PolF64());
