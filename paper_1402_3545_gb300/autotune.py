@@ -1,6 +1,6 @@
 """Autotuner cache: the Smooth tile variant chosen per level, kept in a JSON file keyed by GPU.
 
-tune(op, prec) looks up (GPU name, grid shape, precision, whether lambda^2 varies) in the cache; on a
+tune(op, prec) looks up (GPU name, variant set, grid shape, precision, whether lambda^2 varies) in the cache; on a
 miss it runs the library's tpmg_autotune (which times every variant on the operator's own
 workspace) and stores the result. The cache lives in $TPMG_TUNE_CACHE, else
 ~/.cache/tpmg/tuning.json. Only the schedule changes with the variant, never the per-cell
@@ -14,6 +14,10 @@ import os
 import torch
 
 from . import tpmg
+
+# The library's set of Smooth kernels: raised when a variant gets another kernel or levels are dealt to them
+# differently. A choice that was timed among other kernels is measured again.
+VARIANT_SET = 2
 
 
 def cache_path() -> str:
@@ -43,7 +47,7 @@ def _store(d: dict) -> None:
 
 def key(operator: "tpmg.Operator", prec: int, lambda_varies: bool) -> str:
     gpu = torch.cuda.get_device_name(torch.cuda.current_device())
-    return f"{gpu}|{operator.nx}x{operator.ny}x{operator.nz}|L{operator.L}|prec{prec}|var{int(lambda_varies)}"
+    return f"{gpu}|set{VARIANT_SET}|{operator.nx}x{operator.ny}x{operator.nz}|L{operator.L}|prec{prec}|var{int(lambda_varies)}"
 
 
 def tune(operator: "tpmg.Operator", prec: int, lambda_varies: bool, reps: int = 5, force: bool = False) -> list[int]:
