@@ -1645,7 +1645,7 @@ static void cycle_tasks(tpmg_op* op, int b, const tpmg_params* prm, std::vector<
     auto form_of = [&](int type, int level) {
         const int lf = type == BT_RRS ? level - 1 : level;  // whose factors it uses
         return batched_form(type, op->g.lnx[level], op->g.lny[level], op->g.nz, op->percol[lf],
-                            factor_planes(level_view<PolF32>(op, lf)), op->cx[level] == op->cy[level]);
+                            op->percol[lf] ? factor_planes(level_view<PolF32>(op, lf)) : 0);
     };
     auto task = [&](int type, int level, const void* a, const void* rhs, void* o, void* o2) {
         BTask t;

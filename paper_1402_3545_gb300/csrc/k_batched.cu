@@ -12,16 +12,18 @@
 //
 // Forms of a task (batched_form):
 //  - BF_TILE1, BF_TILE2: Smooth and first line solve on whole columns in shared memory, 128 x 1 or 64 x 2 FP32
-//    columns a tile, as the single-problem solver's (sweep_tile.cuh; here the one-row tile is the faster one); the fused Residual + RestrictSmooth on tiles of 128 x 2 fine
-//    columns (restrict_tile.cuh);
+//    columns a tile, as the single-problem solver's (sweep_tile.cuh; here the one-row tile is the faster one); the
+//    fused Residual + RestrictSmooth on tiles of 128 x 2 fine columns (restrict_tile.cuh);
 //  - BF_COLS: 32 columns of the level in order, planes in parallel over the eight warps, one warp running the
-//    recurrences in shared memory: all other shapes;
+//    recurrences in shared memory, their factors there too: all other shapes;
 //  - Residuals (FP32 and the outer double-word one), Prolongate and the correction: pointwise.
-// Three blocks of 256 threads per SM, set by the tiles' 65 KB at 128 planes. Before, 128-thread blocks marched
-// every column plane by plane, its Thomas values on a stack in L2 (a chain of loads, elimination and stack store
-// per plane, and on the narrow levels one column per thread): 12 problems of 64 .. 512 squared x 32 .. 128 to 1e-9
-// 43.2 ms, 28.7 here, the same bits. What is left: the FP32 tiles (0.55 of the copy rate), the outer residual
-// and correction (20 bytes per cell each) and, once most problems have converged, too few tiles per phase.
+// Three blocks of 256 threads per SM, set by the tiles' 65 KB at 128 planes, or two where a tile's per-column factors
+// take it to 84 KB (BTILE_SMEM2). Ten cycles of 256^2 x 64, 512 x 256 x 128, 128^2 x 64 and 64 x 128 x 32, ms: lambda^2
+// constant 10.4, varying 13.9 (two blocks; 16.9 with those levels on BF_COLS). 256^2 x 200 and 128 x 256 x 200 (BF_COLS)
+// 14.7 and 16.7 (20.2 with a limit of 98 KB, which moves some of their levels to tiles); oblong cells the same. With
+// BF_COLS' factors read from global memory plane by plane the varying ones took 28 and 31 ms.
+// What is left: the FP32 tiles (0.55 of the copy rate), the outer residual and correction (20 bytes per cell each) and,
+// once most problems have converged, too few tiles per phase.
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -36,6 +38,7 @@ constexpr int BPZ = 16;             // planes of a column a pointwise residual t
 constexpr int BCH = 4096;           // cells of a correction tile
 constexpr int BPU = 1024;           // coarse segments of a Prolongate tile
 constexpr size_t BTILE_SMEM = 72 * 1024;  // three blocks of it fit an SM
+constexpr size_t BTILE_SMEM2 = 84 * 1024;  // two: tiles with per-column factors
 
 __device__ __forceinline__ int bwrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
@@ -210,21 +213,30 @@ struct BRhs {
     }
 };
 
-// BF_COLS: out = u + rho M^{-1}(f - A u), rho M^{-1} f, or (u the fine residual) fc = R u, out = rho M^{-1} fc
+// BF_COLS: out = u + rho M^{-1}(f - A u), rho M^{-1} f, or (u the fine residual) fc = R u, out = rho M^{-1} fc.
+// Factors as in sweep_tile.cuh: two tables of nz values behind the planes, or (percol) 1/m_k of the planes before the
+// converged ones, which the elimination turns into w_k.
 template <int MODE, bool SW>
 __device__ void t_cols(const BLevelDesc& L, float rho, const float* u, const float* f, float* fc, float* out, int tile,
                        unsigned char* smem) {
     float* const Z = reinterpret_cast<float*>(smem);
-    const int nz = L.nz, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* const T = Z + (size_t)nz * 32;  // the factor tables where lambda^2 is constant
+    const int nz = L.nz, kw = L.kw, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, clast = nz >= 2 ? nz - 2 : 0;
+    const bool percol = L.percol != 0;
+    float* const T = Z + (size_t)nz * 32;
     const BRhs<MODE, SW> R(L, u, f, tile * 32 + lane);
     constexpr bool GF = MODE == BM_SMOOTH && SW;  // the back substitution yields the result
+    constexpr int TAB = 0, COL = 1, CONV = 2;     // factors: per-plane table, per column and plane, converged
     const size_t pl = R.pl, c = R.q.c;
-    if (!L.percol)
+    float cw = 0.f;  // the converged w_k (that of plane nz-1 meets x = 0)
+    if (percol) {
+        for (int k = warp; k < kw; k += BNW) T[k * 32 + lane] = __ldg(L.finv + (size_t)k * pl + c);
+        cw = __ldg(L.fw + (size_t)clast * pl + c);
+    } else {
         for (int k = threadIdx.x; k < nz; k += BNT) {
             T[k] = __ldg(L.finv + k);
             T[nz + k] = __ldg(L.fw + k);
         }
+    }
     constexpr int D = MODE == BM_SMOOTH ? 2 : 4;
     for (int k = warp; k < nz; k += D * BNW) {
         float r[D];
@@ -240,37 +252,44 @@ __device__ void t_cols(const BLevelDesc& L, float rho, const float* u, const flo
     }
     __syncthreads();
     constexpr int KB = 8;
-    auto fac = [&](int which, int k) {
-        if (!L.percol) return T[which * nz + k];
-        return __ldg((which ? L.fw : L.finv) + (size_t)k * pl + c);
-    };
     if (warp == 0) {
         const float vv = R.vv;
         float d = 0.f;
-        int k = 0;
-        for (; k + KB <= nz; k += KB) {
-            float r[KB], iv[KB];
+        auto forward = [&](auto kind, int k, int ke, float inv) {
+            constexpr int F = decltype(kind)::value;
+            auto factor = [&](int kk) { return F == TAB ? T[kk] : (F == COL ? T[kk * 32 + lane] : inv); };
+            auto step = [&](int kk, float r, float iv) {
+                if (F == COL) T[kk * 32 + lane] = PolF32::mul(vv, iv);
+                d = PolF32::mul(PolF32::fma(vv, d, r), iv);
+                Z[kk * 32 + lane] = d;
+            };
+            for (; k + KB <= ke; k += KB) {
+                float r[KB], iv[KB];
 #pragma unroll
-            for (int t = 0; t < KB; ++t) {
-                r[t] = Z[(k + t) * 32 + lane];
-                iv[t] = fac(0, k + t);
-            }
+                for (int t = 0; t < KB; ++t) {
+                    r[t] = Z[(k + t) * 32 + lane];
+                    iv[t] = factor(k + t);
+                }
 #pragma unroll
-            for (int t = 0; t < KB; ++t) {
-                d = PolF32::mul(PolF32::fma(vv, d, r[t]), iv[t]);
-                Z[(k + t) * 32 + lane] = d;
+                for (int t = 0; t < KB; ++t) step(k + t, r[t], iv[t]);
             }
-        }
-        for (; k < nz; ++k) {
-            d = PolF32::mul(PolF32::fma(vv, d, Z[k * 32 + lane]), fac(0, k));
-            Z[k * 32 + lane] = d;
+            for (; k < ke; ++k) step(k, Z[k * 32 + lane], factor(k));
+        };
+        if (percol) {
+            const float cinv = __ldg(L.finv + (size_t)clast * pl + c), einv = __ldg(L.finv + (size_t)(nz - 1) * pl + c);
+            forward(std::integral_constant<int, COL>(), 0, kw, 0.f);
+            forward(std::integral_constant<int, CONV>(), kw, nz - 1, cinv);
+            forward(std::integral_constant<int, CONV>(), nz - 1, nz, einv);
+        } else {
+            forward(std::integral_constant<int, TAB>(), 0, nz, 0.f);
         }
     }
     if (GF) {
         __syncthreads();
         for (int k = warp; k < nz; k += BNW) {
             const float u0 = u[(size_t)k * pl + c], u1 = u[(size_t)(k + 1 < nz ? k + 1 : k) * pl + c];
-            Z[k * 32 + lane] = PolF32::fma(-fac(1, k), k + 1 < nz ? u1 : 0.f, PolF32::fma(rho, Z[k * 32 + lane], u0));
+            const float w = !percol ? T[nz + k] : (k < kw ? T[k * 32 + lane] : cw);
+            Z[k * 32 + lane] = PolF32::fma(-w, k + 1 < nz ? u1 : 0.f, PolF32::fma(rho, Z[k * 32 + lane], u0));
         }
         __syncthreads();
     }
@@ -280,23 +299,32 @@ __device__ void t_cols(const BLevelDesc& L, float rho, const float* u, const flo
             if (MODE == BM_SMOOTH && !GF) Z[kk * 32 + lane] = xk;
             else if (R.q.act) out[(size_t)kk * pl + c] = GF ? xk : PolF32::mul(rho, xk);
         };
-        int k = nz;
-        for (; k - KB >= 0; k -= KB) {
-            float dk[KB], w[KB];
+        auto backward = [&](auto kind, int k, int ke) {  // planes k-1 .. ke
+            constexpr int F = decltype(kind)::value;
+            auto factor = [&](int kk) { return F == TAB ? T[nz + kk] : (F == COL ? T[kk * 32 + lane] : cw); };
+            for (; k - KB >= ke; k -= KB) {
+                float dk[KB], w[KB];
 #pragma unroll
-            for (int t = 0; t < KB; ++t) {
-                dk[t] = Z[(k - 1 - t) * 32 + lane];
-                w[t] = fac(1, k - 1 - t);
-            }
+                for (int t = 0; t < KB; ++t) {
+                    dk[t] = Z[(k - 1 - t) * 32 + lane];
+                    w[t] = factor(k - 1 - t);
+                }
 #pragma unroll
-            for (int t = 0; t < KB; ++t) {
-                x = PolF32::fma(w[t], x, dk[t]);
-                put(k - 1 - t, x);
+                for (int t = 0; t < KB; ++t) {
+                    x = PolF32::fma(w[t], x, dk[t]);
+                    put(k - 1 - t, x);
+                }
             }
-        }
-        for (; k > 0; --k) {
-            x = PolF32::fma(fac(1, k - 1), x, Z[(k - 1) * 32 + lane]);
-            put(k - 1, x);
+            for (; k > ke; --k) {
+                x = PolF32::fma(factor(k - 1), x, Z[(k - 1) * 32 + lane]);
+                put(k - 1, x);
+            }
+        };
+        if (percol) {
+            backward(std::integral_constant<int, CONV>(), nz, kw);
+            backward(std::integral_constant<int, COL>(), kw, 0);
+        } else {
+            backward(std::integral_constant<int, TAB>(), nz, 0);
         }
     }
     if (MODE == BM_SMOOTH && !GF) {
@@ -447,8 +475,12 @@ __device__ __forceinline__ void tile_task(const BTask& tk, const BLevelDesc& bl,
     constexpr int W = TPB / TR / (int)sizeof(float);
     const int tx = bl.nx / W, by = loc / tx, bx = loc - by * tx;
     const float* u = (const float*)(MODE == MODE_LINESOLVE ? tk.b : tk.a);
-    sweep_tile_body<PolF32, MODE, TR, true, false, false>(lv32(bl), bl.krho, u, (const float*)tk.b, (float*)tk.out, nullptr,
-                                                          bl.kw, nullptr, bx, by, 0, 0, smem);
+    if (MODE == MODE_LINESOLVE || bl.k1.iso)
+        sweep_tile_body<PolF32, MODE, TR, true, false, false>(lv32(bl), bl.krho, u, (const float*)tk.b, (float*)tk.out, nullptr,
+                                                              bl.kw, nullptr, bx, by, 0, 0, smem);
+    else
+        sweep_tile_body<PolF32, MODE, TR, false, false, false>(lv32(bl), bl.krho, u, (const float*)tk.b, (float*)tk.out, nullptr,
+                                                               bl.kw, nullptr, bx, by, 0, 0, smem);
 }
 
 __global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
@@ -511,7 +543,8 @@ __global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
                         const BLevelDesc& bc = pb.lev[tk.level - 1];
                         const XRestrict<PolF32> xr{lv32(bc), bc.krho.coef, 0.25f, o, o2};
                         const int tx = bl.nx / 128, by = loc / tx, bx = loc - by * tx;
-                        restrict_tile_body<PolF32, true, false>(lv32(bl), bl.k1, xr, a, b, bc.kw, bx, by, bsmem);
+                        if (bl.k1.iso) restrict_tile_body<PolF32, true, false>(lv32(bl), bl.k1, xr, a, b, bc.kw, bx, by, bsmem);
+                        else restrict_tile_body<PolF32, false, false>(lv32(bl), bl.k1, xr, a, b, bc.kw, bx, by, bsmem);
                         break;
                     }
                     case BT_PROL:
@@ -533,23 +566,20 @@ __global__ void __launch_bounds__(BNT, 3) k_batched(BatchDesc d) {
 }
 
 // ---------------------------------------------------------------- tasks and launch
-// The vector tiles (cx == cy: their square-cell form) take the levels with the sweeps' arithmetic, all others the
-// 32-column form.
-int batched_form(int type, int nx, int ny, int nz, int percol, int kw, bool square) {
-    const size_t tile = (size_t)nz * TPB + (percol ? (size_t)kw * TPB : 2 * (size_t)nz * sizeof(float));
-    if (type == BT_SMOOTH || type == BT_LS0) {
-        if (!square || !bsweeps(nx, ny) || tile > BTILE_SMEM) return BF_COLS;
-        return nx % 128 == 0 ? BF_TILE1 : BF_TILE2;
-    }
-    if (type == BT_RRS)  // nx, ny of the fine level, percol and kw of the coarse one
-        return square && bsweeps(nx, ny) && nx % 128 == 0 && batched_smem(BT_RRS, BF_TILE1, nz, percol, kw) <= BTILE_SMEM ? BF_TILE1 : -1;
-    return BF_COLS;
+// The vector tiles take the levels with the sweeps' arithmetic, all others the 32-column form.
+int batched_form(int type, int nx, int ny, int nz, int percol, int kw) {
+    if (type != BT_SMOOTH && type != BT_LS0 && type != BT_RRS) return BF_COLS;
+    const int tile = nx % 128 == 0 ? BF_TILE1 : BF_TILE2;
+    const bool fits = bsweeps(nx, ny) && batched_smem(type, tile, nz, percol, kw) <= (percol ? BTILE_SMEM2 : BTILE_SMEM);
+    // (BT_RRS: nx, ny of the fine level, percol and kw of the coarse one)
+    if (type == BT_RRS) return fits && tile == BF_TILE1 ? BF_TILE1 : -1;
+    return fits ? tile : BF_COLS;
 }
 size_t batched_smem(int type, int form, int nz, int percol, int kw) {
     const size_t tables = percol ? 0 : 2 * (size_t)nz * sizeof(float);
     if (type == BT_RRS) return (size_t)(nz + (percol ? kw : 0)) * 256 + tables;
     if (type != BT_SMOOTH && type != BT_LS0 && type != BT_RS) return 0;
-    if (form == BF_COLS) return (size_t)nz * 128 + 2 * (size_t)nz * sizeof(float);
+    if (form == BF_COLS) return (size_t)(nz + (percol ? kw : 0)) * 128 + tables;
     return (size_t)(nz + (percol ? kw : 0)) * TPB + tables;
 }
 int batched_tiles(int type, int form, int nx, int ny, int nz) {
@@ -569,7 +599,7 @@ int batched_tiles(int type, int form, int nx, int ny, int nz) {
 }
 int batched_blocks_per_sm(size_t smem) {
     int nb = 0;
-    if (cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BTILE_SMEM) != cudaSuccess ||
+    if (cudaFuncSetAttribute(k_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BTILE_SMEM2) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batched, BNT, smem) != cudaSuccess)
         return 0;
     return nb;

@@ -483,7 +483,7 @@ struct BatchDesc {
 cudaError_t launch_batched(const BatchDesc& d, int grid, size_t smem, cudaStream_t s);
 // The form a task's tiles take (BT_RRS: nx, ny of the fine level, percol and kw of the coarse one; -1: the two
 // separate tasks), the number of tiles, and the dynamic shared memory of a block
-int batched_form(int type, int nx, int ny, int nz, int percol, int kw, bool square);
+int batched_form(int type, int nx, int ny, int nz, int percol, int kw);
 int batched_tiles(int type, int form, int nx, int ny, int nz);
 size_t batched_smem(int type, int form, int nz, int percol, int kw);
 int batched_blocks_per_sm(size_t smem);
