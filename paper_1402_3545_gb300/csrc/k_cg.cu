@@ -9,6 +9,8 @@
 //   r <- r - alpha_j q ; z <- M^{-1} r ; <r, r> ; <r, z>
 // One thread owns one vertical column; the sums are reduced per block and summed in a fixed order
 // by the finalize kernels (k_util.cu), which also compute alpha and beta on the device.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "sweep_x2.cuh"
 
@@ -488,10 +490,12 @@ __global__ void k_cg_finish(size_t n, const Scalars* __restrict__ sc, typename P
 template <class P>
 static dim3 spmv_march_grid(const Lv<P>& L, int& pz) {
     dim3 g((L.nx / 2 + 31) / 32, (L.ny + SPMV_TY - 1) / SPMV_TY);
-    // one partial sum per block: as many slabs of planes as max_partials leaves room for
-    const int room = max_partials(L.nx, L.ny) / (int)(g.x * g.y);
-    int nzs = (L.nz + SPMV_PZ - 1) / SPMV_PZ;
-    if (nzs > room) nzs = room < 1 ? 1 : room;
+    // SPMV_PZ planes per block, fewer where the blocks would not give every SM two (with 16 everywhere FP32 32 x 42 x 66
+    // took 11.3 us, with the two scalar kernels of a call; 8.8 with a thread per pair of cells); one partial sum per block: as
+    // many slabs of planes as max_partials leaves room for
+    const int cols = (int)(g.x * g.y), room = max_partials(L.nx, L.ny) / cols;
+    int nzs = std::max((L.nz + SPMV_PZ - 1) / SPMV_PZ, std::min(L.nz, (2 * 152 + cols - 1) / cols));
+    nzs = std::min(nzs, std::max(room, 1));
     pz = (L.nz + nzs - 1) / nzs;
     g.z = (L.nz + pz - 1) / pz;
     return g;
