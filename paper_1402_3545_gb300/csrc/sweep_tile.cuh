@@ -605,9 +605,18 @@ static int run_sweep_tile_rows(const Lv<P>& L, double coef, const typename P::S*
     }
 }
 
+// Where the fused Tridiag runs on tiles. Double-word: as the Smooth. FP32, whose two-column sweep is the faster one on
+// large levels (us, tile / sweep; with the call's scalar kernels): 128 x 64 x 16 12 / 13, 160^2 x 64 17 / 37; 256^2 x 32
+// 23 / 19, x 64 30 / 29, x 96 37 / 41; 512^2 x 32 55 / 40, x 96 102 / 104; 1024 x 512 x 16 82 / 37.
+template <class P>
+static bool cg_tile_pays(const Lv<P>& L) {
+    const size_t cols = (size_t)L.nx * L.ny;
+    if (P::id != 1) return tile_pays(L);
+    return L.nz >= 16 && (cols <= 32768 || (cols <= 65536 && L.nz > 64));
+}
 template <class P>
 int cg_tile_blocks(const Lv<P>& L) {
-    if (L.nz > 128 || !L.finv || !L.fw || !(tile_pays(L) || (P::id == 1 && L.nz >= 16))) return -1;
+    if (L.nz > 128 || !L.finv || !L.fw || !cg_tile_pays(L)) return -1;
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(L.v) || (L.fac_percol && (!al(L.finv) || !al(L.fw)))) return -1;
     const int tr = tile_rows<P>(L.nx, L.ny, false);

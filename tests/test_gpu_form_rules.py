@@ -1,0 +1,19 @@
+"""Each side of the rules that deal levels to kernel forms by size: both forms under the comparisons, and their
+tolerances, of the forms' own tests."""
+import pytest
+
+import test_gpu_tiles as tiles
+from paper_1402_3545_gb300 import tpmg
+
+pytestmark = pytest.mark.gpu
+
+
+def ids(s):
+    return "x".join(map(str, s))
+
+
+# FP32: tiles up to 32768 columns from 16 planes, up to 65536 beyond 64, the two-column sweep else
+@pytest.mark.parametrize("lam", [None, 1e3], ids=["varying", "constant"])
+@pytest.mark.parametrize("shape", [(256, 128, 16), (256, 132, 16), (256, 256, 64), (256, 256, 65), (512, 130, 65)], ids=ids)
+def test_fp32_tridiag(shape, lam):
+    tiles.test_tile_line_solve_and_tridiag_match_oracle(tpmg.F32, shape, lam)
