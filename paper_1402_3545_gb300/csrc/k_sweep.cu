@@ -614,6 +614,13 @@ int launch_apply_A_x2(const Lv<P>& L, const typename P::S* x, typename P::S* y, 
 template <class P>
 int launch_line_solve_pp(const Lv<P>& L, const typename P::S* b, typename P::S* x, double scale, const int* done,
                          cudaStream_t s) {
+    // FP32, lambda^2 varying: large levels of up to 64 planes on the four-column tile of a warp where it takes them
+    // (512^2 x 16 10.9 us / 11.9, x 48 26.6 / 30.9; x 96 52.8 / 50.9)
+    if constexpr (std::is_same<P, PolF32>::value)
+        if (L.gstack && L.fac_percol && L.nz <= 64 && (size_t)L.nx * L.ny > 131072) {
+            const int nb = launch_line_solve_x4(L, b, x, scale, done, s);
+            if (nb >= 0) return nb;
+        }
     if constexpr (tile_policy<P>())
         // (the line solve has no stencil to form: it gains wherever the Smooth does, in FP32 on all levels of
         // 16 planes and more: 1024^2 x 128 166 us / 349, 128^2 x 128 10 / 60, 512^2 x 128 varying 77 / 77)
