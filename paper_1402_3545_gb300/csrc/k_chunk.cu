@@ -15,6 +15,8 @@
 // carried value's own rounding enters damped by the products, all below 1.
 // Measured per Smooth inside a graph: 64^2 x 128 16 us (cyclic reduction 30), 128^2 x 128 49 us (thread per
 // column 72), 64^2 x 64 10 us (17); 300 x 150 x 60 with the norm 119 us, 185 with a thread per column.
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace tpmg {
@@ -320,23 +322,30 @@ template int launch_restrict_smooth_chunk<PolF64>(const Lv<PolF64>&, double, con
 template int launch_restrict_smooth_chunk<PolDW>(const Lv<PolF64>&, double, const float2*, double*, double*, const int*,
                                                  cudaStream_t);
 
-// planes per thread of the residual: at most 16 blocks per 128 columns, or 1024, on small levels (room for one
-// partial sum per 8 columns, and for 1216, max_partials), 4 on larger ones, where the columns alone fill the GPU
-static int residual_planes(int nx, int ny, int nz) {
+// Planes per thread of the residual. Small levels: one where that gives at most 1024 blocks (a thread that takes four
+// planes waits for memory four times: FP64 32^2 x 32 3.5 us, 2.6 with one), up to four where that does; with the norm at
+// most 256 where four planes allow it (the sum over the blocks is one block's work: FP64 64^2 x 29 8.9 us with 928
+// blocks, 7.7 with 256). Else as many as leave 16 blocks per 128 columns (room for one partial sum per 8 columns,
+// max_partials), and above CHUNK_MAX_COLS columns, where the columns alone fill the GPU, 4.
+static int residual_planes(int nx, int ny, int nz, bool norm) {
     if ((size_t)nx * ny > (size_t)CHUNK_MAX_COLS) return (nz + 3) / 4;
-    const int four = (nx * ny + 127) / 128 * ((nz + 3) / 4);  // blocks of four planes per thread
-    return four > 1024 ? (nz + 15) / 16 : 4;
+    const int cb = (nx * ny + 127) / 128;
+    auto slabs = [&](int p) { return (nz + p - 1) / p; };
+    int p = 1;
+    while (p < 4 && cb * slabs(p) > (norm ? 256 : 1024)) ++p;
+    if (cb * slabs(p) > 1024) p = std::max(4, (nz + 15) / 16);
+    return slabs(slabs(p));  // in equal parts
 }
 
 template <class P>
 int residual_point_blocks(const Lv<P>& L) {
-    const int pz = residual_planes(L.nx, L.ny, L.nz);
+    const int pz = residual_planes(L.nx, L.ny, L.nz, true);
     return (L.nx * L.ny + 127) / 128 * ((L.nz + pz - 1) / pz);
 }
 template <class P, class PO>
 int launch_residual_point(const Lv<P>& L, const typename P::S* u, const typename P::S* f, typename PO::S* r,
                           double* partials, const int* done, cudaStream_t s) {
-    const int pz = residual_planes(L.nx, L.ny, L.nz);
+    const int pz = residual_planes(L.nx, L.ny, L.nz, partials != nullptr);
     const dim3 g((L.nx * L.ny + 127) / 128, (L.nz + pz - 1) / pz);
     k_residual_point<P, PO><<<g, 128, 0, s>>>(L, sweep_k<P>(L.cx, L.cy, 1.0), u, f, r, partials, done, pz);
     note_launch();

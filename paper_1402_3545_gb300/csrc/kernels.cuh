@@ -357,7 +357,7 @@ int launch_line_solve_chunk(const Lv<PolF64>& L, const double* b, double* x, dou
 template <class PF>
 int launch_restrict_smooth_chunk(const Lv<PolF64>& Lc, double rho, const typename PF::S* rf, double* fc, double* uc,
                                  const int* done, cudaStream_t s);
-// Residual, pointwise, any level and policy; the number of its blocks (= partial sums)
+// Residual, pointwise, any level and policy; the number of its blocks with the norm (= partial sums)
 template <class P>
 int residual_point_blocks(const Lv<P>& L);
 template <class P, class PO>

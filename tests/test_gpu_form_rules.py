@@ -1,8 +1,10 @@
 """Each side of the rules that deal levels to kernel forms by size: both forms under the comparisons, and their
 tolerances, of the forms' own tests."""
 import pytest
+import torch
 
 import test_gpu_tiles as tiles
+from gpu_common import PREC_IDS, PRECS
 from paper_1402_3545_gb300 import tpmg
 
 pytestmark = pytest.mark.gpu
@@ -23,3 +25,19 @@ def test_fp32_tridiag(shape, lam):
 @pytest.mark.parametrize("shape", [(512, 256, 17), (512, 260, 17), (512, 260, 64), (512, 260, 65)], ids=ids)
 def test_fp32_line_solve(shape):
     tiles.test_tile_line_solve_and_tridiag_match_oracle(tpmg.F32, shape, None)
+
+
+# the pointwise Residual's planes per thread: one to four on small levels, fewer blocks with the norm, sixteenths beyond
+@pytest.mark.parametrize("shape", [(8, 8, 256), (34, 20, 8), (64, 64, 29), (64, 64, 256), (128, 128, 13), (192, 126, 29),
+                                   (192, 126, 67), (370, 330, 7)], ids=ids)
+@pytest.mark.parametrize("prec", PRECS, ids=PREC_IDS)
+def test_residual_planes(prec, shape):
+    tiles.test_pointwise_residual_matches_oracle(prec, shape)
+    nx, ny, nz = shape
+    op = tiles.operator(nx, ny, nz, None, nlevels=1)
+    u, f = tiles.fields((nz, ny, nx), prec, 3)
+    r, norm = [torch.empty_like(u) for _ in range(2)], torch.zeros(1, dtype=torch.float64, device="cuda")
+    tpmg.residual(op.op, 1, prec, u, f, r[0], u.numel())
+    tpmg.residual(op.op, 1, prec, u, f, r[1], u.numel(), norm_out=norm)
+    assert torch.equal(*r)
+    op.close()
