@@ -449,12 +449,13 @@ int launch_residual_restrict(const Lv<P>& L, const Lv<P>& Lc, double rho, const 
     if ((Lc.pcr || Lc.chunkw) && (size_t)Lc.nx * Lc.ny <= (size_t)PCR_MAX_COLS && Lc.nz <= 256) return -1;
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     if (!al(u) || !al(f)) return -1;
-    // whole-column tiles (us, tile / marching): FP32 everywhere (1024 x 512 x 64 83 / 134, 512^2 x 128 83-87 /
-    // 126-132, 256^2 x 128 17-19 / 62); double-word, whose arithmetic rather than the chain bounds large levels,
+    // whole-column tiles (us, tile / marching): FP32 (1024 x 512 x 64 83 / 134, 512^2 x 128 83-87 / 126-132, 256^2 x
+    // 128 17-19 / 62) but for large levels of few planes, which leave its eight warps without work (512^2 x 1 6.2 / 3.8,
+    // x 3 6.5-6.9 / 5.6, x 6 7.6-7.9 / 8.4; 896 x 732 x 2 12-13 / 8.8; 256^2 x 1 2.5 / 2.8); double-word, whose arithmetic rather than the chain bounds large levels,
     // where the marching form leaves the GPU idle (with conversions: 256 x 72 x 128 83 / 131, 256^2 x 128
     // 233-239 / 256-264, 384 x 256 347 / 351, but 512^2 x 128 854 / 834 and 384 x 256 x 8 38 / 36)
     if constexpr (tile_policy<P>())
-        if (P::id == 1 || (L.nx * L.ny <= 98304 && L.nz >= 16)) {
+        if (P::id == 1 ? L.nz >= 6 || L.nx * L.ny <= 131072 : L.nx * L.ny <= 98304 && L.nz >= 16) {
             const int nb = launch_restrict_tile<P>(L, Lc, rho, u, f, fc, uc, done, s);
             if (nb >= 0) return nb;
         }

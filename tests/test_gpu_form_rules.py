@@ -41,3 +41,10 @@ def test_residual_planes(prec, shape):
     tpmg.residual(op.op, 1, prec, u, f, r[1], u.numel(), norm_out=norm)
     assert torch.equal(*r)
     op.close()
+
+
+# FP32 Residual + RestrictSmooth: tiles from 6 planes, or up to 131072 fine columns; the marching form else
+@pytest.mark.parametrize("lam", [None, 1e3], ids=["varying", "constant"])
+@pytest.mark.parametrize("shape", [(512, 256, 5), (512, 258, 5), (512, 258, 6), (512, 258, 1)], ids=ids)
+def test_fp32_residual_restriction(shape, lam):
+    tiles.test_restrict_tile_equals_the_two_kernels(tpmg.F32, shape, True, lam)
