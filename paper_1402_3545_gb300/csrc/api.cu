@@ -2520,7 +2520,7 @@ extern "C" tpmg_status tpmg_create_panel_operator(const tpmg_grid* g, double ome
         }
         for (int t = 0; t < 3; ++t)
             if ((st = dalloc((void**)&op->pfac[l][t], lvl_cells(op, l) * sizeof(double))) != TPMG_OK) return fail(st);
-        if (panel_chunked(nx, ny))
+        if (panel_chunked(nx, ny, nz))
             for (int t = 0; t < 2; ++t)
                 if ((st = dalloc((void**)&op->pchunk[l][t], (size_t)nx * ny * ((nz + panel_chunk_planes(nz) - 1) / panel_chunk_planes(nz)) *
                                                                 sizeof(double))) != TPMG_OK)

@@ -38,8 +38,15 @@ enum { PANEL_SMOOTH = 0, PANEL_RESIDUAL = 1, PANEL_LINESOLVE = 2, PANEL_APPLY = 
 // planes per chunk of a column in the chunked sweeps: up to 16 chunks of 4, 8 or 16 planes
 inline int panel_chunk_planes(int nz) { return nz <= 64 ? 4 : (nz <= 128 ? 8 : 16); }
 // Levels that sweep their columns in chunks: where a thread per column leaves the GPU waiting on its
-// recurrences (128^2 x 128 Smooth 193 us with one thread per column at a floor of 36)
-inline bool panel_chunked(int nx, int ny) { return (size_t)nx * ny <= (size_t)CHUNK_MAX_COLS; }
+// recurrences (128^2 x 128 Smooth 193 us with one thread per column at a floor of 36), and not on few planes, where
+// the chunks' barriers and second passes outweigh that. Smooth / with the norm, time in chunks over the other form's:
+// 72^2 x 4 0.85 / 1.05, x 6 0.71 / 0.95; 128^2 x 8 0.87 / 1.17, x 10 0.76 / 1.02; 152^2 x 10 0.78 / 1.15, x 12 0.66 / 1.01;
+// 180^2 x 12 0.92 / 1.36, x 24 0.87 / 1.33, x 32 0.68 / 1.03, x 64 0.73 / 0.97.
+inline bool panel_chunked(int nx, int ny, int nz) {
+    const size_t cols = (size_t)nx * ny;
+    if (cols > (size_t)CHUNK_MAX_COLS) return false;
+    return nz >= (cols <= 10240 ? 6 : (cols <= 16384 ? 10 : (cols <= 24576 ? 12 : 32)));
+}
 // wf, wb: the chunk products, or null
 void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw, double* wf, double* wb, cudaStream_t s);
 // mode PANEL_*: Smooth (coef = rho) and Residual write partial sums of ||f - A u||^2 when partials is
