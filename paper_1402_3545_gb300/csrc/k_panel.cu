@@ -86,8 +86,9 @@ __device__ __forceinline__ T panel_Au(const PanelLvT<T>& L, const PCol<T>& q, co
     return fma(-tc, up, s);
 }
 
-// f - A u at one cell in FP64, nine operations: the vertical and the |T| part of the diagonal share one
-// product with |T|
+// f - A u (APPLY: A u) at one cell in FP64, nine operations: the vertical and the |T| part of the diagonal share
+// one product with |T|
+template <bool APPLY = false>
 __device__ __forceinline__ double panel_res(const PanelLv& L, const PCol<double>& q, const double* __restrict__ x, size_t b,
                                             int k, double fk, double uc, double um, double up) {
     const double xw = q.hw ? __ldg(x + b + q.c - 1) : 0.0;
@@ -95,6 +96,7 @@ __device__ __forceinline__ double panel_res(const PanelLv& L, const PCol<double>
     const double xs = q.hs ? __ldg(x + b + q.c - L.nx) : 0.0;
     const double xn = q.hn ? __ldg(x + b + q.c + L.nx) : 0.0;
     const double v = fma(-__ldg(L.C + k), up, fma(-__ldg(L.B + k), um, __ldg(L.E + k) * uc));
+    if (APPLY) return fma(q.area, v, fma(q.an, xn, fma(q.as, xs, fma(q.ae, xe, fma(q.aw, xw, -q.at * uc)))));
     double r = fma(q.at, uc, fk);
     r = fma(-q.aw, xw, r);
     r = fma(-q.ae, xe, r);
@@ -354,8 +356,8 @@ __global__ void __launch_bounds__(128) k_panel_point(PanelLv L, const double* __
 #pragma unroll 4
         for (int k = k0; k < k1; ++k, b += pl) {
             const double up = k + 1 < nz ? __ldg(u + b + pl + q.c) : 0.0;
-            const double r = panel_res(L, q, u, b, k, MODE == 3 ? 0.0 : __ldg(f + b + q.c), uc, um, up);
-            out[b + q.c] = (TO)(MODE == 3 ? -r : r);
+            const double r = panel_res<MODE == 3>(L, q, u, b, k, MODE == 3 ? 0.0 : __ldg(f + b + q.c), uc, um, up);
+            out[b + q.c] = (TO)r;
             if (MODE == 1 && partials) acc = fma(r, r, acc);
             um = uc;
             uc = up;
@@ -411,7 +413,7 @@ __global__ void __launch_bounds__(128) k_panel_prolongate(int nxc, int nyc, int 
     const size_t plc = (size_t)nxc * nyc, c0 = (size_t)J * nxc + I, cx = (size_t)J * nxc + I2,
                  fo = (size_t)(2 * J) * nxf + i;
     const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
-#pragma unroll 2
+#pragma unroll 4
     for (int k = k0; k < k1; ++k) {
         const T* p = uc + (size_t)k * plc;
         T* o = uf + (size_t)k * 4 * plc + fo;
@@ -523,8 +525,15 @@ void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw,
     note_launch();
 }
 
-// planes per block of the pointwise kernels: 16 where the level fills the GPU with them, else 4
-static int point_planes(int nx, int ny) { return (size_t)nx * ny > 65536 ? 16 : 4; }
+// planes per block of the pointwise kernels with `blocks` blocks a plane: 16 where the level fills the GPU with them,
+// else 4, in equal parts; one or two where that gives at most 1024 blocks (a thread that takes four planes waits for memory
+// four times: 64^2 x 3 prolongation 3.2 us, 2.6 with one)
+static int point_planes(int nx, int ny, int nz, int blocks) {
+    for (int p = 1; p <= 2; ++p)
+        if (blocks * ((nz + p - 1) / p) <= 1024) return p;
+    const int p = (size_t)nx * ny > 65536 ? 16 : 4, slabs = (nz + p - 1) / p;
+    return (nz + slabs - 1) / slabs;
+}
 
 // The chunked sweep where the level has its chunk products (PanelLvT::wf). Returns the number of blocks, or
 // -1 where it does not apply.
@@ -562,10 +571,15 @@ template <int MODE, class TO>
 static int panel_point(const PanelLv& L, const double* u, const double* f, TO* out, double* partials, const int* done,
                        cudaStream_t s) {
     dim3 g = panel_grid(L.nx, L.ny);
-    int pz = point_planes(L.nx, L.ny);
-    if (partials) {  // as many slabs of planes as max_partials leaves room for
-        const int room = max_partials(L.nx, L.ny) / (int)(g.x * g.y);
-        pz = std::max(pz, room > 1 ? (L.nz + room - 1) / room : L.nz);
+    int pz = point_planes(L.nx, L.ny, L.nz, (int)(g.x * g.y));
+    if (partials) {
+        // as many slabs of planes as max_partials leaves room for, of four planes or more, and below the size that takes 16 at
+        // most 1024 blocks (one block adds the sums up: 138 x 446 x 36 62 us with 5040 of them, 58 with 560)
+        const int blocks = (int)(g.x * g.y), least = std::max(pz, 4);
+        int slabs = std::min((L.nz + least - 1) / least, max_partials(L.nx, L.ny) / blocks);
+        if ((size_t)L.nx * L.ny <= 65536) slabs = std::min(slabs, 1024 / blocks);
+        slabs = std::max(slabs, 1);
+        pz = (L.nz + slabs - 1) / slabs;
     }
     g.z = (L.nz + pz - 1) / pz;
     k_panel_point<MODE, TO><<<g, dim3(32, 4), 0, s>>>(L, u, f, out, partials, done, pz);
@@ -615,7 +629,7 @@ void launch_panel_restrict_smooth(const PanelLvT<T>& Lc, double rho, const T* rf
 template <class T>
 void launch_panel_prolongate(int nxc, int nyc, int nz, const T* uc, T* uf, const int* done, cudaStream_t s) {
     dim3 g = panel_grid(2 * nxc, nyc);
-    const int pz = point_planes(2 * nxc, 2 * nyc);
+    const int pz = point_planes(2 * nxc, 2 * nyc, nz, (int)(g.x * g.y));
     g.z = (nz + pz - 1) / pz;
     k_panel_prolongate<T><<<g, dim3(32, 4), 0, s>>>(nxc, nyc, nz, uc, uf, done, pz);
     note_launch();
