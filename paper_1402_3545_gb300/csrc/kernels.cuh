@@ -151,8 +151,10 @@ static constexpr int CHUNK_MAX_COLS = 32768;
 // and without the norm (Smooth without it, us; chunks / the other form):
 //  - cyclic reduction (k_coarse.cu) on small levels of few planes, where the chunks' three barriers outweigh its
 //    operations: 32^2 x 8 5.5 / 3.6, x 32 6.0 / 5.4, x 48 6.4 / 6.8; 64^2 x 8 5.7 / 4.0, x 12 5.9 / 5.9, x 20 6.5 / 7.3;
-//    up to 512 columns a warp scans the chunks: 16^2 x 8 4.5 / 3.6, x 12 4.3 / 4.8; and on the smallest of many
-//    planes, where a level is one wave of either: 8^2 x 160 9.6 / 6.7, 16^2 x 128 6.7 / 6.0;
+//    up to 512 columns a warp scans the chunks: 16^2 x 8 4.5 / 3.6, x 12 4.3 / 4.8; just above, a block takes four columns:
+//    24^2 x 48 6.0 / 5.4, 32 x 24 x 40 6.0 / 5.5, x 48 5.8 / 6.3; and on levels that are one wave of either where their
+//    chunks are longer, beyond 64 planes (RestrictSmooth included): 8^2 x 160 9.6 / 6.7, 20^2 x 72 6.4 / 5.7, x 160 10.0 / 8.3;
+//    24^2 x 96 7.4 / 6.6, x 256 11.1 / 12.5; 32 x 24 x 72 7.2 / 6.7, x 128 7.5 / 8.1;
 //  - the sweep (a thread per column) where the columns alone fill the GPU. With tiles: 96^2 x 8 7.4 / 6.3, x 16
 //    7.3 / 10.4; 128^2 x 24 15.8 / 15.3, x 32 16.0 / 19.7; 192 x 160 x 64 49 / 47. Without (nx % 32 != 0, a slower
 //    sweep): 150^2 x 4 12 / 8; 182 x 178 x 20 29 / 37 but 47 / 41 with the norm, x 32 30 / 48; 450 x 330 x 20
@@ -163,8 +165,9 @@ inline int f64_columns(int nx, int ny, int nz) {
     const size_t cols = (size_t)nx * ny;
     if (nz > 256) return F64_SWEEP;
     if (cols <= (size_t)PCR_MAX_COLS) {
-        const int few = cols <= 512 ? 8 : (cols <= 2048 ? 32 : 12);
-        return nz <= few || (cols <= 256 && nz > 64) ? F64_PCR : F64_CHUNK;
+        const int few = cols <= 512 ? 8 : (cols <= 640 ? 64 : (cols <= 768 ? 40 : (cols <= 2048 ? 32 : 12)));
+        const int many = cols <= 512 ? 256 : (cols <= 640 ? 200 : (cols <= 768 ? 96 : 0));  // from 65 planes to this many
+        return nz <= few || (nz > 64 && nz <= many) ? F64_PCR : F64_CHUNK;
     }
     const bool small = cols <= (size_t)CHUNK_MAX_COLS / 2;
     if (nx % 32 == 0) return small && (nz > 24 || (nz > 8 && cols <= 10240)) ? F64_CHUNK : F64_SWEEP;

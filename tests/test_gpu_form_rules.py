@@ -48,3 +48,10 @@ def test_residual_planes(prec, shape):
 @pytest.mark.parametrize("shape", [(512, 256, 5), (512, 258, 5), (512, 258, 6), (512, 258, 1)], ids=ids)
 def test_fp32_residual_restriction(shape, lam):
     tiles.test_restrict_tile_equals_the_two_kernels(tpmg.F32, shape, True, lam)
+
+
+# native FP64 levels between cyclic reduction and chunks of planes: up to 512, 640 and 768 columns
+@pytest.mark.parametrize("shape", [(20, 20, 65), (16, 32, 256), (24, 24, 64), (24, 24, 65), (24, 24, 200), (24, 24, 201),
+                                   (32, 24, 40), (32, 24, 41), (32, 24, 96), (32, 24, 97)], ids=ids)
+def test_fp64_columns(shape):
+    tiles.test_chunked_columns_match_oracle(shape)
