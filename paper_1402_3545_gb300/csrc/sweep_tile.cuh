@@ -116,6 +116,9 @@ __device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
 // partial sums of <r, r> and, behind them, of <r, z>: with M = U^T D U the elimination gives yh = U^{-T} r
 // and d' = D^{-1} yh, so <r, M^{-1} r> = sum_k yh_k d'_k, and the back substitution does not read r again.
 constexpr int MODE_CGTRI = 16;
+// u's element type: only MODE_CGTRI writes it
+template <class P, int MODE>
+using TileU = std::conditional_t<MODE == MODE_CGTRI, typename P::S, const typename P::S>;
 
 // One tile: columns bx * W .., rows by * TR ...
 // kw: planes whose factors are kept per column in shared memory behind the nz planes of the tile (0
@@ -123,7 +126,7 @@ constexpr int MODE_CGTRI = 16;
 // nparts (both compile-time: as runtime choices their instructions were issued either way). RO: the fields read
 // are not written by the kernel
 template <class P, int MODE, int TR, bool ISO, bool NORM, bool RO>
-__device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>& K, const typename P::S* u,
+__device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>& K, TileU<P, MODE>* u,
                                                 const typename P::S* f, typename P::S* out, double* partials, int kw,
                                                 const Scalars* sc, int bx, int by, int part, int nparts,
                                                 unsigned char* smem_raw) {
@@ -260,7 +263,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
     if constexpr (CG) {
         const R nalpha = P::neg(P::cst(sc->alpha));
         const S* pq = f + (size_t)klo * pl + c;
-        S* pr = const_cast<S*>(u) + (size_t)klo * pl + c;
+        S* pr = u + (size_t)klo * pl + c;
         S* z = Z + klo * NC + zo;
         bool landed = false;
 #pragma unroll 4
@@ -560,7 +563,7 @@ __device__ __forceinline__ void sweep_tile_body(const Lv<P>& L, const SweepK<P>&
 
 template <class P, int MODE, int TR, bool ISO, bool NORM>
 __global__ void __launch_bounds__(TNT, 3)
-    k_sweep_tile(Lv<P> L, SweepK<P> K, const typename P::S* __restrict__ u, const typename P::S* __restrict__ f,
+    k_sweep_tile(Lv<P> L, SweepK<P> K, TileU<P, MODE>* __restrict__ u, const typename P::S* __restrict__ f,
                  typename P::S* __restrict__ out, double* partials, const int* done, int kw, const Scalars* sc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (done && *(volatile const int*)done) return;
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(TNT, 3)
 }
 
 template <class P, int MODE, int TR, bool ISO, bool NORM>
-static int run_sweep_tile(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
+static int run_sweep_tile(const Lv<P>& L, double coef, TileU<P, MODE>* u, const typename P::S* f,
                           typename P::S* out, double* partials, const int* done, cudaStream_t s, const Scalars* sc) {
     typedef typename P::S S;
     int kw = 0;
@@ -592,7 +595,7 @@ static int tile_rows(int nx, int ny, bool two) {
     return nx % (W / 4) == 0 && ny % 4 == 0 && ny / 4 <= MAXR ? 4 : 0;
 }
 template <class P, int MODE, bool ISO, bool NORM>
-static int run_sweep_tile_rows(const Lv<P>& L, double coef, const typename P::S* u, const typename P::S* f,
+static int run_sweep_tile_rows(const Lv<P>& L, double coef, TileU<P, MODE>* u, const typename P::S* f,
                                typename P::S* out, double* partials, const int* done, cudaStream_t s,
                                const Scalars* sc = nullptr) {
     // FP32 Smooth: two rows of 64 columns share their inner rows and so load two rows of u per row instead of
