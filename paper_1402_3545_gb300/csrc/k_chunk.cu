@@ -359,7 +359,6 @@ TPMG_POINT_INST(PolF32, PolF32)
 TPMG_POINT_INST(PolF32B, PolF32B)
 TPMG_POINT_INST(PolDW, PolDW)
 TPMG_POINT_INST(PolDW, PolF32)
-TPMG_POINT_INST(PolF64, PolF32)
 template int residual_point_blocks<PolF64>(const Lv<PolF64>&);
 template int residual_point_blocks<PolF32>(const Lv<PolF32>&);
 template int residual_point_blocks<PolF32B>(const Lv<PolF32B>&);

@@ -499,9 +499,10 @@ int launch_prolongate_x4(int nxc, int nyc, int nz, const typename P::S* uc, type
                                       const int*, cudaStream_t);                                             \
     template int launch_line_solve_pcr<P>(const Lv<P>&, const P::S*, P::S*, double, const int*, cudaStream_t); \
     template int launch_restrict_smooth_pcr<P, P>(const Lv<P>&, double, const P::S*, P::S*, P::S*, const int*, \
-                                                  cudaStream_t);                                             \
-    template int launch_residual_cell<P, P>(const Lv<P>&, const P::S*, const P::S*, P::S*, double*, const int*, \
-                                            cudaStream_t);
+                                                  cudaStream_t);
+#define TPMG_CELL_INST(P, PO) /* (native FP64's small levels are pointwise, k_chunk.cu) */                   \
+    template int launch_residual_cell<P, PO>(const Lv<P>&, const P::S*, const P::S*, PO::S*, double*, const int*, \
+                                             cudaStream_t);
 #define TPMG_PROL_INST(P)                                                                                   \
     template int launch_prolongate_cell<P, P>(int, int, int, const P::S*, P::S*, const int*, cudaStream_t);     \
     template int launch_prolongate_x4<P, P>(int, int, int, const P::S*, P::S*, const int*, cudaStream_t);
@@ -514,6 +515,10 @@ TPMG_PCR_INST(PolF64)
 TPMG_PCR_INST(PolF32)
 TPMG_PCR_INST(PolDW)
 TPMG_PCR_INST(PolF32B)
+TPMG_CELL_INST(PolF32, PolF32)
+TPMG_CELL_INST(PolDW, PolDW)
+TPMG_CELL_INST(PolF32B, PolF32B)
+TPMG_CELL_INST(PolDW, PolF32)
 template int launch_restrict_smooth_pcr<PolF32, PolF32B>(const Lv<PolF32B>&, double, const float*, float*, float*,
                                                          const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
@@ -522,9 +527,5 @@ template int launch_restrict_smooth_pcr<PolDW, PolF64>(const Lv<PolF64>&, double
                                                        const int*, cudaStream_t);
 template int launch_prolongate_cell<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
 template int launch_prolongate_x4<PolF64, PolDW>(int, int, int, const double*, float2*, const int*, cudaStream_t);
-template int launch_residual_cell<PolDW, PolF32>(const Lv<PolDW>&, const float2*, const float2*, float*, double*,
-                                                 const int*, cudaStream_t);
-template int launch_residual_cell<PolF64, PolF32>(const Lv<PolF64>&, const double*, const double*, float*, double*,
-                                                  const int*, cudaStream_t);
 
 }  // namespace tpmg

@@ -422,7 +422,7 @@ int launch_smooth(const Lv<P>& L, double rho, const typename P::S* u, const type
 template <class P, class PO>
 static bool residual_pointwise(const Lv<P>& L, const typename P::S* u, const typename P::S* f, const typename PO::S* r) {
     const size_t cols = (size_t)L.nx * L.ny;
-    if (P::id == 0 && PO::id == 0) return cols <= (size_t)CHUNK_MAX_COLS || (L.nx % 32 != 0 && cols <= 4 * (size_t)CHUNK_MAX_COLS);
+    if (P::id == 0) return cols <= (size_t)CHUNK_MAX_COLS || (L.nx % 32 != 0 && cols <= 4 * (size_t)CHUNK_MAX_COLS);
     return cols > (size_t)PCR_MAX_COLS && cols <= (size_t)CHUNK_MAX_COLS && L.nx % 32 == 0 && (L.ny % 4 == 0 || (L.nx % 64 == 0 && L.ny % 2 == 0));
 }
 template <class P, class PO>
@@ -439,7 +439,7 @@ int launch_residual(const Lv<P>& L, const typename P::S* u, const typename P::S*
                     typename PO::S* r, double* partials, const int* done, cudaStream_t s) {
     if (residual_pointwise<P, PO>(L, u, f, r)) return launch_residual_point<P, PO>(L, u, f, r, partials, done, s);
     int nb;
-    if constexpr (P::id != 0 || PO::id != 0) {  // (native FP64's small levels are pointwise above)
+    if constexpr (P::id != 0) {  // (native FP64's small levels are pointwise above)
         nb = launch_residual_cell<P, PO>(L, u, f, r, partials, done, s);
         if (nb >= 0) return nb;
     }
@@ -505,8 +505,6 @@ template void launch_restrict_smooth<PolF32, PolF32B>(const Lv<PolF32B>&, double
 template void launch_prolongate<PolF32B, PolF32>(int, int, int, const float*, float*, const int*, cudaStream_t);
 template int launch_residual<PolDW, PolF32>(const Lv<PolDW>&, const float2*, const float2*, float*,
                                              double*, const int*, cudaStream_t);
-template int launch_residual<PolF64, PolF32>(const Lv<PolF64>&, const double*, const double*,
-                                              float*, double*, const int*, cudaStream_t);
 template void launch_correct<PolDW>(size_t, float2*, const float*, const int*, cudaStream_t);
 template void launch_restrict_smooth<PolDW, PolF64>(const Lv<PolF64>&, double, const float2*, double*, double*,
                                                     const int*, cudaStream_t);

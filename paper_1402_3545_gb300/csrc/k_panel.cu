@@ -151,15 +151,13 @@ __global__ void __launch_bounds__(128) k_panel_factors(PanelLv L, double* __rest
 }
 
 // MODE 0 Smooth: out = u + coef M^{-1} (f - A u) (Eq. (11)), partial sums of ||f - A u||^2
-// MODE 1 Residual: out = f - A u (stored in TO: the FP64 outer residual of the mixed solve is stored
-//        in FP32), partial sums of ||f - A u||^2
+// MODE 1 Residual (FP32; FP64: k_panel_point): out = f - A u
 // MODE 2 line solve: out = coef M^{-1} u (u is the right-hand side)
-// MODE 3 apply: out = A u
 // T is the arithmetic (double or float); the norm's partial sums are accumulated in T.
 // NORM (FP64 Smooth): with the sums; without them the Smooth takes the form that needs no residual.
-template <int MODE, class T, class TO, bool NORM>
+template <int MODE, class T, bool NORM>
 __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, const T* __restrict__ u,
-                                                     const T* __restrict__ f, TO* out, double* partials,
+                                                     const T* __restrict__ f, T* out, double* partials,
                                                      const int* done) {
     if (done && *(volatile const int*)done) return;
     const PCol<T> q = panel_col(L);
@@ -183,40 +181,34 @@ __global__ void __launch_bounds__(128) k_panel_sweep(PanelLvT<T> L, T coef, cons
             T r;
             if (MODE != 2) {
                 const T up = (k + 1 < nz) ? __ldg(u + b + pl + q.c) : T(0);
-                if constexpr (sizeof(T) == 8) {
-                    r = panel_res(L, q, u, b, k, MODE == 3 ? 0.0 : __ldg(f + b + q.c), uc, um, up);
-                    if (MODE == 3) r = -r;
-                } else {
-                    const T au = panel_Au(L, q, u, b, k, uc, um, up, tb, tc);
-                    r = (MODE == 3) ? au : __ldg(f + b + q.c) - au;
-                }
+                const T fk = __ldg(f + b + q.c);
+                if constexpr (sizeof(T) == 8) r = panel_res(L, q, u, b, k, fk, uc, um, up);
+                else r = fk - panel_Au(L, q, u, b, k, uc, um, up, tb, tc);
                 um = uc;
                 uc = up;
             } else {
                 r = __ldg(u + b + q.c);
             }
-            if (MODE == 0 || MODE == 1) {
-                if (partials) acc = fma(r, r, acc);
-            }
-            if (MODE == 0 || MODE == 2) {
+            if (MODE != 2 && partials) acc = fma(r, r, acc);
+            if (MODE != 1) {
                 dp = fma(__ldg(L.fl + b + q.c), dp, r * __ldg(L.inv + b + q.c));  // forward elimination
                 out[b + q.c] = dp;  // the output field holds d'_k until the back substitution
             } else {
-                out[b + q.c] = (TO)r;
+                out[b + q.c] = r;
             }
             tb = tc;
         }
-        if (MODE == 0 || MODE == 2) {
+        if (MODE != 1) {
             T x = 0;
             for (int k = nz - 1; k >= 0; --k) {
                 const size_t id = (size_t)k * pl + q.c;
-                x = fma(__ldg(L.fw + id), x, (T)out[id]);
+                x = fma(__ldg(L.fw + id), x, out[id]);
                 if constexpr (RHS) out[id] = fma(coef, x, (1.0 - coef) * __ldg(u + id));
                 else out[id] = (MODE == 0) ? fma(coef, x, __ldg(u + id)) : coef * x;
             }
         }
     }
-    if ((MODE == 0 || MODE == 1) && partials) {
+    if (MODE != 2 && partials) {
         const double s = block_sum((double)acc);
         if (threadIdx.x == 0 && threadIdx.y == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
@@ -599,15 +591,10 @@ int launch_panel_sweep(int mode, const PanelLvT<T>& L, double coef, const T* u, 
                                             : panel_chunk<2>(L, coef, u, f, out, nullptr, nullptr, done, s);
         if (nb >= 0) return nb;
     }
-    switch (mode) {
-        case PANEL_SMOOTH:
-            if (partials) k_panel_sweep<0, T, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done);
-            else k_panel_sweep<0, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done);
-            break;
-        case PANEL_RESIDUAL: k_panel_sweep<1, T, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done); break;
-        case PANEL_LINESOLVE: k_panel_sweep<2, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
-        default: k_panel_sweep<3, T, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done); break;
-    }
+    if (mode == PANEL_LINESOLVE) k_panel_sweep<2, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done);
+    else if (mode == PANEL_SMOOTH && partials) k_panel_sweep<0, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done);
+    else if (mode == PANEL_SMOOTH) k_panel_sweep<0, T, false><<<g, b, 0, s>>>(L, c, u, f, out, nullptr, done);
+    else if constexpr (sizeof(T) == 4) k_panel_sweep<1, T, true><<<g, b, 0, s>>>(L, c, u, f, out, partials, done);
     note_launch();
     return (int)(g.x * g.y);
 }

@@ -805,8 +805,6 @@ TPMG_SWEEP_INST(PolDW)
 TPMG_SWEEP_INST(PolF32B)
 template int launch_restrict_smooth_pp<PolF32, PolF32B>(const Lv<PolF32B>&, double, const float*, float*, float*,
                                                         const int*, cudaStream_t);
-template int launch_residual_pp<PolF64, PolF32>(const Lv<PolF64>&, const double*, const double*, float*, double*,
-                                                const int*, cudaStream_t);
 template int launch_residual_pp<PolDW, PolF32>(const Lv<PolDW>&, const float2*, const float2*, float*, double*,
                                                const int*, cudaStream_t);
 template int launch_restrict_smooth_pp<PolDW, PolF64>(const Lv<PolF64>&, double, const float2*, double*, double*,
