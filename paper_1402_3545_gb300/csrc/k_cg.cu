@@ -124,30 +124,46 @@ __device__ __forceinline__ float lane_dn(float x) { return __shfl_down_sync(0xff
 __device__ __forceinline__ dw lane_up(dw x) { return dw{lane_up(x.hi), lane_up(x.lo)}; }
 __device__ __forceinline__ dw lane_dn(dw x) { return dw{lane_dn(x.hi), lane_dn(x.lo)}; }
 
-template <class P, bool ALIGNED>
+// FOLD: the block's w < 32 pairs of SPMV_TY rows lie behind one another in its threads, a warp holds the end of one
+// row and the start of the next; else w = 32, a row per warp
+template <class P, bool ALIGNED, bool FOLD>
 __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<P> K, const Scalars* __restrict__ sc,
                                                                 typename P::S* __restrict__ u,
                                                                 typename P::S* __restrict__ p,
                                                                 const typename P::S* __restrict__ z,
-                                                                typename P::S* __restrict__ q, double* partials, int pz) {
+                                                                typename P::S* __restrict__ q, double* partials, int pz,
+                                                                int w) {
     typedef typename P::R R;
     typedef CgPair<P, ALIGNED> V;
     if (*(volatile const int*)&sc->done) return;
-    const int nx = L.nx, ny = L.ny, nz = L.nz, lane = threadIdx.x;
-    const int i = 2 * (blockIdx.x * 32 + lane), j = blockIdx.y * SPMV_TY + threadIdx.y;
+    const int nx = L.nx, ny = L.ny, nz = L.nz, lane = threadIdx.x & 31;
+    if (!FOLD) w = 32;
+    const int jt = FOLD ? threadIdx.x / w : threadIdx.x >> 5, it = threadIdx.x - jt * w;
+    const int i = 2 * (blockIdx.x * w + it), j = blockIdx.y * SPMV_TY + jt;
     const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
     const size_t pl = (size_t)nx * ny;
     const R alpha = P::cst(sc->alpha), beta = P::cst(sc->beta);
     typename P::Acc acc = 0, cmp = 0;
-    if (j < ny) {  // (a whole warp: one row)
-        const bool act = i < nx;
-        const int ii = act ? i : nx - 2;  // lanes beyond the row repeat its last pair and store nothing
-        const size_t row = (size_t)j * nx, c = row + ii, b0 = (size_t)k0 * pl;
-        const size_t rs = (size_t)wrapc(j - 1, ny) * nx + ii, rn = (size_t)wrapc(j + 1, ny) * nx + ii;
-        // the columns beyond the warp's ends or the row's: every lane loads both (one sector each)
-        const bool lw = lane == 0, le = lane == 31 || i + 2 >= nx;
-        const int iw = i - 2 * lane;
-        const size_t cw = row + wrapc(iw - 1, nx), ce = row + (iw + 64 < nx ? iw + 64 : 0);
+    if (FOLD || j < ny) {  // (else a whole warp: one row)
+        const bool act = i < nx && (!FOLD || (jt < SPMV_TY && j < ny));
+        const int ii = i < nx ? i : nx - 2, jj = j < ny ? j : ny - 1;  // lanes beyond the grid repeat its last pair and store nothing
+        const size_t row = (size_t)jj * nx, c = row + ii, b0 = (size_t)k0 * pl;
+        const size_t rs = (size_t)wrapc(jj - 1, ny) * nx + ii, rn = (size_t)wrapc(jj + 1, ny) * nx + ii;
+        // the columns beyond the ends of the warp, the block's rows and the grid's: every lane loads one on either side,
+        // those that need none the warp's first or last lane's (one sector a row)
+        const bool lw = lane == 0 || (FOLD && it == 0), le = lane == 31 || ii + 2 >= nx || (FOLD && it == w - 1);
+        size_t cw, ce;
+        if (FOLD) {
+            cw = row + wrapc(ii - 1, nx);
+            ce = row + (ii + 2 < nx ? ii + 2 : 0);
+            const size_t first = __shfl_sync(0xffffffffu, cw, 0), last = __shfl_sync(0xffffffffu, ce, 31);
+            if (!lw) cw = first;
+            if (!le) ce = last;
+        } else {
+            const int iw = i - 2 * lane;
+            cw = row + wrapc(iw - 1, nx);
+            ce = row + (iw + 64 < nx ? iw + 64 : 0);
+        }
         const R v0 = P::ld(L.v, c), v1 = P::ld(L.v, c + 1);
         const R d1a = P::add(K.dh, v0), d1b = P::add(K.dh, v1), d2a = P::add(d1a, v0), d2b = P::add(d1b, v1);
         const bool iso = K.iso != 0;
@@ -194,8 +210,7 @@ __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<
         }
     }
     const double s = block_sum(P::acc_get(acc, cmp));
-    if (threadIdx.x == 0 && threadIdx.y == 0)
-        partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+    if (threadIdx.x == 0) partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
 }
 
 template <class P>
@@ -488,13 +503,19 @@ __global__ void k_cg_finish(size_t n, const Scalars* __restrict__ sc, typename P
 
 // the marching SpMV for the FP32-pipe policies (native FP64 keeps the column kernel, bound by its pipe)
 template <class P>
-static dim3 spmv_march_grid(const Lv<P>& L, int& pz) {
-    dim3 g((L.nx / 2 + 31) / 32, (L.ny + SPMV_TY - 1) / SPMV_TY);
-    // SPMV_PZ planes per block, fewer where the blocks would not give every SM two (with 16 everywhere FP32 32 x 42 x 66
-    // took 11.3 us, with the two scalar kernels of a call; 8.8 with a thread per pair of cells); one partial sum per block: as
-    // many slabs of planes as max_partials leaves room for
+static dim3 spmv_march_grid(const Lv<P>& L, int& pz, int& w) {
+    // a row's pairs to its warps; folded, in equal parts, where that leaves a quarter of the lanes or more without a pair
+    // (FP32 78 x 628 x 203 107 us, 70 folded; 34 x 700 x 16 15.5, 9.7)
+    const int pairs = L.nx / 2, parts = (pairs + 31) / 32;
+    w = 4 * pairs > 3 * 32 * parts ? 32 : (pairs + parts - 1) / parts;
+    dim3 g(parts, (L.ny + SPMV_TY - 1) / SPMV_TY);
+    // SPMV_PZ planes per block, fewer where that leaves a quarter of the SMs without one (with 16 everywhere FP32 32 x 42 x 66
+    // took 11.3 us, with the two scalar kernels of a call; 8.8 with a thread per pair of cells; where the SMs are full, more
+    // and shorter slabs cost: double-word 128^2 x 128 80 us with ten, 73 with eight); one partial sum per block: as many
+    // slabs of planes as max_partials leaves room for
     const int cols = (int)(g.x * g.y), room = max_partials(L.nx, L.ny) / cols;
-    int nzs = std::max((L.nz + SPMV_PZ - 1) / SPMV_PZ, std::min(L.nz, (2 * 152 + cols - 1) / cols));
+    int nzs = (L.nz + SPMV_PZ - 1) / SPMV_PZ;
+    if (cols * nzs < 114) nzs = std::max(nzs, std::min(L.nz, (152 + cols - 1) / cols));
     nzs = std::min(nzs, std::max(room, 1));
     pz = (L.nz + nzs - 1) / nzs;
     g.z = (L.nz + pz - 1) / pz;
@@ -503,8 +524,8 @@ static dim3 spmv_march_grid(const Lv<P>& L, int& pz) {
 template <class P>
 int cg_spmv_blocks(const Lv<P>& L) {
     if (L.nx % 2 == 0 && P::id != 0) {
-        int pz;
-        const dim3 g = spmv_march_grid(L, pz);
+        int pz, w;
+        const dim3 g = spmv_march_grid(L, pz, w);
         return (int)(g.x * g.y * g.z);
     }
     return sweep_shape(L.nx, L.ny, L.nz, sizeof(typename P::R), false).nblocks();
@@ -514,12 +535,15 @@ int launch_cg_spmv(const Lv<P>& L, const Scalars* sc, typename P::S* u, typename
                    const typename P::S* z, typename P::S* q, double* partials, cudaStream_t s) {
     if constexpr (P::id != 0)
         if (L.nx % 2 == 0) {
-            int pz;
-            const dim3 g = spmv_march_grid(L, pz), b(32, SPMV_TY);
+            int pz, w;
+            const dim3 g = spmv_march_grid(L, pz, w);
             const SweepK<P> K = sweep_k<P>(L.cx, L.cy, 1.0);
             const bool al = (((uintptr_t)u | (uintptr_t)p | (uintptr_t)z | (uintptr_t)q) & (2 * sizeof(typename P::S) - 1)) == 0;
-            if (al) k_cg_spmv_march<P, true><<<g, b, 0, s>>>(L, K, sc, u, p, z, q, partials, pz);
-            else k_cg_spmv_march<P, false><<<g, b, 0, s>>>(L, K, sc, u, p, z, q, partials, pz);
+            auto run = [&](auto kern) {
+                kern<<<g, (w * SPMV_TY + 31) / 32 * 32, 0, s>>>(L, K, sc, u, p, z, q, partials, pz, w);
+            };
+            if (w == 32) al ? run(k_cg_spmv_march<P, true, false>) : run(k_cg_spmv_march<P, false, false>);
+            else al ? run(k_cg_spmv_march<P, true, true>) : run(k_cg_spmv_march<P, false, true>);
             note_launch();
             return (int)(g.x * g.y * g.z);
         }
