@@ -552,6 +552,9 @@ template <int MODE>
 static int panel_chunk(const PanelLv& L, double coef, const double* u, const double* f, double* out, double* fc,
                        double* partials, const int* done, cudaStream_t s) {
     if (!L.wf || !L.wb) return -1;
+    // with the norm (14 operations a cell) the largest levels are bound by the FP64 pipe but where their planes fill the rows of
+    // chunks: 180^2 x 40 62 us in chunks / 53, 128 x 254 x 169 344 / 276, 180^2 x 96 128 / 152
+    if (MODE == 0 && partials && (size_t)L.nx * L.ny > 28672 && (L.nz < 64 || L.nz > 128)) return -1;
     switch (panel_chunk_planes(L.nz)) {
         case 4: return run_panel_chunk<MODE, 4>(L, coef, u, f, out, fc, partials, done, s);
         case 8: return run_panel_chunk<MODE, 8>(L, coef, u, f, out, fc, partials, done, s);
