@@ -11,8 +11,8 @@
 // Rounding: the tensor cores cut an accumulator's low bits off instead of rounding them, an error that does not
 // average out: same-signed sums lose about half a unit in the last place per MMA (2.6e-5 of the sum in 430 of
 // them). So no accumulator lives long: the thin layers add each MMA's 16 cells to FP32 sums by ordinary
-// additions, the 16 -> 16 layers pass theirs on every D16_FLUSH planes, and biases are ordinary additions, FP32 over 32
-// planes and FP64 from there.
+// additions, the 16 -> 16 layers pass theirs on every D16_FLUSH planes, and biases are ordinary additions,
+// FP32 over 32 planes or a tile's and FP64 from there.
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
@@ -254,8 +254,7 @@ __global__ void __launch_bounds__(D16_NT) k_dw16_march(const __nv_bfloat16* __re
 // 3-plane ring; the thin operand from a 4-plane ring of channel-separated rows, kept twice, once
 // shifted by a cell, so that a lane's pair of cells is one aligned word for every x-shift. Bias
 // gradients: the sum of the A fragments (first layer), or of d4 as it is loaded (last layer).
-// Measured on 256^2 x 64: 65 us (first, cin = 2) and 87 us (last).
-constexpr int THIN_FLUSH = 32;
+// Measured on 256^2 x 64: 65 us (first, cin = 2) and 83 us (last).
 template <int CIN, bool LAST>
 struct ThinShape {
     static constexpr int NCH = LAST ? 3 : CIN;            // thin rows stored per plane row
@@ -281,11 +280,9 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
     const int q8 = lane >> 3, rr = lane & 7, g = lane >> 2, t = lane & 3;
     __shared__ double redb[8][16];
     float acc[SH::NTL][4];
-    // biases: of channels lane / 4 and 8 + lane / 4, or (LAST) of this thread's cells; FP32 sums of up to THIN_FLUSH
-    // planes
+    // biases: of channels lane / 4 and 8 + lane / 4, or (LAST) of this thread's cells; FP32 sums of a tile's planes
     float f0 = 0.f, f1 = 0.f;
     double b0 = 0.0, b1 = 0.0;
-    int since = 0;
     int off[SH::NTL], ddz[SH::NTL];  // word offset within a thin plane, plane offset 0..2, of the lane's columns
 #pragma unroll
     for (int j = 0; j < SH::NTL; ++j) {
@@ -416,17 +413,12 @@ __global__ void __launch_bounds__(256) k_dw_thin(const __nv_bfloat16* __restrict
                 f1 += p1;
             }
             if (z + 1 < ze) store(z + 2);
-            if (++since == THIN_FLUSH) {
-                b0 += f0;
-                b1 += f1;
-                f0 = f1 = 0.f;
-                since = 0;
-            }
         }
         gwait<0>();
+        b0 += f0;  // (not in the loop over the planes, where the compiler adds at every one of them: 23 % of the FP64 pipe)
+        b1 += f1;
+        f0 = f1 = 0.f;
     }
-    b0 += f0;
-    b1 += f1;
     for (int h = 1; h < (LAST ? 32 : 4); h <<= 1) {
         b0 += __shfl_xor_sync(0xffffffffu, b0, h);
         if (!LAST) b1 += __shfl_xor_sync(0xffffffffu, b1, h);
