@@ -136,22 +136,21 @@ __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<
     typedef typename P::R R;
     typedef CgPair<P, ALIGNED> V;
     if (*(volatile const int*)&sc->done) return;
-    const int nx = L.nx, ny = L.ny, nz = L.nz, lane = threadIdx.x & 31;
-    if (!FOLD) w = 32;
-    const int jt = FOLD ? threadIdx.x / w : threadIdx.x >> 5, it = threadIdx.x - jt * w;
-    const int i = 2 * (blockIdx.x * w + it), j = blockIdx.y * SPMV_TY + jt;
+    const int nx = L.nx, ny = L.ny, nz = L.nz, lane = FOLD ? threadIdx.x & 31 : threadIdx.x;
+    const int jt = FOLD ? threadIdx.x / w : threadIdx.y, it = FOLD ? threadIdx.x - jt * w : lane;
+    const int i = 2 * (blockIdx.x * (FOLD ? w : 32) + it), j = blockIdx.y * SPMV_TY + jt;
     const int k0 = blockIdx.z * pz, k1 = k0 + pz < nz ? k0 + pz : nz;
     const size_t pl = (size_t)nx * ny;
     const R alpha = P::cst(sc->alpha), beta = P::cst(sc->beta);
     typename P::Acc acc = 0, cmp = 0;
     if (FOLD || j < ny) {  // (else a whole warp: one row)
         const bool act = i < nx && (!FOLD || (jt < SPMV_TY && j < ny));
-        const int ii = i < nx ? i : nx - 2, jj = j < ny ? j : ny - 1;  // lanes beyond the grid repeat its last pair and store nothing
+        const int ii = i < nx ? i : nx - 2, jj = !FOLD || j < ny ? j : ny - 1;  // lanes beyond repeat the last pair, store nothing
         const size_t row = (size_t)jj * nx, c = row + ii, b0 = (size_t)k0 * pl;
         const size_t rs = (size_t)wrapc(jj - 1, ny) * nx + ii, rn = (size_t)wrapc(jj + 1, ny) * nx + ii;
         // the columns beyond the ends of the warp, the block's rows and the grid's: every lane loads one on either side,
         // those that need none the warp's first or last lane's (one sector a row)
-        const bool lw = lane == 0 || (FOLD && it == 0), le = lane == 31 || ii + 2 >= nx || (FOLD && it == w - 1);
+        const bool lw = lane == 0 || (FOLD && it == 0), le = lane == 31 || i + 2 >= nx || (FOLD && it == w - 1);
         size_t cw, ce;
         if (FOLD) {
             cw = row + wrapc(ii - 1, nx);
@@ -210,7 +209,8 @@ __global__ void __launch_bounds__(32 * SPMV_TY) k_cg_spmv_march(Lv<P> L, SweepK<
         }
     }
     const double s = block_sum(P::acc_get(acc, cmp));
-    if (threadIdx.x == 0) partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+    if (threadIdx.x == 0 && threadIdx.y == 0)
+        partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
 }
 
 template <class P>
@@ -540,7 +540,8 @@ int launch_cg_spmv(const Lv<P>& L, const Scalars* sc, typename P::S* u, typename
             const SweepK<P> K = sweep_k<P>(L.cx, L.cy, 1.0);
             const bool al = (((uintptr_t)u | (uintptr_t)p | (uintptr_t)z | (uintptr_t)q) & (2 * sizeof(typename P::S) - 1)) == 0;
             auto run = [&](auto kern) {
-                kern<<<g, (w * SPMV_TY + 31) / 32 * 32, 0, s>>>(L, K, sc, u, p, z, q, partials, pz, w);
+                const dim3 b = w == 32 ? dim3(32, SPMV_TY) : dim3((w * SPMV_TY + 31) / 32 * 32);
+                kern<<<g, b, 0, s>>>(L, K, sc, u, p, z, q, partials, pz, w);
             };
             if (w == 32) al ? run(k_cg_spmv_march<P, true, false>) : run(k_cg_spmv_march<P, false, false>);
             else al ? run(k_cg_spmv_march<P, true, true>) : run(k_cg_spmv_march<P, false, true>);
