@@ -1444,13 +1444,14 @@ tpmg_status tpmg_autotune(tpmg_op* op, tpmg_precision prec, int reps, int* varia
         for (int v = 0; v < TPMG_NUM_VARIANTS; ++v) {
             if (v >= 8 && pid != 1) continue;  // the four-column tiles are FP32 only
             op->variant[pid][l] = v;
+            // as the cycles run it: without the norm (in native FP64 another kernel), on the finest level one in four with it
             auto run = [&](auto tag) {
                 typedef decltype(tag) P;
                 typedef typename P::S S;
                 Hier& h = op->hier[pid];
-                // without the norm, as all but one Smooth of a cycle run (in native FP64 another kernel)
-                launch_smooth<P>(level_view<P>(op, l), 0.8, (const S*)h.u[l], (const S*)h.f[l], (S*)h.ub[l], nullptr,
-                                 nullptr, s);
+                for (int t = 0; t < (l == op->g.L ? 4 : 1); ++t)
+                    launch_smooth<P>(level_view<P>(op, l), 0.8, (const S*)h.u[l], (const S*)h.f[l], (S*)h.ub[l],
+                                     t == 3 ? op->partials : nullptr, nullptr, s);
             };
             auto once = [&]() {
                 if (pid == 0) run(PolF64());
