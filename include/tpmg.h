@@ -99,7 +99,8 @@ tpmg_status tpmg_grid_level_size(const tpmg_grid* g, int level, int* nx, int* ny
 tpmg_status tpmg_create_operator(const tpmg_grid* g, double omega2, double hx, double hy, double hz,
                                  double lambda2, const double* lambda2_col, tpmg_op** out);
 tpmg_status tpmg_destroy_operator(tpmg_op* op);
-/* Allocates now the workspace a solver in precision `prec` needs (see the conventions above). */
+/* Allocates now the workspace that the multigrid and CG solvers and tpmg_vcycle in precision `prec` need
+ * (TPMG_DW: with that of the coarse levels it runs in native FP64); see the conventions above. */
 tpmg_status tpmg_op_reserve(tpmg_op* op, tpmg_precision prec);
 /* Discrete coefficients of `level`: cx, cy and the HOST copy of v (ny_l*nx_l values), any NULL. */
 tpmg_status tpmg_op_level_coefficients(const tpmg_op* op, int level, double* cx, double* cy,
@@ -117,7 +118,10 @@ tpmg_status tpmg_apply_A(tpmg_op* op, int level, tpmg_precision prec, const void
 tpmg_status tpmg_line_solve(tpmg_op* op, int level, tpmg_precision prec, const void* b, void* x,
                             void* stream);
 /* u_out = u + rho M^{-1}(f - A u): one block-Jacobi smoothing step, Eq. (11)
- * "MultigridSmoother". If norm_out (a DEVICE double) is not NULL it receives ||f - A u||_2. */
+ * "MultigridSmoother". If norm_out (a DEVICE double) is not NULL it receives ||f - A u||_2. Native FP64
+ * (TPMG_F64, and TPMG_DW on levels that run in it) then forms the residual; without norm_out it forms the
+ * same step as (1 - rho) u + rho M^{-1}(f + H u), H the horizontal couplings, which rounds differently in
+ * the last bits. */
 tpmg_status tpmg_smooth(tpmg_op* op, int level, tpmg_precision prec, double rho, const void* u,
                         const void* f, void* u_out, double* norm_out, void* stream);
 /* r = f - A u (kernel "Residual", Sec. 3.1); optional ||r||_2 into the DEVICE double norm_out. */
@@ -142,8 +146,9 @@ tpmg_status tpmg_residual_restrict_smooth(tpmg_op* op, int level, tpmg_precision
                                           const void* u_fine, const void* f_fine, void* f_c, void* u_c,
                                           void* stream);
 /* enable != 0 (the default): V-cycles of this operator fuse Residual and RestrictSmooth wherever
- * tpmg_residual_restrict_smooth's fused kernel applies (in tpmg_mg_solve_batched: wherever the
- * fine level takes its two-column tiles); 0: separate kernels. Same results bit for bit either way.
+ * tpmg_residual_restrict_smooth's fused kernel applies (in tpmg_mg_solve_batched: where the fine
+ * level's nx is a multiple of 128 and ny of 4 and, with varying lambda^2, the coarse factors fit its
+ * tile); 0: separate kernels. Same results bit for bit either way.
  * Invalidates the operator's cached CUDA graphs and batched-solve tables. */
 tpmg_status tpmg_set_fusion(tpmg_op* op, int enable);
 /* u_f += P u_c on fine level `level` (> 1), P the cell-centred bilinear interpolation from level-1
@@ -273,14 +278,17 @@ tpmg_status tpmg_measure_alu_rate(int which, int reps, double* ops_per_s, double
  * of values, or of 256 bytes with even ny, or of 128 bytes with ny a multiple of 4). A level that was
  * never tuned or set takes variant 0 in those precisions where lambda^2 is constant or the level is
  * small; otherwise, in FP32, variant 8 where the level fits one tile per resident warp (nx % 128 == 0),
- * else 5; double-word takes 6 where nx % 64 == 0; otherwise (and in native FP64) variant 3. Variants
- * 8-11 in other precisions run the default.
- * tpmg_autotune times each of them `reps` times on every level of precision `prec` (on the
- * operator's workspace, CUDA events on `stream`) and keeps the fastest per level; if variants_out
+ * else 5; double-word takes 6 where nx % 64 == 0; otherwise variant 3, in native FP64 too. Variants
+ * 8-11 in other precisions run the default. A level that does not sweep its columns has one form and no
+ * variants: at most 4096 columns, in native FP64 also levels of up to 16384 columns (any number where
+ * nx % 32 != 0) whose columns run in chunks of planes.
+ * tpmg_autotune times each of them `reps` times on every level of precision `prec`, without the norm (on
+ * the finest level one Smooth in four with it, as in a V(2,2) cycle), on the operator's workspace by
+ * CUDA events on `stream`, and keeps the fastest per level; if variants_out
  * is not NULL it receives the choice of level l in variants_out[l] (host array of L+1 ints).
- * tpmg_set_variant sets one level's choice (e.g. from a saved tuning table). Both invalidate the
- * operator's cached CUDA graphs. Variants change the schedule, not the per-cell arithmetic (only the
- * grouping of the residual norm's partial sums differs). */
+ * tpmg_set_variant sets one level's choice (e.g. from a saved tuning table; a table is only as good as the
+ * library it was measured with). Both invalidate the operator's cached CUDA graphs. Variants change the
+ * schedule, not the per-cell arithmetic (only the grouping of the residual norm's partial sums differs). */
 #define TPMG_NUM_VARIANTS 12
 tpmg_status tpmg_autotune(tpmg_op* op, tpmg_precision prec, int reps, int* variants_out, void* stream);
 tpmg_status tpmg_set_variant(tpmg_op* op, tpmg_precision prec, int level, int variant);

@@ -66,9 +66,9 @@ __global__ void __launch_bounds__(256) k_cg_spmv(Lv<P> L, const Scalars* __restr
 
 // The fused SpMV with two x-adjacent columns per thread and SPMV_PZ planes per block: the vertical neighbours
 // stay in registers, the x neighbours come from the adjacent lanes, and a plane's six 16-byte loads (DW; 8 bytes
-// in FP32) are in flight together. Bound by DRAM (seven fields); 512^2 x 128 double-word 372 us, 390 with
-// a thread per pair of cells, whose 64-bit divisions for the cell's indices and five stencil loads it does
-// without. Requires nx even; ALIGNED: pair-aligned fields.
+// in FP32) are in flight together. 512^2 x 128 double-word 372 us (seven fields, 277 at the copy rate): DRAM 0.61 busy with
+// a quarter of the warps (114 registers); 390 with a thread per pair of cells, whose 64-bit divisions for the
+// cell's indices and five stencil loads it does without. Requires nx even; ALIGNED: pair-aligned fields.
 constexpr int SPMV_PZ = 16, SPMV_TY = 8;
 template <class P, bool ALIGNED>
 struct CgPair {

@@ -14,7 +14,7 @@
 // The forward-error bound is that of the Thomas algorithm: the second pass is its recurrence, and the
 // carried value's own rounding enters damped by the products, all below 1.
 // Measured per Smooth inside a graph: 64^2 x 128 16 us (cyclic reduction 30), 128^2 x 128 49 us (thread per
-// column 72), 64^2 x 64 10 us (17); 300 x 150 x 60 with the norm 119 us, 185 with a thread per column.
+// column 72), 64^2 x 64 10 us (17); 300 x 150 x 60 with the norm 116 us, 185 with a thread per column.
 #include <algorithm>
 
 #include "kernels.cuh"

@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(256) k_prolongate(int nxc, int nyc, int nz,
 
 // ---------------------------------------------------------------- u += e (FP32 correction)
 // Bound by memory. VEC: four values a thread, their loads before the stores (16-byte aligned fields): a thread that
-// adds one value at a time has only its own 12 bytes in flight. 1024^2 x 128 double-word 403 us, 444 before.
+// adds one value at a time has only its own 12 bytes in flight. 1024^2 x 128 double-word 403 us, 444 that way.
 template <class P, bool VEC>
 __global__ void k_correct(size_t n, typename P::S* __restrict__ u, const float* __restrict__ e,
                           const int* done) {

@@ -79,7 +79,7 @@ __device__ __forceinline__ void share(long nsteps, long& s0, long& s1) {
 // the dx = 1 warps' dy fragments. Rings: 5 planes of dy (10 rows), 3 of x (66 cells a row). Every D16_FLUSH
 // planes (256 MMAs to an accumulator) and at the end the four 16-cell columns add their sums, in order, to the
 // block's in shared memory, [x-shift, dz, dy, half of ci][lane][4], 16 bytes a lane.
-// Measured on 256^2 x 64 (4.2 M cells, 58 GFLOP): 165 us.
+// Measured on 256^2 x 64 (4.2 M cells, 58 GFLOP): 165 us, the tensor pipe 0.59 busy with one block of 12 warps per SM.
 constexpr int D16_NT = 384, D16_DYP = (GY + 2) * GX * ROWB, D16_XP = GY * (GX + 2) * ROWB;
 constexpr int D16_RING = 5 * D16_DYP + 3 * D16_XP;
 constexpr int D16_OUT = 27 * 256 + 16;  // weights, then biases
@@ -472,10 +472,10 @@ __global__ void __launch_bounds__(256) k_reduce_parts(const float* __restrict__ 
 
 // ---------------------------------------------------------------- data gradient of the last layer
 // d3[ci](p) = mask(a3) * sum_d W4[ci][d] d4(p - d): the transposed 16 <- 1 convolution, FP32, taps in
-// ascending order. Bound by the FP32 pipe (432 multiply-adds per cell): a thread owns 2 x 2 cells (32
-// apart in x, so a warp's accesses stay contiguous; two rows share their d4 loads) and reads each
-// weight as part of a 16-byte vector for all four. 225 us before (one cell per thread, one weight
-// load per multiply-add), 137 us now on 256^2 x 64.
+// ascending order. 432 multiply-adds per cell: a thread owns 2 x 2 cells (32 apart in x, so a warp's accesses stay
+// contiguous; two rows share their d4 loads) and reads each weight as part of a 16-byte vector for all four. 136 us
+// on 256^2 x 64: the FP32 pipe 0.40 busy, the issue slots 0.63, with a quarter of the warps (116 registers) that wait
+// for d4; one cell per thread with a weight load per multiply-add takes 225 us.
 __global__ void __launch_bounds__(128) k_bwd_last(const float* __restrict__ d4, const __nv_bfloat16* __restrict__ W,
                                                   const __nv_bfloat16* __restrict__ a3, __nv_bfloat16* __restrict__ d3,
                                                   int nx, int ny, int nz) {

@@ -502,13 +502,15 @@ struct SmoothVariants<PolDW> {
 
 // Where an untuned level smooths on whole columns in shared memory, from both sides' times over 15
 // horizontal sizes, nz = 8 .. 128 and both kinds of lambda^2 (tile / best sweep with its stack in L2, us):
-//  - below 16 planes the sweeps have no chain to speak of: FP32 512^2 x 8 13.5 / 12.2;
-//  - lambda^2 constant: FP32 everywhere else (128^2 x 128 13 / 57, 256^2 35 / 63, 512^2 121 / 124, 1024^2
-//    419 / 480); double-word (with conversions) above 64 planes everywhere (512^2 x 128 919 / 958), below
-//    only on levels of up to 65536 columns (320 x 200 x 32 72 / 74, 512^2 x 32 255 / 249);
-//  - lambda^2 varying: the factors of the planes share the shared memory, two blocks per SM remain, and
-//    only levels too small to fill the GPU gain: FP32 256^2 x 128 42 / 46, 448 x 256 62 / 67, but 512 x 256
-//    76 / 71; double-word 128^2 x 128 90 / 96, 160^2 136 / 143, but 256^2 319 / 265.
+//  - below 16 planes the sweeps have no chain to speak of: FP32 512^2 x 8 11.9 / 9.9;
+//  - lambda^2 constant: FP32 everywhere else (128^2 x 128 9.0 / 48, 256^2 31 / 59, 512^2 110 / 122, 1024^2 397 / 530; few
+//    planes on large levels about even: 1024 x 512 x 16 37 / 37, 1024^2 x 16 74 / 69); double-word (with conversions)
+//    above 64 planes everywhere (512^2 x 128 476 / 544, x 64 245 / 277), below only on levels of up to 65536 columns
+//    (320 x 200 x 32 36 / 43; 512^2 x 32 136 / 142, x 16 77 / 76);
+//  - lambda^2 varying: the factors of the planes share the shared memory, two blocks per SM remain, and levels that fill
+//    the GPU gain nothing: FP32 256^2 x 128 37 / 53, 448 x 256 56 / 65, 512 x 256 68 / 69, 512^2 123 / 120 (but 1024 x 512
+//    224 / 264, which this line leaves to the sweep); double-word 128^2 x 128 52 / 76, 160^2 81 / 93, 256 x 128 109 / 105,
+//    256^2 198 / 157.
 template <class P>
 bool tile_pays(const Lv<P>& L) {
     const size_t cols = (size_t)L.nx * L.ny;

@@ -423,10 +423,10 @@ void launch_cg_finish(size_t n, const Scalars* sc, typename P::S* u, const typen
 // ---------------------------------------------------------------- batched persistent solver (k_batched.cu)
 // Many independent problems of different sizes advance through one mixed-precision iterative
 // refinement together, inside one cooperative persistent launch: the work of each step of the
-// cycle ("phase") is cut into tiles of 32 x BTY columns over all problems; a bounded grid barrier
+// cycle ("phase") is cut into tiles over all problems (batched_form); a bounded grid barrier
 // separates the phases. Per-problem state decides which problems are still active.
-// BT_RRS: Residual of level `level` and RestrictSmooth onto level-1 in one two-column sweep
-// (a = u, b = f of the fine level, out = f_c, out2 = u_c), where the fine level takes 64 x BTY tiles
+// BT_RRS: Residual of level `level` and RestrictSmooth onto level-1 in one tile (a = u, b = f of the fine
+// level, out = f_c, out2 = u_c)
 enum { BT_OUTRES = 0, BT_FINAL = 1, BT_LS0 = 2, BT_SMOOTH = 3, BT_RESID = 4, BT_RS = 5, BT_PROL = 6, BT_CORR = 7,
        BT_RRS = 8 };
 // forms of a task's tiles (k_batched.cu)

@@ -11,7 +11,8 @@
 // threads, one of which alone runs the coarse recurrence, plane by plane between two block barriers.
 // The per-cell arithmetic and its order are the same, so the results are the same bits.
 // Measured: FP32 1024 x 512 x 64 83 us (4.0 TB/s of algorithmic traffic; 134 plane-marching), 512^2 x 128 83
-// (132), 256^2 x 128 17 (62); bound by the issue and latency of the loads (six 16-byte loads per 16 cells).
+// (132), 256^2 x 128 17 (62); bound by the latency of the loads (six of 16 bytes per 16 cells; 119 registers leave a
+// fifth of the warps, DRAM 0.51 busy). Levels of few planes leave the warps without work (launch_residual_restrict).
 #pragma once
 #include <type_traits>
 

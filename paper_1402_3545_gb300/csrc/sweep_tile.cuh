@@ -15,7 +15,7 @@
 // Up to three blocks per SM overlap one another's phases. The plane-marching sweeps keep one plane's
 // loads, elimination and stack store of every column in one chain, and their Thomas stack in a
 // global scratch (8 or 16 bytes of L2 traffic per cell); here nothing but the fields moves.
-// Measured, FP32: Smooth 1024^2 x 128 395 us (528 marching; 4.1 TB/s of algorithmic traffic), 128^2 x 128 8.8 (76);
+// Measured, FP32: Smooth 1024^2 x 128 397 us (530 marching; 4.1 TB/s of algorithmic traffic), 128^2 x 128 9.0 (48);
 // line solve 165 (345; 6.5 TB/s). A Smooth tile of 128 planes takes 48 000 cycles among three: step 1 half, step 2
 // 16 %, step 3 14 %, step 4 20 %. No single rate is reached (DRAM 0.46, L2 0.32, shared-memory wavefronts 0.48):
 // with all loads but one taken out it still takes 276 us, so the phases' own work bounds it, not the traffic alone.
