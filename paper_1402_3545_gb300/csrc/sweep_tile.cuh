@@ -608,14 +608,16 @@ static int run_sweep_tile_rows(const Lv<P>& L, double coef, TileU<P, MODE>* u, c
     }
 }
 
-// Where the fused Tridiag runs on tiles. Double-word: as the Smooth. FP32, whose two-column sweep is the faster one on
-// large levels (us, tile / sweep; with the call's scalar kernels): 128 x 64 x 16 12 / 13, 160^2 x 64 17 / 37; 256^2 x 32
-// 23 / 19, x 64 30 / 29, x 96 37 / 41; 512^2 x 32 55 / 40, x 96 102 / 104; 1024 x 512 x 16 82 / 37.
+// Where the fused Tridiag runs on tiles. Double-word: as the Smooth. FP32: everywhere from 16 planes (against one column a
+// thread: 352^2 x 70 CG iteration 138 us, 237), but on large levels that take the two-column sweep, the faster one there
+// (us, tile / sweep; with the call's scalar kernels): 128 x 64 x 16 12 / 13, 160^2 x 64 17 / 37; 256^2 x 32 23 / 19, x 64
+// 30 / 29, x 96 37 / 41; 512^2 x 32 55 / 40, x 96 102 / 104; 1024 x 512 x 16 82 / 37.
 template <class P>
 static bool cg_tile_pays(const Lv<P>& L) {
     const size_t cols = (size_t)L.nx * L.ny;
     if (P::id != 1) return tile_pays(L);
-    return L.nz >= 16 && (cols <= 32768 || (cols <= 65536 && L.nz > 64));
+    const bool pairs = L.gstack && L.nx % 64 == 0 && L.ny % 2 == 0;
+    return L.nz >= 16 && (!pairs || cols <= 32768 || (cols <= 65536 && L.nz > 64));
 }
 template <class P>
 int cg_tile_blocks(const Lv<P>& L) {
