@@ -289,7 +289,7 @@ static tpmg_status ensure_factors(tpmg_op* op, int pid, int top = 0) {
         // small levels: factor products of the columns in chunks (native FP64), parallel-cyclic-reduction factors
         // of the cell-parallel kernels
         const size_t cols = (size_t)op->g.lnx[l] * op->g.lny[l];
-        const int f64 = f64_columns(op->g.lnx[l], op->g.lny[l], op->g.nz);
+        const int f64 = f64_columns(op->g.lnx[l], op->g.lny[l], op->g.nz, op->percol[l] != 0);
         if (pid == 0 && f64 == F64_CHUNK) {
             const Lv<PolF64> L = level_view<PolF64>(op, l);
             TRY(dalloc((void**)&op->chunkw[l], chunk_count(L) * eb));

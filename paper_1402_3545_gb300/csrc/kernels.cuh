@@ -154,19 +154,23 @@ static constexpr int CHUNK_MAX_COLS = 32768;
 //    up to 512 columns a warp scans the chunks: 16^2 x 8 4.5 / 3.6, x 12 4.3 / 4.8; just above, a block takes four columns:
 //    24^2 x 48 6.0 / 5.4, 32 x 24 x 40 6.0 / 5.5, x 48 5.8 / 6.3; and on levels that are one wave of either where their
 //    chunks are longer, beyond 64 planes (RestrictSmooth included): 8^2 x 160 9.6 / 6.7, 20^2 x 72 6.4 / 5.7, x 160 10.0 / 8.3;
-//    24^2 x 96 7.4 / 6.6, x 256 11.1 / 12.5; 32 x 24 x 72 7.2 / 6.7, x 128 7.5 / 8.1;
+//    24^2 x 96 7.4 / 6.6, x 256 11.1 / 12.5; 32 x 24 x 72 7.2 / 6.7, x 128 7.5 / 8.1; with lambda^2 varying, where cyclic
+//    reduction reads two factors per cell and step, to fewer planes (20^2 x 72 1.09 of its time, x 128 0.89; 24^2 x 96 1.13,
+//    x 160 0.94; 26 x 24 x 186 0.85);
 //  - the sweep (a thread per column) where the columns alone fill the GPU. With tiles: 96^2 x 8 7.4 / 6.3, x 16
 //    7.3 / 10.4; 128^2 x 24 15.8 / 15.3, x 32 16.0 / 19.7; 192 x 160 x 64 49 / 47. Without (nx % 32 != 0, a slower
 //    sweep): 150^2 x 4 12 / 8; 182 x 178 x 20 29 / 37 but 47 / 41 with the norm, x 32 30 / 48; 450 x 330 x 20
 //    121 / 125, x 32 125 / 207, x 64 229 / 552;
 //  - chunks of planes (k_chunk.cu) else.
 enum { F64_SWEEP = 0, F64_CHUNK = 1, F64_PCR = 2 };
-inline int f64_columns(int nx, int ny, int nz) {
+inline int f64_columns(int nx, int ny, int nz, bool percol) {
     const size_t cols = (size_t)nx * ny;
     if (nz > 256) return F64_SWEEP;
     if (cols <= (size_t)PCR_MAX_COLS) {
-        const int few = cols <= 512 ? 8 : (cols <= 640 ? 64 : (cols <= 768 ? 40 : (cols <= 2048 ? 32 : 12)));
-        const int many = cols <= 512 ? 256 : (cols <= 640 ? 200 : (cols <= 768 ? 96 : 0));  // from 65 planes to this many
+        const int few = cols <= 512 ? 8 : (cols <= 608 ? 64 : (cols <= 752 ? 48 : (cols <= 912 ? 40 : (cols <= 2048 ? 32 : 12))));
+        // from 65 planes to this many
+        const int many = percol ? (cols <= 256 ? 256 : (cols <= 512 ? 80 : (cols <= 608 ? 128 : (cols <= 912 ? 80 : 0))))
+                                : (cols <= 512 ? 256 : (cols <= 608 ? 200 : (cols <= 752 ? 160 : (cols <= 912 ? 96 : 0))));
         return nz <= few || (nz > 64 && nz <= many) ? F64_PCR : F64_CHUNK;
     }
     const bool small = cols <= (size_t)CHUNK_MAX_COLS / 2;

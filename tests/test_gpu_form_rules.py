@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import test_gpu_tiles as tiles
-from gpu_common import PREC_IDS, PRECS
+from gpu_common import PREC_IDS, PRECS, make_problem
 from paper_1402_3545_gb300 import tpmg
 
 pytestmark = pytest.mark.gpu
@@ -52,8 +52,12 @@ def test_fp32_residual_restriction(shape, lam):
     tiles.test_restrict_tile_equals_the_two_kernels(tpmg.F32, shape, True, lam)
 
 
-# native FP64 levels between cyclic reduction and chunks of planes: up to 512, 640 and 768 columns
-@pytest.mark.parametrize("shape", [(20, 20, 65), (16, 32, 256), (24, 24, 64), (24, 24, 65), (24, 24, 200), (24, 24, 201),
-                                   (32, 24, 40), (32, 24, 41), (32, 24, 96), (32, 24, 97)], ids=ids)
-def test_fp64_columns(shape):
+# native FP64 levels between cyclic reduction and chunks of planes: up to 512, 608, 752 and 912 columns
+@pytest.mark.parametrize("lam,shape", [(None, s) for s in ((20, 20, 80), (20, 20, 81), (24, 24, 64), (24, 24, 128), (24, 24, 129),
+                                                          (26, 24, 48), (26, 24, 49), (32, 24, 80), (32, 24, 81))] +
+                         [(1e3, s) for s in ((20, 20, 65), (16, 32, 256), (24, 24, 200), (24, 24, 201), (26, 24, 160), (26, 24, 161),
+                                             (32, 24, 40), (32, 24, 41), (32, 24, 96), (32, 24, 97))],
+                         ids=lambda v: ids(v) if isinstance(v, tuple) else ("varying" if v is None else "constant"))
+def test_fp64_columns(shape, lam, monkeypatch):
+    monkeypatch.setattr(tiles, "make_problem", lambda *size: make_problem(*size, lam=lam))
     tiles.test_chunked_columns_match_oracle(shape)
