@@ -260,25 +260,34 @@ __global__ void __launch_bounds__(256) k_residual_cell(Lv<P> L, const typename P
 }
 
 // ---------------------------------------------------------------- Prolongate (pointwise)
-// u_f += P u_c at fine cell (i, j, k): cell-centred bilinear weights 9/16, 3/16, 3/16, 1/16
-template <class P, class PF>
+// u_f += P u_c at fine cell (i, j, k): cell-centred bilinear weights 9/16, 3/16, 3/16, 1/16. PAIR: a thread takes the
+// fine rows 2 J and 2 J + 1, which share their x part: four operations per cell on the FP64 pipe instead of five
+template <class P, class PF, bool PAIR>
 __global__ void __launch_bounds__(256) k_prolongate_cell(int nxc, int nyc, int nz, const typename P::S* __restrict__ uc,
                                                          typename PF::S* __restrict__ uf, const int* done) {
     typedef typename P::R R;
     if (done && *(volatile const int*)done) return;
-    const int nxf = 2 * nxc, nyf = 2 * nyc;
-    const size_t plf = (size_t)nxf * nyf, plc = (size_t)nxc * nyc, n = plf * nz;
+    const int nxf = 2 * nxc, nr = PAIR ? nyc : 2 * nyc;
+    const size_t plc = (size_t)nxc * nyc, pl = (size_t)nxf * nr, n = pl * nz;
     const R w9 = P::cst(0.5625), w3 = P::cst(0.1875), w1 = P::cst(0.0625);
     for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < n; id += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(id % nxf), j = (int)((id / nxf) % nyf), k = (int)(id / plf);
-        const int I = i >> 1, J = j >> 1;
-        const int I2 = cwrap((i & 1) ? I + 1 : I - 1, nxc), J2 = cwrap((j & 1) ? J + 1 : J - 1, nyc);
-        const size_t bc = (size_t)k * plc;
-        R val = P::mul(w9, P::ld(uc, bc + (size_t)J * nxc + I));
-        val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J * nxc + I2)));
-        val = P::add(val, P::mul(w3, P::ld(uc, bc + (size_t)J2 * nxc + I)));
-        val = P::add(val, P::mul(w1, P::ld(uc, bc + (size_t)J2 * nxc + I2)));
-        PF::st(uf, id, PF::add(PF::ld_plain(uf, id), Conv<P, PF>::f(val)));
+        const int i = (int)(id % nxf), j = (int)((id / nxf) % nr) * (PAIR ? 2 : 1), k = (int)(id / pl);
+        const int I = i >> 1, J = j >> 1, I2 = cwrap((i & 1) ? I + 1 : I - 1, nxc);
+        const size_t bc = (size_t)k * plc, r = bc + (size_t)J * nxc, f = 4 * bc + (size_t)j * nxf + i;
+        const typename PF::R o0 = PF::ld_plain(uf, f), o1 = PF::ld_plain(uf, PAIR ? f + nxf : f);
+        R h = P::mul(w9, P::ld(uc, r + I));
+        h = P::add(h, P::mul(w3, P::ld(uc, r + I2)));
+        auto sum = [&](int J2) {  // with the y neighbour's row
+            const size_t q = bc + (size_t)cwrap(J2, nyc) * nxc;
+            const R v = P::add(h, P::mul(w3, P::ld(uc, q + I)));
+            return P::add(v, P::mul(w1, P::ld(uc, q + I2)));
+        };
+        const R v0 = sum((j & 1) ? J + 1 : J - 1);
+        if (PAIR) {
+            const R v1 = sum(J + 1);
+            PF::st(uf, f + nxf, PF::add(o1, Conv<P, PF>::f(v1)));
+        }
+        PF::st(uf, f, PF::add(o0, Conv<P, PF>::f(v0)));
     }
 }
 
@@ -469,8 +478,13 @@ template <class P, class PF>
 int launch_prolongate_cell(int nxc, int nyc, int nz, const typename P::S* uc, typename PF::S* uf, const int* done,
                            cudaStream_t s) {
     if ((size_t)nxc * nyc > (size_t)PCR_MAX_COLS / 4) return -1;  // fine level at most PCR_MAX_COLS columns
-    const int nb = cell_blocks((size_t)4 * nxc * nyc * nz);
-    k_prolongate_cell<P, PF><<<nb, 256, 0, s>>>(nxc, nyc, nz, uc, uf, done);
+    // pairs where they still give each SM its blocks (FP64 128 x 32 x 171 8.2 us, 9.6 cell by cell); below, where the loads'
+    // latency is all there is, cell by cell (32^2 x 8 2.3, 2.5 in pairs)
+    const size_t n = (size_t)4 * nxc * nyc * nz;
+    const bool pair = n > 131072;
+    const int nb = cell_blocks(pair ? n / 2 : n);
+    if (pair) k_prolongate_cell<P, PF, true><<<nb, 256, 0, s>>>(nxc, nyc, nz, uc, uf, done);
+    else k_prolongate_cell<P, PF, false><<<nb, 256, 0, s>>>(nxc, nyc, nz, uc, uf, done);
     note_launch();
     return nb;
 }

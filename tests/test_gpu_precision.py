@@ -77,7 +77,8 @@ def test_gradient_sums_of_one_sign_match_64_bit_sums(cin, shape):
 
 
 @pytest.mark.parametrize("what,shape,by", [("box", (130, 66, 3), 0), ("box", (130, 66, 3), 1), ("box", (32, 32, 8), 0),
-                                           ("panel", (66, 64, 5), 0)], ids=["vector", "any-alignment", "cells", "panel"])
+                                           ("box", (64, 62, 96), 0), ("panel", (66, 64, 5), 0)],
+                         ids=["vector", "any-alignment", "cells", "pairs-of-cells", "panel"])
 def test_prolongation_rounds_once_relative_to_the_fine_field(what, shape, by):
     """u_f + P u_c with a correction of a tenth of u_f, as in a V-cycle, in native FP64 against extended precision.
     The correctly rounded sum has the r.m.s. error e of one rounding; P u_c adds at most five of a tenth of its size:
