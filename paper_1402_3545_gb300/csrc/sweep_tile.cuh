@@ -611,13 +611,16 @@ static int run_sweep_tile_rows(const Lv<P>& L, double coef, TileU<P, MODE>* u, c
 // Where the fused Tridiag runs on tiles. Double-word: as the Smooth. FP32: everywhere from 16 planes (against one column a
 // thread: 352^2 x 70 CG iteration 138 us, 237), but on large levels that take the two-column sweep, the faster one there
 // (us, tile / sweep; with the call's scalar kernels): 128 x 64 x 16 12 / 13, 160^2 x 64 17 / 37; 256^2 x 32 23 / 19, x 64
-// 30 / 29, x 96 37 / 41; 512^2 x 32 55 / 40, x 96 102 / 104; 1024 x 512 x 16 82 / 37.
+// 30 / 29, x 96 37 / 41; 512^2 x 32 55 / 40, x 96 102 / 104; 1024 x 512 x 16 82 / 37. In between, as long as three blocks an
+// SM take the level in one wave, tiles from 24 planes: tile over sweep, 34816 to 58368 columns, 1.07-1.10 at 16 planes,
+// 0.91-1.00 at 24, 0.73-0.84 at 48.
 template <class P>
 static bool cg_tile_pays(const Lv<P>& L) {
     const size_t cols = (size_t)L.nx * L.ny;
     if (P::id != 1) return tile_pays(L);
     const bool pairs = L.gstack && L.nx % 64 == 0 && L.ny % 2 == 0;
-    return L.nz >= 16 && (!pairs || cols <= 32768 || (cols <= 65536 && L.nz > 64));
+    const int from = cols <= 32768 ? 16 : cols <= 3 * 152 * 128 ? 24 : 65;
+    return L.nz >= 16 && (!pairs || (cols <= 65536 && L.nz >= from));
 }
 template <class P>
 int cg_tile_blocks(const Lv<P>& L) {

@@ -14,11 +14,11 @@ def ids(s):
     return "x".join(map(str, s))
 
 
-# FP32: tiles from 16 planes; where there is the two-column sweep (nx a multiple of 64) up to 32768 columns, up to 65536
-# beyond 64 planes
+# FP32: tiles from 16 planes; where there is the two-column sweep (nx a multiple of 64) up to 32768 columns, up to 58368
+# from 24 planes and up to 65536 beyond 64
 @pytest.mark.parametrize("lam", [None, 1e3], ids=["varying", "constant"])
-@pytest.mark.parametrize("shape", [(256, 128, 16), (256, 132, 16), (256, 256, 64), (256, 256, 65), (512, 130, 65),
-                                   (352, 132, 17), (96, 704, 40), (352, 132, 15)], ids=ids)
+@pytest.mark.parametrize("shape", [(256, 128, 16), (256, 132, 16), (256, 132, 23), (256, 228, 24),
+                                   (256, 232, 24), (256, 256, 64), (256, 256, 65), (512, 130, 65), (352, 132, 17), (96, 704, 40), (352, 132, 15)], ids=ids)
 def test_fp32_tridiag(shape, lam):
     tiles.test_tile_line_solve_and_tridiag_match_oracle(tpmg.F32, shape, lam)
 
