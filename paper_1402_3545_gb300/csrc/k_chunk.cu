@@ -323,7 +323,7 @@ template int launch_restrict_smooth_chunk<PolDW>(const Lv<PolF64>&, double, cons
                                                  cudaStream_t);
 
 // Planes per thread of the residual. Small levels: one where that gives at most 1024 blocks (a thread that takes four
-// planes waits for memory four times: FP64 32^2 x 32 3.5 us, 2.6 with one), up to four where that does; with the norm at
+// planes waits for memory four times: FP64 32^2 x 32 3.5 us, 2.6 with one), two or four where that does; with the norm at
 // most 256 where four planes allow it (the sum over the blocks is one block's work: FP64 64^2 x 29 8.9 us with 928
 // blocks, 7.7 with 256). Else as many as leave 16 blocks per 128 columns (room for one partial sum per 8 columns,
 // max_partials), and above CHUNK_MAX_COLS columns, where the columns alone fill the GPU, 4.
@@ -332,7 +332,7 @@ static int residual_planes(int nx, int ny, int nz, bool norm) {
     const int cb = (nx * ny + 127) / 128;
     auto slabs = [&](int p) { return (nz + p - 1) / p; };
     int p = 1;
-    while (p < 4 && cb * slabs(p) > (norm ? 256 : 1024)) ++p;
+    while (p < 4 && cb * slabs(p) > (norm ? 256 : 1024)) p *= 2;
     if (cb * slabs(p) > 1024) p = std::max(4, (nz + 15) / 16);
     return slabs(slabs(p));  // in equal parts
 }
