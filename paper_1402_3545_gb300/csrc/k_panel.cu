@@ -568,9 +568,10 @@ static int panel_point(const PanelLv& L, const double* u, const double* f, TO* o
     dim3 g = panel_grid(L.nx, L.ny);
     int pz = point_planes(L.nx, L.ny, L.nz, (int)(g.x * g.y));
     if (partials) {
-        // as many slabs of planes as max_partials leaves room for, of four planes or more, and below the size that takes 16 at
-        // most 1024 blocks (one block adds the sums up: 138 x 446 x 36 62 us with 5040 of them, 58 with 560)
-        const int blocks = (int)(g.x * g.y), least = std::max(pz, 4);
+        // as many slabs of planes as max_partials leaves room for, of four planes or more unless 256 blocks do with fewer (32 x
+        // 28 x 3 5.4 us with one, 6.4 with three), and below the size that takes 16 at most 1024 blocks (one block adds the
+        // sums up: 138 x 446 x 36 62 us with 5040 of them, 58 with 560)
+        const int blocks = (int)(g.x * g.y), least = blocks * ((L.nz + pz - 1) / pz) <= 256 ? pz : std::max(pz, 4);
         int slabs = std::min((L.nz + least - 1) / least, max_partials(L.nx, L.ny) / blocks);
         if ((size_t)L.nx * L.ny <= 65536) slabs = std::min(slabs, 1024 / blocks);
         slabs = std::max(slabs, 1);
