@@ -507,7 +507,6 @@ static dim3 spmv_march_grid(const Lv<P>& L, int& pz, int& w) {
     // a row's pairs to its warps; folded, in equal parts, where that leaves a quarter of the lanes or more without a pair
     // (FP32 78 x 628 x 203 107 us, 70 folded; 34 x 700 x 16 15.5, 9.7)
     const int pairs = L.nx / 2, parts = (pairs + 31) / 32;
-    w = 4 * pairs > 3 * 32 * parts ? 32 : (pairs + parts - 1) / parts;
     dim3 g(parts, (L.ny + SPMV_TY - 1) / SPMV_TY);
     // SPMV_PZ planes per block, fewer where that leaves a quarter of the SMs without one (with 16 everywhere FP32 32 x 42 x 66
     // took 11.3 us, with the two scalar kernels of a call; 8.8 with a thread per pair of cells; where the SMs are full, more
@@ -515,7 +514,17 @@ static dim3 spmv_march_grid(const Lv<P>& L, int& pz, int& w) {
     // slabs of planes as max_partials leaves room for
     const int cols = (int)(g.x * g.y), room = max_partials(L.nx, L.ny) / cols;
     int nzs = (L.nz + SPMV_PZ - 1) / SPMV_PZ;
-    if (cols * nzs < 114) nzs = std::max(nzs, std::min(L.nz, (152 + cols - 1) / cols));
+    bool fold = 4 * pairs <= 3 * 32 * parts;
+    int from = 114, upto = 152;
+    if (P::id == 1 && fold) {
+        // FP32's folded rows wait longer per plane: fewer planes still, three blocks an SM where there would not be two (88 x
+        // 180 x 45 16.7 us with one, 11.2 with three, 11.9 a row per warp); a row per warp between (88 x 180 x 128 19.0 us, 16.3)
+        from = 2 * 152;
+        upto = 3 * 152;
+        fold = parts == 1 || cols * nzs < from || cols * nzs >= upto;
+    }
+    w = fold ? (pairs + parts - 1) / parts : 32;
+    if (cols * nzs < from) nzs = std::max(nzs, std::min(L.nz, (upto + cols - 1) / cols));
     nzs = std::min(nzs, std::max(room, 1));
     pz = (L.nz + nzs - 1) / nzs;
     g.z = (L.nz + pz - 1) / pz;

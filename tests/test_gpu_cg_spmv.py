@@ -8,7 +8,8 @@ from gpu_common import PREC_IDS, PRECS
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(640, 136, 33), (66, 600, 32), (130, 1200, 17), (200, 96, 5), (34, 700, 33), (78, 131, 17)],
+@pytest.mark.parametrize("shape", [(640, 136, 33), (66, 600, 32), (130, 1200, 17), (200, 96, 5), (34, 700, 33), (78, 131, 17), (88, 180, 45),
+                                   (88, 90, 203)],
                          ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("prec", PRECS, ids=PREC_IDS)
 def test_cg_spmv_matches_oracle(prec, shape):
