@@ -618,9 +618,9 @@ template <class P>
 int launch_line_solve_pp(const Lv<P>& L, const typename P::S* b, typename P::S* x, double scale, const int* done,
                          cudaStream_t s) {
     // FP32, lambda^2 varying: large levels of up to 64 planes on the four-column tile of a warp where it takes them
-    // (512^2 x 16 10.9 us / 11.9, x 48 26.6 / 30.9; x 96 52.8 / 50.9)
+    // (512^2 x 16 10.9 us / 11.9, x 48 26.6 / 30.9; x 96 52.8 / 50.9; 512 x 400 x 48 22.1 / 19.2, 256 x 520 x 48 19.3 / 11.5)
     if constexpr (std::is_same<P, PolF32>::value)
-        if (L.gstack && L.fac_percol && L.nz <= 64 && (size_t)L.nx * L.ny > 131072) {
+        if (L.gstack && L.fac_percol && L.nz <= 64 && (size_t)L.nx * L.ny >= 262144) {
             const int nb = launch_line_solve_x4(L, b, x, scale, done, s);
             if (nb >= 0) return nb;
         }

@@ -23,8 +23,9 @@ def test_fp32_tridiag(shape, lam):
     tiles.test_tile_line_solve_and_tridiag_match_oracle(tpmg.F32, shape, lam)
 
 
-# FP32, lambda^2 varying, above 131072 columns: the four-column tile of a warp up to 64 planes
-@pytest.mark.parametrize("shape", [(512, 256, 17), (512, 260, 17), (512, 260, 64), (512, 260, 65)], ids=ids)
+# FP32, lambda^2 varying, from 262144 columns: the four-column tile of a warp up to 64 planes
+@pytest.mark.parametrize("shape", [(512, 256, 17), (512, 260, 17), (512, 260, 64), (512, 260, 65), (512, 510, 17), (512, 512, 17),
+                                   (512, 516, 64), (512, 516, 65)], ids=ids)
 def test_fp32_line_solve(shape):
     tiles.test_tile_line_solve_and_tridiag_match_oracle(tpmg.F32, shape, None)
 
