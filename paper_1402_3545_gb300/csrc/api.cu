@@ -224,9 +224,9 @@ static size_t elem_bytes(int pid) { return pid == 1 ? 4 : 8; }
 
 static tpmg_status ensure_common(tpmg_op* op) {
     if (!op->partials) {
-        // a half holds any level's sums, and at least 152 x 8: the grid-stride reductions of flexible CG use up to
-        // that many blocks
-        op->max_parts = 152 * 8;
+        // a half holds any level's sums, and at least MIN_PARTIALS: the grid-stride reductions of flexible CG use up to
+        // 152 x 8 blocks
+        op->max_parts = MIN_PARTIALS;
         for (int l = 1; l <= op->g.L; ++l) op->max_parts = std::max(op->max_parts, max_partials(op->g.lnx[l], op->g.lny[l]));
         TRY(dalloc((void**)&op->partials, sizeof(double) * 2 * (size_t)op->max_parts));
     }

@@ -518,8 +518,9 @@ void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw,
 }
 
 // planes per block of the pointwise kernels with `blocks` blocks a plane: 16 where the level fills the GPU with them (8 in
-// the prolongation, whose threads take two fine rows: 896 x 144 x 14 17.0 us, 18.4 with 16 planes), else 4, in equal parts; one or two where that gives at most 1024 blocks (a thread that takes four planes waits for memory
-// four times: 64^2 x 3 prolongation 3.2 us, 2.6 with one)
+// the prolongation, whose threads take two fine rows: 896 x 144 x 14 17.0 us, 18.4 with 16 planes), else 4, in equal
+// parts; one or two where that gives at most 1024 blocks (a thread that takes four planes waits for memory four times:
+// 64^2 x 3 prolongation 3.2 us, 2.6 with one)
 static int point_planes(int nx, int ny, int nz, int blocks, int most = 16) {
     for (int p = 1; p <= 2; ++p)
         if (blocks * ((nz + p - 1) / p) <= 1024) return p;
@@ -569,11 +570,12 @@ static int panel_point(const PanelLv& L, const double* u, const double* f, TO* o
     int pz = point_planes(L.nx, L.ny, L.nz, (int)(g.x * g.y));
     if (partials) {
         // as many slabs of planes as max_partials leaves room for, of four planes or more unless 256 blocks do with fewer (32 x
-        // 28 x 3 5.4 us with one, 6.4 with three), and below the size that takes 16 at most 1024 blocks (one block adds the
-        // sums up: 138 x 446 x 36 62 us with 5040 of them, 58 with 560)
+        // 28 x 3 5.4 us with one, 6.4 with three), and below the size that takes 16 at most MIN_PARTIALS blocks (one block
+        // adds the sums up: 138 x 446 x 36 62 us with 5040 of them, 58 with 560; fewer leave the last round of blocks short: 134
+        // x 258 x 130 119 us with 975, 109 with 1300)
         const int blocks = (int)(g.x * g.y), least = blocks * ((L.nz + pz - 1) / pz) <= 256 ? pz : std::max(pz, 4);
-        int slabs = std::min((L.nz + least - 1) / least, max_partials(L.nx, L.ny) / blocks);
-        if ((size_t)L.nx * L.ny <= 65536) slabs = std::min(slabs, 1024 / blocks);
+        int slabs = std::min((L.nz + least - 1) / least, std::max(max_partials(L.nx, L.ny), MIN_PARTIALS) / blocks);
+        if ((size_t)L.nx * L.ny <= 65536) slabs = std::min(slabs, MIN_PARTIALS / blocks);
         slabs = std::max(slabs, 1);
         pz = (L.nz + slabs - 1) / slabs;
     }

@@ -261,6 +261,7 @@ struct Shape {
 // Thomas stack: two values (forward-eliminated rhs and w_k = v/m_k) per level per thread.
 Shape sweep_shape(int nx, int ny, int nz, int bytes_per_value, bool stack);
 int max_partials(int nx, int ny);
+constexpr int MIN_PARTIALS = 1536;  // room for partial sums that every operator has
 
 // ---------------------------------------------------------------- launchers (k_sweep.cu)
 // Thomas factors of level L into finv/fw (per cell when percol, else a table of nz entries).
