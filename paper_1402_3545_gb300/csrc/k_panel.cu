@@ -517,14 +517,14 @@ void launch_panel_factors(const PanelLv& L, double* inv, double* fl, double* fw,
     note_launch();
 }
 
-// planes per block of the pointwise kernels with `blocks` blocks a plane: 16 where the level fills the GPU with them (8 in
-// the prolongation, whose threads take two fine rows: 896 x 144 x 14 17.0 us, 18.4 with 16 planes), else 4, in equal
-// parts; one or two where that gives at most 1024 blocks (a thread that takes four planes waits for memory four times:
-// 64^2 x 3 prolongation 3.2 us, 2.6 with one)
-static int point_planes(int nx, int ny, int nz, int blocks, int most = 16) {
+// planes per block of the pointwise kernels with `blocks` blocks a plane: 16 where the level fills the GPU with them, else
+// 4, in equal parts, half as many where a thread takes two rows (the prolongation: 896 x 144 x 14 17.0 us, 18.4 with 16
+// planes; 448 x 10 x 77 4.8, 5.4 with four); one or two where that gives at most 1024 blocks (a thread that takes four
+// planes waits for memory four times: 64^2 x 3 prolongation 3.2 us, 2.6 with one)
+static int point_planes(int nx, int ny, int nz, int blocks, int rows = 1) {
     for (int p = 1; p <= 2; ++p)
         if (blocks * ((nz + p - 1) / p) <= 1024) return p;
-    const int p = (size_t)nx * ny > 65536 ? most : 4, slabs = (nz + p - 1) / p;
+    const int p = (size_t)nx * ny > 65536 ? 16 / rows : 4 / rows, slabs = (nz + p - 1) / p;
     return (nz + slabs - 1) / slabs;
 }
 
@@ -622,7 +622,7 @@ void launch_panel_restrict_smooth(const PanelLvT<T>& Lc, double rho, const T* rf
 template <class T>
 void launch_panel_prolongate(int nxc, int nyc, int nz, const T* uc, T* uf, const int* done, cudaStream_t s) {
     dim3 g = panel_grid(2 * nxc, nyc);
-    const int pz = point_planes(2 * nxc, 2 * nyc, nz, (int)(g.x * g.y), 8);
+    const int pz = point_planes(2 * nxc, 2 * nyc, nz, (int)(g.x * g.y), 2);
     g.z = (nz + pz - 1) / pz;
     k_panel_prolongate<T><<<g, dim3(32, 4), 0, s>>>(nxc, nyc, nz, uc, uf, done, pz);
     note_launch();
